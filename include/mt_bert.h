@@ -209,7 +209,9 @@ int mt_poll_status(mt_model* m, void* stream, uint32_t* flags);
  * otherwise room for trunk_layers + max branch_layers + 1 ints). */
 int mt_plan_summary(const mt_model* m, uint64_t task_mask, int32_t* n_layers, int32_t* n_waves,
                     int32_t* trunk_depth, int32_t* groups_per_wave);
-/* Kernel launches one mt_forward at batch = max_batch, seq = max_seq enqueues for this mask. */
+/* Kernel launches one mt_forward at batch = max_batch, seq = max_seq enqueues for this mask.  Before mt_bind_memory the
+ * device is not known and the count is that of the plan without the launches that join several steps of a layer
+ * (option "qkv_attention"). */
 int mt_plan_launches(const mt_model* m, uint64_t task_mask, int32_t* n_launches);
 
 /* Launch plans currently cached (host side; no device access).  mt_forward keeps one plan per distinct
@@ -265,6 +267,10 @@ int mt_plan_cache_size(const mt_model* m);
  * differ in the last bits from the unsplit projection, within every tolerance of the tests; the choice depends on
  * the rows of one layer and on options only, never on the tasks asked for or on how many layers share a launch,
  * so a merged model and its tasks run alone still agree bit for bit.  Not with "fp8_gemm".
+ * key "qkv_attention" (0/1, default 1, any time): with the packed layout, bf16 operands, seq <= 64 and batch x seq >= 256
+ * the layers on all tokens run their Q/K/V projection and attention as one launch, over windows of 128 rows that hold
+ * whole sequences (1), or as two launches (0).  Logits agree to rounding (the keys of a sequence are summed over in
+ * other groups of 16).
  * key "overlap_cls" (0/1, default 1, any time): where a wave holds layers on all tokens and last branch
  * layers, the first-token attention of the latter runs on a stream the library creates for itself (in
  * mt_bind_memory), forked from the caller's stream after the wave's Q/K/V projection and joined before the next

@@ -104,12 +104,15 @@ struct DumpCopy {
   bool compact;  // [B, H]: first tokens only
 };
 // One chunk of a wave: the QKV projection of all its layers in one launch, then the rest of the
-// layer for the layers computed on every token (`full`).  The last layers of task branches are
+// layer for the layers computed on every token (`full`).  With `fused_qkv` the layers on every token have projection
+// and attention in one launch (`qa`), and `qkv` holds the last branch layers only.  The last layers of task branches are
 // needed for the first token of every sequence only: in their wave they get the QKV projection (keys
 // and values of all tokens) and the first-token attention (`attn_cls`, `n_cls` groups); the rest of
 // those layers, a few rows each, is run for all tasks together after the last wave (a `cls tail` step).
 struct Chunk {
   QuantParams q_in;   // 8-bit operands: the layers' inputs, quantised row by row before the Q/K/V projection
+  bool fused_qkv = false;
+  QkvAttnParams qa;
   GemmParams qkv;
   AttnParams attn;
   ClsAttnParams attn_cls;
@@ -230,6 +233,7 @@ struct mt_model {
   bool pack_tokens;  // packed token layout: only valid tokens are stored and computed
   bool cls_only;     // the last layer of a task branch is evaluated for the first token of a sequence only
   int64_t expected_tokens;  // caller's estimate of the valid tokens per batch (0 = every row); tunes tile shapes only
+  bool qkv_attention; // Q/K/V projection and attention of layers on all tokens in one launch where it applies (use_qkv_attention)
   bool attention_tc;  // attention on tcgen05 with tensor-memory accumulators when seq <= 128 (else mma.sync)
   int32_t gemm_pair;  // GEMMs as pairs of CTAs on 256-row tiles (cta_group::2): 0 never, 1 always, 2 by launch size
   bool early_heads;  // every task's head (and first-token tail) runs right after the wave that finishes its branch
@@ -255,7 +259,7 @@ struct mt_model {
   int sm_device, sm_limit;
 
   // workspace layout (byte offsets)
-  size_t ws_status, ws_rows_valid, ws_row_start, ws_tok, ws_seg, ws_len, ws_logits, ws_pooled, ws_partial, ws_trunk[2], ws_task0,
+  size_t ws_status, ws_rows_valid, ws_row_start, ws_windows, ws_row_info, ws_tok, ws_seg, ws_len, ws_logits, ws_pooled, ws_partial, ws_trunk[2], ws_task0,
       ws_slot0, ws_cls0, ws_dump0;
   size_t slot_q_off, cls_q_off;   // 8-bit scratch inside a slot / inside a task's first-token scratch
   size_t cls_bytes, cls_h_bytes, cls_h32_bytes;  // per-task first-token scratch and its [B,H] bf16 / fp32 pieces
@@ -360,6 +364,8 @@ void layout_workspace(mt_model* m) {
   m->ws_status = take(256);
   m->ws_rows_valid = take(256);
   m->ws_row_start = take((static_cast<size_t>(m->max_batch) + 1) * 4);
+  m->ws_windows = take(256 + static_cast<size_t>(m->max_batch) * sizeof(int2));   // the count, then the windows
+  m->ws_row_info = take(M * sizeof(int2));
   m->ws_tok = take(M * 4);
   m->ws_seg = take(M * 4);
   m->ws_len = take(static_cast<size_t>(m->max_batch) * 4);
@@ -508,6 +514,20 @@ int32_t use_pair(const mt_model* m, int64_t rows, int64_t groups) {
   if (m->gemm_pair != 2) return m->gemm_pair;
   return rows * groups >= 12288 ? 1 : 0;
 }
+// Whether the layers on all tokens of a forward have their Q/K/V projection and attention in one launch: packed
+// layout, bf16 operands, sequences of at most 64 tokens, of which a 128-row window holds two or more and is well filled
+// (256 x 16: 1.18 against 1.62 ms per forward; 256 x 64, lengths U[8, 64]: 3.48 against 3.73).  Sequences of 65 to 128 tokens
+// fill windows only when their lengths are nearly equal (256 x 128 full: 10.78 against 11.04 ms; with lengths U[16, 128]
+// 128 x 128 takes 1.6 % longer), and longer ones would project the keys again for every tile of queries.  Below 256
+// rows a launch has too few units (one per window and head) to fill the SMs.
+bool use_qkv_attention(const mt_model* m, int64_t rows, int32_t seq) {
+  return m->qkv_attention && m->d_workspace != nullptr && m->pack_tokens && m->attention_tc && !m->fp8 && seq <= kWindowRows / 2 &&
+         rows >= 256;
+}
+int32_t* window_count(const mt_model* m) { return reinterpret_cast<int32_t*>(m->d_workspace + m->ws_windows); }
+int2* window_list(const mt_model* m) { return reinterpret_cast<int2*>(m->d_workspace + m->ws_windows + 256); }
+int2* row_info(const mt_model* m) { return reinterpret_cast<int2*>(m->d_workspace + m->ws_row_info); }
+
 // Tile width of a grouped GEMM launch (see gemm_block_n).  `rows` are the rows the launch is sized for;
 // with the packed token layout only the valid tokens are in use, and the caller's estimate of their
 // number (option "expected_tokens"), when given, replaces it.
@@ -705,11 +725,15 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   const size_t act = m->act_bytes;
   const size_t qkv_bytes = pad256(static_cast<size_t>(m->max_batch) * m->max_seq * 3 * H * 2);
   const int32_t* row_start = reinterpret_cast<const int32_t*>(m->d_workspace + m->ws_row_start);
+  int32_t n_full = 0;
+  for (size_t i = 0; i < count; ++i) n_full += is_cls_op(m, ops[first + i]) ? 0 : 1;
+  ck->fused_qkv = use_qkv_attention(m, M, seq) && n_full > 0;
+  const int32_t n_qkv = static_cast<int32_t>(count) - (ck->fused_qkv ? n_full : 0);
   memset(&ck->qkv, 0, sizeof(ck->qkv));
-  ck->qkv.n_groups = static_cast<int32_t>(count);
+  ck->qkv.n_groups = n_qkv;
   ck->qkv.M = M; ck->qkv.N = 3 * H; ck->qkv.K = H;
-  ck->qkv.pair = use_pair(m, M, static_cast<int64_t>(count));
-  choose_block_n(m, &ck->qkv, kEpiBias, false, static_cast<int32_t>(count));
+  ck->qkv.pair = use_pair(m, M, n_qkv);
+  choose_block_n(m, &ck->qkv, kEpiBias, false, n_qkv);
   memset(&ck->q_in, 0, sizeof(ck->q_in));
   if (m->fp8) {
     ck->qkv.fp8 = 1;
@@ -722,8 +746,13 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   }
   ck->qkv.m_valid = reinterpret_cast<const int32_t*>(m->d_workspace + m->ws_rows_valid);
   ck->qkv.status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
-  int32_t n_full = 0;
-  for (size_t i = 0; i < count; ++i) n_full += is_cls_op(m, ops[first + i]) ? 0 : 1;
+  memset(&ck->qa, 0, sizeof(ck->qa));
+  ck->qa.heads = m->trunk.heads;
+  ck->qa.max_windows = batch;
+  ck->qa.n_windows = window_count(m);
+  ck->qa.windows = window_list(m);
+  ck->qa.row_info = row_info(m);
+  ck->qa.status = ck->qkv.status;
   init_tail(m, &ck->full, M, false, n_full);
   ck->n_cls = 0;
   memset(&ck->attn, 0, sizeof(ck->attn));
@@ -736,6 +765,7 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   ck->attn.tensor_memory = (m->attention_tc && seq <= kAttnTensorMemoryMaxSeq) ? 1 : 0;
   ck->attn.status = ck->qkv.status;
 
+  int n_qkv_set = 0;
   for (size_t i = 0; i < count; ++i) {
     const OpDesc& op = ops[first + i];
     const LayerOffsets* lo;
@@ -761,25 +791,32 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
     // 1. qkv = in . [Wq;Wk;Wv]^T + [bq;bk;bv] on every token (the three matrices and biases are
     //    contiguous in the arena); keys and values are needed for all tokens even in a `cls` layer
     const QuantScratch qs = m->fp8 ? slot_quant(m, slot) : QuantScratch{};
-    if (m->fp8) {
-      ck->q_in.x[i] = in; ck->q_in.q[i] = qs.xq; ck->q_in.scale[i] = qs.sx;
-      if ((e = set_gemm_group(&ck->qkv, static_cast<int>(i), kEpiBias, qs.xq, m->d_weights + lo->q_qkv, w_ptr(m, lo->bq),
-                              nullptr, qkv)) != cudaSuccess)
-        return e;
-      ck->qkv.group[i].scale_x = qs.sx;
-      ck->qkv.group[i].scale_w = reinterpret_cast<const float*>(m->d_weights + lo->s_qkv);
-    } else if ((e = set_gemm_group(&ck->qkv, static_cast<int>(i), kEpiBias, in, w_ptr(m, lo->wq), w_ptr(m, lo->bq), nullptr,
-                                   qkv)) != cudaSuccess) {
-      return e;
-    }
     const bool cls = is_cls_op(m, op);
+    if (m->fp8) { ck->q_in.x[i] = in; ck->q_in.q[i] = qs.xq; ck->q_in.scale[i] = qs.sx; }
+    const void* x_op = m->fp8 ? static_cast<const void*>(qs.xq) : in;   // the projection's operands
+    const void* w_op = m->fp8 ? static_cast<const void*>(m->d_weights + lo->q_qkv) : w_ptr(m, lo->wq);
+    const float* w_scale = m->fp8 ? reinterpret_cast<const float*>(m->d_weights + lo->s_qkv) : nullptr;
+    if (ck->fused_qkv && !cls) {
+      const int a = ck->qa.n_groups;
+      if ((e = make_tmap(&ck->qa.tmap_x[a], x_op, M, H, 64, 64, false)) != cudaSuccess ||
+          (e = make_tmap(&ck->qa.tmap_w[a], w_op, 3 * H, H, 64, 64, false)) != cudaSuccess)
+        return e;
+      ck->qa.bias[a] = w_ptr(m, lo->bq);
+      ck->qa.ctx[a] = ctx;
+      ck->qa.n_groups = a + 1;
+    } else {
+      const int a = n_qkv_set++;
+      if ((e = set_gemm_group(&ck->qkv, a, kEpiBias, x_op, w_op, w_ptr(m, lo->bq), nullptr, qkv)) != cudaSuccess) return e;
+      ck->qkv.group[a].scale_x = qs.sx;
+      ck->qkv.group[a].scale_w = w_scale;
+    }
     if (!cls) {
       // 2. ctx = attention(qkv) for every token; 3-7 on every token
       const int a = ck->full.count;
       ck->attn.qkv[a] = qkv;
       ck->attn.ctx[a] = ctx;
       ck->attn.n_groups = a + 1;
-      if (ck->attn.tensor_memory &&
+      if (!ck->fused_qkv && ck->attn.tensor_memory &&
           ((e = make_tmap(&ck->attn.tmap_qkv[a], qkv, M, 3 * H, kAttnTileRows, kHeadDim, false)) != cudaSuccess ||
            (e = make_tmap(&ck->attn.tmap_qkv64[a], qkv, M, 3 * H, kAttnTileRows / 2, kHeadDim, false)) != cudaSuccess))
         return e;
@@ -826,10 +863,13 @@ cudaError_t build_cls_tail(const mt_model* m, const std::vector<int32_t>& tasks,
   return cudaSuccess;
 }
 
-int32_t chunk_launches(const mt_model* m, const std::vector<OpDesc>& ops, size_t first, size_t count, int64_t rows) {
+int32_t chunk_launches(const mt_model* m, const std::vector<OpDesc>& ops, size_t first, size_t count, int64_t rows,
+                       int32_t seq) {
   size_t n_cls = 0;
   for (size_t i = 0; i < count; ++i) n_cls += is_cls_op(m, ops[first + i]) ? 1 : 0;
-  return 1 + (m->fp8 ? 1 : 0) + (n_cls < count ? 1 + tail_launches(m, static_cast<int32_t>(count - n_cls), rows) : 0) +
+  // (projection and attention in one launch: the projection of its own serves the last branch layers only)
+  const bool fused = use_qkv_attention(m, rows, seq) && n_cls < count;
+  return (fused && n_cls == 0 ? 0 : 1) + (m->fp8 ? 1 : 0) + (n_cls < count ? 1 + tail_launches(m, static_cast<int32_t>(count - n_cls), rows) : 0) +
          (n_cls > 0 ? 1 : 0);
 }
 // Active tasks whose last branch layer is finished on first tokens right after wave w (1-based):
@@ -886,8 +926,9 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
         ht.compact = compact ? 1 : 0;
         st.head_tasks.push_back(t);
         if (st.pool_gemm) {
-          cudaError_t e = set_gemm_group(&st.pool, static_cast<int>(i), kEpiBiasTanhF32, ht.hidden, ht.pool_w, ht.pool_b,
-                                         nullptr, st.heads.pooled + i * static_cast<size_t>(batch) * m->trunk.hidden);
+          float* pooled = st.heads.pooled + i * static_cast<size_t>(batch) * m->trunk.hidden;
+          cudaError_t e = set_gemm_group(&st.pool, static_cast<int>(i), kEpiBiasTanhF32, ht.hidden, ht.pool_w,
+                                                          ht.pool_b, nullptr, pooled);
           if (e != cudaSuccess) heads_error = e;
         }
       }
@@ -937,7 +978,7 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
       cudaError_t e = build_chunk(m, ops, first, count, batch, seq, &st.chunk);
       if (e != cudaSuccess) return e;
       plan->steps.push_back(std::move(st));
-      plan->launches += chunk_launches(m, ops, first, count, static_cast<int64_t>(batch) * seq);
+      plan->launches += chunk_launches(m, ops, first, count, static_cast<int64_t>(batch) * seq, seq);
     }
     {
       // first-token tails: of the tasks finishing in this wave (early_heads), or of all tasks after the last wave
@@ -996,6 +1037,7 @@ int mt_create(const mt_trunk_config* trunk, const mt_task_config* tasks, int32_t
   m->cls_only = true;
   m->early_heads = false;
   m->gemm_pair = 2;
+  m->qkv_attention = true;
   m->attention_tc = true;
   m->expected_tokens = 0;
   m->pool_gemm = true;
@@ -1136,6 +1178,11 @@ int mt_set_option(mt_model* m, const char* key, int64_t value) {
   }
   if (strcmp(key, "pool_gemm") == 0) {
     m->pool_gemm = value != 0;
+    m->plans.clear();
+    return MT_OK;
+  }
+  if (strcmp(key, "qkv_attention") == 0) {
+    m->qkv_attention = value != 0;
     m->plans.clear();
     return MT_OK;
   }
@@ -1323,7 +1370,7 @@ int mt_plan_launches(const mt_model* m, uint64_t task_mask, int32_t* n_launches)
       const std::vector<OpDesc>& ops = s.waves[w - 1];
       for (size_t first = 0; first < ops.size(); first += m->n_slots)
         n += chunk_launches(m, ops, first, std::min<size_t>(m->n_slots, ops.size() - first),
-                            static_cast<int64_t>(m->max_batch) * m->max_seq);
+                            static_cast<int64_t>(m->max_batch) * m->max_seq, m->max_seq);
       const size_t n_cls_tasks = cls_tasks_after_wave(m, s, w).size();
       for (size_t first = 0; first < n_cls_tasks; first += kMaxGroups)
         n += tail_launches(m, static_cast<int32_t>(std::min<size_t>(kMaxGroups, n_cls_tasks - first)), m->max_batch);
@@ -1450,11 +1497,14 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
   } while (0)
 
   int32_t* row_start = reinterpret_cast<int32_t*>(m->d_workspace + m->ws_row_start);
+  const bool fused_qkv = use_qkv_attention(m, static_cast<int64_t>(batch) * seq, seq);
   MT_LAUNCH(launch_row_starts(d_lengths, batch, seq, m->pack_tokens ? 1 : 0, row_start,
-                              reinterpret_cast<int32_t*>(m->d_workspace + m->ws_rows_valid), stream),
+                              reinterpret_cast<int32_t*>(m->d_workspace + m->ws_rows_valid), fused_qkv ? window_count(m) : nullptr,
+                              fused_qkv ? window_list(m) : nullptr, stream),
             "row-start kernel");
   EmbedParams ep;
   ep.row_start = row_start;
+  ep.row_info = fused_qkv ? row_info(m) : nullptr;
   ep.packed = m->pack_tokens ? 1 : 0;
   ep.token_ids = d_token_ids; ep.segment_ids = d_segment_ids; ep.lengths = d_lengths;
   ep.word = w_ptr(m, m->emb_word); ep.pos = w_ptr(m, m->emb_pos); ep.type = w_ptr(m, m->emb_type);
@@ -1479,7 +1529,10 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
       ck.attn.lengths = d_lengths;
       ck.attn_cls.lengths = d_lengths;
       if (m->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(ck.q_in, stream), "quantising the layer inputs");
-      MT_TIMED(MT_CLASS_QKV, launch_gemm(ck.qkv, kEpiBias, m->sm_count, stream), "QKV GEMM");
+      if (ck.fused_qkv)
+        MT_TIMED(MT_CLASS_QKV, launch_qkv_attention(ck.qa, m->sm_count, stream), "QKV projection + attention kernel");
+      if (ck.qkv.n_groups > 0)
+        MT_TIMED(MT_CLASS_QKV, launch_gemm(ck.qkv, kEpiBias, m->sm_count, stream), "QKV GEMM");
       const bool beside = m->overlap_cls && m->side_stream != nullptr && !m->profile && ck.n_cls > 0 && ck.full.count > 0;
       if (beside) {
         MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
@@ -1488,7 +1541,7 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
         MT_LAUNCH(cudaEventRecord(m->ev_join, m->side_stream), "joining the side stream");
         side_pending = true;
       }
-      if (ck.full.count > 0) MT_TIMED(MT_CLASS_ATTENTION, launch_attention(ck.attn, stream), "attention kernel");
+      if (ck.full.count > 0 && !ck.fused_qkv) MT_TIMED(MT_CLASS_ATTENTION, launch_attention(ck.attn, stream), "attention kernel");
       if (ck.n_cls > 0 && !beside)
         MT_TIMED(MT_CLASS_ATTENTION, launch_cls_attention(ck.attn_cls, stream), "first-token attention kernel");
       if (ck.full.count > 0) MT_TAIL(&ck.full);
@@ -1814,6 +1867,7 @@ int mt_kernel_embed(const int32_t* d_token_ids, const int32_t* d_segment_ids, co
   p.batch = batch; p.seq = seq; p.hidden = hidden; p.vocab = vocab; p.type_vocab = type_vocab; p.eps = eps;
   p.status = d_status;
   p.row_start = nullptr;
+  p.row_info = nullptr;
   p.packed = 0;
   return launch_embed(p, as_stream(stream)) == cudaSuccess ? MT_OK : MT_ERR_CUDA;
 }

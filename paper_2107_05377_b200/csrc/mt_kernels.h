@@ -156,6 +156,23 @@ constexpr int kAttnTileRows = 128;   // rows of the Q/K/V boxes of the tensor ma
 cudaError_t launch_attention(const AttnParams& p, cudaStream_t stream);
 cudaError_t launch_attention_tc(const AttnParams& p, cudaStream_t stream);
 
+// Q/K/V projection and attention in one launch (qkv_attention_tcgen05): sequences of at most 128 tokens in the packed
+// layout.  Work is dealt out over windows - runs of whole consecutive sequences that fit in 128 rows - built on the
+// device by launch_row_starts; row_info tells every row which rows are its own sequence.
+struct alignas(64) QkvAttnParams {
+  CUtensorMap tmap_x[kMaxGroups];      // layer input: dims {H, rows}, box {64, 64}
+  CUtensorMap tmap_w[kMaxGroups];      // [Wq; Wk; Wv]: dims {H, 3H}, box {64, 64}
+  const bf16* bias[kMaxGroups];        // [3H]
+  bf16* ctx[kMaxGroups];               // [rows, H]
+  const int32_t* n_windows;            // device scalar
+  const int2* windows;                 // device: {first row, rows} of every window
+  const int2* row_info;                // device: {first row, row after the last} of the sequence a row belongs to
+  int32_t n_groups, heads, max_windows;
+  uint32_t* status;
+};
+constexpr int kWindowRows = 128;       // rows of a window = longest sequence this kernel takes
+cudaError_t launch_qkv_attention(const QkvAttnParams& p, int sm_count, cudaStream_t stream);
+
 // Attention of the first token of every sequence only (the last layer of a task branch: its head
 // reads nothing but that row).  Writes the context compactly, ctx[b, :], and gathers the fp32
 // residual of that row from the layer input, res[b, :] = in32[row_start[b], :].
@@ -229,6 +246,7 @@ struct EmbedParams {
   bf16* out;
   float* out32;  // may be null
   const int32_t* row_start;  // [B + 1] or null (padded layout)
+  int2* row_info;            // null, or (packed layout) {first row, row after the last} of the row's sequence, per row
   int32_t packed;            // 1: positions >= length are skipped
   int32_t batch, seq, hidden, vocab, type_vocab;
   float eps;
@@ -282,9 +300,11 @@ cudaError_t launch_wait_probe(unsigned long long limit_ns, int arrive, uint32_t*
                               int* ok_out, cudaStream_t stream);
 
 // row_start[b] for b = 0..batch and *rows_valid = row_start[batch]: b * seq (padded) or the running sum
-// of the lengths clamped to [1, seq] (packed).
+// of the lengths clamped to [1, seq] (packed).  With windows != null (packed, seq <= kWindowRows) also the windows of
+// qkv_attention_tcgen05: *n_windows <= batch runs of consecutive sequences, each filled until the next sequence would
+// not fit in kWindowRows rows.
 cudaError_t launch_row_starts(const int32_t* lengths, int32_t batch, int32_t seq, int32_t packed, int32_t* row_start,
-                              int32_t* rows_valid, cudaStream_t stream);
+                              int32_t* rows_valid, int32_t* n_windows, int2* windows, cudaStream_t stream);
 // padded[b*seq + pos] = packed[row_start[b] + pos] for pos < length, 0 elsewhere (bf16 rows of `hidden`).
 // With compact != 0 the source is [B, H] (first tokens only) and only position 0 of a sequence is filled.
 cudaError_t launch_unpack_rows(const bf16* packed, const int32_t* lengths, const int32_t* row_start, bf16* padded,

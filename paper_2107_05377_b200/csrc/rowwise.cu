@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(kRowThreads) embed_kernel(const EmbedParams p)
     len = len < 1 ? 1 : (len > p.seq ? p.seq : len);
     if (p.packed && pos >= len) return;  // packed layout: padded positions do not exist
     out_row = p.row_start[b] + pos;
+    if (p.row_info != nullptr && lane == 0) p.row_info[out_row] = make_int2(out_row - pos, out_row - pos + len);
   }
   const bf16* w = p.word + static_cast<size_t>(tok) * H;
   const bf16* q = p.pos + static_cast<size_t>(pos) * H;
@@ -273,13 +274,15 @@ __global__ void __launch_bounds__(kRowThreads) quantize_rows_kernel(const QuantP
   }
 }
 
-// One warp: inclusive scan of the clamped lengths in chunks of 32.
+// One warp: inclusive scan of the clamped lengths in chunks of 32, and the windows (next fit: a window is closed by the
+// first sequence that would not fit in kWindowRows rows; a ballot finds it, one step per window).
 __global__ void row_starts_kernel(const int32_t* lengths, int32_t batch, int32_t seq, int32_t packed,
-                                  int32_t* row_start, int32_t* rows_valid) {
+                                  int32_t* row_start, int32_t* rows_valid, int32_t* n_windows, int2* windows) {
   const int lane = threadIdx.x;
   grid_dependency_wait();
   grid_launch_dependents();
   int carry = 0;
+  int win_first = 0, win_count = 0;   // first row of the open window, windows closed so far
   for (int base = 0; base < batch; base += 32) {
     const int b = base + lane;
     int n = 0;
@@ -297,11 +300,26 @@ __global__ void row_starts_kernel(const int32_t* lengths, int32_t batch, int32_t
       if (lane >= o) incl += up;
     }
     if (b < batch) row_start[b] = carry + incl - n;
+    if (windows != nullptr) {
+      // (lanes past the batch end where the last sequence does: they close nothing that it does not)
+      for (;;) {
+        const unsigned over = __ballot_sync(0xffffffffu, carry + incl - win_first > kWindowRows);
+        if (over == 0) break;
+        const int next = __shfl_sync(0xffffffffu, carry + incl - n, __ffs(over) - 1);   // where that sequence starts
+        if (lane == 0) windows[win_count] = make_int2(win_first, next - win_first);
+        ++win_count;
+        win_first = next;
+      }
+    }
     carry += __shfl_sync(0xffffffffu, incl, 31);
   }
   if (lane == 0) {
     row_start[batch] = carry;
     *rows_valid = carry;
+    if (windows != nullptr) {
+      windows[win_count] = make_int2(win_first, carry - win_first);   // (the last sequence is always in the open one)
+      *n_windows = win_count + 1;
+    }
   }
 }
 
@@ -332,9 +350,10 @@ cudaError_t launch_quantize_rows(const QuantParams& p, cudaStream_t stream) {
 }
 
 cudaError_t launch_row_starts(const int32_t* lengths, int32_t batch, int32_t seq, int32_t packed, int32_t* row_start,
-                              int32_t* rows_valid, cudaStream_t stream) {
-  if (batch < 1 || seq < 1) return cudaErrorInvalidValue;
-  row_starts_kernel<<<1, 32, 0, stream>>>(lengths, batch, seq, packed, row_start, rows_valid);
+                              int32_t* rows_valid, int32_t* n_windows, int2* windows, cudaStream_t stream) {
+  if (batch < 1 || seq < 1 || (windows != nullptr && (n_windows == nullptr || packed == 0 || seq > kWindowRows)))
+    return cudaErrorInvalidValue;
+  row_starts_kernel<<<1, 32, 0, stream>>>(lengths, batch, seq, packed, row_start, rows_valid, n_windows, windows);
   return cudaGetLastError();
 }
 
