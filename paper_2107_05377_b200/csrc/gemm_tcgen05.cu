@@ -481,8 +481,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
         }
         fence_async_shared();
         __syncwarp();
-        if (lane == 0 && rows_in_range) {
-          tma_store_2d(&p.tmap_out[g], my_stage + buf * kStagingBytes, col, out_row0);
+        if (lane == 0) {
+          // (a group per chunk even where nothing is stored: the waits above count groups to know which buffer is free)
+          if (rows_in_range) tma_store_2d(&p.tmap_out[g], my_stage + buf * kStagingBytes, col, out_row0);
           tma_store_commit();
         }
         ++n_done;
