@@ -44,20 +44,29 @@ constexpr int kStagingBytes = 4096;  // 32 rows x 128 bytes, one epilogue chunk 
 #endif
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kBookBytes = 512 + 1024;   // barriers/bookkeeping + slack for manual 1024-byte alignment
-__host__ __device__ constexpr int gemm_a_bytes() { return kGemmBlockM * kGemmBlockK * 2; }
+// LOW = 64 or 32: tiles of that many rows and 64 columns (launches of few rows; 0: the full 128).  The MMA still covers 128
+// rows, of which the others are whatever follows in shared memory; their rows of the accumulator are never read.
+// Their stages hold kGemmLowKBlocks k-blocks, fetched by one copy each (three-dimensional tensor maps).
+__host__ __device__ constexpr int gemm_a_bytes(int low = 0) {
+  return (low ? low * kGemmLowKBlocks : kGemmBlockM) * kGemmBlockK * 2;
+}
 // A CTA of a pair stages only its half of the W tile.
-__host__ __device__ constexpr int gemm_b_bytes(int bn, bool pair) { return (pair ? bn / 2 : bn) * kGemmBlockK * 2; }
+__host__ __device__ constexpr int gemm_b_bytes(int bn, bool pair, int low = 0) {
+  return (pair ? bn / 2 : bn) * kGemmBlockK * 2 * (low ? kGemmLowKBlocks : 1);
+}
 __host__ __device__ constexpr int gemm_staging_bufs(int bn, bool pair, int epi) {
   return epi == kEpiBiasResidual ? 2 : ((bn == 256 && !pair) ? 1 : MT_GEMM_NBUF);
 }
-__host__ __device__ constexpr int gemm_stages(int bn, bool pair, int epi) {
-  const int room = kSmemLimit - kBookBytes - kNumEpilogueWarps * gemm_staging_bufs(bn, pair, epi) * kStagingBytes;
-  const int s = room / (gemm_a_bytes() + gemm_b_bytes(bn, pair));
+// Epilogue warps with rows to work on: all eight, or (LOW) those whose quarter of tensor memory the tile's rows reach.
+__host__ __device__ constexpr int gemm_staging_warps(int low) { return low ? kNumEpilogueWarps / 4 * (low / 32) : kNumEpilogueWarps; }
+__host__ __device__ constexpr int gemm_stages(int bn, bool pair, int epi, int low = 0) {
+  const int room = kSmemLimit - kBookBytes - gemm_staging_warps(low) * gemm_staging_bufs(bn, pair, epi) * kStagingBytes;
+  const int s = room / (gemm_a_bytes(low) + gemm_b_bytes(bn, pair, low));
   return s > 8 ? 8 : s;
 }
-__host__ __device__ constexpr int gemm_smem_bytes(int bn, bool pair, int epi) {
-  return gemm_stages(bn, pair, epi) * (gemm_a_bytes() + gemm_b_bytes(bn, pair)) +
-         kNumEpilogueWarps * gemm_staging_bufs(bn, pair, epi) * kStagingBytes + kBookBytes;
+__host__ __device__ constexpr int gemm_smem_bytes(int bn, bool pair, int epi, int low = 0) {
+  return gemm_stages(bn, pair, epi, low) * (gemm_a_bytes(low) + gemm_b_bytes(bn, pair, low)) +
+         gemm_staging_warps(low) * gemm_staging_bufs(bn, pair, epi) * kStagingBytes + kBookBytes;
 }
 
 // ---- the kernel -------------------------------------------------------------------------------
@@ -70,15 +79,27 @@ __host__ __device__ constexpr int gemm_smem_bytes(int bn, bool pair, int epi) {
 // FP8: the operands are E4M3 bytes with one fp32 scale per row of X and per row of W (GemmParams::scale_x,
 // scale_w); a shared-memory row of 128 bytes then holds 128 elements of K, an instruction covers 32 of them,
 // and the epilogue multiplies the accumulator by scale_x[row] * scale_w[column] before the bias.
-template <int BN, int EPI, bool PAIR, bool FP8 = false>
+// LOW: tiles of 64 or 32 rows and 64 columns.  A launch of one or two row blocks is a chain of latencies: with 16 (12) KB a
+// k-block all twelve of K = 768 fit in the ring, so the whole operands are asked for at once; a stage is four k-blocks, so
+// that a copy, a wait and a commit are paid for three times and not twelve (each costs the issuing warp 100 to 200 clocks);
+// more CTAs share the launch; and X, which comes in at about 30 bytes per clock and CTA once the previous kernel has
+// ended (32 KB after 1.15 us, 96 KB after 2.3), is a half or a quarter of the full tile's.  128 rows of the eight-task tree:
+// accumulator complete 2.8 us after the dependency wait against 3.3 with 128-row tiles of the same width, results bf16
+// 0.6 us later (straight from registers) against 1.1 to 1.7.
+template <int BN, int EPI, bool PAIR, bool FP8 = false, int LOW = 0>
 __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __grid_constant__ GemmParams p) {
   static_assert(!FP8 || !PAIR, "the 8-bit operands run as single CTAs");
   constexpr int KB_ELEMS = FP8 ? 2 * kGemmBlockK : kGemmBlockK;   // elements of K in a 128-byte row
-  constexpr int STAGES = gemm_stages(BN, PAIR, EPI);
-  constexpr int A_BYTES = gemm_a_bytes();
-  constexpr int B_BYTES = gemm_b_bytes(BN, PAIR);   // this CTA's part of the W tile
+  static_assert(LOW == 0 || LOW == 64 || LOW == 32, "tile heights implemented: 128, 64, 32");
+  static_assert(LOW == 0 || (BN == 64 && !PAIR && !FP8), "low tiles: 64 columns, single CTAs, bf16");
+  constexpr int STAGES = gemm_stages(BN, PAIR, EPI, LOW);
+  constexpr int A_BYTES = gemm_a_bytes(LOW);
+  constexpr int KPS = LOW ? kGemmLowKBlocks : 1;         // k-blocks of a stage
+  constexpr int B_BYTES = gemm_b_bytes(BN, PAIR, LOW);   // this CTA's part of the W tile
   constexpr int NBUF = gemm_staging_bufs(BN, PAIR, EPI);
-  constexpr int TILE_M = PAIR ? 2 * kGemmBlockM : kGemmBlockM;
+  constexpr int TILE_M = PAIR ? 2 * kGemmBlockM : (LOW ? LOW : kGemmBlockM);
+  constexpr int MMA_M = LOW ? kGemmBlockM : TILE_M;
+  constexpr int STAGING_WARPS = gemm_staging_warps(LOW);
   constexpr int ACC_ARRIVALS = PAIR ? 2 * kNumEpilogueWarps : kNumEpilogueWarps;
   constexpr uint32_t TMEM_COLS = BN == 64 ? 128 : (BN == 128 ? 256 : 512);  // two accumulators; a power of two >= 32
   static_assert(BN == 64 || BN == 128 || BN == 192 || BN == 256, "tile widths implemented: 64, 128, 192, 256");
@@ -90,7 +111,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
   const uint32_t sA = smem_u32(smem);
   const uint32_t sB = sA + STAGES * A_BYTES;
   const uint32_t sStage = sB + STAGES * B_BYTES;          // kNumEpilogueWarps x NBUF x 4 KB
-  uint8_t* book = smem + STAGES * (A_BYTES + B_BYTES) + kNumEpilogueWarps * NBUF * kStagingBytes;
+  uint8_t* book = smem + STAGES * (A_BYTES + B_BYTES) + STAGING_WARPS * NBUF * kStagingBytes;
   const uint32_t bar_full = smem_u32(book);               // STAGES x 8 bytes
   const uint32_t bar_empty = bar_full + 8 * STAGES;       // STAGES x 8 bytes
   const uint32_t bar_acc_full = bar_empty + 8 * STAGES;   // 2 x 8 bytes
@@ -107,7 +128,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
 
   const int n_tiles_n = p.N / BN;
   const int k_splits = p.k_splits > 1 ? p.k_splits : 1;   // ranges of K (> 1 only with the partial-sum epilogue)
-  const int k_blocks = p.K / KB_ELEMS / k_splits;         // k-blocks of one tile
+  const int k_blocks = p.K / KB_ELEMS / KPS / k_splits;   // k-blocks (LOW: stages of KPS k-blocks) of one tile
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -161,7 +182,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
           tma_load_2d_pair(sB + s * B_BYTES, &p.tmap_w[g], (kb0 + s) * KB_ELEMS, n0, bar_full_count + 8 * s);
         } else {
           mbar_add_tx(bar_full + 8 * s, B_BYTES);
-          tma_load_2d(sB + s * B_BYTES, &p.tmap_w[g], (kb0 + s) * KB_ELEMS, n0, bar_full + 8 * s);
+          if (LOW) tma_load_3d(sB + s * B_BYTES, &p.tmap_w[g], 0, n0, (kb0 + s) * KPS, bar_full + 8 * s);
+          else tma_load_2d(sB + s * B_BYTES, &p.tmap_w[g], (kb0 + s) * KB_ELEMS, n0, bar_full + 8 * s);
         }
       }
     }
@@ -218,9 +240,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
               tma_load_2d_pair(sB + stage * B_BYTES, &p.tmap_w[g], (kb0 + kb) * KB_ELEMS, n0, bar_full_count + 8 * stage);
           } else {
             mbar_expect_tx(bar_full + 8 * stage, A_BYTES + (w_on_its_way ? 0 : B_BYTES));
-            tma_load_2d(sA + stage * A_BYTES, &p.tmap_x[g], (kb0 + kb) * KB_ELEMS, m0, bar_full + 8 * stage);
-            if (!w_on_its_way)
-              tma_load_2d(sB + stage * B_BYTES, &p.tmap_w[g], (kb0 + kb) * KB_ELEMS, n0, bar_full + 8 * stage);
+            if (LOW) tma_load_3d(sA + stage * A_BYTES, &p.tmap_x[g], 0, m0, (kb0 + kb) * KPS, bar_full + 8 * stage);
+            else tma_load_2d(sA + stage * A_BYTES, &p.tmap_x[g], (kb0 + kb) * KB_ELEMS, m0, bar_full + 8 * stage);
+            if (!w_on_its_way) {
+              if (LOW) tma_load_3d(sB + stage * B_BYTES, &p.tmap_w[g], 0, n0, (kb0 + kb) * KPS, bar_full + 8 * stage);
+              else tma_load_2d(sB + stage * B_BYTES, &p.tmap_w[g], (kb0 + kb) * KB_ELEMS, n0, bar_full + 8 * stage);
+            }
           }
           ++issued;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -248,7 +273,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
     // The whole warp walks the loop and waits on the barriers (it stays converged); the elected lane issues.
     const bool leader = elect_one();
     if (rank == 0) {
-      constexpr uint32_t idesc = FP8 ? umma_idesc_e4m3(TILE_M, BN) : umma_idesc_bf16(TILE_M, BN);
+      constexpr uint32_t idesc = FP8 ? umma_idesc_e4m3(MMA_M, BN) : umma_idesc_bf16(MMA_M, BN);
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
@@ -263,14 +288,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
           if (!mbar_wait(bar_full + 8 * stage, phase, abort_flag)) { ok = false; break; }
           tc_fence_after();
           if (leader) {
-            const uint64_t da = smem_desc_sw128(sA + stage * A_BYTES);
-            const uint64_t db = smem_desc_sw128(sB + stage * B_BYTES);
 #pragma unroll
-            for (int k = 0; k < kGemmBlockK / 16; ++k) {
+            for (int i = 0; i < KPS * (kGemmBlockK / 16); ++i) {
+              constexpr int PER_KB = kGemmBlockK / 16;
+              const int k = i % PER_KB;
+              const uint64_t da = smem_desc_sw128(sA + stage * A_BYTES + i / PER_KB * (A_BYTES / KPS));
+              const uint64_t db = smem_desc_sw128(sB + stage * B_BYTES + i / PER_KB * (B_BYTES / KPS));
               // advancing one instruction along K (16 bf16 or 32 E4M3 = 32 bytes) inside the swizzled row: +2 in the address field
-              if (FP8) umma_e4m3(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
-              else if (PAIR) umma_bf16_pair(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
-              else umma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+              if (FP8) umma_e4m3(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | i) != 0 ? 1u : 0u);
+              else if (PAIR) umma_bf16_pair(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | i) != 0 ? 1u : 0u);
+              else umma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | i) != 0 ? 1u : 0u);
             }
             if (PAIR) umma_commit_pair(bar_empty + 8 * stage); else umma_commit(bar_empty + 8 * stage);
           }
@@ -291,11 +318,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
     const int quarter = warp & 3;                       // TMEM lanes this warp may read
     const int col_group = e >> 2;                       // which share of the column chunks
     constexpr int COL_GROUPS = kNumEpilogueWarps / 4;
-    constexpr int CHUNK_COLS = (EPI == kEpiBiasResidual || EPI == kEpiBiasTanhF32 || EPI == kEpiPartialF32) ? 32 : 64;
+    constexpr int CHUNK_COLS = (LOW || EPI == kEpiBiasResidual || EPI == kEpiBiasTanhF32 || EPI == kEpiPartialF32) ? 32 : 64;
     constexpr int CHUNKS = BN / CHUNK_COLS;
-    const uint32_t my_stage = sStage + static_cast<uint32_t>(e * NBUF * kStagingBytes);
+    const bool has_rows = LOW == 0 || quarter < LOW / 32;                // (LOW) the others only keep the barriers' counts
+    const int slot = LOW ? col_group * (LOW / 32) + quarter : e;         // (not used without rows)
+    const uint32_t my_stage = sStage + static_cast<uint32_t>(slot * NBUF * kStagingBytes);
     const uint32_t my_res_bar = bar_res + 16 * e;       // two barriers, one per staging buffer
-    uint8_t* my_stage_ptr = smem + STAGES * (A_BYTES + B_BYTES) + e * NBUF * kStagingBytes;
+    uint8_t* my_stage_ptr = smem + STAGES * (A_BYTES + B_BYTES) + slot * NBUF * kStagingBytes;
     int acc = 0;
     uint32_t acc_phase = 0;
     int buf = 0;                  // staging buffer of the next chunk
@@ -319,7 +348,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
     // its present chunk has read it, so up to two requests are kept in flight: both chunks of a 128-wide tile
     // are asked for before the tile's main loop ends (at the kernel's start for a CTA's first tile) instead of
     // the second one only when the first is being worked on.
-    int req_tile = worker, req_chunk = col_group;   // the next chunk to ask for
+    int req_tile = has_rows ? worker : total_tiles, req_chunk = col_group;   // the next chunk to ask for
     int n_req = 0, n_done = 0;                      // chunks asked for / chunks whose store has been issued
     auto refill = [&]() {
       while (n_req < n_done + 2 && req_tile < total_tiles) {
@@ -341,6 +370,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
       const int n0 = (rem - g * n_tiles_n) * BN;
       // (partial sums) the tile's range of K writes its own rows of the output
       const int out_row0 = m0 + quarter * 32 + (EPI == kEpiPartialF32 ? (rem_s % k_splits) * p.split_pitch : 0);
+      // (LOW) the tile's bias - this warp has one chunk of 32 columns - is on its way while the MMAs run
+      uint4 low_bias[LOW ? 4 : 1];
+      if (LOW && EPI != kEpiPartialF32 && has_rows) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          low_bias[LOW ? q : 0] = __ldg(reinterpret_cast<const uint4*>(p.group[g].bias + n0 + col_group * 32) + q);
+      }
       // warp-uniform decisions: the TMEM loads below are warp-collective
       if (!__all_sync(0xffffffffu, mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag))) break;
       tc_fence_after();
@@ -354,7 +390,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
         col_scale = p.group[g].scale_w;
       }
 #pragma unroll 1
-      for (int chunk = col_group; chunk < CHUNKS; chunk += COL_GROUPS) {
+      for (int chunk = has_rows ? col_group : CHUNKS; chunk < CHUNKS; chunk += COL_GROUPS) {
         const int col = n0 + chunk * CHUNK_COLS;
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
                                static_cast<uint32_t>(acc * BN + chunk * CHUNK_COLS);
@@ -384,7 +420,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
           const uint4* bias4 = reinterpret_cast<const uint4*>(bias + col);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const uint4 b = __ldg(bias4 + q);
+            const uint4 b = LOW ? low_bias[LOW ? q : 0] : __ldg(bias4 + q);
             const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
             float4* s0 = reinterpret_cast<float4*>(sbuf + staging_off(lane, 2 * q));
             float4* s1 = reinterpret_cast<float4*>(sbuf + staging_off(lane, 2 * q + 1));
@@ -424,7 +460,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
           const uint4* bias4 = reinterpret_cast<const uint4*>(bias + col);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const uint4 b = __ldg(bias4 + q);
+            const uint4 b = LOW ? low_bias[LOW ? q : 0] : __ldg(bias4 + q);
             const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
             float4 r0, r1;
             r0.x = tanhf(__uint_as_float(v[q * 8 + 0]) + bf16_lo(bw[0]));
@@ -438,6 +474,31 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
             *reinterpret_cast<float4*>(sbuf + staging_off(lane, 2 * q)) = r0;
             *reinterpret_cast<float4*>(sbuf + staging_off(lane, 2 * q + 1)) = r1;
           }
+        } else if (LOW) {
+          // bf16 results of few rows: 32 columns per thread (every warp with rows has some), straight from registers
+          uint32_t v[32];
+          tmem_ld_32x32(taddr, v);
+          tmem_ld_wait();
+          const int row = m0 + quarter * 32 + lane;
+          bf16* out = static_cast<bf16*>(p.group[g].out) + static_cast<size_t>(row) * p.N + col;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint4 b = low_bias[LOW ? q : 0];
+            const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
+            uint32_t ow[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              float x0 = __uint_as_float(v[q * 8 + 2 * j]) + bf16_lo(bw[j]);
+              float x1 = __uint_as_float(v[q * 8 + 2 * j + 1]) + bf16_hi(bw[j]);
+              if (EPI == kEpiBiasGelu) {
+                x0 = gelu_fitted(x0);
+                x1 = gelu_fitted(x1);
+              }
+              ow[j] = pack_bf16(x0, x1);
+            }
+            if (row < m_rows) *reinterpret_cast<uint4*>(out + q * 8) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
+          }
+          continue;
         } else {
           // the store that last read this staging buffer must be done with it
           if (lane == 0) {
@@ -528,20 +589,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
   }
 }
 
-template <int BN, int EPI, bool PAIR, bool FP8 = false>
+template <int BN, int EPI, bool PAIR, bool FP8 = false, int LOW = 0>
 cudaError_t launch_one(const GemmParams& p, int sm_count, cudaStream_t stream) {
-  auto kernel = gemm_bf16_tcgen05<BN, EPI, PAIR, FP8>;
+  auto kernel = gemm_bf16_tcgen05<BN, EPI, PAIR, FP8, LOW>;
   static PerDeviceOnce once;   // per instantiation
   cudaError_t err = per_device_once(once, [&](int) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(BN, PAIR, EPI));
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(BN, PAIR, EPI, LOW));
   });
   if (err != cudaSuccess) return err;
-  constexpr int tile_m = PAIR ? 2 * kGemmBlockM : kGemmBlockM;
+  constexpr int tile_m = PAIR ? 2 * kGemmBlockM : (LOW ? LOW : kGemmBlockM);
   const int tiles = ((p.M + tile_m - 1) / tile_m) * (p.N / BN) * p.n_groups * (p.k_splits > 1 ? p.k_splits : 1);
   const int workers_max = PAIR ? sm_count / 2 : sm_count;
   const int workers = tiles < workers_max ? tiles : workers_max;
   if (workers <= 0) return cudaSuccess;
-  return launch_kernel(kernel, dim3(PAIR ? 2 * workers : workers), dim3(kGemmThreads), gemm_smem_bytes(BN, PAIR, EPI), stream,
+  return launch_kernel(kernel, dim3(PAIR ? 2 * workers : workers), dim3(kGemmThreads), gemm_smem_bytes(BN, PAIR, EPI, LOW), stream,
                        p, PAIR ? 2u : 1u);
 }
 
@@ -572,6 +633,18 @@ cudaError_t launch_any(const GemmParams& p, int epilogue, int sm_count, cudaStre
     case 64:
       if constexpr (!PAIR) return launch_bn<64, PAIR>(p, epilogue, sm_count, stream);
       return cudaErrorInvalidValue;
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int LOW>
+cudaError_t launch_low(const GemmParams& p, int epilogue, int sm_count, cudaStream_t stream) {
+  switch (epilogue) {
+    case kEpiBias: return launch_one<64, kEpiBias, false, false, LOW>(p, sm_count, stream);
+    case kEpiBiasGelu: return launch_one<64, kEpiBiasGelu, false, false, LOW>(p, sm_count, stream);
+    case kEpiBiasResidual: return launch_one<64, kEpiBiasResidual, false, false, LOW>(p, sm_count, stream);
+    case kEpiBiasTanhF32: return launch_one<64, kEpiBiasTanhF32, false, false, LOW>(p, sm_count, stream);
+    case kEpiPartialF32: return launch_one<64, kEpiPartialF32, false, false, LOW>(p, sm_count, stream);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -611,6 +684,20 @@ int gemm_block_n(int N, int epilogue, int64_t rows, int groups, bool pair, int s
   }
   return best;
 }
+// Low tiles (64 rows x 64 columns, 32 rows where a layer has no more; single CTAs) where a launch has so few rows that all
+// of them run at once: then the chain of k-blocks one CTA walks is what the launch costs, not the bytes it stages.  (32-row
+// tiles of more rows read the weights that much more often: 1 x 128 tokens 397 us per forward against 386.)  Never changes
+// a bit.
+void gemm_choose_low(GemmParams* p, int groups, int sm_count) {
+  const int splits = p->k_splits > 1 ? p->k_splits : 1;
+  if (p->fp8 || p->N % 64 != 0 || p->K % (kGemmBlockK * kGemmLowKBlocks * splits) != 0) return;
+  const int low = p->M <= 32 ? 32 : 64;
+  const int64_t tiles = static_cast<int64_t>((p->M + low - 1) / low) * (p->N / 64) * (groups < 1 ? 1 : groups) * splits;
+  if (tiles > sm_count) return;
+  p->low = low;
+  p->pair = 0;
+  p->block_n = 64;
+}
 int gemm_out_box_cols(int epilogue) {
   return (epilogue == kEpiBiasResidual || epilogue == kEpiBiasTanhF32 || epilogue == kEpiPartialF32) ? 32 : 64;
 }
@@ -631,6 +718,12 @@ cudaError_t launch_gemm(const GemmParams& p, int epilogue, int sm_count, cudaStr
     if (epilogue == kEpiBiasGelu && p.block_n == 256) return launch_one<256, kEpiBiasGelu, false, true>(p, sm_count, stream);
     if (epilogue == kEpiBiasResidual && p.block_n == 128) return launch_one<128, kEpiBiasResidual, false, true>(p, sm_count, stream);
     return cudaErrorInvalidValue;
+  }
+  if (p.low != 0) {
+    if (p.pair || p.block_n != 64 || p.K % (kGemmBlockK * kGemmLowKBlocks * (p.k_splits > 1 ? p.k_splits : 1)) != 0)
+      return cudaErrorInvalidValue;
+    return p.low == 64 ? launch_low<64>(p, epilogue, sm_count, stream)
+                       : (p.low == 32 ? launch_low<32>(p, epilogue, sm_count, stream) : cudaErrorInvalidValue);
   }
   return p.pair ? launch_any<true>(p, epilogue, sm_count, stream) : launch_any<false>(p, epilogue, sm_count, stream);
 }

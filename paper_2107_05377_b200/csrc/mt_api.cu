@@ -93,6 +93,7 @@ struct LayerTail {
   // launches of few rows: the FFN-down projection as partial sums over `down_splits` ranges of K, put together
   // (ranges in order, bias, residual) by the LayerNorm kernel after it
   int32_t down_splits = 1;
+  int32_t out_splits = 1;    // the same for the attention-output projection
   GemmLnParams attn_out_ln, ffn_down_ln;
   // 8-bit operands: the inputs of the FFN-up and FFN-down projections are quantised row by row first
   bool fp8 = false;
@@ -177,6 +178,22 @@ cudaError_t make_tmap(CUtensorMap* map, const void* base, int64_t rows, int64_t 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Tensor map of a row-major bf16 matrix [rows, cols] as {64, rows, cols / 64}: a box is some rows of several k-blocks, one
+// behind the other in shared memory, each with the 128-byte swizzle.
+cudaError_t make_tmap_kblocks(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows) {
+  EncodeTiledFn enc = nullptr;
+  cudaError_t err = get_encoder(&enc);
+  if (err != cudaSuccess) return err;
+  const cuuint64_t dims[3] = {kGemmBlockK, static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(cols / kGemmBlockK)};
+  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * sizeof(bf16), kGemmBlockK * sizeof(bf16)};
+  const cuuint32_t box[3] = {kGemmBlockK, static_cast<cuuint32_t>(box_rows), kGemmLowKBlocks};
+  const cuuint32_t elem[3] = {1, 1, 1};
+  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, elem,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 // Tensor map of a row-major matrix [rows, cols] of bytes (E4M3 operands) accessed in boxes of box_rows x 128.
 cudaError_t make_tmap_u8(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows) {
   EncodeTiledFn enc = nullptr;
@@ -203,6 +220,9 @@ cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, co
   if (g->fp8 != 0) {
     if ((e = make_tmap_u8(&g->tmap_x[i], x, M, K, kGemmBlockM)) != cudaSuccess) return e;
     if ((e = make_tmap_u8(&g->tmap_w[i], w, N, K, g->block_n)) != cudaSuccess) return e;
+  } else if (g->low != 0) {
+    if ((e = make_tmap_kblocks(&g->tmap_x[i], x, M, K, g->low)) != cudaSuccess) return e;
+    if ((e = make_tmap_kblocks(&g->tmap_w[i], w, N, K, 64)) != cudaSuccess) return e;
   } else {
     if ((e = make_tmap(&g->tmap_x[i], x, M, K, kGemmBlockM, kGemmBlockK, false)) != cudaSuccess) return e;
     if ((e = make_tmap(&g->tmap_w[i], w, N, K, g->block_n / (g->pair != 0 ? 2 : 1), kGemmBlockK, false)) != cudaSuccess) return e;
@@ -210,6 +230,7 @@ cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, co
   if ((e = make_tmap(&g->tmap_out[i], y, M, N, 32, gemm_out_box_cols(epilogue), f32_out)) != cudaSuccess) return e;
   if (res && (e = make_tmap(&g->tmap_res[i], residual, M, N, 32, 32, true)) != cudaSuccess) return e;
   g->group[i].bias = bias;
+  g->group[i].out = y;
   return cudaSuccess;
 }
 
@@ -573,7 +594,15 @@ int32_t down_split_count(const mt_model* m, int64_t rows) {
   if (m->ffn_down_split == 0 || m->fp8 || rows > kSplitRowsMax) return 1;
   return (m->trunk.ffn / kGemmBlockK) % kDownSplits == 0 ? kDownSplits : 1;
 }
-// Launches of steps 3-7 for `groups` layers.
+// The same for the attention-output projection, which a LayerNorm follows too: ranges of kGemmLowKBlocks k-blocks, a
+// single stage of the low tiles each (three for a hidden size of 768, four for 1024; 1 x 128 tokens: 377 us per forward
+// against 386, 4 x 128: 500 against 505).
+int32_t out_split_count(const mt_model* m, int64_t rows) {
+  const int32_t kb = m->trunk.hidden / kGemmBlockK;
+  if (m->ffn_down_split == 0 || m->fp8 || rows > kSplitRowsMax || kb % kGemmLowKBlocks != 0) return 1;
+  return kb / kGemmLowKBlocks <= kDownSplits ? kb / kGemmLowKBlocks : 1;
+}
+// Launches of steps 3-7 for `groups` layers (before mt_bind_memory; afterwards plans are built and counted).
 int32_t tail_launches(const mt_model* m, int32_t groups, int64_t rows) {
   const bool fused = use_fused_ln(m, groups, rows);
   // 8-bit operands: two quantisations, and the FFN-down projection keeps its LayerNorm as a launch of its own;
@@ -593,7 +622,14 @@ void init_tail(const mt_model* m, LayerTail* t, int32_t rows, bool all_rows_vali
     g->m_valid = rows_valid;
     g->status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
   };
-  init_gemm(&t->attn_out, H, H, kEpiBiasResidual);
+  t->out_splits = out_split_count(m, rows);
+  init_gemm(&t->attn_out, H, H, t->out_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual);
+  if (t->out_splits > 1) {
+    t->attn_out.k_splits = t->out_splits;
+    t->attn_out.split_pitch = static_cast<int32_t>(split_pitch(rows));
+    t->attn_out.block_n = gemm_block_n(H, kEpiPartialF32, rows, groups * t->out_splits, false, m->sm_count);
+    t->attn_out.pair = 0;
+  }
   init_gemm(&t->ffn_up, F, H, kEpiBiasGelu);
   t->down_splits = down_split_count(m, rows);
   if (t->down_splits > 1) {
@@ -605,6 +641,8 @@ void init_tail(const mt_model* m, LayerTail* t, int32_t rows, bool all_rows_vali
   } else {
     init_gemm(&t->ffn_down, H, F, kEpiBiasResidual);
   }
+  if (!m->fp8)
+    for (GemmParams* g : {&t->attn_out, &t->ffn_up, &t->ffn_down}) gemm_choose_low(g, groups, m->sm_count);
   t->fp8 = m->fp8;
   if (m->fp8) {
     // E4M3 operands: single CTAs, 256-wide tiles (128 with the residual epilogue)
@@ -626,7 +664,7 @@ void init_tail(const mt_model* m, LayerTail* t, int32_t rows, bool all_rows_vali
   t->ln1.hidden = t->ln2.hidden = H;
   t->ln1.eps = t->ln2.eps = m->trunk.ln_eps;
   t->count = 0;
-  t->ln_fused = use_fused_ln(m, groups, rows);
+  t->ln_fused = use_fused_ln(m, groups, rows) && t->out_splits == 1;
   t->ln_wide = fused_ln_kind(m, groups, rows) == 2;
   t->down_fused = t->ln_fused && !m->fp8 && t->down_splits == 1;
   if (t->ln_fused) {
@@ -648,9 +686,24 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
                         float* u, bf16* h1, float* h1_32, bf16* f, bf16* out, float* out32, const QuantScratch* qs) {
   const int i = t->count;
   cudaError_t e;
-  if ((e = set_gemm_group(&t->attn_out, i, kEpiBiasResidual, ctx, w_ptr(m, lo->wo), w_ptr(m, lo->bo), residual, u)) !=
-      cudaSuccess)
+  // partial sums of a split projection: range s of this group writes rows [s * pitch, s * pitch + rows) of the group's piece
+  // of the partial-sum scratch; the LayerNorm kernel adds the ranges, the bias and the residual
+  auto set_partial = [&](GemmParams* g, int32_t splits, LayerNormParams* ln, const bf16* x, size_t w, size_t b,
+                         const float* res) -> cudaError_t {
+    const size_t pitch = static_cast<size_t>(g->split_pitch);
+    float* part = reinterpret_cast<float*>(m->d_workspace + m->ws_partial) + static_cast<size_t>(i) * splits * pitch * m->trunk.hidden;
+    cudaError_t err = set_gemm_group(g, i, kEpiPartialF32, x, w_ptr(m, w), nullptr, nullptr, part);
+    if (err != cudaSuccess) return err;
+    ln->part[i] = part; ln->residual[i] = res; ln->bias[i] = w_ptr(m, b);
+    ln->n_parts = splits; ln->part_pitch = static_cast<int32_t>(pitch);
+    return make_tmap(&g->tmap_out[i], part, static_cast<int>(splits * pitch), g->N, 32, 32, true);
+  };
+  if (t->out_splits > 1) {
+    if ((e = set_partial(&t->attn_out, t->out_splits, &t->ln1, ctx, lo->wo, lo->bo, residual)) != cudaSuccess) return e;
+  } else if ((e = set_gemm_group(&t->attn_out, i, kEpiBiasResidual, ctx, w_ptr(m, lo->wo), w_ptr(m, lo->bo), residual, u)) !=
+             cudaSuccess) {
     return e;
+  }
   t->ln1.x[i] = u; t->ln1.gamma[i] = w_ptr(m, lo->ln1_g); t->ln1.beta[i] = w_ptr(m, lo->ln1_b);
   t->ln1.y[i] = h1; t->ln1.y32[i] = h1_32;
   if (t->fp8) {
@@ -673,18 +726,7 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
         cudaSuccess)
       return e;
     if (t->down_splits > 1) {
-      // partial sums: range s of this group writes rows [s * pitch, s * pitch + rows) of the group's piece of the
-      // partial-sum scratch; the LayerNorm kernel adds the ranges, the bias and the residual
-      const size_t pitch = static_cast<size_t>(t->ffn_down.split_pitch);
-      float* part = reinterpret_cast<float*>(m->d_workspace + m->ws_partial) +
-                    static_cast<size_t>(i) * t->down_splits * pitch * m->trunk.hidden;
-      if ((e = set_gemm_group(&t->ffn_down, i, kEpiPartialF32, f, w_ptr(m, lo->w2), nullptr, nullptr, part)) != cudaSuccess)
-        return e;
-      if ((e = make_tmap(&t->ffn_down.tmap_out[i], part, static_cast<int>(t->down_splits * pitch), t->ffn_down.N, 32, 32,
-                         true)) != cudaSuccess)
-        return e;
-      t->ln2.part[i] = part; t->ln2.residual[i] = h1_32; t->ln2.bias[i] = w_ptr(m, lo->b2);
-      t->ln2.n_parts = t->down_splits; t->ln2.part_pitch = static_cast<int32_t>(pitch);
+      if ((e = set_partial(&t->ffn_down, t->down_splits, &t->ln2, f, lo->w2, lo->b2, h1_32)) != cudaSuccess) return e;
     } else if ((e = set_gemm_group(&t->ffn_down, i, kEpiBiasResidual, f, w_ptr(m, lo->w2), w_ptr(m, lo->b2), h1_32, u)) !=
                cudaSuccess) {
       return e;
@@ -734,6 +776,7 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   ck->qkv.M = M; ck->qkv.N = 3 * H; ck->qkv.K = H;
   ck->qkv.pair = use_pair(m, M, n_qkv);
   choose_block_n(m, &ck->qkv, kEpiBias, false, n_qkv);
+  if (!m->fp8) gemm_choose_low(&ck->qkv, n_qkv, m->sm_count);
   memset(&ck->q_in, 0, sizeof(ck->q_in));
   if (m->fp8) {
     ck->qkv.fp8 = 1;
@@ -863,13 +906,10 @@ cudaError_t build_cls_tail(const mt_model* m, const std::vector<int32_t>& tasks,
   return cudaSuccess;
 }
 
-int32_t chunk_launches(const mt_model* m, const std::vector<OpDesc>& ops, size_t first, size_t count, int64_t rows,
-                       int32_t seq) {
+int32_t chunk_launches(const mt_model* m, const std::vector<OpDesc>& ops, size_t first, size_t count, int64_t rows) {
   size_t n_cls = 0;
   for (size_t i = 0; i < count; ++i) n_cls += is_cls_op(m, ops[first + i]) ? 1 : 0;
-  // (projection and attention in one launch: the projection of its own serves the last branch layers only)
-  const bool fused = use_qkv_attention(m, rows, seq) && n_cls < count;
-  return (fused && n_cls == 0 ? 0 : 1) + (m->fp8 ? 1 : 0) + (n_cls < count ? 1 + tail_launches(m, static_cast<int32_t>(count - n_cls), rows) : 0) +
+  return 1 + (m->fp8 ? 1 : 0) + (n_cls < count ? 1 + tail_launches(m, static_cast<int32_t>(count - n_cls), rows) : 0) +
          (n_cls > 0 ? 1 : 0);
 }
 // Active tasks whose last branch layer is finished on first tokens right after wave w (1-based):
@@ -885,9 +925,26 @@ std::vector<int32_t> cls_tasks_after_wave(const mt_model* m, const Schedule& s, 
   return out;
 }
 
+// Kernel launches of a built plan: the row starts, the embedding, and what mt_forward_tokens does for every step.
+int32_t plan_launches(const Plan& plan) {
+  auto tail = [](const LayerTail& t) {
+    return t.count == 0 ? 0 : (t.ln_fused ? 1 : 2) + 1 + (t.down_fused ? 1 : 2) + (t.fp8 ? 2 : 0);
+  };
+  int32_t n = 2;
+  for (const PlanStep& st : plan.steps) {
+    if (st.kind == 0) {
+      const Chunk& ck = st.chunk;
+      n += (ck.q_in.n_groups > 0 ? 1 : 0) + (ck.fused_qkv ? 1 : 0) + (ck.qkv.n_groups > 0 ? 1 : 0);
+      n += (ck.full.count > 0 && !ck.fused_qkv ? 1 : 0) + (ck.n_cls > 0 ? 1 : 0) + tail(ck.full);
+    } else {
+      n += st.kind == 2 ? tail(st.tail) : (st.kind == 3 ? 1 : 2);
+    }
+  }
+  return n;
+}
+
 cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int32_t seq, Plan* plan) {
   plan->steps.clear();
-  plan->launches = 2;  // row starts, embedding
   // Pooler + head of a set of tasks.  Tasks whose final state is compact ([B, H], one row per sequence:
   // the last branch layer was evaluated on first tokens only) get their pooler as one grouped GEMM on
   // the tensor cores, Y_t = tanh(X_t . Wp_t^T + bp_t) in fp32, followed by the head kernel; the others
@@ -913,6 +970,7 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
         st.pool.pair = 0;
         st.pool.block_n = gemm_block_n(st.pool.N, kEpiBiasTanhF32, batch, static_cast<int>(count), false, m->sm_count);
         st.pool.m_valid = nullptr;
+        gemm_choose_low(&st.pool, static_cast<int>(count), m->sm_count);
         st.pool.status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
       }
       for (size_t i = 0; i < count; ++i) {
@@ -933,7 +991,6 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
         }
       }
       plan->steps.push_back(std::move(st));
-      plan->launches += 2;
     }
   };
   // Token-level tasks: one linear map on every valid token of the final state, written by position.
@@ -958,7 +1015,6 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
         st.head_tasks.push_back(t);
       }
       plan->steps.push_back(std::move(st));
-      plan->launches += 1;
     }
   };
   auto add_heads = [&](const std::vector<int32_t>& tasks) {
@@ -978,7 +1034,6 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
       cudaError_t e = build_chunk(m, ops, first, count, batch, seq, &st.chunk);
       if (e != cudaSuccess) return e;
       plan->steps.push_back(std::move(st));
-      plan->launches += chunk_launches(m, ops, first, count, static_cast<int64_t>(batch) * seq, seq);
     }
     {
       // first-token tails: of the tasks finishing in this wave (early_heads), or of all tasks after the last wave
@@ -988,12 +1043,12 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
         st.kind = 2;
         cudaError_t e = build_cls_tail(m, tasks, first, std::min<size_t>(kMaxGroups, tasks.size() - first), batch, &st);
         if (e != cudaSuccess) return e;
-        plan->launches += tail_launches(m, st.tail.count, batch);
         plan->steps.push_back(std::move(st));
       }
     }
     add_heads(s.heads[w]);
   }
+  plan->launches = plan_launches(*plan);
   return heads_error;
 }
 
@@ -1364,13 +1419,20 @@ int mt_plan_launches(const mt_model* m, uint64_t task_mask, int32_t* n_launches)
   if (m == nullptr || n_launches == nullptr) return MT_ERR_INVALID_ARG;
   Schedule s;
   if (!build_schedule(m, task_mask, &s)) return fail(m, MT_ERR_INVALID_ARG, "task_mask selects no task");
+  if (m->d_workspace != nullptr) {
+    Plan plan;
+    cudaError_t e = build_plan(m, s, m->max_batch, m->max_seq, &plan);
+    if (e != cudaSuccess) return fail_cuda(m, e, "building the launch plan");
+    *n_launches = plan.launches;
+    return MT_OK;
+  }
   int32_t n = 2;  // row starts, embedding
   for (size_t w = 0; w <= s.waves.size(); ++w) {
     if (w >= 1) {
       const std::vector<OpDesc>& ops = s.waves[w - 1];
       for (size_t first = 0; first < ops.size(); first += m->n_slots)
         n += chunk_launches(m, ops, first, std::min<size_t>(m->n_slots, ops.size() - first),
-                            static_cast<int64_t>(m->max_batch) * m->max_seq, m->max_seq);
+                            static_cast<int64_t>(m->max_batch) * m->max_seq);
       const size_t n_cls_tasks = cls_tasks_after_wave(m, s, w).size();
       for (size_t first = 0; first < n_cls_tasks; first += kMaxGroups)
         n += tail_launches(m, static_cast<int32_t>(std::min<size_t>(kMaxGroups, n_cls_tasks - first)), m->max_batch);
@@ -1479,7 +1541,8 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
                                               : launch_gemm_ln(t_->attn_out_ln, stream),                              \
                "attention output GEMM + LayerNorm");                                                                   \
     } else {                                                                                                           \
-      MT_TIMED(MT_CLASS_ATTN_OUT, launch_gemm(t_->attn_out, kEpiBiasResidual, m->sm_count, stream), "attention output GEMM"); \
+      MT_TIMED(MT_CLASS_ATTN_OUT, launch_gemm(t_->attn_out, t_->out_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual,    \
+                                              m->sm_count, stream), "attention output GEMM");                         \
       MT_TIMED(MT_CLASS_LN1, launch_layernorm(t_->ln1, stream), "LayerNorm 1");                                        \
     }                                                                                                                  \
     if (t_->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_h1, stream), "quantising the FFN input");         \

@@ -16,6 +16,7 @@ typedef __nv_bfloat16 bf16;
 constexpr int kMaxGroups = 8;      // layers fused into one grouped launch
 constexpr int kHeadDim = 64;       // the only head width implemented
 constexpr int kGemmBlockM = 128;   // rows of one GEMM tile (one tcgen05 accumulator = 128 TMEM lanes)
+constexpr int kGemmLowKBlocks = 4;  // k-blocks of a stage of the low tiles (GemmParams::low)
 constexpr int kGemmBlockK = 64;    // bf16 elements per 128-byte swizzled shared-memory row
 
 constexpr uint32_t kFlagBadToken = 0x1u;
@@ -102,6 +103,7 @@ enum GemmEpilogue { kEpiBias = 0, kEpiBiasGelu = 1, kEpiBiasResidual = 2, kEpiBi
 // The output and the residual are reached through the tensor maps of GemmParams.
 struct GemmGroup {
   const bf16* bias;
+  void* out;             // (low tiles with bf16 results) the output by pointer
   const float* scale_x;  // (8-bit operands) one scale per row of X, [M]
   const float* scale_w;  // (8-bit operands) one scale per row of W, [N]
 };
@@ -117,6 +119,8 @@ struct alignas(64) GemmParams {
   const int32_t* m_valid;  // device scalar: rows actually in use (<= M); null = all M rows
   int32_t pair;            // 1: run as pairs of CTAs on 256-row tiles (the W maps then fetch half a tile's rows)
   int32_t block_n;         // tile width along N: 128, 192 or 256 (gemm_block_n); N % block_n == 0
+  int32_t low;             // 64 or 32: tiles of that many rows (block_n 64, single CTAs, bf16); 0: 128.  The X and W maps are
+                           // then dims {64, rows, K / 64}, box {64, low | 64, kGemmLowKBlocks}
   int32_t k_splits;        // ranges K is split into (kEpiPartialF32 only; otherwise 1): (K / 64) % k_splits == 0
   int32_t split_pitch;     // rows between the outputs of consecutive ranges (a multiple of 128, >= M)
   int32_t fp8;             // 1: X and W are E4M3 bytes (maps of uint8, boxes of 128 bytes of K) with row scales;
@@ -130,6 +134,7 @@ struct alignas(64) GemmParams {
 // re-read X less; narrower ones waste less of the last round.  Every output element is accumulated
 // over K in the same order whatever the width, so the choice never changes a result.
 int gemm_block_n(int N, int epilogue, int64_t rows, int groups, bool pair, int sm_count);
+void gemm_choose_low(GemmParams* p, int groups, int sm_count);   // after N, M, K, k_splits and block_n are set
 // Width in elements of the 128-byte output box (64 bf16 or 32 fp32 columns; 32 rows).
 int gemm_out_box_cols(int epilogue);
 cudaError_t launch_gemm(const GemmParams& p, int epilogue, int sm_count, cudaStream_t stream);
