@@ -377,16 +377,8 @@ __global__ void __launch_bounds__(kLnThreads, 1) gemm_ln_tcgen05(const __grid_co
   }
 }
 
-}  // namespace
-
-bool gemm_ln_supported(int N) { return N == 768 || N == 1024; }
-
-cudaError_t launch_gemm_ln(const GemmLnParams& p, cudaStream_t stream) {
-  if (p.n_groups < 1 || p.n_groups > kMaxGroups || !gemm_ln_supported(p.N) || p.K % kGemmBlockK != 0 || p.K < kGemmBlockK ||
-      p.M < 1)
-    return cudaErrorInvalidValue;
-  const int cluster_size = p.N / kLnBlockN;
-  // per device: shared-memory opt-in and, per cluster size, the number of clusters that fit the GPU at once
+// Clusters of this kernel that are resident on the current device at once (and, once per device, its launch set-up).
+cudaError_t resident_clusters(int cluster_size, int* fit_out) {
   static PerDeviceOnce once;
   static int max_clusters[kMaxDevices][2] = {};
   int dev = 0;
@@ -414,7 +406,27 @@ cudaError_t launch_gemm_ln(const GemmLnParams& p, cudaStream_t stream) {
     return cudaSuccess;
   }, &dev);
   if (err != cudaSuccess) return err;
-  const int fit = max_clusters[dev][cluster_size == 8 ? 1 : 0];
+  *fit_out = max_clusters[dev][cluster_size == 8 ? 1 : 0];
+  return cudaSuccess;
+}
+
+}  // namespace
+
+bool gemm_ln_supported(int N) { return N == 768 || N == 1024; }
+
+int gemm_ln_resident(int N) {
+  int fit = 0;
+  return gemm_ln_supported(N) && resident_clusters(N / kLnBlockN, &fit) == cudaSuccess ? fit : 0;
+}
+
+cudaError_t launch_gemm_ln(const GemmLnParams& p, cudaStream_t stream) {
+  if (p.n_groups < 1 || p.n_groups > kMaxGroups || !gemm_ln_supported(p.N) || p.K % kGemmBlockK != 0 || p.K < kGemmBlockK ||
+      p.M < 1)
+    return cudaErrorInvalidValue;
+  const int cluster_size = p.N / kLnBlockN;
+  int fit = 0;
+  cudaError_t err = resident_clusters(cluster_size, &fit);
+  if (err != cudaSuccess) return err;
   if (fit < 1) return cudaErrorLaunchOutOfResources;
   const int tiles = ((p.M + kGemmBlockM - 1) / kGemmBlockM) * p.n_groups;
   const int clusters = tiles < fit ? tiles : fit;

@@ -578,7 +578,20 @@ int fused_ln_kind(const mt_model* m, int32_t groups, int64_t rows) {
   int64_t in_use = rows;
   if (m->pack_tokens && m->expected_tokens > 0 && m->expected_tokens < in_use) in_use = m->expected_tokens;
   if (in_use * groups <= 1024) return 0;
-  return groups == 1 ? 1 : 2;
+  if (m->d_workspace == nullptr) return groups == 1 ? 1 : 2;   // (the device is not known yet)
+  // The row blocks are dealt out in rounds over the clusters that are resident at once (22 of six CTAs, 45 of three), and a
+  // block's epilogue is not hidden behind anything in the last round: the fused launch is the faster one while the rounds
+  // are well filled.  One layer, blocks of 128 rows, us per forward of seven layers, fused / separate: 10 blocks 414 / 396,
+  // 12: 419 / 404, 16: 466 / 497, 20: 502 / 545, 24 (two rounds): 586 / 506, 32: 638 / 610, 40: 739 / 779, 64: 1098 / 1121.
+  // (With ragged lengths fewer rows are in use than the launch is planned for - 32 blocks planned, 18 in use: 1683 / 1730
+  // for the 21-task tree - hence the line at 70 and not at 80 of 100 for more than one round.)  Two layers (wide tiles),
+  // forwards of the eight-task tree: 10 + 10 blocks 790 / 772, 18 + 18: 1052 / 1048, 20 + 20: 1114 / 1132.
+  const int64_t tiles = (in_use + kGemmBlockM - 1) / kGemmBlockM * groups;
+  const int64_t fit = groups == 1 ? gemm_ln_resident(m->trunk.hidden) : gemm_ln_wide_resident(m->trunk.hidden);
+  if (fit < 1) return 0;
+  const int64_t rounds = (tiles + fit - 1) / fit;
+  if (groups == 1) return 100 * tiles >= (rounds == 1 ? 64 : 70) * rounds * fit ? 1 : 0;
+  return 100 * tiles >= 85 * rounds * fit ? 2 : 0;
 }
 bool use_fused_ln(const mt_model* m, int32_t groups, int64_t rows) { return fused_ln_kind(m, groups, rows) != 0; }
 // Ranges the K of the FFN-down projection is split into.  A launch of few rows has few tiles, and each walks

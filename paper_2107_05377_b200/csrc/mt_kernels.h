@@ -237,10 +237,12 @@ struct alignas(64) GemmLnParams {
 };
 // N must be 768 or 1024 (clusters of 6 or 8 CTAs), K a multiple of 64.
 bool gemm_ln_supported(int N);
+int gemm_ln_resident(int N);        // clusters resident on the current device at once (0: error)
 cudaError_t launch_gemm_ln(const GemmLnParams& p, cudaStream_t stream);
 // The same on 128 x 256 accumulator tiles, clusters of N / 256 CTAs (tmap_w256 and residual filled): identical bits,
 // half the CTAs per row block and full-rate tcgen05.mma - for launches with many row blocks.
 bool gemm_ln_wide_supported(int N);
+int gemm_ln_wide_resident(int N);
 cudaError_t launch_gemm_ln_wide(const GemmLnParams& p, cudaStream_t stream);
 
 struct EmbedParams {
