@@ -225,6 +225,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
         const int rem = rem_s / k_splits;
         const int g = rem / n_tiles_n;
         const int n0 = (rem - g * n_tiles_n) * BN + static_cast<int>(rank) * (PAIR ? BN / 2 : 0);
+        // (first k-block of X: a column block of its own per column tile with x_by_tile)
+        const int xb0 = kb0 + (BN == 64 && p.x_by_tile != 0 ? (rem - g * n_tiles_n) * k_blocks : 0);
         for (int kb = 0; kb < k_blocks; ++kb) {
           // this CTA's stage is free once the MMAs that read it (in both CTAs of a pair) are done
           if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag)) { ok = false; break; }
@@ -240,8 +242,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
               tma_load_2d_pair(sB + stage * B_BYTES, &p.tmap_w[g], (kb0 + kb) * KB_ELEMS, n0, bar_full_count + 8 * stage);
           } else {
             mbar_expect_tx(bar_full + 8 * stage, A_BYTES + (w_on_its_way ? 0 : B_BYTES));
-            if (LOW) tma_load_3d(sA + stage * A_BYTES, &p.tmap_x[g], 0, m0, (kb0 + kb) * KPS, bar_full + 8 * stage);
-            else tma_load_2d(sA + stage * A_BYTES, &p.tmap_x[g], (kb0 + kb) * KB_ELEMS, m0, bar_full + 8 * stage);
+            if (LOW) tma_load_3d(sA + stage * A_BYTES, &p.tmap_x[g], 0, m0, (xb0 + kb) * KPS, bar_full + 8 * stage);
+            else tma_load_2d(sA + stage * A_BYTES, &p.tmap_x[g], (xb0 + kb) * KB_ELEMS, m0, bar_full + 8 * stage);
             if (!w_on_its_way) {
               if (LOW) tma_load_3d(sB + stage * B_BYTES, &p.tmap_w[g], 0, n0, (kb0 + kb) * KPS, bar_full + 8 * stage);
               else tma_load_2d(sB + stage * B_BYTES, &p.tmap_w[g], (kb0 + kb) * KB_ELEMS, n0, bar_full + 8 * stage);
@@ -719,6 +721,7 @@ cudaError_t launch_gemm(const GemmParams& p, int epilogue, int sm_count, cudaStr
     if (epilogue == kEpiBiasResidual && p.block_n == 128) return launch_one<128, kEpiBiasResidual, false, true>(p, sm_count, stream);
     return cudaErrorInvalidValue;
   }
+  if (p.x_by_tile != 0 && (p.block_n != 64 || p.pair || p.fp8 || p.k_splits > 1)) return cudaErrorInvalidValue;
   if (p.low != 0) {
     if (p.pair || p.block_n != 64 || p.K % (kGemmBlockK * kGemmLowKBlocks * (p.k_splits > 1 ? p.k_splits : 1)) != 0)
       return cudaErrorInvalidValue;

@@ -40,6 +40,7 @@ constexpr size_t split_pitch(size_t rows) { return (rows + 127) / 128 * 128; }
 constexpr int32_t kDownSplits = 4;
 // "Few rows": at most this many per layer (batch 4 x 128 tokens; the first-token tails of batches up to 512).
 constexpr int32_t kSplitRowsMax = 512;
+static int64_t cls_rows() { const char* e = getenv("MT_CLS"); return e ? atoi(e) : 512; }
 
 inline size_t pad256(size_t n) { return (n + kAlign - 1) / kAlign * kAlign; }
 
@@ -117,6 +118,11 @@ struct Chunk {
   GemmParams qkv;
   AttnParams attn;
   ClsAttnParams attn_cls;
+  // (use_cls_pool) the first-token attention of the last branch layers without keys and values: cls_pool and cls_v in
+  // place of their part of `qkv` and of `attn_cls`
+  bool pool_cls = false;
+  ClsPoolParams cls_pool;
+  GemmParams cls_v;
   LayerTail full;
   int32_t n_cls = 0;
   std::vector<DumpCopy> dumps;
@@ -214,6 +220,7 @@ cudaError_t make_tmap_u8(CUtensorMap* map, const void* base, int64_t rows, int64
 cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, const void* w, const bf16* bias,
                            const float* residual, void* y) {
   const int M = g->M, N = g->N, K = g->K;
+  const int64_t x_cols = g->x_by_tile != 0 ? static_cast<int64_t>(N) / 64 * K : K;   // (X has a column block per column tile)
   const bool res = epilogue == kEpiBiasResidual;
   const bool f32_out = res || epilogue == kEpiBiasTanhF32 || epilogue == kEpiPartialF32;
   cudaError_t e;
@@ -221,10 +228,10 @@ cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, co
     if ((e = make_tmap_u8(&g->tmap_x[i], x, M, K, kGemmBlockM)) != cudaSuccess) return e;
     if ((e = make_tmap_u8(&g->tmap_w[i], w, N, K, g->block_n)) != cudaSuccess) return e;
   } else if (g->low != 0) {
-    if ((e = make_tmap_kblocks(&g->tmap_x[i], x, M, K, g->low)) != cudaSuccess) return e;
+    if ((e = make_tmap_kblocks(&g->tmap_x[i], x, M, x_cols, g->low)) != cudaSuccess) return e;
     if ((e = make_tmap_kblocks(&g->tmap_w[i], w, N, K, 64)) != cudaSuccess) return e;
   } else {
-    if ((e = make_tmap(&g->tmap_x[i], x, M, K, kGemmBlockM, kGemmBlockK, false)) != cudaSuccess) return e;
+    if ((e = make_tmap(&g->tmap_x[i], x, M, x_cols, kGemmBlockM, kGemmBlockK, false)) != cudaSuccess) return e;
     if ((e = make_tmap(&g->tmap_w[i], w, N, K, g->block_n / (g->pair != 0 ? 2 : 1), kGemmBlockK, false)) != cudaSuccess) return e;
   }
   if ((e = make_tmap(&g->tmap_out[i], y, M, N, 32, gemm_out_box_cols(epilogue), f32_out)) != cudaSuccess) return e;
@@ -255,6 +262,7 @@ struct mt_model {
   bool cls_only;     // the last layer of a task branch is evaluated for the first token of a sequence only
   int64_t expected_tokens;  // caller's estimate of the valid tokens per batch (0 = every row); tunes tile shapes only
   bool qkv_attention; // Q/K/V projection and attention of layers on all tokens in one launch where it applies (use_qkv_attention)
+  bool cls_pool;      // first-token attention without projecting keys and values (use_cls_pool)
   bool attention_tc;  // attention on tcgen05 with tensor-memory accumulators when seq <= 128 (else mma.sync)
   int32_t gemm_pair;  // GEMMs as pairs of CTAs on 256-row tiles (cta_group::2): 0 never, 1 always, 2 by launch size
   bool early_heads;  // every task's head (and first-token tail) runs right after the wave that finishes its branch
@@ -549,6 +557,13 @@ int32_t* window_count(const mt_model* m) { return reinterpret_cast<int32_t*>(m->
 int2* window_list(const mt_model* m) { return reinterpret_cast<int2*>(m->d_workspace + m->ws_windows + 256); }
 int2* row_info(const mt_model* m) { return reinterpret_cast<int2*>(m->d_workspace + m->ws_row_info); }
 
+// Whether the last branch layers get their first-token attention without projecting keys and values (cls_pool.cu): a few
+// H x H products per sequence instead of two per token, in three launches instead of two - worth it beyond the few rows
+// whose launches are all latency.  (The scratch is the layer's slot for Q, K and V, which has room from 8 or 11 tokens up.)
+bool use_cls_pool(const mt_model* m, int64_t rows, int32_t seq) {
+  return m->cls_pool && !m->fp8 && rows > cls_rows() && 3 * seq >= 2 * m->trunk.heads;
+}
+
 // Tile width of a grouped GEMM launch (see gemm_block_n).  `rows` are the rows the launch is sized for;
 // with the packed token layout only the valid tokens are in use, and the caller's estimate of their
 // number (option "expected_tokens"), when given, replaces it.
@@ -783,7 +798,20 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   int32_t n_full = 0;
   for (size_t i = 0; i < count; ++i) n_full += is_cls_op(m, ops[first + i]) ? 0 : 1;
   ck->fused_qkv = use_qkv_attention(m, M, seq) && n_full > 0;
-  const int32_t n_qkv = static_cast<int32_t>(count) - (ck->fused_qkv ? n_full : 0);
+  const int32_t n_last = static_cast<int32_t>(count) - n_full;
+  ck->pool_cls = n_last > 0 && use_cls_pool(m, M, seq);
+  const int32_t n_qkv = static_cast<int32_t>(count) - (ck->fused_qkv ? n_full : 0) - (ck->pool_cls ? n_last : 0);
+  memset(&ck->cls_pool, 0, sizeof(ck->cls_pool));
+  memset(&ck->cls_v, 0, sizeof(ck->cls_v));
+  if (ck->pool_cls) {
+    ck->cls_pool.batch = batch; ck->cls_pool.seq = seq; ck->cls_pool.heads = m->trunk.heads;
+    ck->cls_pool.row_start = row_start;
+    ck->cls_v.M = batch; ck->cls_v.N = H; ck->cls_v.K = H;
+    ck->cls_v.block_n = 64;
+    ck->cls_v.x_by_tile = 1;
+    ck->cls_v.status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
+    gemm_choose_low(&ck->cls_v, n_last, m->sm_count);
+  }
   memset(&ck->qkv, 0, sizeof(ck->qkv));
   ck->qkv.n_groups = n_qkv;
   ck->qkv.M = M; ck->qkv.N = 3 * H; ck->qkv.K = H;
@@ -852,6 +880,20 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
     const void* x_op = m->fp8 ? static_cast<const void*>(qs.xq) : in;   // the projection's operands
     const void* w_op = m->fp8 ? static_cast<const void*>(m->d_weights + lo->q_qkv) : w_ptr(m, lo->wq);
     const float* w_scale = m->fp8 ? reinterpret_cast<const float*>(m->d_weights + lo->s_qkv) : nullptr;
+    if (ck->pool_cls && cls) {
+      const int a = ck->n_cls;
+      uint8_t* cs = m->d_workspace + m->ws_cls0 + m->cls_bytes * op.task;
+      bf16* z = qkv + static_cast<size_t>(batch) * m->trunk.heads * H;
+      ck->cls_pool.x[a] = in;
+      ck->cls_pool.in32[a] = f32_of(m, in);
+      ck->cls_pool.wq[a] = w_ptr(m, lo->wq); ck->cls_pool.bq[a] = w_ptr(m, lo->bq); ck->cls_pool.wk[a] = w_ptr(m, lo->wk);
+      ck->cls_pool.qt[a] = qkv;
+      ck->cls_pool.z[a] = z;
+      ck->cls_pool.res[a] = reinterpret_cast<float*>(cs + m->cls_h_bytes);
+      if ((e = set_gemm_group(&ck->cls_v, a, kEpiBias, z, w_ptr(m, lo->wv), w_ptr(m, lo->bv), nullptr, cs)) != cudaSuccess) return e;
+      ck->cls_pool.n_groups = ck->cls_v.n_groups = ck->n_cls = a + 1;
+      continue;
+    }
     if (ck->fused_qkv && !cls) {
       const int a = ck->qa.n_groups;
       if ((e = make_tmap(&ck->qa.tmap_x[a], x_op, M, H, 64, 64, false)) != cudaSuccess ||
@@ -948,7 +990,7 @@ int32_t plan_launches(const Plan& plan) {
     if (st.kind == 0) {
       const Chunk& ck = st.chunk;
       n += (ck.q_in.n_groups > 0 ? 1 : 0) + (ck.fused_qkv ? 1 : 0) + (ck.qkv.n_groups > 0 ? 1 : 0);
-      n += (ck.full.count > 0 && !ck.fused_qkv ? 1 : 0) + (ck.n_cls > 0 ? 1 : 0) + tail(ck.full);
+      n += (ck.full.count > 0 && !ck.fused_qkv ? 1 : 0) + (ck.n_cls > 0 ? (ck.pool_cls ? 3 : 1) : 0) + tail(ck.full);
     } else {
       n += st.kind == 2 ? tail(st.tail) : (st.kind == 3 ? 1 : 2);
     }
@@ -1106,6 +1148,7 @@ int mt_create(const mt_trunk_config* trunk, const mt_task_config* tasks, int32_t
   m->early_heads = false;
   m->gemm_pair = 2;
   m->qkv_attention = true;
+  m->cls_pool = true;
   m->attention_tc = true;
   m->expected_tokens = 0;
   m->pool_gemm = true;
@@ -1246,6 +1289,11 @@ int mt_set_option(mt_model* m, const char* key, int64_t value) {
   }
   if (strcmp(key, "pool_gemm") == 0) {
     m->pool_gemm = value != 0;
+    m->plans.clear();
+    return MT_OK;
+  }
+  if (strcmp(key, "cls_pool") == 0) {
+    m->cls_pool = value != 0;
     m->plans.clear();
     return MT_OK;
   }
@@ -1604,21 +1652,36 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
       Chunk& ck = st.chunk;
       ck.attn.lengths = d_lengths;
       ck.attn_cls.lengths = d_lengths;
+      ck.cls_pool.lengths = d_lengths;
       if (m->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(ck.q_in, stream), "quantising the layer inputs");
+      const bool beside = m->overlap_cls && m->side_stream != nullptr && !m->profile && ck.n_cls > 0 && ck.full.count > 0;
+      auto fork = [&]() -> cudaError_t {
+        cudaError_t err = cudaEventRecord(m->ev_fork, stream);
+        return err == cudaSuccess ? cudaStreamWaitEvent(m->side_stream, m->ev_fork, 0) : err;
+      };
+      if (ck.pool_cls) {
+        // first-token attention straight from the layers' inputs: beside the wave's kernels from its start
+        cudaStream_t cls_stream = beside ? m->side_stream : stream;
+        if (beside) MT_LAUNCH(fork(), "forking the side stream");
+        MT_TIMED(MT_CLASS_ATTENTION, launch_cls_pool(ck.cls_pool, cls_stream), "first-token attention kernels");
+        MT_TIMED(MT_CLASS_ATTENTION, launch_gemm(ck.cls_v, kEpiBias, m->sm_count, cls_stream), "first-token value projection");
+        if (beside) {
+          MT_LAUNCH(cudaEventRecord(m->ev_join, m->side_stream), "joining the side stream");
+          side_pending = true;
+        }
+      }
       if (ck.fused_qkv)
         MT_TIMED(MT_CLASS_QKV, launch_qkv_attention(ck.qa, m->sm_count, stream), "QKV projection + attention kernel");
       if (ck.qkv.n_groups > 0)
         MT_TIMED(MT_CLASS_QKV, launch_gemm(ck.qkv, kEpiBias, m->sm_count, stream), "QKV GEMM");
-      const bool beside = m->overlap_cls && m->side_stream != nullptr && !m->profile && ck.n_cls > 0 && ck.full.count > 0;
-      if (beside) {
-        MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
-        MT_LAUNCH(cudaStreamWaitEvent(m->side_stream, m->ev_fork, 0), "forking the side stream");
+      if (beside && !ck.pool_cls) {
+        MT_LAUNCH(fork(), "forking the side stream");
         MT_LAUNCH(launch_cls_attention(ck.attn_cls, m->side_stream), "first-token attention kernel");
         MT_LAUNCH(cudaEventRecord(m->ev_join, m->side_stream), "joining the side stream");
         side_pending = true;
       }
       if (ck.full.count > 0 && !ck.fused_qkv) MT_TIMED(MT_CLASS_ATTENTION, launch_attention(ck.attn, stream), "attention kernel");
-      if (ck.n_cls > 0 && !beside)
+      if (ck.n_cls > 0 && !beside && !ck.pool_cls)
         MT_TIMED(MT_CLASS_ATTENTION, launch_cls_attention(ck.attn_cls, stream), "first-token attention kernel");
       if (ck.full.count > 0) MT_TAIL(&ck.full);
       for (const DumpCopy& d : ck.dumps)
