@@ -225,8 +225,8 @@ int mt_plan_cache_size(const mt_model* m);
  * key "debug_capture" (0/1): keep a copy of every layer output for mt_debug_copy_hidden (changes
  * mt_workspace_bytes); both must be set before mt_bind_memory.  key "profile" (0/1): see
  * mt_profile_read.  key "cls_only_last_layer" (0/1, default 1, any time): the last
- * layer of every task branch is evaluated for the first token of each sequence only (keys and values
- * still for all tokens) because the pooler reads nothing else; mt_debug_copy_hidden then returns that
+ * layer of every task branch is evaluated for the first token of each sequence only (which still attends
+ * to all tokens) because the pooler reads nothing else; mt_debug_copy_hidden then returns that
  * layer's state at position 0 and zeros elsewhere.  key "early_heads" (0/1, default 0, any time): see mt_forward_events.
  * key "pack_tokens" (0/1, default 1, any time): store
  * and compute only the valid tokens of every sequence (rows of sequence b follow those of b-1) instead
@@ -272,11 +272,16 @@ int mt_plan_cache_size(const mt_model* m);
  * the layers on all tokens run their Q/K/V projection and attention as one launch, over windows of 128 rows that hold
  * whole sequences (1), or as two launches (0).  Logits agree to rounding (the keys of a sequence are summed over in
  * other groups of 16).
- * key "overlap_cls" (0/1, default 1, any time): where a wave holds layers on all tokens and last branch
- * layers, the first-token attention of the latter runs on a stream the library creates for itself (in
- * mt_bind_memory), forked from the caller's stream after the wave's Q/K/V projection and joined before the next
- * step, so that it overlaps the wave's other kernels; the caller sees ordinary single-stream semantics,
- * also under stream capture.  Same results.
+ * key "cls_pool" (0/1, default 1, any time): with bf16 operands and batch x seq > 512 the first-token attention of
+ * the last branch layers runs without projecting keys and values: the query is taken through the key matrix and
+ * the attended mean of the inputs through the value matrix (1), or as a Q/K/V projection and an attention over it (0).
+ * Logits agree to rounding.
+ * key "overlap_cls" (0/1, default 1, any time): first-token attention beside layers on all tokens runs on a stream
+ * that the library creates for itself (in mt_bind_memory), so that it overlaps their kernels.  With "cls_pool" it is
+ * forked from the caller's stream before the wave before last and joined before the first-token tails (with
+ * "early_heads" it stays on the caller's stream); without, it is forked after its wave's Q/K/V projection and
+ * joined before the next step.  The caller sees ordinary single-stream semantics, also under stream capture.
+ * Same results.
  * key "pool_gemm" (0/1, default 1, any time): the pooler of tasks whose last branch layer was evaluated on
  * first tokens only runs as one grouped GEMM with a tanh epilogue on the tensor cores (1) or in the
  * row-wise pooler kernel (0, also used for every other task); logits agree to rounding.

@@ -40,7 +40,6 @@ constexpr size_t split_pitch(size_t rows) { return (rows + 127) / 128 * 128; }
 constexpr int32_t kDownSplits = 4;
 // "Few rows": at most this many per layer (batch 4 x 128 tokens; the first-token tails of batches up to 512).
 constexpr int32_t kSplitRowsMax = 512;
-static int64_t cls_rows() { const char* e = getenv("MT_CLS"); return e ? atoi(e) : 512; }
 
 inline size_t pad256(size_t n) { return (n + kAlign - 1) / kAlign * kAlign; }
 
@@ -118,17 +117,15 @@ struct Chunk {
   GemmParams qkv;
   AttnParams attn;
   ClsAttnParams attn_cls;
-  // (use_cls_pool) the first-token attention of the last branch layers without keys and values: cls_pool and cls_v in
-  // place of their part of `qkv` and of `attn_cls`
-  bool pool_cls = false;
-  ClsPoolParams cls_pool;
-  GemmParams cls_v;
   LayerTail full;
   int32_t n_cls = 0;
   std::vector<DumpCopy> dumps;
 };
 struct PlanStep {
-  int kind;  // 0 = chunk, 1 = heads, 2 = cls tail, 3 = token-level heads
+  int kind;  // 0 = chunk, 1 = heads, 2 = cls tail, 3 = token-level heads, 4 = first-token attention without keys and values
+  ClsPoolParams cls_pool;           // (4)
+  GemmParams cls_v;
+  bool beside = false;              // (4) on the side stream, joined before the first-token tails
   TokenHeadParams token_heads;
   Chunk chunk;
   HeadParams heads;
@@ -140,6 +137,7 @@ struct PlanStep {
 };
 struct Plan {
   std::vector<PlanStep> steps;
+  bf16* embedding = nullptr;   // where the embedding output goes (StateBufs)
   int32_t launches = 0;
   uint64_t last_use = 0;  // stamp of the last forward that ran this plan (least recently used goes first)
 };
@@ -290,7 +288,7 @@ struct mt_model {
   // workspace layout (byte offsets)
   size_t ws_status, ws_rows_valid, ws_row_start, ws_windows, ws_row_info, ws_tok, ws_seg, ws_len, ws_logits, ws_pooled, ws_partial, ws_trunk[2], ws_task0,
       ws_slot0, ws_cls0, ws_dump0;
-  size_t slot_q_off, cls_q_off;   // 8-bit scratch inside a slot / inside a task's first-token scratch
+  size_t slot_q_off, cls_q_off, cls_pool_off;   // 8-bit scratch inside a slot / inside a task's first-token scratch
   size_t cls_bytes, cls_h_bytes, cls_h32_bytes;  // per-task first-token scratch and its [B,H] bf16 / fp32 pieces
   size_t act_bytes;    // max_batch*max_seq*hidden bf16
   size_t act32_bytes;  // the same tensor in fp32
@@ -425,6 +423,10 @@ void layout_workspace(mt_model* m) {
     const size_t B = static_cast<size_t>(m->max_batch);
     m->cls_bytes += pad256(B * H) + pad256(B * F) + 2 * pad256(B * 4);
   }
+  // ... and q~ and z of the attention without keys and values, bf16 [B, heads, H] each
+  m->cls_pool_off = m->cls_bytes;
+  if (!m->fp8 && 3 * m->max_seq >= 2 * m->trunk.heads)
+    m->cls_bytes += 2 * pad256(static_cast<size_t>(m->max_batch) * m->trunk.heads * H * 2);
   m->ws_cls0 = off;
   off += m->cls_bytes * m->tasks.size();
   m->n_dump = 0;
@@ -559,9 +561,13 @@ int2* row_info(const mt_model* m) { return reinterpret_cast<int2*>(m->d_workspac
 
 // Whether the last branch layers get their first-token attention without projecting keys and values (cls_pool.cu): a few
 // H x H products per sequence instead of two per token, in three launches instead of two - worth it beyond the few rows
-// whose launches are all latency.  (The scratch is the layer's slot for Q, K and V, which has room from 8 or 11 tokens up.)
+// whose launches are all latency (1 x 128 tokens: 408 us per forward against 379; 23 x 101 on the 33-layer paper tree: 994
+// against 1005; 32 x 128: 1009 against 1046, 1555 against 1704 with 21 tasks; 256 x 128: 10.09 ms against 11.11).
+// The line depends on the rows of one layer alone, so a task gets the same bits whatever runs beside it.  Sequences of so
+// few tokens that q~ and z [B, heads, H] would outweigh K and V stay where they were.
+bool cls_pool_scratch(const mt_model* m) { return !m->fp8 && 3 * m->max_seq >= 2 * m->trunk.heads; }
 bool use_cls_pool(const mt_model* m, int64_t rows, int32_t seq) {
-  return m->cls_pool && !m->fp8 && rows > cls_rows() && 3 * seq >= 2 * m->trunk.heads;
+  return m->cls_pool && m->cls_only && cls_pool_scratch(m) && rows > kSplitRowsMax && 3 * seq >= 2 * m->trunk.heads;
 }
 
 // Tile width of a grouped GEMM launch (see gemm_block_n).  `rows` are the rows the launch is sized for;
@@ -789,8 +795,29 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
   return cudaSuccess;
 }
 
+// Where the state of a trunk depth lives.  Every reader but one runs in the next wave, so two buffers taken in turn are
+// enough; the first-token attention without keys and values (use_cls_pool) reads its layer's input as late as just before
+// the first-token tails.  The input of a branch's second or later layer is the task's own buffer, which nothing writes
+// before the tails; the trunk state that a one-layer branch reads is put into that task's buffer, otherwise unused so far.
+struct StateBufs {
+  std::vector<bf16*> depth;
+};
+StateBufs place_states(const mt_model* m, const Schedule& s, bool pool) {
+  StateBufs b;
+  for (int32_t d = 0; d <= s.trunk_depth; ++d) b.depth.push_back(trunk_buf(m, d));
+  if (pool)
+    for (const std::vector<OpDesc>& ops : s.waves)
+      for (const OpDesc& op : ops)
+        if (is_cls_op(m, op) && op.layer == 1) b.depth[m->tasks[op.task].cfg.fork_depth] = task_buf(m, op.task);
+  return b;
+}
+bf16* layer_input(const mt_model* m, const StateBufs& bufs, const OpDesc& op) {
+  if (op.task < 0) return bufs.depth[op.layer - 1];
+  return op.layer == 1 ? bufs.depth[m->tasks[op.task].cfg.fork_depth] : task_buf(m, op.task);
+}
+
 cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_t first, size_t count, int32_t batch,
-                        int32_t seq, Chunk* ck) {
+                        int32_t seq, const StateBufs& bufs, Chunk* ck) {
   const int32_t M = batch * seq, H = m->trunk.hidden;
   const size_t act = m->act_bytes;
   const size_t qkv_bytes = pad256(static_cast<size_t>(m->max_batch) * m->max_seq * 3 * H * 2);
@@ -798,20 +825,7 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   int32_t n_full = 0;
   for (size_t i = 0; i < count; ++i) n_full += is_cls_op(m, ops[first + i]) ? 0 : 1;
   ck->fused_qkv = use_qkv_attention(m, M, seq) && n_full > 0;
-  const int32_t n_last = static_cast<int32_t>(count) - n_full;
-  ck->pool_cls = n_last > 0 && use_cls_pool(m, M, seq);
-  const int32_t n_qkv = static_cast<int32_t>(count) - (ck->fused_qkv ? n_full : 0) - (ck->pool_cls ? n_last : 0);
-  memset(&ck->cls_pool, 0, sizeof(ck->cls_pool));
-  memset(&ck->cls_v, 0, sizeof(ck->cls_v));
-  if (ck->pool_cls) {
-    ck->cls_pool.batch = batch; ck->cls_pool.seq = seq; ck->cls_pool.heads = m->trunk.heads;
-    ck->cls_pool.row_start = row_start;
-    ck->cls_v.M = batch; ck->cls_v.N = H; ck->cls_v.K = H;
-    ck->cls_v.block_n = 64;
-    ck->cls_v.x_by_tile = 1;
-    ck->cls_v.status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
-    gemm_choose_low(&ck->cls_v, n_last, m->sm_count);
-  }
+  const int32_t n_qkv = static_cast<int32_t>(count) - (ck->fused_qkv ? n_full : 0);
   memset(&ck->qkv, 0, sizeof(ck->qkv));
   ck->qkv.n_groups = n_qkv;
   ck->qkv.M = M; ck->qkv.N = 3 * H; ck->qkv.K = H;
@@ -852,18 +866,9 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   int n_qkv_set = 0;
   for (size_t i = 0; i < count; ++i) {
     const OpDesc& op = ops[first + i];
-    const LayerOffsets* lo;
-    bf16 *in, *out;
-    if (op.task < 0) {
-      lo = &m->trunk_layers[op.layer - 1];
-      in = trunk_buf(m, op.layer - 1);
-      out = trunk_buf(m, op.layer);
-    } else {
-      const TaskEntry& te = m->tasks[op.task];
-      lo = &te.layers[op.layer - 1];
-      in = op.layer == 1 ? trunk_buf(m, te.cfg.fork_depth) : task_buf(m, op.task);
-      out = task_buf(m, op.task);
-    }
+    const LayerOffsets* lo = op.task < 0 ? &m->trunk_layers[op.layer - 1] : &m->tasks[op.task].layers[op.layer - 1];
+    bf16* in = layer_input(m, bufs, op);
+    bf16* out = op.task < 0 ? bufs.depth[op.layer] : task_buf(m, op.task);
     uint8_t* slot = m->d_workspace + m->ws_slot0 + m->slot_bytes * i;
     bf16* qkv = reinterpret_cast<bf16*>(slot);
     bf16* ctx = reinterpret_cast<bf16*>(slot + qkv_bytes);
@@ -880,20 +885,6 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
     const void* x_op = m->fp8 ? static_cast<const void*>(qs.xq) : in;   // the projection's operands
     const void* w_op = m->fp8 ? static_cast<const void*>(m->d_weights + lo->q_qkv) : w_ptr(m, lo->wq);
     const float* w_scale = m->fp8 ? reinterpret_cast<const float*>(m->d_weights + lo->s_qkv) : nullptr;
-    if (ck->pool_cls && cls) {
-      const int a = ck->n_cls;
-      uint8_t* cs = m->d_workspace + m->ws_cls0 + m->cls_bytes * op.task;
-      bf16* z = qkv + static_cast<size_t>(batch) * m->trunk.heads * H;
-      ck->cls_pool.x[a] = in;
-      ck->cls_pool.in32[a] = f32_of(m, in);
-      ck->cls_pool.wq[a] = w_ptr(m, lo->wq); ck->cls_pool.bq[a] = w_ptr(m, lo->bq); ck->cls_pool.wk[a] = w_ptr(m, lo->wk);
-      ck->cls_pool.qt[a] = qkv;
-      ck->cls_pool.z[a] = z;
-      ck->cls_pool.res[a] = reinterpret_cast<float*>(cs + m->cls_h_bytes);
-      if ((e = set_gemm_group(&ck->cls_v, a, kEpiBias, z, w_ptr(m, lo->wv), w_ptr(m, lo->bv), nullptr, cs)) != cudaSuccess) return e;
-      ck->cls_pool.n_groups = ck->cls_v.n_groups = ck->n_cls = a + 1;
-      continue;
-    }
     if (ck->fused_qkv && !cls) {
       const int a = ck->qa.n_groups;
       if ((e = make_tmap(&ck->qa.tmap_x[a], x_op, M, H, 64, 64, false)) != cudaSuccess ||
@@ -933,6 +924,42 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
       ck->attn_cls.res[a] = reinterpret_cast<float*>(cs + m->cls_h_bytes);
       ck->attn_cls.n_groups = ck->n_cls = a + 1;
     }
+  }
+  return cudaSuccess;
+}
+
+// First-token attention without keys and values of up to kMaxGroups last branch layers.
+cudaError_t build_cls_pool(const mt_model* m, const std::vector<OpDesc>& ops, size_t first, size_t count, int32_t batch, int32_t seq,
+                           const StateBufs& bufs, PlanStep* st) {
+  const int32_t H = m->trunk.hidden;
+  st->kind = 4;
+  ClsPoolParams& p = st->cls_pool;
+  GemmParams& v = st->cls_v;
+  memset(&p, 0, sizeof(p));
+  memset(&v, 0, sizeof(v));
+  p.batch = batch; p.seq = seq; p.heads = m->trunk.heads;
+  p.row_start = reinterpret_cast<const int32_t*>(m->d_workspace + m->ws_row_start);
+  v.M = batch; v.N = H; v.K = H;
+  v.block_n = 64;
+  v.x_by_tile = 1;
+  v.status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
+  gemm_choose_low(&v, static_cast<int32_t>(count), m->sm_count);
+  for (size_t i = 0; i < count; ++i) {
+    const OpDesc& op = ops[first + i];
+    const LayerOffsets& lo = m->tasks[op.task].layers[op.layer - 1];
+    bf16* in = layer_input(m, bufs, op);
+    uint8_t* cs = m->d_workspace + m->ws_cls0 + m->cls_bytes * op.task;
+    bf16* qt = reinterpret_cast<bf16*>(cs + m->cls_pool_off);
+    bf16* z = qt + pad256(static_cast<size_t>(m->max_batch) * m->trunk.heads * H * 2) / 2;
+    p.x[i] = in;
+    p.in32[i] = f32_of(m, in);
+    p.wq[i] = w_ptr(m, lo.wq); p.bq[i] = w_ptr(m, lo.bq); p.wk[i] = w_ptr(m, lo.wk);
+    p.qt[i] = qt;
+    p.z[i] = z;
+    p.res[i] = reinterpret_cast<float*>(cs + m->cls_h_bytes);
+    cudaError_t e = set_gemm_group(&v, static_cast<int>(i), kEpiBias, z, w_ptr(m, lo.wv), w_ptr(m, lo.bv), nullptr, cs);
+    if (e != cudaSuccess) return e;
+    p.n_groups = v.n_groups = static_cast<int32_t>(i) + 1;
   }
   return cudaSuccess;
 }
@@ -990,9 +1017,9 @@ int32_t plan_launches(const Plan& plan) {
     if (st.kind == 0) {
       const Chunk& ck = st.chunk;
       n += (ck.q_in.n_groups > 0 ? 1 : 0) + (ck.fused_qkv ? 1 : 0) + (ck.qkv.n_groups > 0 ? 1 : 0);
-      n += (ck.full.count > 0 && !ck.fused_qkv ? 1 : 0) + (ck.n_cls > 0 ? (ck.pool_cls ? 3 : 1) : 0) + tail(ck.full);
+      n += (ck.full.count > 0 && !ck.fused_qkv ? 1 : 0) + (ck.n_cls > 0 ? 1 : 0) + tail(ck.full);
     } else {
-      n += st.kind == 2 ? tail(st.tail) : (st.kind == 3 ? 1 : 2);
+      n += st.kind == 2 ? tail(st.tail) : (st.kind == 4 ? 3 : (st.kind == 3 ? 1 : 2));
     }
   }
   return n;
@@ -1000,6 +1027,9 @@ int32_t plan_launches(const Plan& plan) {
 
 cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int32_t seq, Plan* plan) {
   plan->steps.clear();
+  const bool pool = use_cls_pool(m, static_cast<int64_t>(batch) * seq, seq);
+  const StateBufs bufs = place_states(m, s, pool);
+  plan->embedding = bufs.depth[0];
   // Pooler + head of a set of tasks.  Tasks whose final state is compact ([B, H], one row per sequence:
   // the last branch layer was evaluated on first tokens only) get their pooler as one grouped GEMM on
   // the tensor cores, Y_t = tanh(X_t . Wp_t^T + bp_t) in fp32, followed by the head kernel; the others
@@ -1032,7 +1062,7 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
         const int32_t t = tasks[first + i];
         const TaskEntry& te = m->tasks[t];
         HeadTask& ht = st.heads.task[i];
-        ht.hidden = te.cfg.branch_layers == 0 ? trunk_buf(m, te.cfg.fork_depth) : task_buf(m, t);
+        ht.hidden = te.cfg.branch_layers == 0 ? bufs.depth[te.cfg.fork_depth] : task_buf(m, t);
         ht.pool_w = w_ptr(m, te.pool_w); ht.pool_b = w_ptr(m, te.pool_b);
         ht.cls_w = w_ptr(m, te.cls_w); ht.cls_b = w_ptr(m, te.cls_b);
         ht.num_classes = te.cfg.num_classes; ht.col0 = te.col0;
@@ -1064,7 +1094,7 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
       for (size_t i = 0; i < count; ++i) {
         const int32_t t = tasks[first + i];
         const TaskEntry& te = m->tasks[t];
-        th.hidden_state[i] = te.cfg.branch_layers == 0 ? trunk_buf(m, te.cfg.fork_depth) : task_buf(m, t);
+        th.hidden_state[i] = te.cfg.branch_layers == 0 ? bufs.depth[te.cfg.fork_depth] : task_buf(m, t);
         th.cls_w[i] = w_ptr(m, te.cls_w); th.cls_b[i] = w_ptr(m, te.cls_b);
         th.num_classes[i] = te.cfg.num_classes; th.col0[i] = te.col0;
         st.head_tasks.push_back(t);
@@ -1081,12 +1111,33 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
   };
   add_heads(s.heads[0]);
   for (size_t w = 1; w <= s.waves.size(); ++w) {
-    const std::vector<OpDesc>& ops = s.waves[w - 1];
+    std::vector<OpDesc> ops = s.waves[w - 1];
+    if (pool) {
+      // The first-token attention is no part of the wave.  That of all waves but the last goes beside the last two, from the
+      // start of the one before last, when all its inputs are there: one fork and one join per forward, where a fork
+      // and a join per wave cost the caller's stream the overlap of two launches each (23 x 101: 994 us against 1027;
+      // 32 x 128: 1009 against 1032).  With option "early_heads" each stays in its own wave, since its tail follows at once.
+      std::vector<OpDesc> now;
+      const size_t last = s.waves.size();
+      const bool beside = !m->early_heads && w + 1 == last;
+      for (size_t v = 1; v <= w; ++v)
+        if (m->early_heads || w == last ? v == w : beside)
+          for (const OpDesc& op : s.waves[v - 1])
+            if (is_cls_op(m, op)) now.push_back(op);
+      for (size_t first = 0; first < now.size(); first += kMaxGroups) {
+        PlanStep st;
+        cudaError_t e = build_cls_pool(m, now, first, std::min<size_t>(kMaxGroups, now.size() - first), batch, seq, bufs, &st);
+        if (e != cudaSuccess) return e;
+        st.beside = beside;
+        plan->steps.push_back(std::move(st));
+      }
+      ops.erase(std::remove_if(ops.begin(), ops.end(), [&](const OpDesc& op) { return is_cls_op(m, op); }), ops.end());
+    }
     for (size_t first = 0; first < ops.size(); first += m->n_slots) {
       const size_t count = std::min<size_t>(m->n_slots, ops.size() - first);
       PlanStep st;
       st.kind = 0;
-      cudaError_t e = build_chunk(m, ops, first, count, batch, seq, &st.chunk);
+      cudaError_t e = build_chunk(m, ops, first, count, batch, seq, bufs, &st.chunk);
       if (e != cudaSuccess) return e;
       plan->steps.push_back(std::move(st));
     }
@@ -1633,7 +1684,7 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
   ep.token_ids = d_token_ids; ep.segment_ids = d_segment_ids; ep.lengths = d_lengths;
   ep.word = w_ptr(m, m->emb_word); ep.pos = w_ptr(m, m->emb_pos); ep.type = w_ptr(m, m->emb_type);
   ep.gamma = w_ptr(m, m->emb_ln_g); ep.beta = w_ptr(m, m->emb_ln_b);
-  ep.out = trunk_buf(m, 0);
+  ep.out = plan.embedding;
   ep.out32 = f32_of(m, ep.out);
   ep.batch = batch; ep.seq = seq; ep.hidden = m->trunk.hidden; ep.vocab = m->trunk.vocab_size;
   ep.type_vocab = m->trunk.type_vocab; ep.eps = m->trunk.ln_eps; ep.status = status;
@@ -1642,46 +1693,32 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
     MT_LAUNCH(cudaMemcpyAsync(m->d_workspace + m->ws_dump0, ep.out, act_used, cudaMemcpyDeviceToDevice, stream),
               "debug capture");
 
+  bool pool_pending = false;   // ... of a step of kind 4: waited for before the first-token tails
   bool side_pending = false;   // work on the side stream that the caller's stream has not waited for yet
   for (PlanStep& st : plan.steps) {
-    if (side_pending) {
+    if (side_pending || (pool_pending && st.kind == 2)) {
       MT_LAUNCH(cudaStreamWaitEvent(stream, m->ev_join, 0), "joining the side stream");
-      side_pending = false;
+      side_pending = pool_pending = false;
     }
     if (st.kind == 0) {
       Chunk& ck = st.chunk;
       ck.attn.lengths = d_lengths;
       ck.attn_cls.lengths = d_lengths;
-      ck.cls_pool.lengths = d_lengths;
       if (m->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(ck.q_in, stream), "quantising the layer inputs");
       const bool beside = m->overlap_cls && m->side_stream != nullptr && !m->profile && ck.n_cls > 0 && ck.full.count > 0;
-      auto fork = [&]() -> cudaError_t {
-        cudaError_t err = cudaEventRecord(m->ev_fork, stream);
-        return err == cudaSuccess ? cudaStreamWaitEvent(m->side_stream, m->ev_fork, 0) : err;
-      };
-      if (ck.pool_cls) {
-        // first-token attention straight from the layers' inputs: beside the wave's kernels from its start
-        cudaStream_t cls_stream = beside ? m->side_stream : stream;
-        if (beside) MT_LAUNCH(fork(), "forking the side stream");
-        MT_TIMED(MT_CLASS_ATTENTION, launch_cls_pool(ck.cls_pool, cls_stream), "first-token attention kernels");
-        MT_TIMED(MT_CLASS_ATTENTION, launch_gemm(ck.cls_v, kEpiBias, m->sm_count, cls_stream), "first-token value projection");
-        if (beside) {
-          MT_LAUNCH(cudaEventRecord(m->ev_join, m->side_stream), "joining the side stream");
-          side_pending = true;
-        }
-      }
       if (ck.fused_qkv)
         MT_TIMED(MT_CLASS_QKV, launch_qkv_attention(ck.qa, m->sm_count, stream), "QKV projection + attention kernel");
       if (ck.qkv.n_groups > 0)
         MT_TIMED(MT_CLASS_QKV, launch_gemm(ck.qkv, kEpiBias, m->sm_count, stream), "QKV GEMM");
-      if (beside && !ck.pool_cls) {
-        MT_LAUNCH(fork(), "forking the side stream");
+      if (beside) {
+        MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
+        MT_LAUNCH(cudaStreamWaitEvent(m->side_stream, m->ev_fork, 0), "forking the side stream");
         MT_LAUNCH(launch_cls_attention(ck.attn_cls, m->side_stream), "first-token attention kernel");
         MT_LAUNCH(cudaEventRecord(m->ev_join, m->side_stream), "joining the side stream");
         side_pending = true;
       }
       if (ck.full.count > 0 && !ck.fused_qkv) MT_TIMED(MT_CLASS_ATTENTION, launch_attention(ck.attn, stream), "attention kernel");
-      if (ck.n_cls > 0 && !beside && !ck.pool_cls)
+      if (ck.n_cls > 0 && !beside)
         MT_TIMED(MT_CLASS_ATTENTION, launch_cls_attention(ck.attn_cls, stream), "first-token attention kernel");
       if (ck.full.count > 0) MT_TAIL(&ck.full);
       for (const DumpCopy& d : ck.dumps)
@@ -1689,6 +1726,20 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
                                   d.compact ? static_cast<size_t>(batch) * m->trunk.hidden * sizeof(bf16) : act_used,
                                   cudaMemcpyDeviceToDevice, stream),
                   "debug capture");
+    } else if (st.kind == 4) {
+      st.cls_pool.lengths = d_lengths;
+      const bool beside = st.beside && m->overlap_cls && m->side_stream != nullptr && !m->profile;
+      cudaStream_t on = beside ? m->side_stream : stream;
+      if (beside) {
+        MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
+        MT_LAUNCH(cudaStreamWaitEvent(on, m->ev_fork, 0), "forking the side stream");
+      }
+      MT_TIMED(MT_CLASS_ATTENTION, launch_cls_pool(st.cls_pool, on), "first-token attention kernels");
+      MT_TIMED(MT_CLASS_ATTENTION, launch_gemm(st.cls_v, kEpiBias, m->sm_count, on), "first-token value projection");
+      if (beside) {
+        MT_LAUNCH(cudaEventRecord(m->ev_join, on), "joining the side stream");
+        pool_pending = true;
+      }
     } else if (st.kind == 2) {
       MT_TAIL(&st.tail);
       for (const DumpCopy& d : st.dumps)
@@ -1715,7 +1766,7 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
             MT_LAUNCH(cudaEventRecord(reinterpret_cast<cudaEvent_t>(task_events[t]), stream), "recording a task event");
     }
   }
-  if (side_pending) MT_LAUNCH(cudaStreamWaitEvent(stream, m->ev_join, 0), "joining the side stream");
+  if (side_pending || pool_pending) MT_LAUNCH(cudaStreamWaitEvent(stream, m->ev_join, 0), "joining the side stream");
 #undef MT_TAIL
 #undef MT_TIMED
 #undef MT_LAUNCH
