@@ -30,8 +30,15 @@
 namespace mt {
 namespace {
 
-constexpr int kNumEpilogueWarps = 8;
-constexpr int kGemmThreads = 32 * (2 + kNumEpilogueWarps);
+// Epilogue warps of a CTA.  bf16 results of wide pair tiles: 16 warps, each one chunk of 64 columns of the tile with a staging
+// buffer of its own.  With K = 768 a tile's main loop is some 9 thousand clocks, and eight warps with two chunks each
+// - GELU is 16 clocks of the special-function unit per element, and two warps per scheduler cannot hide the trips to tensor memory,
+// staging and bias in between - took as long: 32768 x 3072 x 768 190 -> 128 us with GELU, 159 -> 121 us without; 256 x 128
+// tokens 2.47 -> 2.14 ms of FFN-up projections per forward.
+__host__ __device__ constexpr int gemm_epilogue_warps(int bn, bool pair, int epi) {
+  return pair && bn >= 192 && (epi == kEpiBias || epi == kEpiBiasGelu) ? 16 : 8;
+}
+__host__ __device__ constexpr int gemm_threads(int bn, bool pair, int epi) { return 32 * (2 + gemm_epilogue_warps(bn, pair, epi)); }
 
 constexpr int kStagingBytes = 4096;  // 32 rows x 128 bytes, one epilogue chunk of one warp
 // Shared memory of a CTA: the ring of operand stages, the epilogue warps' staging buffers, bookkeeping.
@@ -55,18 +62,20 @@ __host__ __device__ constexpr int gemm_b_bytes(int bn, bool pair, int low = 0) {
   return (pair ? bn / 2 : bn) * kGemmBlockK * 2 * (low ? kGemmLowKBlocks : 1);
 }
 __host__ __device__ constexpr int gemm_staging_bufs(int bn, bool pair, int epi) {
-  return epi == kEpiBiasResidual ? 2 : ((bn == 256 && !pair) ? 1 : MT_GEMM_NBUF);
+  return epi == kEpiBiasResidual ? 2 : (((bn == 256 && !pair) || gemm_epilogue_warps(bn, pair, epi) == 16) ? 1 : MT_GEMM_NBUF);
 }
 // Epilogue warps with rows to work on: all eight, or (LOW) those whose quarter of tensor memory the tile's rows reach.
-__host__ __device__ constexpr int gemm_staging_warps(int low) { return low ? kNumEpilogueWarps / 4 * (low / 32) : kNumEpilogueWarps; }
+__host__ __device__ constexpr int gemm_staging_warps(int bn, bool pair, int epi, int low) {
+  return low ? 2 * (low / 32) : gemm_epilogue_warps(bn, pair, epi);
+}
 __host__ __device__ constexpr int gemm_stages(int bn, bool pair, int epi, int low = 0) {
-  const int room = kSmemLimit - kBookBytes - gemm_staging_warps(low) * gemm_staging_bufs(bn, pair, epi) * kStagingBytes;
+  const int room = kSmemLimit - kBookBytes - gemm_staging_warps(bn, pair, epi, low) * gemm_staging_bufs(bn, pair, epi) * kStagingBytes;
   const int s = room / (gemm_a_bytes(low) + gemm_b_bytes(bn, pair, low));
   return s > 8 ? 8 : s;
 }
 __host__ __device__ constexpr int gemm_smem_bytes(int bn, bool pair, int epi, int low = 0) {
   return gemm_stages(bn, pair, epi, low) * (gemm_a_bytes(low) + gemm_b_bytes(bn, pair, low)) +
-         gemm_staging_warps(low) * gemm_staging_bufs(bn, pair, epi) * kStagingBytes + kBookBytes;
+         gemm_staging_warps(bn, pair, epi, low) * gemm_staging_bufs(bn, pair, epi) * kStagingBytes + kBookBytes;
 }
 
 // ---- the kernel -------------------------------------------------------------------------------
@@ -87,7 +96,7 @@ __host__ __device__ constexpr int gemm_smem_bytes(int bn, bool pair, int epi, in
 // accumulator complete 2.8 us after the dependency wait against 3.3 with 128-row tiles of the same width, results bf16
 // 0.6 us later (straight from registers) against 1.1 to 1.7.
 template <int BN, int EPI, bool PAIR, bool FP8 = false, int LOW = 0>
-__global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __grid_constant__ GemmParams p) {
+__global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI), 1) gemm_bf16_tcgen05(const __grid_constant__ GemmParams p) {
   static_assert(!FP8 || !PAIR, "the 8-bit operands run as single CTAs");
   constexpr int KB_ELEMS = FP8 ? 2 * kGemmBlockK : kGemmBlockK;   // elements of K in a 128-byte row
   static_assert(LOW == 0 || LOW == 64 || LOW == 32, "tile heights implemented: 128, 64, 32");
@@ -99,8 +108,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
   constexpr int NBUF = gemm_staging_bufs(BN, PAIR, EPI);
   constexpr int TILE_M = PAIR ? 2 * kGemmBlockM : (LOW ? LOW : kGemmBlockM);
   constexpr int MMA_M = LOW ? kGemmBlockM : TILE_M;
-  constexpr int STAGING_WARPS = gemm_staging_warps(LOW);
-  constexpr int ACC_ARRIVALS = PAIR ? 2 * kNumEpilogueWarps : kNumEpilogueWarps;
+  constexpr int STAGING_WARPS = gemm_staging_warps(BN, PAIR, EPI, LOW);
+  constexpr int EPI_WARPS = gemm_epilogue_warps(BN, PAIR, EPI);
+  constexpr int ACC_ARRIVALS = PAIR ? 2 * EPI_WARPS : EPI_WARPS;
   constexpr uint32_t TMEM_COLS = BN == 64 ? 128 : (BN == 128 ? 256 : 512);  // two accumulators; a power of two >= 32
   static_assert(BN == 64 || BN == 128 || BN == 192 || BN == 256, "tile widths implemented: 64, 128, 192, 256");
   static_assert(BN != 64 || !PAIR, "64-wide tiles (launches of a few rows) run as single CTAs");
@@ -110,14 +120,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sA = smem_u32(smem);
   const uint32_t sB = sA + STAGES * A_BYTES;
-  const uint32_t sStage = sB + STAGES * B_BYTES;          // kNumEpilogueWarps x NBUF x 4 KB
+  const uint32_t sStage = sB + STAGES * B_BYTES;          // EPI_WARPS x NBUF x 4 KB
   uint8_t* book = smem + STAGES * (A_BYTES + B_BYTES) + STAGING_WARPS * NBUF * kStagingBytes;
   const uint32_t bar_full = smem_u32(book);               // STAGES x 8 bytes
   const uint32_t bar_empty = bar_full + 8 * STAGES;       // STAGES x 8 bytes
   const uint32_t bar_acc_full = bar_empty + 8 * STAGES;   // 2 x 8 bytes
   const uint32_t bar_acc_empty = bar_acc_full + 16;       // 2 x 8 bytes
-  const uint32_t bar_res = bar_acc_empty + 16;            // kNumEpilogueWarps x 2 x 8 bytes
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(book + 8 * (2 * STAGES + 4 + 2 * kNumEpilogueWarps));
+  const uint32_t bar_res = bar_acc_empty + 16;            // EPI_WARPS x 2 x 8 bytes
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(book + 8 * (2 * STAGES + 4 + 2 * EPI_WARPS));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5;
@@ -139,7 +149,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
       mbar_init(bar_acc_full + 8 * a, 1);
       mbar_init(bar_acc_empty + 8 * a, ACC_ARRIVALS);
     }
-    for (int i = 0; i < 2 * kNumEpilogueWarps; ++i) mbar_init(bar_res + 8 * i, 1);
+    for (int i = 0; i < 2 * EPI_WARPS; ++i) mbar_init(bar_res + 8 * i, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -319,7 +329,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
     const int e = warp - 2;
     const int quarter = warp & 3;                       // TMEM lanes this warp may read
     const int col_group = e >> 2;                       // which share of the column chunks
-    constexpr int COL_GROUPS = kNumEpilogueWarps / 4;
+    constexpr int COL_GROUPS = EPI_WARPS / 4;
     constexpr int CHUNK_COLS = (LOW || EPI == kEpiBiasResidual || EPI == kEpiBiasTanhF32 || EPI == kEpiPartialF32) ? 32 : 64;
     constexpr int CHUNKS = BN / CHUNK_COLS;
     const bool has_rows = LOW == 0 || quarter < LOW / 32;                // (LOW) the others only keep the barriers' counts
@@ -379,6 +389,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
         for (int q = 0; q < 4; ++q)
           low_bias[LOW ? q : 0] = __ldg(reinterpret_cast<const uint4*>(p.group[g].bias + n0 + col_group * 32) + q);
       }
+      // the tile's bias (a line per 64 columns) into L1 ahead of its use: a trip to L2 for each chunk otherwise
+      if (!LOW && EPI != kEpiPartialF32 && lane < BN / 64) asm volatile("prefetch.global.L1 [%0];" ::"l"(p.group[g].bias + n0 + lane * 64));
       // warp-uniform decisions: the TMEM loads below are warp-collective
       if (!__all_sync(0xffffffffu, mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag))) break;
       tc_fence_after();
@@ -533,9 +545,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_tcgen05(const __gri
                 float x0 = __uint_as_float(v[q * 8 + 2 * j]) + bf16_lo(bw[j]);
                 float x1 = __uint_as_float(v[q * 8 + 2 * j + 1]) + bf16_hi(bw[j]);
                 if (EPI == kEpiBiasGelu) {
-                  x0 = gelu_fitted(x0);
-                  x1 = gelu_fitted(x1);
-                }
+                x0 = gelu_fitted(x0);
+                x1 = gelu_fitted(x1);
+              }
                 ow[j] = pack_bf16(x0, x1);
               }
               *reinterpret_cast<uint4*>(sbuf + staging_off(lane, half * 4 + q)) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
@@ -604,7 +616,7 @@ cudaError_t launch_one(const GemmParams& p, int sm_count, cudaStream_t stream) {
   const int workers_max = PAIR ? sm_count / 2 : sm_count;
   const int workers = tiles < workers_max ? tiles : workers_max;
   if (workers <= 0) return cudaSuccess;
-  return launch_kernel(kernel, dim3(PAIR ? 2 * workers : workers), dim3(kGemmThreads), gemm_smem_bytes(BN, PAIR, EPI, LOW), stream,
+  return launch_kernel(kernel, dim3(PAIR ? 2 * workers : workers), dim3(gemm_threads(BN, PAIR, EPI)), gemm_smem_bytes(BN, PAIR, EPI, LOW), stream,
                        p, PAIR ? 2u : 1u);
 }
 
