@@ -249,16 +249,14 @@ int mt_plan_cache_size(const mt_model* m);
  * for bit.
  * key "sm_limit" (>= 0, default 0 = all; any time): size the persistent GEMM grids for at most this many SMs
  * (for callers that share the GPU between several streams and want to leave room; measured no gain).
- * key "fused_ln" (0 never; 1 always, on 128-column tiles; 3 always, on 256-column tiles; 2 = chosen per launch, the
- * default: launches of at most "fused_ln_max_groups" (default 2) layers on all tokens - one layer on 128-column
- * tiles, more on 256-column tiles - and launches of at most "fused_ln_max_rows" (default 0) rows per layer; any
+ * key "fused_ln" (0 never; 1 always, on 128-column tiles; 3 always, on 256 x 256 tiles of CTA pairs; 2 = chosen per
+ * launch, the default: launches of at most "fused_ln_max_groups" (default 8) layers on all tokens whose row blocks fill
+ * the clusters that are resident at once, and launches of at most "fused_ln_max_rows" (default 0) rows per layer; any
  * time): the attention-output and FFN-down projections carry the LayerNorm that follows them: the CTAs holding the
- * column blocks of the same 128 rows form a thread-block cluster and exchange per-row statistics through
+ * column blocks of the same 128 or 256 rows form a thread-block cluster and exchange per-row statistics through
  * distributed shared memory, so the pre-normalisation sum never goes to global memory and no LayerNorm launch
  * follows.  All settings give the same bits (every LayerNorm of the library sums its row statistics over the same
- * 64-column segments in the same order, every projection sums over K in one sequence).  Measured: faster than the
- * separate launches while the launch is a single round of tiles (one or two layers of the 32 x 128 batch), slower
- * beyond, where the separate LayerNorm hides the same latencies behind full occupancy.
+ * 64-column segments in the same order, every projection sums over K in one sequence).
  * key "ffn_down_split" (0/1, default 1, any time): launches of at most 512 rows per layer (batch x seq up to
  * 4 x 128, and the first-token rows of the last branch layers for batches up to 512) run the FFN-down projection
  * as partial sums over four ranges of K - four times as many tiles, each a quarter as long -, and the attention-output
@@ -377,7 +375,7 @@ int mt_kernel_linear_layernorm(const void* d_x, const void* d_w, const void* d_b
                                const void* d_gamma, const void* d_beta, void* d_y, void* d_y_f32, int32_t M,
                                int32_t N, int32_t K, float eps, uint32_t* d_status, void* stream);
 /* The same with the accumulator tile width chosen by the caller: 128 (clusters of N / 128 CTAs, as above) or 256
- * (clusters of N / 256 CTAs; tcgen05.mma at its full rate, for launches with many row blocks).  Identical bits. */
+ * (256 x 256 tiles of CTA pairs, clusters of N / 256 pairs; for launches with many row blocks).  Identical bits. */
 int mt_kernel_linear_layernorm_tiles(const void* d_x, const void* d_w, const void* d_bias, const void* d_residual,
                                      const void* d_gamma, const void* d_beta, void* d_y, void* d_y_f32, int32_t M,
                                      int32_t N, int32_t K, float eps, int32_t tile_cols, uint32_t* d_status, void* stream);

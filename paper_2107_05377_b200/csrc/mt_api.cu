@@ -86,10 +86,9 @@ struct LayerTail {
   GemmParams attn_out, ffn_up, ffn_down;
   LayerNormParams ln1, ln2;
   int32_t count = 0;
-  // each residual GEMM together with the LayerNorm after it, as one cluster launch (option "fused_ln")
-  bool ln_fused = false;
-  bool ln_wide = false;      // ... on 128 x 256 accumulator tiles (clusters of N / 256): launches with many row blocks
-  bool down_fused = false;   // the FFN-down projection too (not with 8-bit operands: that GEMM is the plain kernel)
+  // each residual GEMM together with the LayerNorm after it, as one cluster launch (fused_ln_kind: 0 no, 1 on 128-column
+  // tiles, 2 on 256 x 256 tiles of CTA pairs); the FFN-down projection not with 8-bit operands (that GEMM is the plain kernel)
+  int32_t out_ln = 0, down_ln = 0;
   // launches of few rows: the FFN-down projection as partial sums over `down_splits` ranges of K, put together
   // (ranges in order, bias, residual) by the LayerNorm kernel after it
   int32_t down_splits = 1;
@@ -579,42 +578,44 @@ void choose_block_n(const mt_model* m, GemmParams* g, int epilogue, bool all_row
   g->block_n = gemm_block_n(g->N, epilogue, rows, groups < 1 ? 1 : groups, g->pair != 0, m->sm_count);
 }
 
-// Whether the residual GEMMs of `groups` layers carry their LayerNorm (see GemmLnParams): 0 no, 1 on 128-column
-// tiles (clusters of N / 128 CTAs), 2 on 256-column tiles (clusters of N / 256).  All three ways give the same bits,
-// so the default chooses by the launch.  The fused epilogue is a chain of latencies (statistics through the
-// cluster, staged stores) run by eight warps per CTA; it only beats the separate LayerNorm launch, which hides the
-// same latencies behind full occupancy, while the whole launch is a single round of tiles.  Measured on the
-// 32 x 128 batch (about 2409 valid rows per layer): one layer per launch - narrow tiles, 12.5 + 23.4 us against
-// 8.8 + 6 + 20.1 + 6 us; two layers - wide tiles, 18.2 + 32.8 us against 18.9 + 40.1 us for the narrow ones; three
-// layers - separate launches, 15 + 8 + 40 + 8 us against 25 + 60 us (narrow) or 31 + 62 us (wide).
+// Whether the residual GEMMs of `groups` layers carry their LayerNorm (see GemmLnParams): 0 no, 1 on 128-column tiles
+// (clusters of N / 128 CTAs over 128 rows), 2 on 256 x 256 tiles of CTA pairs (clusters of N / 256 pairs over 256 rows).
+// All three ways give the same bits, so the default chooses by the launch.  The row blocks are dealt out in rounds over the
+// clusters that are resident at once (22 of six CTAs), and the epilogue of the last round - a chain of latencies: residual,
+// statistics through the cluster, staged stores - is not hidden behind anything, so fusing pays while the rounds are
+// well filled; the separate GEMM's tiles are smaller and a LayerNorm launch hides its latencies behind full occupancy, but
+// the pair costs 20 bytes of memory traffic per element against 12.
 // The first-token tails (a few rows per layer) keep the separate launches unless fused_ln_max_rows says otherwise.
 int fused_ln_kind(const mt_model* m, int32_t groups, int64_t rows) {
   if (groups < 1 || !gemm_ln_supported(m->trunk.hidden) || m->fused_ln == 0) return 0;
   if (m->fused_ln == 1) return 1;
   if (m->fused_ln == 3) return 2;
   if (rows <= m->fused_ln_max_rows) return 1;
-  if (rows <= m->max_batch || groups > m->fused_ln_max_groups) return 0;   // a first-token tail, or many layers
+  if (rows <= m->max_batch || groups > m->fused_ln_max_groups) return 0;   // a first-token tail, or too many layers
   // few rows in all (small batches): the row-wise LayerNorm is a 3 us launch and the plain GEMM has the shorter
   // epilogue (measured at 128 and 512 rows: 6.9 + 2.7 against 10.8 us, 17.1 + 2.7 against 21.3 us)
   int64_t in_use = rows;
   if (m->pack_tokens && m->expected_tokens > 0 && m->expected_tokens < in_use) in_use = m->expected_tokens;
   if (in_use * groups <= 1024) return 0;
-  if (m->d_workspace == nullptr) return groups == 1 ? 1 : 2;   // (the device is not known yet)
-  // The row blocks are dealt out in rounds over the clusters that are resident at once (22 of six CTAs, 45 of three), and a
-  // block's epilogue is not hidden behind anything in the last round: the fused launch is the faster one while the rounds
-  // are well filled.  One layer, blocks of 128 rows, us per forward of seven layers, fused / separate: 10 blocks 414 / 396,
-  // 12: 419 / 404, 16: 466 / 497, 20: 502 / 545, 24 (two rounds): 586 / 506, 32: 638 / 610, 40: 739 / 779, 64: 1098 / 1121.
-  // (With ragged lengths fewer rows are in use than the launch is planned for - 32 blocks planned, 18 in use: 1683 / 1730
-  // for the 21-task tree - hence the line at 70 and not at 80 of 100 for more than one round.)  Two layers (wide tiles),
-  // forwards of the eight-task tree: 10 + 10 blocks 790 / 772, 18 + 18: 1052 / 1048, 20 + 20: 1114 / 1132.
+  if (m->d_workspace == nullptr) return groups == 1 ? 1 : (groups == 2 ? 2 : 0);   // (the device is not known yet)
+  // One layer in a single round of narrow tiles, blocks of 128 rows, us per forward of seven layers, fused / separate: 10
+  // blocks 414 / 396, 12: 419 / 404, 16: 466 / 497, 20: 502 / 545; two rounds 24: 586 / 506, 32: 638 / 610, 40: 739 / 779.
+  // Pairs, the same forward, blocks of 256 rows, pairs / narrow / separate: 17 of a round of 22 901 / 959 / 921, 20: 1005 /
+  // 1070 / 1119, 24 (two rounds): 1432 / 1282 / 1238, 28: 1580 / 1469 / 1467, 40: 1829 / 1996 / 2043.  Several layers: 21
+  // tasks 32 x 128, 16 blocks each: 1531 from the line at 75 of 100, 1618 with it at 70; 256 x 128 9.31 ms / 9.40 / 9.75 (there
+  // the memory traffic is energy, which sets the clock).  With ragged lengths fewer rows are in use than the launch is
+  // planned for, unless the caller has said how many: two layers of 10 planned blocks, 5 in use: 1023 / 990 separate - hence
+  // the higher line for several layers in one round, and narrow tiles for 32 planned blocks of 128, 18 in use (1683 / 1730).
   const int64_t tiles = (in_use + kGemmBlockM - 1) / kGemmBlockM * groups;
-  const int64_t fit = groups == 1 ? gemm_ln_resident(m->trunk.hidden) : gemm_ln_wide_resident(m->trunk.hidden);
-  if (fit < 1) return 0;
-  const int64_t rounds = (tiles + fit - 1) / fit;
-  if (groups == 1) return 100 * tiles >= (rounds == 1 ? 64 : 70) * rounds * fit ? 1 : 0;
-  return 100 * tiles >= 85 * rounds * fit ? 2 : 0;
+  const int64_t fit = gemm_ln_resident(m->trunk.hidden), fit_pair = gemm_ln_pair_resident(m->trunk.hidden);
+  if (fit < 1 || fit_pair < 1) return 0;
+  if (groups == 1 && tiles <= fit) return 100 * tiles >= 64 * fit ? 1 : 0;
+  const int64_t tiles_pair = (in_use + 2 * kGemmBlockM - 1) / (2 * kGemmBlockM) * groups;
+  const int64_t rounds_pair = (tiles_pair + fit_pair - 1) / fit_pair;
+  const bool rows_known = !m->pack_tokens || m->expected_tokens > 0;
+  if (100 * tiles_pair >= (rounds_pair == 1 && groups > 1 && !rows_known ? 95 : 75) * rounds_pair * fit_pair) return 2;
+  return groups == 1 && tiles <= 2 * fit && 100 * tiles >= 70 * 2 * fit ? 1 : 0;
 }
-bool use_fused_ln(const mt_model* m, int32_t groups, int64_t rows) { return fused_ln_kind(m, groups, rows) != 0; }
 // Ranges the K of the FFN-down projection is split into.  A launch of few rows has few tiles, and each walks
 // K = F by itself (48 k-blocks one after the other for BERT-base) while most SMs have none: four ranges, each a
 // tile of its own, shorten that chain fourfold, and the LayerNorm kernel that follows adds the four partial
@@ -638,7 +639,7 @@ int32_t out_split_count(const mt_model* m, int64_t rows) {
 }
 // Launches of steps 3-7 for `groups` layers (before mt_bind_memory; afterwards plans are built and counted).
 int32_t tail_launches(const mt_model* m, int32_t groups, int64_t rows) {
-  const bool fused = use_fused_ln(m, groups, rows);
+  const bool fused = fused_ln_kind(m, groups, rows) != 0;
   // 8-bit operands: two quantisations, and the FFN-down projection keeps its LayerNorm as a launch of its own;
   // so does a projection whose K is split
   return (fused ? 3 : 5) + (m->fp8 ? 2 + (fused ? 1 : 0) : 0) + (fused && down_split_count(m, rows) > 1 ? 1 : 0);
@@ -698,10 +699,9 @@ void init_tail(const mt_model* m, LayerTail* t, int32_t rows, bool all_rows_vali
   t->ln1.hidden = t->ln2.hidden = H;
   t->ln1.eps = t->ln2.eps = m->trunk.ln_eps;
   t->count = 0;
-  t->ln_fused = use_fused_ln(m, groups, rows) && t->out_splits == 1;
-  t->ln_wide = fused_ln_kind(m, groups, rows) == 2;
-  t->down_fused = t->ln_fused && !m->fp8 && t->down_splits == 1;
-  if (t->ln_fused) {
+  t->out_ln = t->out_splits == 1 ? fused_ln_kind(m, groups, rows) : 0;
+  t->down_ln = !m->fp8 && t->out_splits == 1 && t->down_splits == 1 ? fused_ln_kind(m, groups, rows) : 0;
+  if (t->out_ln != 0 || t->down_ln != 0) {
     auto init_ln = [&](GemmLnParams* g, int32_t K) {
       memset(g, 0, sizeof(*g));
       g->M = rows; g->N = H; g->K = K;
@@ -770,14 +770,12 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
   t->ln2.y[i] = out; t->ln2.y32[i] = out32;
   t->count = i + 1;
   t->attn_out.n_groups = t->ffn_up.n_groups = t->ffn_down.n_groups = t->ln1.n_groups = t->ln2.n_groups = t->count;
-  if (t->ln_fused) {
+  if (t->out_ln != 0 || t->down_ln != 0) {
     auto set_ln = [&](GemmLnParams* g, const void* x, size_t w, size_t b, size_t gamma, size_t beta, const float* res,
                       bf16* y, float* y32) -> cudaError_t {
       cudaError_t err;
       if ((err = make_tmap(&g->tmap_x[i], x, g->M, g->K, kGemmBlockM, kGemmBlockK, false)) != cudaSuccess) return err;
       if ((err = make_tmap(&g->tmap_w[i], w_ptr(m, w), g->N, g->K, 128, kGemmBlockK, false)) != cudaSuccess) return err;
-      if ((err = make_tmap(&g->tmap_w256[i], w_ptr(m, w), g->N, g->K, 256, kGemmBlockK, false)) != cudaSuccess) return err;
-      g->residual[i] = res;
       if ((err = make_tmap(&g->tmap_res[i], res, g->M, g->N, 32, 32, true)) != cudaSuccess) return err;
       if ((err = make_tmap(&g->tmap_y[i], y, g->M, g->N, 32, 64, false)) != cudaSuccess) return err;
       if ((err = make_tmap(&g->tmap_y32[i], y32, g->M, g->N, 32, 32, true)) != cudaSuccess) return err;
@@ -788,7 +786,7 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
     // (a state is its bf16 copy followed by room for its fp32 copy: the fp32 result always has a home)
     float* out32_home = out32 != nullptr ? out32 : f32_of(m, out);
     if ((e = set_ln(&t->attn_out_ln, ctx, lo->wo, lo->bo, lo->ln1_g, lo->ln1_b, residual, h1, h1_32)) != cudaSuccess) return e;
-    if (t->down_fused &&
+    if (t->down_ln != 0 &&
         (e = set_ln(&t->ffn_down_ln, f, lo->w2, lo->b2, lo->ln2_g, lo->ln2_b, h1_32, out, out32_home)) != cudaSuccess)
       return e;
   }
@@ -1010,7 +1008,7 @@ std::vector<int32_t> cls_tasks_after_wave(const mt_model* m, const Schedule& s, 
 // Kernel launches of a built plan: the row starts, the embedding, and what mt_forward_tokens does for every step.
 int32_t plan_launches(const Plan& plan) {
   auto tail = [](const LayerTail& t) {
-    return t.count == 0 ? 0 : (t.ln_fused ? 1 : 2) + 1 + (t.down_fused ? 1 : 2) + (t.fp8 ? 2 : 0);
+    return t.count == 0 ? 0 : (t.out_ln != 0 ? 1 : 2) + 1 + (t.down_ln != 0 ? 1 : 2) + (t.fp8 ? 2 : 0);
   };
   int32_t n = 2;
   for (const PlanStep& st : plan.steps) {
@@ -1207,7 +1205,7 @@ int mt_create(const mt_trunk_config* trunk, const mt_task_config* tasks, int32_t
   m->side_stream = nullptr;
   m->ev_fork = m->ev_join = nullptr;
   m->fused_ln = 2;
-  m->fused_ln_max_groups = 2;
+  m->fused_ln_max_groups = kMaxGroups;
   m->ffn_down_split = 1;
   m->fused_ln_max_rows = 0;
   m->last_lengths = nullptr;
@@ -1648,9 +1646,9 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
 #define MT_TAIL(tail)                                                                                                  \
   do {                                                                                                                 \
     LayerTail* t_ = (tail);                                                                                            \
-    if (t_->ln_fused) {                                                                                                \
-      MT_TIMED(MT_CLASS_ATTN_OUT, t_->ln_wide ? launch_gemm_ln_wide(t_->attn_out_ln, stream)                          \
-                                              : launch_gemm_ln(t_->attn_out_ln, stream),                              \
+    if (t_->out_ln != 0) {                                                                                             \
+      MT_TIMED(MT_CLASS_ATTN_OUT, t_->out_ln == 2 ? launch_gemm_ln_pair(t_->attn_out_ln, stream)                       \
+                                                  : launch_gemm_ln(t_->attn_out_ln, stream),                           \
                "attention output GEMM + LayerNorm");                                                                   \
     } else {                                                                                                           \
       MT_TIMED(MT_CLASS_ATTN_OUT, launch_gemm(t_->attn_out, t_->out_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual,    \
@@ -1660,9 +1658,9 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
     if (t_->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_h1, stream), "quantising the FFN input");         \
     MT_TIMED(MT_CLASS_FFN_UP, launch_gemm(t_->ffn_up, kEpiBiasGelu, m->sm_count, stream), "FFN up GEMM");              \
     if (t_->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_f, stream), "quantising the FFN intermediate");   \
-    if (t_->down_fused) {                                                                                              \
-      MT_TIMED(MT_CLASS_FFN_DOWN, t_->ln_wide ? launch_gemm_ln_wide(t_->ffn_down_ln, stream)                          \
-                                              : launch_gemm_ln(t_->ffn_down_ln, stream),                              \
+    if (t_->down_ln != 0) {                                                                                            \
+      MT_TIMED(MT_CLASS_FFN_DOWN, t_->down_ln == 2 ? launch_gemm_ln_pair(t_->ffn_down_ln, stream)                      \
+                                                   : launch_gemm_ln(t_->ffn_down_ln, stream),                          \
                "FFN down GEMM + LayerNorm");                                                                           \
     } else {                                                                                                           \
       MT_TIMED(MT_CLASS_FFN_DOWN, launch_gemm(t_->ffn_down, t_->down_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual,   \
@@ -1965,7 +1963,6 @@ int mt_kernel_linear_layernorm_tiles(const void* d_x, const void* d_w, const voi
   p.n_groups = 1; p.M = M; p.N = N; p.K = K; p.eps = eps; p.status = d_status;
   if (make_tmap(&p.tmap_x[0], d_x, M, K, kGemmBlockM, kGemmBlockK, false) != cudaSuccess ||
       make_tmap(&p.tmap_w[0], d_w, N, K, 128, kGemmBlockK, false) != cudaSuccess ||
-      make_tmap(&p.tmap_w256[0], d_w, N, K, 256, kGemmBlockK, false) != cudaSuccess ||
       make_tmap(&p.tmap_res[0], d_residual, M, N, 32, 32, true) != cudaSuccess ||
       make_tmap(&p.tmap_y[0], d_y, M, N, 32, 64, false) != cudaSuccess ||
       make_tmap(&p.tmap_y32[0], d_y_f32, M, N, 32, 32, true) != cudaSuccess)
@@ -1973,8 +1970,7 @@ int mt_kernel_linear_layernorm_tiles(const void* d_x, const void* d_w, const voi
   p.bias[0] = static_cast<const bf16*>(d_bias);
   p.gamma[0] = static_cast<const bf16*>(d_gamma);
   p.beta[0] = static_cast<const bf16*>(d_beta);
-  p.residual[0] = static_cast<const float*>(d_residual);
-  const cudaError_t e = tile_cols == 256 ? launch_gemm_ln_wide(p, as_stream(stream)) : launch_gemm_ln(p, as_stream(stream));
+  const cudaError_t e = tile_cols == 256 ? launch_gemm_ln_pair(p, as_stream(stream)) : launch_gemm_ln(p, as_stream(stream));
   return e == cudaSuccess ? MT_OK : MT_ERR_CUDA;
 }
 

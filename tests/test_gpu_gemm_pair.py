@@ -1,0 +1,51 @@
+"""GEMMs on pairs of CTAs where their tiles can go wrong - one row, rows around a CTA's 128 and a pair's 256, more row blocks
+than clusters fit the GPU at once, fewer k-blocks than stages, both cluster sizes: the same bits as the single CTAs (and the
+separate LayerNorm) that other tests hold against the oracle, and nothing written beyond the last row."""
+import pytest
+import torch
+
+from paper_2107_05377_b200 import binding as mt
+
+pytestmark = pytest.mark.gpu
+
+
+def draw(M, N, K, seed=0):
+    gen = torch.Generator(device="cuda").manual_seed(seed + M)
+    rnd = lambda *shape, scale=1.0: torch.randn(*shape, device="cuda", generator=gen) * scale   # noqa: E731
+    return (rnd(M, K).bfloat16(), rnd(N, K, scale=0.05).bfloat16(), rnd(N).bfloat16(), rnd(M, N), rnd(N).bfloat16(),
+            rnd(N).bfloat16())
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 768, 64), (127, 768, 128), (128, 768, 192), (129, 768, 320), (255, 768, 768),
+                                   (257, 768, 768), (5633, 768, 64), (11265, 768, 256), (129, 1024, 64), (4097, 1024, 320)])
+def test_residual_and_layernorm_on_pair_tiles(M, N, K):
+    x, w, b, res, gamma, beta = draw(M, N, K)
+    y = torch.full((M + 3, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+    y32 = torch.full((M + 3, N), float("nan"), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    mt.mt_kernel_linear_layernorm(x, w, b, res, gamma, beta, y[:M], y32[:M], 1e-12, status=status, tile_cols=256)
+    u, z, z32 = torch.empty_like(res), torch.empty_like(y[:M]), torch.empty_like(res)
+    mt.mt_kernel_linear(x, w, b, res, u, 2)
+    mt.mt_kernel_layernorm(u, gamma, beta, z, 1e-12, y_f32=z32)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(y32[:M], z32) and torch.equal(y[:M], z)
+    assert torch.isnan(y[M:].float()).all() and torch.isnan(y32[M:]).all(), "rows beyond M were written"
+
+
+@pytest.mark.parametrize("block_n", [192, 256])
+@pytest.mark.parametrize("epilogue", [0, 1])
+@pytest.mark.parametrize("M,K", [(1, 64), (129, 768), (257, 64), (20000, 128)])
+def test_bf16_results_of_pair_tiles(M, K, epilogue, block_n):
+    N = 768
+    x, w, b, _, _, _ = draw(M, N, K, seed=1)
+    out = {}
+    for pair in (True, False):
+        out[pair] = torch.full((M + 3, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+        mt.lib().mt_kernel_linear_force_block_n(block_n if pair else 128)
+        try:
+            mt.mt_kernel_linear(x, w, b, None, out[pair][:M], epilogue, cta_pair=pair)
+        finally:
+            mt.lib().mt_kernel_linear_force_block_n(0)
+        assert torch.isnan(out[pair][M:].float()).all(), "rows beyond M were written"
+    assert torch.equal(out[True][:M], out[False][:M])
