@@ -314,15 +314,42 @@ __global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadParams p) 
   }
 }
 
-// Row-wise E4M3 quantisation (QuantParams): one warp per row; the row is read twice (bf16 from L2), first for
-// its largest magnitude, then to scale and convert.  Every decision is taken in fp32 with IEEE operations
+// Row-wise E4M3 quantisation (QuantParams): one warp per row, first for its largest magnitude, then to
+// scale and convert.  Every decision is taken in fp32 with IEEE operations
 // that no compiler option can change: scale = amax * (1/448), y = x / scale, code = cvt.rn.satfinite.e4m3.
 __device__ __forceinline__ uint32_t cvt_e4m3x2(float hi, float lo) {
   uint16_t r;
   asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
   return r;
 }
-__global__ void __launch_bounds__(kRowThreads) quantize_rows_kernel(const QuantParams p) {
+// x / scale rounded to nearest, from the correctly rounded reciprocal of scale: a product, its exact remainder and one
+// correction (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990: the result is the
+// correctly rounded quotient, as long as nothing under- or overflows and scale's significand is not all ones).  A
+// zero keeps the sign of x, which the correction would lose.
+__device__ __forceinline__ float divide_by(float x, float scale, float rcp) {
+  const float q = x * rcp;
+  return copysignf(fmaf(fmaf(-q, scale, x), rcp, q), x);
+}
+template <bool EXACT>
+__device__ __forceinline__ uint2 quantize8(const uint4& u, float scale, float rcp) {
+  float f[8];
+  unpack8(u, f);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) f[i] = EXACT ? __fdiv_rn(f[i], scale) : divide_by(f[i], scale, rcp);
+  return make_uint2(cvt_e4m3x2(f[1], f[0]) | (cvt_e4m3x2(f[3], f[2]) << 16), cvt_e4m3x2(f[5], f[4]) | (cvt_e4m3x2(f[7], f[6]) << 16));
+}
+__device__ __forceinline__ __nv_bfloat162 amax8(const uint4& u, __nv_bfloat162 amax) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) amax = __hmax2(amax, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&w[i])));
+  return amax;
+}
+// V: 16-byte vectors of a row per lane, held in registers between the two steps (0: any length, read twice).  A row of
+// 3072 values then has twelve loads per lane in flight instead of one or two and is read once, and the division is three
+// multiply-adds instead of some ten instructions and a branch.  20000 rows of 3072 values: 124 -> 58 us, of 768: 34 -> 16,
+// of 4096: 170 -> 79; forward of 64 x 128 tokens with 8-bit projections 1774 -> 1660 us, 4 x 64 622 -> 555.
+template <int V>
+__global__ void __launch_bounds__(kRowThreads, V >= 16 ? 3 : 4) quantize_rows_kernel(const QuantParams p) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = blockIdx.y;
   int rows = p.rows;
@@ -331,28 +358,32 @@ __global__ void __launch_bounds__(kRowThreads) quantize_rows_kernel(const QuantP
   grid_launch_dependents();
   const int row = blockIdx.x * (kRowThreads / 32) + warp;
   if (row >= rows) return;
-  const bf16* x = p.x[g] + static_cast<size_t>(row) * p.cols;
-  float amax = 0.f;
-  for (int c = lane * 8; c < p.cols; c += 256) {
-    float f[8];
-    unpack8(__ldg(reinterpret_cast<const uint4*>(x + c)), f);
+  const uint4* x = reinterpret_cast<const uint4*>(p.x[g] + static_cast<size_t>(row) * p.cols) + lane;
+  const int vectors = V > 0 ? V : p.cols / 256;
+  uint4 u[V > 0 ? V : 1];
+  __nv_bfloat162 amax2 = __float2bfloat162_rn(0.f);   // (bf16 magnitudes compare exactly)
+  if (V > 0) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) amax = fmaxf(amax, fabsf(f[i]));
+    for (int v = 0; v < V; ++v) u[v] = __ldg(x + v * 32);
+#pragma unroll
+    for (int v = 0; v < V; ++v) amax2 = amax8(u[v], amax2);
+  } else {
+    for (int v = 0; v < vectors; ++v) amax2 = amax8(__ldg(x + v * 32), amax2);
   }
+  float amax = fmaxf(__low2float(amax2), __high2float(amax2));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   const float scale = amax == 0.f ? 1.0f : __fmul_rn(amax, 1.0f / 448.0f);
   if (lane == 0) p.scale[g][row] = scale;
-  uint8_t* q = p.q[g] + static_cast<size_t>(row) * p.cols;
-  for (int c = lane * 8; c < p.cols; c += 256) {
-    float f[8];
-    unpack8(__ldg(reinterpret_cast<const uint4*>(x + c)), f);
+  uint2* q = reinterpret_cast<uint2*>(p.q[g] + static_cast<size_t>(row) * p.cols) + lane;
+  // (the quotients that decide a code are between 2^-10 and 448: with scale in this range no remainder underflows)
+  const bool plain = scale > 0x1p-60f && scale < 0x1p60f && (__float_as_uint(scale) & 0x7FFFFFu) != 0x7FFFFFu;
+  if (V > 0 && plain) {
+    const float rcp = __frcp_rn(scale);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) f[i] = __fdiv_rn(f[i], scale);
-    uint2 out;
-    out.x = cvt_e4m3x2(f[1], f[0]) | (cvt_e4m3x2(f[3], f[2]) << 16);
-    out.y = cvt_e4m3x2(f[5], f[4]) | (cvt_e4m3x2(f[7], f[6]) << 16);
-    *reinterpret_cast<uint2*>(q + c) = out;
+    for (int v = 0; v < (V > 0 ? V : 1); ++v) q[v * 32] = quantize8<false>(u[v], scale, rcp);
+  } else {
+    for (int v = 0; v < vectors; ++v) q[v * 32] = quantize8<true>(__ldg(x + v * 32), scale, 0.f);
   }
 }
 
@@ -428,7 +459,13 @@ cudaError_t launch_quantize_rows(const QuantParams& p, cudaStream_t stream) {
   if (p.n_groups < 1 || p.n_groups > kMaxGroups || p.rows < 1 || p.cols < 256 || p.cols % 256 != 0) return cudaErrorInvalidValue;
   const int rows_per_cta = kRowThreads / 32;
   dim3 grid((p.rows + rows_per_cta - 1) / rows_per_cta, p.n_groups);
-  return launch_kernel(quantize_rows_kernel, grid, dim3(kRowThreads), 0, stream, p);
+  switch (p.cols) {   // the hidden and FFN sizes of the two BERT models
+    case 768: return launch_kernel(quantize_rows_kernel<3>, grid, dim3(kRowThreads), 0, stream, p);
+    case 1024: return launch_kernel(quantize_rows_kernel<4>, grid, dim3(kRowThreads), 0, stream, p);
+    case 3072: return launch_kernel(quantize_rows_kernel<12>, grid, dim3(kRowThreads), 0, stream, p);
+    case 4096: return launch_kernel(quantize_rows_kernel<16>, grid, dim3(kRowThreads), 0, stream, p);
+    default: return launch_kernel(quantize_rows_kernel<0>, grid, dim3(kRowThreads), 0, stream, p);
+  }
 }
 
 cudaError_t launch_row_starts(const int32_t* lengths, int32_t batch, int32_t seq, int32_t packed, int32_t* row_start,
