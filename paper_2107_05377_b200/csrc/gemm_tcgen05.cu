@@ -30,15 +30,17 @@
 namespace mt {
 namespace {
 
-// Epilogue warps of a CTA.  bf16 results of wide pair tiles: 16 warps, each one chunk of 64 columns of the tile with a staging
-// buffer of its own.  With K = 768 a tile's main loop is some 9 thousand clocks, and eight warps with two chunks each
-// - GELU is 16 clocks of the special-function unit per element, and two warps per scheduler cannot hide the trips to tensor memory,
-// staging and bias in between - took as long: 32768 x 3072 x 768 190 -> 128 us with GELU, 159 -> 121 us without; 256 x 128
-// tokens 2.47 -> 2.14 ms of FFN-up projections per forward.
-__host__ __device__ constexpr int gemm_epilogue_warps(int bn, bool pair, int epi) {
-  return pair && bn >= 192 && (epi == kEpiBias || epi == kEpiBiasGelu) ? 16 : 8;
+// Epilogue warps of a CTA.  bf16 results of wide tiles: one warp per row quarter and chunk of 64 columns (12 at 192 columns, 16
+// at 256), each with a staging buffer of its own; the others eight.  With K = 768 a tile's main loop is some 9 thousand
+// clocks (of a pair; half of that with 8-bit operands), and eight warps with two chunks each - GELU is 16 clocks of the
+// special-function unit per element, and two warps per scheduler cannot hide the trips to tensor memory, staging and bias in
+// between - took as long: 32768 x 3072 x 768 190 -> 128 us with GELU, 159 -> 121 us without; 256 x 128 tokens 2.47 -> 2.14 ms of
+// FFN-up projections per forward; 12 x 128 on 192-column tiles 771 -> 764 us; 64 x 128 with 8-bit operands 1646 -> 1638.  Not
+// for bf16 on 256-column tiles of single CTAs, whose ring would lose its fourth stage (21 tasks 32 x 128: 1520 -> 1532).
+__host__ __device__ constexpr int gemm_epilogue_warps(int bn, bool pair, int epi, bool fp8) {
+  return epi != kEpiBias && epi != kEpiBiasGelu ? 8 : (bn == 192 ? 12 : (bn == 256 && (pair || fp8) ? 16 : 8));
 }
-__host__ __device__ constexpr int gemm_threads(int bn, bool pair, int epi) { return 32 * (2 + gemm_epilogue_warps(bn, pair, epi)); }
+__host__ __device__ constexpr int gemm_threads(int bn, bool pair, int epi, bool fp8) { return 32 * (2 + gemm_epilogue_warps(bn, pair, epi, fp8)); }
 
 constexpr int kStagingBytes = 4096;  // 32 rows x 128 bytes, one epilogue chunk of one warp
 // Shared memory of a CTA: the ring of operand stages, the epilogue warps' staging buffers, bookkeeping.
@@ -61,21 +63,21 @@ __host__ __device__ constexpr int gemm_a_bytes(int low = 0) {
 __host__ __device__ constexpr int gemm_b_bytes(int bn, bool pair, int low = 0) {
   return (pair ? bn / 2 : bn) * kGemmBlockK * 2 * (low ? kGemmLowKBlocks : 1);
 }
-__host__ __device__ constexpr int gemm_staging_bufs(int bn, bool pair, int epi) {
-  return epi == kEpiBiasResidual ? 2 : (((bn == 256 && !pair) || gemm_epilogue_warps(bn, pair, epi) == 16) ? 1 : MT_GEMM_NBUF);
+__host__ __device__ constexpr int gemm_staging_bufs(int bn, bool pair, int epi, bool fp8) {
+  return epi == kEpiBiasResidual ? 2 : (((bn == 256 && !pair) || gemm_epilogue_warps(bn, pair, epi, fp8) > 8) ? 1 : MT_GEMM_NBUF);
 }
 // Epilogue warps with rows to work on: all eight, or (LOW) those whose quarter of tensor memory the tile's rows reach.
-__host__ __device__ constexpr int gemm_staging_warps(int bn, bool pair, int epi, int low) {
-  return low ? 2 * (low / 32) : gemm_epilogue_warps(bn, pair, epi);
+__host__ __device__ constexpr int gemm_staging_warps(int bn, bool pair, int epi, bool fp8, int low) {
+  return low ? 2 * (low / 32) : gemm_epilogue_warps(bn, pair, epi, fp8);
 }
-__host__ __device__ constexpr int gemm_stages(int bn, bool pair, int epi, int low = 0) {
-  const int room = kSmemLimit - kBookBytes - gemm_staging_warps(bn, pair, epi, low) * gemm_staging_bufs(bn, pair, epi) * kStagingBytes;
+__host__ __device__ constexpr int gemm_stages(int bn, bool pair, int epi, bool fp8, int low = 0) {
+  const int room = kSmemLimit - kBookBytes - gemm_staging_warps(bn, pair, epi, fp8, low) * gemm_staging_bufs(bn, pair, epi, fp8) * kStagingBytes;
   const int s = room / (gemm_a_bytes(low) + gemm_b_bytes(bn, pair, low));
   return s > 8 ? 8 : s;
 }
-__host__ __device__ constexpr int gemm_smem_bytes(int bn, bool pair, int epi, int low = 0) {
-  return gemm_stages(bn, pair, epi, low) * (gemm_a_bytes(low) + gemm_b_bytes(bn, pair, low)) +
-         gemm_staging_warps(bn, pair, epi, low) * gemm_staging_bufs(bn, pair, epi) * kStagingBytes + kBookBytes;
+__host__ __device__ constexpr int gemm_smem_bytes(int bn, bool pair, int epi, bool fp8, int low = 0) {
+  return gemm_stages(bn, pair, epi, fp8, low) * (gemm_a_bytes(low) + gemm_b_bytes(bn, pair, low)) +
+         gemm_staging_warps(bn, pair, epi, fp8, low) * gemm_staging_bufs(bn, pair, epi, fp8) * kStagingBytes + kBookBytes;
 }
 
 // ---- the kernel -------------------------------------------------------------------------------
@@ -96,20 +98,20 @@ __host__ __device__ constexpr int gemm_smem_bytes(int bn, bool pair, int epi, in
 // accumulator complete 2.8 us after the dependency wait against 3.3 with 128-row tiles of the same width, results bf16
 // 0.6 us later (straight from registers) against 1.1 to 1.7.
 template <int BN, int EPI, bool PAIR, bool FP8 = false, int LOW = 0>
-__global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI), 1) gemm_bf16_tcgen05(const __grid_constant__ GemmParams p) {
+__global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16_tcgen05(const __grid_constant__ GemmParams p) {
   static_assert(!FP8 || !PAIR, "the 8-bit operands run as single CTAs");
   constexpr int KB_ELEMS = FP8 ? 2 * kGemmBlockK : kGemmBlockK;   // elements of K in a 128-byte row
   static_assert(LOW == 0 || LOW == 64 || LOW == 32, "tile heights implemented: 128, 64, 32");
   static_assert(LOW == 0 || (BN == 64 && !PAIR && !FP8), "low tiles: 64 columns, single CTAs, bf16");
-  constexpr int STAGES = gemm_stages(BN, PAIR, EPI, LOW);
+  constexpr int STAGES = gemm_stages(BN, PAIR, EPI, FP8, LOW);
   constexpr int A_BYTES = gemm_a_bytes(LOW);
   constexpr int KPS = LOW ? kGemmLowKBlocks : 1;         // k-blocks of a stage
   constexpr int B_BYTES = gemm_b_bytes(BN, PAIR, LOW);   // this CTA's part of the W tile
-  constexpr int NBUF = gemm_staging_bufs(BN, PAIR, EPI);
+  constexpr int NBUF = gemm_staging_bufs(BN, PAIR, EPI, FP8);
   constexpr int TILE_M = PAIR ? 2 * kGemmBlockM : (LOW ? LOW : kGemmBlockM);
   constexpr int MMA_M = LOW ? kGemmBlockM : TILE_M;
-  constexpr int STAGING_WARPS = gemm_staging_warps(BN, PAIR, EPI, LOW);
-  constexpr int EPI_WARPS = gemm_epilogue_warps(BN, PAIR, EPI);
+  constexpr int STAGING_WARPS = gemm_staging_warps(BN, PAIR, EPI, FP8, LOW);
+  constexpr int EPI_WARPS = gemm_epilogue_warps(BN, PAIR, EPI, FP8);
   constexpr int ACC_ARRIVALS = PAIR ? 2 * EPI_WARPS : EPI_WARPS;
   constexpr uint32_t TMEM_COLS = BN == 64 ? 128 : (BN == 128 ? 256 : 512);  // two accumulators; a power of two >= 32
   static_assert(BN == 64 || BN == 128 || BN == 192 || BN == 256, "tile widths implemented: 64, 128, 192, 256");
@@ -608,7 +610,7 @@ cudaError_t launch_one(const GemmParams& p, int sm_count, cudaStream_t stream) {
   auto kernel = gemm_bf16_tcgen05<BN, EPI, PAIR, FP8, LOW>;
   static PerDeviceOnce once;   // per instantiation
   cudaError_t err = per_device_once(once, [&](int) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(BN, PAIR, EPI, LOW));
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(BN, PAIR, EPI, FP8, LOW));
   });
   if (err != cudaSuccess) return err;
   constexpr int tile_m = PAIR ? 2 * kGemmBlockM : (LOW ? LOW : kGemmBlockM);
@@ -616,7 +618,7 @@ cudaError_t launch_one(const GemmParams& p, int sm_count, cudaStream_t stream) {
   const int workers_max = PAIR ? sm_count / 2 : sm_count;
   const int workers = tiles < workers_max ? tiles : workers_max;
   if (workers <= 0) return cudaSuccess;
-  return launch_kernel(kernel, dim3(PAIR ? 2 * workers : workers), dim3(gemm_threads(BN, PAIR, EPI)), gemm_smem_bytes(BN, PAIR, EPI, LOW), stream,
+  return launch_kernel(kernel, dim3(PAIR ? 2 * workers : workers), dim3(gemm_threads(BN, PAIR, EPI, FP8)), gemm_smem_bytes(BN, PAIR, EPI, FP8, LOW), stream,
                        p, PAIR ? 2u : 1u);
 }
 

@@ -1,4 +1,4 @@
-"""GEMMs on pairs of CTAs where their tiles can go wrong - one row, rows around a CTA's 128 and a pair's 256, more row blocks
+"""GEMMs on pairs of CTAs and on wide tiles where their tiles can go wrong - one row, rows around a CTA's 128 and a pair's 256, more row blocks
 than clusters fit the GPU at once, fewer k-blocks than stages, both cluster sizes: the same bits as the single CTAs (and the
 separate LayerNorm) that other tests hold against the oracle, and nothing written beyond the last row."""
 import pytest
@@ -36,16 +36,17 @@ def test_residual_and_layernorm_on_pair_tiles(M, N, K):
 @pytest.mark.parametrize("block_n", [192, 256])
 @pytest.mark.parametrize("epilogue", [0, 1])
 @pytest.mark.parametrize("M,K", [(1, 64), (129, 768), (257, 64), (20000, 128)])
-def test_bf16_results_of_pair_tiles(M, K, epilogue, block_n):
+def test_bf16_results_of_wide_tiles(M, K, epilogue, block_n):
     N = 768
     x, w, b, _, _, _ = draw(M, N, K, seed=1)
     out = {}
-    for pair in (True, False):
-        out[pair] = torch.full((M + 3, N), float("nan"), dtype=torch.bfloat16, device="cuda")
-        mt.lib().mt_kernel_linear_force_block_n(block_n if pair else 128)
+    for pair, bn in ((True, block_n), (False, block_n), (False, 128)):
+        out[pair, bn] = torch.full((M + 3, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+        mt.lib().mt_kernel_linear_force_block_n(bn)
         try:
-            mt.mt_kernel_linear(x, w, b, None, out[pair][:M], epilogue, cta_pair=pair)
+            mt.mt_kernel_linear(x, w, b, None, out[pair, bn][:M], epilogue, cta_pair=pair)
         finally:
             mt.lib().mt_kernel_linear_force_block_n(0)
-        assert torch.isnan(out[pair][M:].float()).all(), "rows beyond M were written"
-    assert torch.equal(out[True][:M], out[False][:M])
+        assert torch.isnan(out[pair, bn][M:].float()).all(), "rows beyond M were written"
+    assert torch.equal(out[True, block_n][:M], out[False, 128][:M])
+    assert torch.equal(out[False, block_n][:M], out[False, 128][:M])
