@@ -87,11 +87,20 @@ def tasks_of(cfg):
 
 def gemm_flops_per_forward(cfg, n_layers, m_rows, first_token_layers=0, batch=0):
     """FLOPs of the four linear maps of n_layers encoder layers over m_rows tokens.  Of those layers,
-    first_token_layers (the last layer of each task branch) need the Q/K/V projection on every token
-    but the other three maps only on the first token of each of the `batch` sequences."""
+    first_token_layers (the last layer of each task branch) need the attention output and FFN maps only on the first
+    token of each of the `batch` sequences; their attention projects neither keys nor values (see
+    first_token_attention_flops)."""
     h, f = cfg.hidden, cfg.ffn
     qkv, rest = 2.0 * 3 * h * h, 2.0 * (h * h + 2 * h * f)
-    return (n_layers - first_token_layers) * m_rows * (qkv + rest) + first_token_layers * (m_rows * qkv + batch * rest)
+    return (n_layers - first_token_layers) * m_rows * (qkv + rest) + first_token_layers * batch * rest
+
+
+def first_token_attention_flops(cfg, lengths):
+    """FLOPs of one last branch layer's attention for the first tokens of sequences of these lengths: three H x H products
+    per sequence (query, query through the key matrix, attended mean through the value matrix) and, per head, a pass over
+    the sequence's inputs for the scores and one for the mean."""
+    h = cfg.hidden
+    return len(lengths) * 2.0 * 3 * h * h + 4.0 * cfg.heads * h * float(lengths.sum())
 
 
 def oracle_threads():
@@ -461,8 +470,9 @@ def main():
         padded_flops = gemm_flops_per_forward(cfg, plan["layers"], m_rows) + \
             plan["layers"] * BATCH * 4.0 * cfg.hidden * SEQ * SEQ
         valid_flops = gemm_flops + sum(
-            plan["layers"] * 4.0 * cfg.hidden * float((batches[i % N_INPUT_BATCHES].lengths.astype(np.float64) ** 2).sum())
-            for i in range(args.steps))
+            (plan["layers"] - n_first) * 4.0 * cfg.hidden * float((n.astype(np.float64) ** 2).sum())
+            + n_first * first_token_attention_flops(cfg, n)
+            for n in (batches[i % N_INPUT_BATCHES].lengths for i in range(args.steps)))
         value = aggregate_throughput(world, BATCH, args.steps, total_ms * 1e-3)
         out = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -484,8 +494,8 @@ def main():
                     "d2h_bytes_per_step": BATCH * cfg.total_classes * 4},
             "roofline": {"bound": "tensor", "kernel": "gemm_bf16_tcgen05 and gemm_ln_tcgen05 (QKV, attention-out, FFN-up, FFN-down launches; the two "
                                    "residual GEMMs include the LayerNorm after them)",
-                         "flops": "valid tokens only; the last layer of each branch counts its Q/K/V projection on all "
-                                  "tokens and the rest on one token per sequence",
+                         "flops": "valid tokens only; the last layer of each branch counts its attention-output and FFN maps on one token "
+                                  "per sequence",
                          "achieved": achieved, "peak": peaks["tflops"], "unit": "TFLOP/s",
                          "frac": achieved / peaks["tflops"], "peak_source": peaks["source"],
                          "peak_nominal": NOMINAL_BF16_TFLOPS, "frac_of_nominal": achieved / NOMINAL_BF16_TFLOPS,
