@@ -742,7 +742,11 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
   t->ln1.y[i] = h1; t->ln1.y32[i] = h1_32;
   if (t->fp8) {
     // h1 and f are quantised row by row into the scratch; the projections read those and the 8-bit weights
+    // (h1 by the LayerNorm itself where that is a launch of its own)
     t->q_h1.x[i] = h1; t->q_h1.q[i] = qs->h1q; t->q_h1.scale[i] = qs->sh1;
+    if (t->out_ln == 0) {
+      t->ln1.q[i] = qs->h1q; t->ln1.scale[i] = qs->sh1;
+    }
     t->q_f.x[i] = f; t->q_f.q[i] = qs->fq; t->q_f.scale[i] = qs->sf;
     t->q_h1.n_groups = t->q_f.n_groups = i + 1;
     if ((e = set_gemm_group(&t->ffn_up, i, kEpiBiasGelu, qs->h1q, m->d_weights + lo->q_w1, w_ptr(m, lo->b1), nullptr, f)) !=
@@ -1008,7 +1012,7 @@ std::vector<int32_t> cls_tasks_after_wave(const mt_model* m, const Schedule& s, 
 // Kernel launches of a built plan: the row starts, the embedding, and what mt_forward_tokens does for every step.
 int32_t plan_launches(const Plan& plan) {
   auto tail = [](const LayerTail& t) {
-    return t.count == 0 ? 0 : (t.out_ln != 0 ? 1 : 2) + 1 + (t.down_ln != 0 ? 1 : 2) + (t.fp8 ? 2 : 0);
+    return t.count == 0 ? 0 : (t.out_ln != 0 ? 1 : 2) + 1 + (t.down_ln != 0 ? 1 : 2) + (t.fp8 ? (t.out_ln != 0 ? 2 : 1) : 0);
   };
   int32_t n = 2;
   for (const PlanStep& st : plan.steps) {
@@ -1655,7 +1659,8 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
                                               m->sm_count, stream), "attention output GEMM");                         \
       MT_TIMED(MT_CLASS_LN1, launch_layernorm(t_->ln1, stream), "LayerNorm 1");                                        \
     }                                                                                                                  \
-    if (t_->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_h1, stream), "quantising the FFN input");         \
+    if (t_->fp8 && t_->out_ln != 0)                                                                                    \
+      MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_h1, stream), "quantising the FFN input");                    \
     MT_TIMED(MT_CLASS_FFN_UP, launch_gemm(t_->ffn_up, kEpiBiasGelu, m->sm_count, stream), "FFN up GEMM");              \
     if (t_->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_f, stream), "quantising the FFN intermediate");   \
     if (t_->down_ln != 0) {                                                                                            \

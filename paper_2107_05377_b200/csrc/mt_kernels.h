@@ -228,6 +228,8 @@ struct LayerNormParams {
   float* y32[kMaxGroups];
   int32_t n_groups, rows, hidden;
   const int32_t* rows_valid;  // device scalar: rows actually in use (<= rows); null = all
+  uint8_t* q[kMaxGroups];     // not null in group 0: E4M3 codes of the bf16 rows [rows, hidden] too, ...
+  float* scale[kMaxGroups];   // ... and their scales [rows] (see QuantParams)
   float eps;
 };
 cudaError_t launch_layernorm(const LayerNormParams& p, cudaStream_t stream);

@@ -13,9 +13,62 @@ constexpr int kRowThreads = 256;  // 8 rows per CTA
 constexpr int64_t kRowPerCtaMax = 32 * 148;   // rows x groups up to which LayerNorm takes a CTA per row: 32 per SM
 constexpr int kMaxParts = 4;       // ranges of K a row can be put together from (LayerNormParams::n_parts)
 
+__device__ __forceinline__ uint32_t cvt_e4m3x2(float hi, float lo) {
+  uint16_t r;
+  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+// x / scale rounded to nearest, from the correctly rounded reciprocal of scale: a product, its exact remainder and one
+// correction (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990: the result is the
+// correctly rounded quotient, as long as nothing under- or overflows and scale's significand is not all ones).  A
+// zero keeps the sign of x, which the correction would lose.
+__device__ __forceinline__ float divide_by(float x, float scale, float rcp) {
+  const float q = x * rcp;
+  return copysignf(fmaf(fmaf(-q, scale, x), rcp, q), x);
+}
+template <bool EXACT>
+__device__ __forceinline__ uint2 quantize8(const uint4& u, float scale, float rcp) {
+  float f[8];
+  unpack8(u, f);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) f[i] = EXACT ? __fdiv_rn(f[i], scale) : divide_by(f[i], scale, rcp);
+  return make_uint2(cvt_e4m3x2(f[1], f[0]) | (cvt_e4m3x2(f[3], f[2]) << 16), cvt_e4m3x2(f[5], f[4]) | (cvt_e4m3x2(f[7], f[6]) << 16));
+}
+__device__ __forceinline__ __nv_bfloat162 amax8(const uint4& u, __nv_bfloat162 amax) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) amax = __hmax2(amax, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&w[i])));
+  return amax;
+}
+// Scale of a row with this largest magnitude, and its codes from 16-byte vectors in registers.
+__device__ __forceinline__ float row_scale(float amax) { return amax == 0.f ? 1.0f : __fmul_rn(amax, 1.0f / 448.0f); }
+// (the quotients that decide a code are between 2^-10 and 448: with scale in this range no remainder underflows)
+__device__ __forceinline__ bool plain_division(float scale) {
+  return scale > 0x1p-60f && scale < 0x1p60f && (__float_as_uint(scale) & 0x7FFFFFu) != 0x7FFFFFu;
+}
+__device__ __forceinline__ float warp_max(__nv_bfloat162 amax2) {
+  float amax = fmaxf(__low2float(amax2), __high2float(amax2));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  return amax;
+}
+template <int V>
+__device__ __forceinline__ void store_codes(const uint4 (&u)[V], uint2* q, float scale) {   // vector v to q[v * 32]
+  if (plain_division(scale)) {
+    const float rcp = __frcp_rn(scale);
+#pragma unroll
+    for (int v = 0; v < V; ++v) q[v * 32] = quantize8<false>(u[v], scale, rcp);
+  } else {
+#pragma unroll
+    for (int v = 0; v < V; ++v) q[v * 32] = quantize8<true>(u[v], scale, 0.f);
+  }
+}
+
 // PARTS: the row is put together from the partial sums of a split projection (LayerNormParams::n_parts > 0); a
 // separate instantiation, so that the plain kernel keeps its registers and occupancy.
-template <int V, bool PARTS>
+// QUANT: the bf16 row that leaves is quantised as well, codes and scale as by quantize_rows_kernel, which would be a launch
+// and a pass over the rows of its own (8-bit projections: 64 x 128 tokens 1657 -> 1641 us, 24 x 100 861 -> 844).
+template <int V, bool PARTS, bool QUANT>
 __global__ void __launch_bounds__(kRowThreads) layernorm_kernel(const LayerNormParams p) {
   constexpr int H = V * 256;
   const int lane = threadIdx.x & 31;
@@ -79,14 +132,23 @@ __global__ void __launch_bounds__(kRowThreads) layernorm_kernel(const LayerNormP
     }
   }
   float* y32 = p.y32[g] != nullptr ? p.y32[g] + static_cast<size_t>(row) * H : nullptr;
-  normalise_store<V>(x, p.gamma[g], p.beta[g], p.y[g] + static_cast<size_t>(row) * H, y32, lane, p.eps);
+  uint4 y8[V];
+  normalise_store<V>(x, p.gamma[g], p.beta[g], p.y[g] + static_cast<size_t>(row) * H, y32, lane, p.eps, y8);
+  if (QUANT) {
+    __nv_bfloat162 amax2 = __float2bfloat162_rn(0.f);
+#pragma unroll
+    for (int v = 0; v < V; ++v) amax2 = amax8(y8[v], amax2);
+    const float scale = row_scale(warp_max(amax2));
+    if (lane == 0) p.scale[g][row] = scale;
+    store_codes(y8, reinterpret_cast<uint2*>(p.q[g] + static_cast<size_t>(row) * H) + lane, scale);
+  }
 }
 
 // The same for few rows: one CTA of V warps per row, warp v on columns v * 256 .. + 255.  A launch of a few hundred rows is
 // one row's chain of latencies, which this shortens: a third (a quarter) of the loads, sums and stores per lane, the
 // warps' segments exchanged through shared memory.  Same segments, same additions, same bits.  (128 rows: 0.95 us after the
 // dependency wait against 1.7 with a warp per row; put together from four ranges 1.5 against 3.9.)
-template <int V, bool PARTS>
+template <int V, bool PARTS, bool QUANT>
 __global__ void __launch_bounds__(V * 32) layernorm_row_kernel(const LayerNormParams p) {
   constexpr int H = V * 256;
   constexpr int S = V * 4;
@@ -156,10 +218,23 @@ __global__ void __launch_bounds__(V * 32) layernorm_row_kernel(const LayerNormPa
   unpack8(beta8, bt);
 #pragma unroll
   for (int i = 0; i < 8; ++i) y[i] = fmaf(__fmul_rn(x[i] - mean, rstd), gm[i], bt[i]);
-  *reinterpret_cast<uint4*>(p.y[g] + at) = pack8(y);
+  const uint4 y8[1] = {pack8(y)};
+  *reinterpret_cast<uint4*>(p.y[g] + at) = y8[0];
   if (p.y32[g] != nullptr) {
     *reinterpret_cast<float4*>(p.y32[g] + at) = make_float4(y[0], y[1], y[2], y[3]);
     *reinterpret_cast<float4*>(p.y32[g] + at + 4) = make_float4(y[4], y[5], y[6], y[7]);
+  }
+  if (QUANT) {
+    __shared__ float largest[V];
+    const float mine = warp_max(amax8(y8[0], __float2bfloat162_rn(0.f)));
+    if (lane == 0) largest[v] = mine;
+    __syncthreads();
+    float amax = largest[0];
+#pragma unroll
+    for (int i = 1; i < V; ++i) amax = fmaxf(amax, largest[i]);
+    const float scale = row_scale(amax);
+    if (threadIdx.x == 0) p.scale[g][row] = scale;
+    store_codes(y8, reinterpret_cast<uint2*>(p.q[g] + at), scale);
   }
 }
 
@@ -317,33 +392,6 @@ __global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadParams p) 
 // Row-wise E4M3 quantisation (QuantParams): one warp per row, first for its largest magnitude, then to
 // scale and convert.  Every decision is taken in fp32 with IEEE operations
 // that no compiler option can change: scale = amax * (1/448), y = x / scale, code = cvt.rn.satfinite.e4m3.
-__device__ __forceinline__ uint32_t cvt_e4m3x2(float hi, float lo) {
-  uint16_t r;
-  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-// x / scale rounded to nearest, from the correctly rounded reciprocal of scale: a product, its exact remainder and one
-// correction (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990: the result is the
-// correctly rounded quotient, as long as nothing under- or overflows and scale's significand is not all ones).  A
-// zero keeps the sign of x, which the correction would lose.
-__device__ __forceinline__ float divide_by(float x, float scale, float rcp) {
-  const float q = x * rcp;
-  return copysignf(fmaf(fmaf(-q, scale, x), rcp, q), x);
-}
-template <bool EXACT>
-__device__ __forceinline__ uint2 quantize8(const uint4& u, float scale, float rcp) {
-  float f[8];
-  unpack8(u, f);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) f[i] = EXACT ? __fdiv_rn(f[i], scale) : divide_by(f[i], scale, rcp);
-  return make_uint2(cvt_e4m3x2(f[1], f[0]) | (cvt_e4m3x2(f[3], f[2]) << 16), cvt_e4m3x2(f[5], f[4]) | (cvt_e4m3x2(f[7], f[6]) << 16));
-}
-__device__ __forceinline__ __nv_bfloat162 amax8(const uint4& u, __nv_bfloat162 amax) {
-  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) amax = __hmax2(amax, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&w[i])));
-  return amax;
-}
 // V: 16-byte vectors of a row per lane, held in registers between the two steps (0: any length, read twice).  A row of
 // 3072 values then has twelve loads per lane in flight instead of one or two and is read once, and the division is three
 // multiply-adds instead of some ten instructions and a branch.  20000 rows of 3072 values: 124 -> 58 us, of 768: 34 -> 16,
@@ -370,18 +418,11 @@ __global__ void __launch_bounds__(kRowThreads, V >= 16 ? 3 : 4) quantize_rows_ke
   } else {
     for (int v = 0; v < vectors; ++v) amax2 = amax8(__ldg(x + v * 32), amax2);
   }
-  float amax = fmaxf(__low2float(amax2), __high2float(amax2));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-  const float scale = amax == 0.f ? 1.0f : __fmul_rn(amax, 1.0f / 448.0f);
+  const float scale = row_scale(warp_max(amax2));
   if (lane == 0) p.scale[g][row] = scale;
   uint2* q = reinterpret_cast<uint2*>(p.q[g] + static_cast<size_t>(row) * p.cols) + lane;
-  // (the quotients that decide a code are between 2^-10 and 448: with scale in this range no remainder underflows)
-  const bool plain = scale > 0x1p-60f && scale < 0x1p60f && (__float_as_uint(scale) & 0x7FFFFFu) != 0x7FFFFFu;
-  if (V > 0 && plain) {
-    const float rcp = __frcp_rn(scale);
-#pragma unroll
-    for (int v = 0; v < (V > 0 ? V : 1); ++v) q[v * 32] = quantize8<false>(u[v], scale, rcp);
+  if (V > 0) {
+    store_codes(u, q, scale);
   } else {
     for (int v = 0; v < vectors; ++v) q[v * 32] = quantize8<true>(__ldg(x + v * 32), scale, 0.f);
   }
@@ -529,27 +570,27 @@ cudaError_t launch_token_heads(const TokenHeadParams& p, cudaStream_t stream) {
   return cudaErrorInvalidValue;
 }
 
+namespace {
+template <int V, bool PARTS>
+cudaError_t launch_layernorm_as(const LayerNormParams& p, bool row_per_cta, cudaStream_t stream) {
+  const bool quant = p.q[0] != nullptr;
+  if (row_per_cta) {
+    auto kernel = quant ? layernorm_row_kernel<V, PARTS, true> : layernorm_row_kernel<V, PARTS, false>;
+    return launch_kernel(kernel, dim3(p.rows, p.n_groups), dim3(V * 32), 0, stream, p);
+  }
+  auto kernel = quant ? layernorm_kernel<V, PARTS, true> : layernorm_kernel<V, PARTS, false>;
+  return launch_kernel(kernel, dim3((p.rows + kRowThreads / 32 - 1) / (kRowThreads / 32), p.n_groups), dim3(kRowThreads), 0, stream, p);
+}
+}  // namespace
+
 cudaError_t launch_layernorm(const LayerNormParams& p, cudaStream_t stream) {
   if (p.n_groups < 1 || p.n_groups > kMaxGroups || p.rows < 1 || p.n_parts < 0 || p.n_parts > kMaxParts) return cudaErrorInvalidValue;
   // Few rows in all: a CTA per row, for its shorter chain; beyond that a warp per row, which takes fewer instructions per
   // row.  (6 x 128 tokens, launches of up to 4608 rows: 0.635 ms per forward with the line here, 0.647 with it at 1184, 0.682
   // without.)
-  if (static_cast<int64_t>(p.rows) * p.n_groups <= kRowPerCtaMax) {
-    dim3 grid(p.rows, p.n_groups);
-    if (p.hidden == 768 && p.n_parts > 0) return launch_kernel(layernorm_row_kernel<3, true>, grid, dim3(96), 0, stream, p);
-    if (p.hidden == 768) return launch_kernel(layernorm_row_kernel<3, false>, grid, dim3(96), 0, stream, p);
-    if (p.hidden == 1024 && p.n_parts > 0) return launch_kernel(layernorm_row_kernel<4, true>, grid, dim3(128), 0, stream, p);
-    if (p.hidden == 1024) return launch_kernel(layernorm_row_kernel<4, false>, grid, dim3(128), 0, stream, p);
-    return cudaErrorInvalidValue;
-  }
-  dim3 grid((p.rows + kRowThreads / 32 - 1) / (kRowThreads / 32), p.n_groups);
-  if (p.n_parts > 0) {
-    if (p.hidden == 768) return launch_kernel(layernorm_kernel<3, true>, grid, dim3(kRowThreads), 0, stream, p);
-    if (p.hidden == 1024) return launch_kernel(layernorm_kernel<4, true>, grid, dim3(kRowThreads), 0, stream, p);
-    return cudaErrorInvalidValue;
-  }
-  if (p.hidden == 768) return launch_kernel(layernorm_kernel<3, false>, grid, dim3(kRowThreads), 0, stream, p);
-  if (p.hidden == 1024) return launch_kernel(layernorm_kernel<4, false>, grid, dim3(kRowThreads), 0, stream, p);
+  const bool row_per_cta = static_cast<int64_t>(p.rows) * p.n_groups <= kRowPerCtaMax;
+  if (p.hidden == 768) return p.n_parts > 0 ? launch_layernorm_as<3, true>(p, row_per_cta, stream) : launch_layernorm_as<3, false>(p, row_per_cta, stream);
+  if (p.hidden == 1024) return p.n_parts > 0 ? launch_layernorm_as<4, true>(p, row_per_cta, stream) : launch_layernorm_as<4, false>(p, row_per_cta, stream);
   return cudaErrorInvalidValue;
 }
 

@@ -78,7 +78,7 @@ __device__ __forceinline__ void merge_segments(const float (&seg_mean)[S], const
 // so the eight lanes l / 8 == j of vector v hold segment v * 4 + j) and writes it.
 template <int V>
 __device__ __forceinline__ void normalise_store(float (&x)[V][8], const bf16* gamma, const bf16* beta, bf16* out,
-                                                float* out32, int lane, float eps) {
+                                                float* out32, int lane, float eps, uint4* out8 = nullptr) {
   constexpr int H = V * 256;
   constexpr int S = V * 4;
   float seg_mean[S], seg_m2[S];
@@ -107,7 +107,9 @@ __device__ __forceinline__ void normalise_store(float (&x)[V][8], const bf16* ga
     unpack8(__ldg(reinterpret_cast<const uint4*>(beta + col)), b);
 #pragma unroll
     for (int i = 0; i < 8; ++i) y[i] = fmaf(__fmul_rn(x[v][i] - mean, rstd), g[i], b[i]);
-    *reinterpret_cast<uint4*>(out + col) = pack8(y);
+    const uint4 y8 = pack8(y);
+    *reinterpret_cast<uint4*>(out + col) = y8;
+    if (out8 != nullptr) out8[v] = y8;   // (the same 16 bytes for the caller)
     if (out32 != nullptr) {
       *reinterpret_cast<float4*>(out32 + col) = make_float4(y[0], y[1], y[2], y[3]);
       *reinterpret_cast<float4*>(out32 + col + 4) = make_float4(y[4], y[5], y[6], y[7]);

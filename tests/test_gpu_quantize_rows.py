@@ -8,6 +8,8 @@ import torch
 
 from oracle import fp8_oracle as f8
 from paper_2107_05377_b200 import binding as mt
+from paper_2107_05377_b200 import synth
+from gpu_util import cached_weights, dev_batch
 
 pytestmark = pytest.mark.gpu
 
@@ -36,3 +38,26 @@ def test_codes_and_scales_equal_the_oracle(rows, cols):
     want_q, want_s = f8.quantize_rows(xt.float().numpy().astype(np.float64))
     assert np.array_equal(s.cpu().numpy(), want_s)
     assert np.array_equal(q.cpu().numpy(), want_q)
+
+
+BASE = synth.TreeConfig(trunk_layers=2, tasks=(synth.TaskSpec(2, 2, 3), synth.TaskSpec(1, 1, 2), synth.TaskSpec(2, 0, 2)))
+WIDE = synth.TreeConfig(hidden=1024, heads=16, ffn=4096, trunk_layers=2, vocab_size=2000, tasks=BASE.tasks)
+
+
+@pytest.mark.parametrize("cfg,B,S", [(BASE, 1, 31), (BASE, 20, 64), (BASE, 48, 128), (WIDE, 5, 128), (WIDE, 41, 128)])
+def test_layernorm_that_quantises_gives_the_bits_of_the_separate_launch(cfg, B, S):
+    """fused_ln 0: the LayerNorm before the FFN writes the codes (a CTA or a warp per row, by the rows of the launch); 1 and
+    3: it is part of the projection (beyond 512 rows) and the rows are quantised by a launch of its own."""
+    _, blob, _ = cached_weights(cfg, 5, random_affine=True)
+    batch = synth.make_batch(cfg, B, S, max(1, S // 4), S, seed=2)
+    model = mt.MTModel(cfg, B, S, fp8_gemm=True)
+    model.load_weights(blob)
+    out = {}
+    for fused in (0, 1, 3):
+        model.set_option("fused_ln", fused)
+        out[fused] = torch.full((B, cfg.total_classes), float("nan"), device="cuda")
+        model.forward(*dev_batch(batch), out[fused])
+        torch.cuda.synchronize()
+        assert model.poll_status() == 0
+    assert torch.isfinite(out[0]).all()
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[3])
