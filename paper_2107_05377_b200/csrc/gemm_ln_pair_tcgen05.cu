@@ -257,7 +257,10 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
         const float4 r = *reinterpret_cast<const float4*>(my_stage_ptr + staging_off(lane, c));
         res[4 * c] = r.x; res[4 * c + 1] = r.y; res[4 * c + 2] = r.z; res[4 * c + 3] = r.w;
       }
-      __syncwarp();   // every lane has read the box
+      // every lane has read the box: its reads complete before the next box may land in their place (the copy is another
+      // proxy's write, which a warp barrier alone does not order behind them)
+      fence_async_shared();
+      __syncwarp();
       if (lane == 0) {
         mbar_expect_tx(my_res_bar, kLpStagingBytes);
         tma_load_2d(my_stage, &p.tmap_res[g], col0 + 32, row0, my_res_bar);
