@@ -259,9 +259,8 @@ int mt_plan_cache_size(const mt_model* m);
  * 64-column segments in the same order, every projection sums over K in one sequence).
  * key "ffn_down_split" (0/1, default 1, any time): launches of at most 512 rows per layer (batch x seq up to
  * 4 x 128, and the first-token rows of the last branch layers for batches up to 512) run the FFN-down projection
- * as partial sums over four ranges of K - four times as many tiles, each a quarter as long -, and the attention-output
- * projection over three (four for hidden 1024); the LayerNorm kernel after each adds the ranges in order, then the bias
- * and the residual.  Such a launch has so few tiles that
+ * as partial sums over four ranges of K - four times as many tiles, each a quarter as long - and the LayerNorm
+ * kernel after it adds the ranges in order, then the bias and the residual.  Such a launch has so few tiles that
  * the chain of k-blocks one CTA walks is what it costs.  The sum over K is then taken range by range: results
  * differ in the last bits from the unsplit projection, within every tolerance of the tests; the choice depends on
  * the rows of one layer and on options only, never on the tasks asked for or on how many layers share a launch,

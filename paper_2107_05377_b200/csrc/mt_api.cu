@@ -92,7 +92,6 @@ struct LayerTail {
   // launches of few rows: the FFN-down projection as partial sums over `down_splits` ranges of K, put together
   // (ranges in order, bias, residual) by the LayerNorm kernel after it
   int32_t down_splits = 1;
-  int32_t out_splits = 1;    // the same for the attention-output projection
   GemmLnParams attn_out_ln, ffn_down_ln;
   // 8-bit operands: the inputs of the FFN-up and FFN-down projections are quantised row by row first
   bool fp8 = false;
@@ -629,14 +628,6 @@ int32_t down_split_count(const mt_model* m, int64_t rows) {
   if (m->ffn_down_split == 0 || m->fp8 || rows > kSplitRowsMax) return 1;
   return (m->trunk.ffn / kGemmBlockK) % kDownSplits == 0 ? kDownSplits : 1;
 }
-// The same for the attention-output projection, which a LayerNorm follows too: ranges of kGemmLowKBlocks k-blocks, a
-// single stage of the low tiles each (three for a hidden size of 768, four for 1024; 1 x 128 tokens: 377 us per forward
-// against 386, 4 x 128: 500 against 505).
-int32_t out_split_count(const mt_model* m, int64_t rows) {
-  const int32_t kb = m->trunk.hidden / kGemmBlockK;
-  if (m->ffn_down_split == 0 || m->fp8 || rows > kSplitRowsMax || kb % kGemmLowKBlocks != 0) return 1;
-  return kb / kGemmLowKBlocks <= kDownSplits ? kb / kGemmLowKBlocks : 1;
-}
 // Launches of steps 3-7 for `groups` layers (before mt_bind_memory; afterwards plans are built and counted).
 int32_t tail_launches(const mt_model* m, int32_t groups, int64_t rows) {
   const bool fused = fused_ln_kind(m, groups, rows) != 0;
@@ -657,14 +648,7 @@ void init_tail(const mt_model* m, LayerTail* t, int32_t rows, bool all_rows_vali
     g->m_valid = rows_valid;
     g->status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
   };
-  t->out_splits = out_split_count(m, rows);
-  init_gemm(&t->attn_out, H, H, t->out_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual);
-  if (t->out_splits > 1) {
-    t->attn_out.k_splits = t->out_splits;
-    t->attn_out.split_pitch = static_cast<int32_t>(split_pitch(rows));
-    t->attn_out.block_n = gemm_block_n(H, kEpiPartialF32, rows, groups * t->out_splits, false, m->sm_count);
-    t->attn_out.pair = 0;
-  }
+  init_gemm(&t->attn_out, H, H, kEpiBiasResidual);
   init_gemm(&t->ffn_up, F, H, kEpiBiasGelu);
   t->down_splits = down_split_count(m, rows);
   if (t->down_splits > 1) {
@@ -699,8 +683,8 @@ void init_tail(const mt_model* m, LayerTail* t, int32_t rows, bool all_rows_vali
   t->ln1.hidden = t->ln2.hidden = H;
   t->ln1.eps = t->ln2.eps = m->trunk.ln_eps;
   t->count = 0;
-  t->out_ln = t->out_splits == 1 ? fused_ln_kind(m, groups, rows) : 0;
-  t->down_ln = !m->fp8 && t->out_splits == 1 && t->down_splits == 1 ? fused_ln_kind(m, groups, rows) : 0;
+  t->out_ln = fused_ln_kind(m, groups, rows);
+  t->down_ln = !m->fp8 && t->down_splits == 1 ? t->out_ln : 0;
   if (t->out_ln != 0 || t->down_ln != 0) {
     auto init_ln = [&](GemmLnParams* g, int32_t K) {
       memset(g, 0, sizeof(*g));
@@ -720,24 +704,9 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
                         float* u, bf16* h1, float* h1_32, bf16* f, bf16* out, float* out32, const QuantScratch* qs) {
   const int i = t->count;
   cudaError_t e;
-  // partial sums of a split projection: range s of this group writes rows [s * pitch, s * pitch + rows) of the group's piece
-  // of the partial-sum scratch; the LayerNorm kernel adds the ranges, the bias and the residual
-  auto set_partial = [&](GemmParams* g, int32_t splits, LayerNormParams* ln, const bf16* x, size_t w, size_t b,
-                         const float* res) -> cudaError_t {
-    const size_t pitch = static_cast<size_t>(g->split_pitch);
-    float* part = reinterpret_cast<float*>(m->d_workspace + m->ws_partial) + static_cast<size_t>(i) * splits * pitch * m->trunk.hidden;
-    cudaError_t err = set_gemm_group(g, i, kEpiPartialF32, x, w_ptr(m, w), nullptr, nullptr, part);
-    if (err != cudaSuccess) return err;
-    ln->part[i] = part; ln->residual[i] = res; ln->bias[i] = w_ptr(m, b);
-    ln->n_parts = splits; ln->part_pitch = static_cast<int32_t>(pitch);
-    return make_tmap(&g->tmap_out[i], part, static_cast<int>(splits * pitch), g->N, 32, 32, true);
-  };
-  if (t->out_splits > 1) {
-    if ((e = set_partial(&t->attn_out, t->out_splits, &t->ln1, ctx, lo->wo, lo->bo, residual)) != cudaSuccess) return e;
-  } else if ((e = set_gemm_group(&t->attn_out, i, kEpiBiasResidual, ctx, w_ptr(m, lo->wo), w_ptr(m, lo->bo), residual, u)) !=
-             cudaSuccess) {
+  if ((e = set_gemm_group(&t->attn_out, i, kEpiBiasResidual, ctx, w_ptr(m, lo->wo), w_ptr(m, lo->bo), residual, u)) !=
+      cudaSuccess)
     return e;
-  }
   t->ln1.x[i] = u; t->ln1.gamma[i] = w_ptr(m, lo->ln1_g); t->ln1.beta[i] = w_ptr(m, lo->ln1_b);
   t->ln1.y[i] = h1; t->ln1.y32[i] = h1_32;
   if (t->fp8) {
@@ -764,7 +733,18 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
         cudaSuccess)
       return e;
     if (t->down_splits > 1) {
-      if ((e = set_partial(&t->ffn_down, t->down_splits, &t->ln2, f, lo->w2, lo->b2, h1_32)) != cudaSuccess) return e;
+      // partial sums: range s of this group writes rows [s * pitch, s * pitch + rows) of the group's piece of the
+      // partial-sum scratch; the LayerNorm kernel adds the ranges, the bias and the residual
+      const size_t pitch = static_cast<size_t>(t->ffn_down.split_pitch);
+      float* part = reinterpret_cast<float*>(m->d_workspace + m->ws_partial) +
+                    static_cast<size_t>(i) * t->down_splits * pitch * m->trunk.hidden;
+      if ((e = set_gemm_group(&t->ffn_down, i, kEpiPartialF32, f, w_ptr(m, lo->w2), nullptr, nullptr, part)) != cudaSuccess)
+        return e;
+      if ((e = make_tmap(&t->ffn_down.tmap_out[i], part, static_cast<int>(t->down_splits * pitch), t->ffn_down.N, 32, 32,
+                         true)) != cudaSuccess)
+        return e;
+      t->ln2.part[i] = part; t->ln2.residual[i] = h1_32; t->ln2.bias[i] = w_ptr(m, lo->b2);
+      t->ln2.n_parts = t->down_splits; t->ln2.part_pitch = static_cast<int32_t>(pitch);
     } else if ((e = set_gemm_group(&t->ffn_down, i, kEpiBiasResidual, f, w_ptr(m, lo->w2), w_ptr(m, lo->b2), h1_32, u)) !=
                cudaSuccess) {
       return e;
@@ -1655,8 +1635,7 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
                                                   : launch_gemm_ln(t_->attn_out_ln, stream),                           \
                "attention output GEMM + LayerNorm");                                                                   \
     } else {                                                                                                           \
-      MT_TIMED(MT_CLASS_ATTN_OUT, launch_gemm(t_->attn_out, t_->out_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual,    \
-                                              m->sm_count, stream), "attention output GEMM");                         \
+      MT_TIMED(MT_CLASS_ATTN_OUT, launch_gemm(t_->attn_out, kEpiBiasResidual, m->sm_count, stream), "attention output GEMM"); \
       MT_TIMED(MT_CLASS_LN1, launch_layernorm(t_->ln1, stream), "LayerNorm 1");                                        \
     }                                                                                                                  \
     if (t_->fp8 && t_->out_ln != 0)                                                                                    \

@@ -1,7 +1,8 @@
-"""Forwards of few rows: low GEMM tiles (64 and 32 rows), projections as partial sums, a LayerNorm CTA per row.  Parity with
+"""Forwards of few rows: low GEMM tiles (64 and 32 rows), the FFN-down projection as partial sums, a LayerNorm CTA per row.  Parity with
 the oracle at every hidden state where the sizes can go wrong: a single row, tiles just full and just begun, the last
 size before full tiles and the first after, and a hidden size of 1024 (more k-blocks than the ring of stages holds);
 and the same bits from run to run."""
+import numpy as np
 import pytest
 import torch
 
@@ -35,3 +36,23 @@ def test_forwards_of_few_rows_match_the_oracle(cfg, B, S):
         model.forward(tok, seg, lens, again)
         torch.cuda.synchronize()
         assert torch.equal(again, logits)
+
+
+@pytest.mark.parametrize("cfg,B,S", [(BASE, 1, 8), (BASE, 3, 57), (BASE, 4, 128), (WIDE, 1, 100)])
+def test_only_the_ffn_down_projection_is_summed_range_by_range(cfg, B, S):
+    """With FFN-down weights of zero its partial sums are zero in every order, so option "ffn_down_split" must not change a
+    bit: the attention-output projection of a launch of few rows is summed over K in one sequence like every other."""
+    w = synth.make_weights(cfg, seed=5, random_affine=True)
+    for layer in w["trunk"] + [one for task in w["tasks"] for one in task["layers"]]:
+        layer["w2"] = np.zeros_like(layer["w2"])
+    batch = synth.make_batch(cfg, B, S, max(1, S // 4), S, seed=8)
+    model = mt.MTModel(cfg, B, S)
+    model.load_weights(synth.pack_weights(cfg, w))
+    out = {}
+    for split in (0, 1):
+        model.set_option("ffn_down_split", split)
+        out[split] = torch.full((B, cfg.total_classes), float("nan"), device="cuda")
+        model.forward(*dev_batch(batch), out[split])
+        torch.cuda.synchronize()
+        assert model.poll_status() == 0
+    assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
