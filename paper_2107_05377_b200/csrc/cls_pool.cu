@@ -7,9 +7,16 @@
 // three H x H products of n rows and a pass over n rows of K and V: at 32768 rows the projections were 80 us per layer.
 //
 //   cls_query_kernel : q = x_0 Wq^T + bq (bf16), then q~_h = q_h Wk_h (bf16 [B, heads, H])
-//   cls_pool_kernel  : scores q~_h . x_j / 8, softmax over j < length, z_h = sum_j p_j x_j (bf16 [B, heads, H]);
-//                      also gathers the first token's fp32 residual
+//   cls_pool_kernel  : scores q~_h . x_j / 8, softmax over j < length, z_h = sum_j p_j x_j ([B, heads, 2, H]: a bf16 and
+//                      the bf16 of what it leaves of the sum); also gathers the first token's fp32 residual
 //   (the third step, ctx_h = z_h Wv_h^T + bv, is a launch of gemm_bf16_tcgen05 whose X columns follow the head)
+//
+// Rounding.  The route over keys and values rounds each k_j and v_j to bf16, errors that differ from key to key and
+// average out over them, and takes the probabilities in fp32.  Here p_j and z are therefore each two bf16 terms (the value
+// and its remainder, 16 bits together): with one term for each a layer that is little but this attention is 2.87e-3 from fp64
+// where the other route is 2.40e-3 (48 sequences of 20 to 40 tokens), since z is rounded after the mean; with two 2.35e-3.  q~
+// in one term errs no more than rounding every k_j does.  Both second terms together: 32 x 128 tokens 1040 -> 1043 us per
+// forward, 23 x 101 on the 33-layer paper tree 1053 -> 1059, 16 x 512 2029 -> 2044.
 //
 // Both use mma.sync m16n8k16: a head's row is one of 12 or 16, which is just the 16 rows of that instruction (a tcgen05
 // accumulator would be seven eighths empty), and what bounds them is the reading of weights and of x.  The operands'
@@ -49,10 +56,26 @@ __device__ __forceinline__ void mma_rows4(float (&c)[4][4], const uint32_t (&a)[
   mma_16816(c[3], a[0], a[1], a[2], a[3], __byte_perm(r0.y, r1.y, 0x7632), __byte_perm(r2.y, r3.y, 0x7632));
 }
 // Row g (half 0) or g + 8 (half 1) of the four tiles: this lane's columns t * 8 .. + 7 of the block of 32.
-__device__ __forceinline__ uint4 pack_row(const float (&c)[4][4], int half, float scale) {
+__device__ __forceinline__ uint4 pack_row(const float (&c)[4][4], int half) {
   const int i = 2 * half;
-  return make_uint4(pack_bf16(c[0][i] * scale, c[1][i] * scale), pack_bf16(c[2][i] * scale, c[3][i] * scale),
-                    pack_bf16(c[0][i + 1] * scale, c[1][i + 1] * scale), pack_bf16(c[2][i + 1] * scale, c[3][i + 1] * scale));
+  return make_uint4(pack_bf16(c[0][i], c[1][i]), pack_bf16(c[2][i], c[3][i]), pack_bf16(c[0][i + 1], c[1][i + 1]),
+                    pack_bf16(c[2][i + 1], c[3][i + 1]));
+}
+// The same of c * scale, as a bf16 and the bf16 of what that leaves.
+__device__ __forceinline__ void split_row(const float (&c)[4][4], int half, float scale, uint4* hi, uint4* lo) {
+  float d[4][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) d[j][2 * half + i] = c[j][2 * half + i] * scale;
+  *hi = pack_row(d, half);
+  const uint32_t w[4] = {hi->x, hi->y, hi->z, hi->w};   // (columns 2 k and 2 k + 1 of the block's row: tiles 0, 1 or 2, 3)
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    d[2 * (k & 1)][2 * half + (k >> 1)] -= bf16_lo(w[k]);
+    d[2 * (k & 1) + 1][2 * half + (k >> 1)] -= bf16_hi(w[k]);
+  }
+  *lo = pack_row(d, half);
 }
 
 // One CTA = (16 RT sequences, head, layer).  Warp w makes columns w * 8 .. + 7 of q (its rows of Wq are asked for before the
@@ -137,7 +160,7 @@ __global__ void __launch_bounds__(kCpThreads) cls_query_kernel(const ClsPoolPara
       for (int half = 0; half < 2; ++half) {
         const int b = b0 + r * 16 + g + 8 * half;
         if (b < p.batch)
-          *reinterpret_cast<uint4*>(p.qt[layer] + (static_cast<size_t>(b) * p.heads + head) * H + base + t * 8) = pack_row(c, half, 1.0f);
+          *reinterpret_cast<uint4*>(p.qt[layer] + (static_cast<size_t>(b) * p.heads + head) * H + base + t * 8) = pack_row(c, half);
       }
     }
   }
@@ -147,7 +170,7 @@ __global__ void __launch_bounds__(kCpThreads) cls_query_kernel(const ClsPoolPara
 // into its own three buffers, adds its part of the scores (16 heads x 16 keys), and accumulates its columns of z.  Between
 // the two the warps add their parts and take the softmax (running maximum; a warp has two heads, a lane one key of one).
 template <int V>
-__global__ void __launch_bounds__(kCpThreads, 2) cls_pool_kernel(const ClsPoolParams p) {
+__global__ void __launch_bounds__(kCpThreads, V == 3 ? 2 : 1) cls_pool_kernel(const ClsPoolParams p) {
   constexpr int H = V * 256;
   constexpr int COLS = V * 32;                // columns of a warp
   constexpr int PITCH = COLS * 2 + 16;        // bytes of a row in a warp's buffer
@@ -155,8 +178,8 @@ __global__ void __launch_bounds__(kCpThreads, 2) cls_pool_kernel(const ClsPoolPa
   constexpr int P_PITCH = kCpKeys * 2 + 16;
   extern __shared__ uint8_t smem[];
   float* parts = reinterpret_cast<float*>(smem + kCpStages * kCpWarps * BUF);           // [warp][head][key]
-  uint8_t* probs = reinterpret_cast<uint8_t*>(parts + kCpWarps * 16 * kCpPartPitch);    // [head][key, permuted] bf16
-  float* factor = reinterpret_cast<float*>(probs + 16 * P_PITCH);                       // [head]: rescaling, at the end 1 / sum
+  uint8_t* probs = reinterpret_cast<uint8_t*>(parts + kCpWarps * 16 * kCpPartPitch);    // [term][head][key, permuted] bf16
+  float* factor = reinterpret_cast<float*>(probs + 2 * 16 * P_PITCH);                   // [head]: rescaling, at the end 1 / sum
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const int b = blockIdx.x, layer = blockIdx.y;
@@ -252,7 +275,10 @@ __global__ void __launch_bounds__(kCpThreads, 2) cls_pool_kernel(const ClsPoolPa
       l_run = fmaf(l_run, alpha, sum);
       m_run = m;
       // key t + 4 i goes to place 4 t + i: what a lane of the second product reads as one word pair
-      *reinterpret_cast<bf16*>(probs + my_head * P_PITCH + ((my_key & 3) * 4 + (my_key >> 2)) * 2) = __float2bfloat16(pj);
+      uint8_t* place = probs + my_head * P_PITCH + ((my_key & 3) * 4 + (my_key >> 2)) * 2;
+      const bf16 p_hi = __float2bfloat16(pj);
+      *reinterpret_cast<bf16*>(place) = p_hi;
+      *reinterpret_cast<bf16*>(place + 16 * P_PITCH) = __float2bfloat16(pj - __bfloat162float(p_hi));
       if (my_key == 0) factor[my_head] = alpha;
     }
     __syncthreads();
@@ -269,14 +295,21 @@ __global__ void __launch_bounds__(kCpThreads, 2) cls_pool_kernel(const ClsPoolPa
     }
 #pragma unroll
     for (int kk = 0; kk < kCpKeys / 16; ++kk) {
-      const uint2 lo = *reinterpret_cast<const uint2*>(probs + g * P_PITCH + (kk * 16 + t * 4) * 2);
-      const uint2 hi = *reinterpret_cast<const uint2*>(probs + (g + 8) * P_PITCH + (kk * 16 + t * 4) * 2);
-      const uint32_t a[4] = {lo.x, hi.x, lo.y, hi.y};
+      uint32_t a[2][4];   // rows g and g + 8 of the two terms
+#pragma unroll
+      for (int term = 0; term < 2; ++term) {
+        const uint8_t* pr = probs + (term * 16 + g) * P_PITCH + (kk * 16 + t * 4) * 2;
+        const uint2 lower = *reinterpret_cast<const uint2*>(pr);
+        const uint2 upper = *reinterpret_cast<const uint2*>(pr + 8 * P_PITCH);
+        a[term][0] = lower.x; a[term][1] = upper.x; a[term][2] = lower.y; a[term][3] = upper.y;
+      }
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         const uint8_t* at = xs + (kk * 16 + t) * PITCH + v * 64 + g * 8;
-        mma_rows4(z[v], a, *reinterpret_cast<const uint2*>(at), *reinterpret_cast<const uint2*>(at + 4 * PITCH),
-                  *reinterpret_cast<const uint2*>(at + 8 * PITCH), *reinterpret_cast<const uint2*>(at + 12 * PITCH));
+        const uint2 r0 = *reinterpret_cast<const uint2*>(at), r1 = *reinterpret_cast<const uint2*>(at + 4 * PITCH);
+        const uint2 r2 = *reinterpret_cast<const uint2*>(at + 8 * PITCH), r3 = *reinterpret_cast<const uint2*>(at + 12 * PITCH);
+        mma_rows4(z[v], a[1], r0, r1, r2, r3);
+        mma_rows4(z[v], a[0], r0, r1, r2, r3);
       }
     }
     __syncwarp();   // (every lane has read the buffer that the next request refills)
@@ -289,9 +322,14 @@ __global__ void __launch_bounds__(kCpThreads, 2) cls_pool_kernel(const ClsPoolPa
     const int head = g + 8 * half;
     if (head >= p.heads) continue;
     const float inv = factor[head];
-    bf16* out = p.z[layer] + (static_cast<size_t>(b) * p.heads + head) * H + warp * COLS + t * 8;
+    bf16* out = p.z[layer] + (static_cast<size_t>(b) * p.heads + head) * 2 * H + warp * COLS + t * 8;
 #pragma unroll
-    for (int v = 0; v < V; ++v) *reinterpret_cast<uint4*>(out + v * 32) = pack_row(z[v], half, inv);
+    for (int v = 0; v < V; ++v) {
+      uint4 z_hi, z_lo;
+      split_row(z[v], half, inv, &z_hi, &z_lo);
+      *reinterpret_cast<uint4*>(out + v * 32) = z_hi;
+      *reinterpret_cast<uint4*>(out + H + v * 32) = z_lo;
+    }
   }
 }
 
@@ -306,7 +344,7 @@ cudaError_t launch_query(const ClsPoolParams& p, cudaStream_t stream) {
 }
 template <int V>
 cudaError_t launch_pool(const ClsPoolParams& p, cudaStream_t stream) {
-  constexpr int smem = kCpStages * kCpWarps * kCpKeys * (V * 64 + 16) + kCpWarps * 16 * kCpPartPitch * 4 + 16 * (kCpKeys * 2 + 16) + 64;
+  constexpr int smem = kCpStages * kCpWarps * kCpKeys * (V * 64 + 16) + kCpWarps * 16 * kCpPartPitch * 4 + 2 * 16 * (kCpKeys * 2 + 16) + 64;
   auto kernel = cls_pool_kernel<V>;
   static PerDeviceOnce once;
   cudaError_t err = per_device_once(once, [&](int) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });

@@ -141,6 +141,8 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
   const int n_tiles_n = p.N / BN;
   const int k_splits = p.k_splits > 1 ? p.k_splits : 1;   // ranges of K (> 1 only with the partial-sum epilogue)
   const int k_blocks = p.K / KB_ELEMS / KPS / k_splits;   // k-blocks (LOW: stages of KPS k-blocks) of one tile
+  // k-block of W that k-block kb of X meets (x_by_tile 2: the second half of X goes over W once more)
+  auto w_block = [&](int kb) { return BN == 64 && p.x_by_tile == 2 && 2 * kb >= k_blocks ? kb - k_blocks / 2 : kb; };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -194,8 +196,8 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
           tma_load_2d_pair(sB + s * B_BYTES, &p.tmap_w[g], (kb0 + s) * KB_ELEMS, n0, bar_full_count + 8 * s);
         } else {
           mbar_add_tx(bar_full + 8 * s, B_BYTES);
-          if (LOW) tma_load_3d(sB + s * B_BYTES, &p.tmap_w[g], 0, n0, (kb0 + s) * KPS, bar_full + 8 * s);
-          else tma_load_2d(sB + s * B_BYTES, &p.tmap_w[g], (kb0 + s) * KB_ELEMS, n0, bar_full + 8 * s);
+          if (LOW) tma_load_3d(sB + s * B_BYTES, &p.tmap_w[g], 0, n0, w_block(kb0 + s) * KPS, bar_full + 8 * s);
+          else tma_load_2d(sB + s * B_BYTES, &p.tmap_w[g], w_block(kb0 + s) * KB_ELEMS, n0, bar_full + 8 * s);
         }
       }
     }
@@ -257,8 +259,8 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
             if (LOW) tma_load_3d(sA + stage * A_BYTES, &p.tmap_x[g], 0, m0, (xb0 + kb) * KPS, bar_full + 8 * stage);
             else tma_load_2d(sA + stage * A_BYTES, &p.tmap_x[g], (xb0 + kb) * KB_ELEMS, m0, bar_full + 8 * stage);
             if (!w_on_its_way) {
-              if (LOW) tma_load_3d(sB + stage * B_BYTES, &p.tmap_w[g], 0, n0, (kb0 + kb) * KPS, bar_full + 8 * stage);
-              else tma_load_2d(sB + stage * B_BYTES, &p.tmap_w[g], (kb0 + kb) * KB_ELEMS, n0, bar_full + 8 * stage);
+              if (LOW) tma_load_3d(sB + stage * B_BYTES, &p.tmap_w[g], 0, n0, w_block(kb0 + kb) * KPS, bar_full + 8 * stage);
+              else tma_load_2d(sB + stage * B_BYTES, &p.tmap_w[g], w_block(kb0 + kb) * KB_ELEMS, n0, bar_full + 8 * stage);
             }
           }
           ++issued;
@@ -706,7 +708,7 @@ int gemm_block_n(int N, int epilogue, int64_t rows, int groups, bool pair, int s
 // a bit.
 void gemm_choose_low(GemmParams* p, int groups, int sm_count) {
   const int splits = p->k_splits > 1 ? p->k_splits : 1;
-  if (p->fp8 || p->N % 64 != 0 || p->K % (kGemmBlockK * kGemmLowKBlocks * splits) != 0) return;
+  if (p->fp8 || p->N % 64 != 0 || p->K % (kGemmBlockK * kGemmLowKBlocks * splits * (p->x_by_tile > 1 ? p->x_by_tile : 1)) != 0) return;
   const int low = p->M <= 32 ? 32 : 64;
   const int64_t tiles = static_cast<int64_t>((p->M + low - 1) / low) * (p->N / 64) * (groups < 1 ? 1 : groups) * splits;
   if (tiles > sm_count) return;
@@ -735,7 +737,9 @@ cudaError_t launch_gemm(const GemmParams& p, int epilogue, int sm_count, cudaStr
     if (epilogue == kEpiBiasResidual && p.block_n == 128) return launch_one<128, kEpiBiasResidual, false, true>(p, sm_count, stream);
     return cudaErrorInvalidValue;
   }
-  if (p.x_by_tile != 0 && (p.block_n != 64 || p.pair || p.fp8 || p.k_splits > 1)) return cudaErrorInvalidValue;
+  if (p.x_by_tile != 0 && (p.x_by_tile < 0 || p.x_by_tile > 2 || p.block_n != 64 || p.pair || p.fp8 || p.k_splits > 1 ||
+                           p.K % (p.x_by_tile * kGemmBlockK * (p.low != 0 ? kGemmLowKBlocks : 1)) != 0))
+    return cudaErrorInvalidValue;
   if (p.low != 0) {
     if (p.pair || p.block_n != 64 || p.K % (kGemmBlockK * kGemmLowKBlocks * (p.k_splits > 1 ? p.k_splits : 1)) != 0)
       return cudaErrorInvalidValue;

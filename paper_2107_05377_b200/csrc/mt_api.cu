@@ -217,6 +217,7 @@ cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, co
                            const float* residual, void* y) {
   const int M = g->M, N = g->N, K = g->K;
   const int64_t x_cols = g->x_by_tile != 0 ? static_cast<int64_t>(N) / 64 * K : K;   // (X has a column block per column tile)
+  const int64_t w_cols = g->x_by_tile != 0 ? K / g->x_by_tile : K;
   const bool res = epilogue == kEpiBiasResidual;
   const bool f32_out = res || epilogue == kEpiBiasTanhF32 || epilogue == kEpiPartialF32;
   cudaError_t e;
@@ -225,10 +226,10 @@ cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, co
     if ((e = make_tmap_u8(&g->tmap_w[i], w, N, K, g->block_n)) != cudaSuccess) return e;
   } else if (g->low != 0) {
     if ((e = make_tmap_kblocks(&g->tmap_x[i], x, M, x_cols, g->low)) != cudaSuccess) return e;
-    if ((e = make_tmap_kblocks(&g->tmap_w[i], w, N, K, 64)) != cudaSuccess) return e;
+    if ((e = make_tmap_kblocks(&g->tmap_w[i], w, N, w_cols, 64)) != cudaSuccess) return e;
   } else {
     if ((e = make_tmap(&g->tmap_x[i], x, M, x_cols, kGemmBlockM, kGemmBlockK, false)) != cudaSuccess) return e;
-    if ((e = make_tmap(&g->tmap_w[i], w, N, K, g->block_n / (g->pair != 0 ? 2 : 1), kGemmBlockK, false)) != cudaSuccess) return e;
+    if ((e = make_tmap(&g->tmap_w[i], w, N, w_cols, g->block_n / (g->pair != 0 ? 2 : 1), kGemmBlockK, false)) != cudaSuccess) return e;
   }
   if ((e = make_tmap(&g->tmap_out[i], y, M, N, 32, gemm_out_box_cols(epilogue), f32_out)) != cudaSuccess) return e;
   if (res && (e = make_tmap(&g->tmap_res[i], residual, M, N, 32, 32, true)) != cudaSuccess) return e;
@@ -421,10 +422,10 @@ void layout_workspace(mt_model* m) {
     const size_t B = static_cast<size_t>(m->max_batch);
     m->cls_bytes += pad256(B * H) + pad256(B * F) + 2 * pad256(B * 4);
   }
-  // ... and q~ and z of the attention without keys and values, bf16 [B, heads, H] each
+  // ... and q~ and z of the attention without keys and values, bf16 [B, heads, H] and [B, heads, 2, H]
   m->cls_pool_off = m->cls_bytes;
   if (!m->fp8 && 3 * m->max_seq >= 2 * m->trunk.heads)
-    m->cls_bytes += 2 * pad256(static_cast<size_t>(m->max_batch) * m->trunk.heads * H * 2);
+    m->cls_bytes += 3 * pad256(static_cast<size_t>(m->max_batch) * m->trunk.heads * H * 2);
   m->ws_cls0 = off;
   off += m->cls_bytes * m->tasks.size();
   m->n_dump = 0;
@@ -921,9 +922,9 @@ cudaError_t build_cls_pool(const mt_model* m, const std::vector<OpDesc>& ops, si
   memset(&v, 0, sizeof(v));
   p.batch = batch; p.seq = seq; p.heads = m->trunk.heads;
   p.row_start = reinterpret_cast<const int32_t*>(m->d_workspace + m->ws_row_start);
-  v.M = batch; v.N = H; v.K = H;
+  v.M = batch; v.N = H; v.K = 2 * H;
   v.block_n = 64;
-  v.x_by_tile = 1;
+  v.x_by_tile = 2;
   v.status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
   gemm_choose_low(&v, static_cast<int32_t>(count), m->sm_count);
   for (size_t i = 0; i < count; ++i) {

@@ -121,7 +121,8 @@ struct alignas(64) GemmParams {
   int32_t block_n;         // tile width along N: 128, 192 or 256 (gemm_block_n); N % block_n == 0
   int32_t low;             // 64 or 32: tiles of that many rows (block_n 64, single CTAs, bf16); 0: 128.  The X and W maps are
                            // then dims {64, rows, K / 64}, box {64, low | 64, kGemmLowKBlocks}
-  int32_t x_by_tile;       // 1: column tile n (block_n 64) multiplies columns n K .. n K + K - 1 of X, which has N / 64 * K of them
+  int32_t x_by_tile;       // s = 1 or 2: column tile n (block_n 64) multiplies columns n K .. n K + K - 1 of X, which has N / 64 * K
+                           // of them: s pieces of K / s columns, summands of X, each against all K / s columns of W
   int32_t k_splits;        // ranges K is split into (kEpiPartialF32 only; otherwise 1): (K / 64) % k_splits == 0
   int32_t split_pitch;     // rows between the outputs of consecutive ranges (a multiple of 128, >= M)
   int32_t fp8;             // 1: X and W are E4M3 bytes (maps of uint8, boxes of 128 bytes of K) with row scales;
@@ -194,7 +195,7 @@ struct ClsAttnParams {
 cudaError_t launch_cls_attention(const ClsAttnParams& p, cudaStream_t stream);
 
 // The same without keys and values (cls_pool.cu): q~ = Wk^T (Wq x_0 + bq) per head, softmax over q~ . x_j / 8, z = the
-// weighted sum of the rows x_j per head; the context is then z Wv^T + bv, a GEMM with GemmParams::x_by_tile.  Two launches.
+// weighted sum of the rows x_j per head; the context is then z Wv^T + bv, a GEMM with GemmParams::x_by_tile 2.  Two launches.
 // Also gathers the fp32 residual, res[b, :] = in32[row_start[b], :].
 struct ClsPoolParams {
   const bf16* x[kMaxGroups];     // layer input [rows, H]
@@ -203,7 +204,7 @@ struct ClsPoolParams {
   const bf16* bq[kMaxGroups];
   const bf16* wk[kMaxGroups];
   bf16* qt[kMaxGroups];          // scratch [B, heads, H]: q~
-  bf16* z[kMaxGroups];           // [B, heads, H]
+  bf16* z[kMaxGroups];           // [B, heads, 2, H]: a bf16 and the bf16 of what it leaves
   float* res[kMaxGroups];        // [B, H]
   const int32_t* lengths;
   const int32_t* row_start;      // [B + 1]
