@@ -598,14 +598,13 @@ int fused_ln_kind(const mt_model* m, int32_t groups, int64_t rows) {
   if (m->pack_tokens && m->expected_tokens > 0 && m->expected_tokens < in_use) in_use = m->expected_tokens;
   if (in_use * groups <= 1024) return 0;
   if (m->d_workspace == nullptr) return groups == 1 ? 1 : (groups == 2 ? 2 : 0);   // (the device is not known yet)
-  // One layer in a single round of narrow tiles, blocks of 128 rows, us per forward of seven layers, fused / separate: 10
-  // blocks 414 / 396, 12: 419 / 404, 16: 466 / 497, 20: 502 / 545; two rounds 24: 586 / 506, 32: 638 / 610, 40: 739 / 779.
-  // Pairs, the same forward, blocks of 256 rows, pairs / narrow / separate: 17 of a round of 22 901 / 959 / 921, 20: 1005 /
-  // 1070 / 1119, 24 (two rounds): 1432 / 1282 / 1238, 28: 1580 / 1469 / 1467, 40: 1829 / 1996 / 2043.  Several layers: 21
-  // tasks 32 x 128, 16 blocks each: 1531 from the line at 75 of 100, 1618 with it at 70; 256 x 128 9.31 ms / 9.40 / 9.75 (there
-  // the memory traffic is energy, which sets the clock).  With ragged lengths fewer rows are in use than the launch is
-  // planned for, unless the caller has said how many: two layers of 10 planned blocks, 5 in use: 1023 / 990 separate - hence
-  // the higher line for several layers in one round, and narrow tiles for 32 planned blocks of 128, 18 in use (1683 / 1730).
+  // In blocks of 128 rows (pairs: 256), us per forward, fused / separate, the eight-task tree asked for one task (ten layers, one
+  // per wave) at sequence length 128, full lengths.  One layer in a single round of narrow tiles: 12 blocks 610 / 579, 16:
+  // 642 / 637, 20: 706 / 706, with nine sixteenths of the rows in use 16: 620 / 613, 24: 673 / 678; two rounds 24: 857 / 725, 32:
+  // 934 / 866.  Pairs, 18 of a round of 22: 911 / 917, 20: 977 / 1073, 22: 995 / 1071, 24 (two rounds): 1255 / 1107, 36: 1589 /
+  // 1570, 40: 1675 / 1830, 44: 1791 / 1986, 64 (three): 2535 / 2647.  Several layers: 21 tasks 32 x 128, 16 blocks each: 1531
+  // from the line at 75 of 100, 1618 with it at 70; 256 x 128 9.31 ms / 9.75 (there the memory traffic is energy, which sets
+  // the clock).
   const int64_t tiles = (in_use + kGemmBlockM - 1) / kGemmBlockM * groups;
   const int64_t fit = gemm_ln_resident(m->trunk.hidden), fit_pair = gemm_ln_pair_resident(m->trunk.hidden);
   if (fit < 1 || fit_pair < 1) return 0;
@@ -613,8 +612,20 @@ int fused_ln_kind(const mt_model* m, int32_t groups, int64_t rows) {
   const int64_t tiles_pair = (in_use + 2 * kGemmBlockM - 1) / (2 * kGemmBlockM) * groups;
   const int64_t rounds_pair = (tiles_pair + fit_pair - 1) / fit_pair;
   const bool rows_known = !m->pack_tokens || m->expected_tokens > 0;
-  if (100 * tiles_pair >= (rounds_pair == 1 && groups > 1 && !rows_known ? 95 : 75) * rounds_pair * fit_pair) return 2;
-  return groups == 1 && tiles <= 2 * fit && 100 * tiles >= 70 * 2 * fit ? 1 : 0;
+  const bool pairs_fill = 100 * tiles_pair >= (rounds_pair == 1 && groups > 1 && !rows_known ? 95 : 75) * rounds_pair * fit_pair;
+  if (rows_known || groups > 1 || m->fp8) return pairs_fill ? 2 : 0;   // (8-bit: the separate LayerNorm quantises as well)
+  // One layer whose valid rows are not known: a batch of lengths U[S/8, S] uses nine sixteenths of the rows that the launch is
+  // planned for, a round of pairs takes as long with ten row blocks as with twenty, and the separate projection's tile width is
+  // that of the planned rows.  So the choice has to stand at both ends (full lengths / nine sixteenths, us as above):
+  //  - the separate projection's 128-column tiles fit in one round: separate (24 blocks: 725 / 678; narrow 857 / 673);
+  //  - nine sixteenths are one round of narrow tiles: narrow (28: 920 / 666, separate 846 / 742, pairs 861 / 760; 36: 975 /
+  //    721, 917 / 820, 911 / 813; hidden 1024, 24: 1548 / 1149, 1545 / 1170, 1436 / 1311);
+  //  - beyond, pairs if they fill their rounds, or if two rounds planned are one of use while the separate projection
+  //    keeps its second (48: 1255 / 873, 1107 / 993; 64: 1504 / 1041, 1463 / 1217; hidden 1024, 40: 2334 / 1492, 2314 / 1663).
+  const int64_t columns = m->trunk.hidden / 128;
+  if (tiles * columns <= m->sm_count) return 0;
+  if (9 * tiles <= 16 * fit) return 1;
+  return pairs_fill || (rounds_pair == 2 && 9 * tiles * columns > 16 * m->sm_count) ? 2 : 0;
 }
 // Ranges the K of the FFN-down projection is split into.  A launch of few rows has few tiles, and each walks
 // K = F by itself (48 k-blocks one after the other for BERT-base) while most SMs have none: four ranges, each a

@@ -46,3 +46,27 @@ def task_triples(cfg):
 def dev_batch(batch):
     return (torch.from_numpy(batch.token_ids).cuda(), torch.from_numpy(batch.segment_ids).cuda(),
             torch.from_numpy(batch.lengths).cuda())
+
+
+def captured_kernels(run):
+    """[(name, grid, block)] of the kernels that ``run`` launches, in order of capture, read from a CUDA graph."""
+    from cuda.bindings import driver
+
+    def ok(result):
+        assert result[0] == driver.CUresult.CUDA_SUCCESS, result[0]
+        return result[1:]
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    run()                          # (plans are built outside the capture)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        run()
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    count = ok(driver.cuGraphGetNodes(raw, 0))[1]
+    out = []
+    for node in ok(driver.cuGraphGetNodes(raw, count))[0]:
+        if ok(driver.cuGraphNodeGetType(node))[0] != driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        p = ok(driver.cuGraphKernelNodeGetParams(node))[0]
+        name = ok(driver.cuFuncGetName(p.func))[0] if int(p.func) else ok(driver.cuKernelGetName(p.kern))[0]
+        out.append((name.decode(), (p.gridDimX, p.gridDimY, p.gridDimZ), (p.blockDimX, p.blockDimY, p.blockDimZ)))
+    return out

@@ -1,0 +1,46 @@
+"""What a forward launches, read from a captured graph: which kernel carries the residual projections of a plan that does not know
+how many of its rows are in use."""
+import pytest
+import torch
+
+from paper_2107_05377_b200 import binding as mt
+from paper_2107_05377_b200 import synth
+from gpu_util import cached_weights, captured_kernels, dev_batch
+
+pytestmark = pytest.mark.gpu
+
+# two layers on all tokens, one per wave, and a last branch layer
+ONE = synth.TreeConfig(trunk_layers=2, vocab_size=2000, tasks=(synth.TaskSpec(2, 1, 2),))
+WIDE = synth.TreeConfig(hidden=1024, heads=16, ffn=4096, trunk_layers=2, vocab_size=2000, tasks=(synth.TaskSpec(2, 1, 2),))
+
+
+def model_and_run(cfg, B, S, lo=16, **options):
+    _, blob, _ = cached_weights(cfg, 1)
+    model = mt.MTModel(cfg, B, S)
+    model.load_weights(blob)
+    for key, value in options.items():
+        model.set_option(key, value)
+    batch = synth.make_batch(cfg, B, S, lo, S, seed=4)
+    ids = dev_batch(batch)
+    logits = torch.empty(B, cfg.total_classes, device="cuda")
+    return model, lambda: model.forward(*ids, logits)
+
+
+# Row blocks that need every branch of the rule for launches of one layer: a single round of narrow tiles, the separate
+# projection in one round of its own, narrow tiles in up to 16/9 rounds, pairs that fill their rounds, pairs whose two
+# planned rounds are one of use.  (Both ends of 16/9: 25 and 39 blocks at 22 resident clusters.)
+@pytest.mark.parametrize("cfg,B,known,kind", [
+    (ONE, 20, False, "narrow"), (ONE, 24, False, "separate"), (ONE, 25, False, "narrow"), (ONE, 28, False, "narrow"),
+    (ONE, 39, False, "narrow"), (ONE, 40, False, "pair"), (ONE, 48, False, "pair"), (ONE, 64, False, "pair"),
+    (ONE, 28, True, "separate"), (ONE, 32, True, "separate"), (ONE, 40, True, "pair"), (ONE, 48, True, "separate"),
+    (WIDE, 18, False, "separate"), (WIDE, 24, False, "narrow"), (WIDE, 28, False, "pair"), (WIDE, 32, False, "separate")])
+def test_kernel_of_the_residual_projections_of_one_layer(cfg, B, known, kind):
+    S = 128
+    model, run = model_and_run(cfg, B, S, **({"expected_tokens": B * S} if known else {}))
+    names = [name for name, _, _ in captured_kernels(run)]
+    count = {"narrow": sum("gemm_ln_tcgen05" in n for n in names), "pair": sum("gemm_ln_pair_tcgen05" in n for n in names)}
+    want = {"narrow": 0, "pair": 0}
+    if kind != "separate":
+        want[kind] = 4                       # attention output and FFN-down of the two layers on all tokens
+    assert count == want, names
+    assert model.poll_status() == 0
