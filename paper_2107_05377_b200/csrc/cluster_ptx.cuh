@@ -84,5 +84,11 @@ __device__ __forceinline__ void tmem_st_32x16(uint32_t taddr, const uint32_t (&r
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// Clusters to launch of those that fit the device, for a caller that gives a launch this many SMs (at least one cluster).
+inline int cap_clusters(int fit, int cluster_size, int sm_count) {
+  const int given = sm_count / cluster_size > 0 ? sm_count / cluster_size : 1;
+  return fit < given ? fit : given;
+}
+
 }  // namespace
 }  // namespace mt

@@ -414,12 +414,13 @@ cudaError_t resident_clusters(int cluster_size, int* fit_out) {
 
 bool gemm_ln_supported(int N) { return N == 768 || N == 1024; }
 
-int gemm_ln_resident(int N) {
+int gemm_ln_resident(int N, int sm_count) {
   int fit = 0;
-  return gemm_ln_supported(N) && resident_clusters(N / kLnBlockN, &fit) == cudaSuccess ? fit : 0;
+  if (!gemm_ln_supported(N) || resident_clusters(N / kLnBlockN, &fit) != cudaSuccess) return 0;
+  return cap_clusters(fit, N / kLnBlockN, sm_count);
 }
 
-cudaError_t launch_gemm_ln(const GemmLnParams& p, cudaStream_t stream) {
+cudaError_t launch_gemm_ln(const GemmLnParams& p, int sm_count, cudaStream_t stream) {
   if (p.n_groups < 1 || p.n_groups > kMaxGroups || !gemm_ln_supported(p.N) || p.K % kGemmBlockK != 0 || p.K < kGemmBlockK ||
       p.M < 1)
     return cudaErrorInvalidValue;
@@ -428,6 +429,7 @@ cudaError_t launch_gemm_ln(const GemmLnParams& p, cudaStream_t stream) {
   cudaError_t err = resident_clusters(cluster_size, &fit);
   if (err != cudaSuccess) return err;
   if (fit < 1) return cudaErrorLaunchOutOfResources;
+  fit = cap_clusters(fit, cluster_size, sm_count);
   const int tiles = ((p.M + kGemmBlockM - 1) / kGemmBlockM) * p.n_groups;
   const int clusters = tiles < fit ? tiles : fit;
   return launch_kernel(gemm_ln_tcgen05, dim3(clusters * cluster_size), dim3(kLnThreads), kLnSmemBytes, stream, p,

@@ -606,7 +606,7 @@ int fused_ln_kind(const mt_model* m, int32_t groups, int64_t rows) {
   // from the line at 75 of 100, 1618 with it at 70; 256 x 128 9.31 ms / 9.75 (there the memory traffic is energy, which sets
   // the clock).
   const int64_t tiles = (in_use + kGemmBlockM - 1) / kGemmBlockM * groups;
-  const int64_t fit = gemm_ln_resident(m->trunk.hidden), fit_pair = gemm_ln_pair_resident(m->trunk.hidden);
+  const int64_t fit = gemm_ln_resident(m->trunk.hidden, m->sm_count), fit_pair = gemm_ln_pair_resident(m->trunk.hidden, m->sm_count);
   if (fit < 1 || fit_pair < 1) return 0;
   if (groups == 1 && tiles <= fit) return 100 * tiles >= 64 * fit ? 1 : 0;
   const int64_t tiles_pair = (in_use + 2 * kGemmBlockM - 1) / (2 * kGemmBlockM) * groups;
@@ -1643,8 +1643,8 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
   do {                                                                                                                 \
     LayerTail* t_ = (tail);                                                                                            \
     if (t_->out_ln != 0) {                                                                                             \
-      MT_TIMED(MT_CLASS_ATTN_OUT, t_->out_ln == 2 ? launch_gemm_ln_pair(t_->attn_out_ln, stream)                       \
-                                                  : launch_gemm_ln(t_->attn_out_ln, stream),                           \
+      MT_TIMED(MT_CLASS_ATTN_OUT, t_->out_ln == 2 ? launch_gemm_ln_pair(t_->attn_out_ln, m->sm_count, stream)          \
+                                                  : launch_gemm_ln(t_->attn_out_ln, m->sm_count, stream),              \
                "attention output GEMM + LayerNorm");                                                                   \
     } else {                                                                                                           \
       MT_TIMED(MT_CLASS_ATTN_OUT, launch_gemm(t_->attn_out, kEpiBiasResidual, m->sm_count, stream), "attention output GEMM"); \
@@ -1655,8 +1655,8 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
     MT_TIMED(MT_CLASS_FFN_UP, launch_gemm(t_->ffn_up, kEpiBiasGelu, m->sm_count, stream), "FFN up GEMM");              \
     if (t_->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_f, stream), "quantising the FFN intermediate");   \
     if (t_->down_ln != 0) {                                                                                            \
-      MT_TIMED(MT_CLASS_FFN_DOWN, t_->down_ln == 2 ? launch_gemm_ln_pair(t_->ffn_down_ln, stream)                      \
-                                                   : launch_gemm_ln(t_->ffn_down_ln, stream),                          \
+      MT_TIMED(MT_CLASS_FFN_DOWN, t_->down_ln == 2 ? launch_gemm_ln_pair(t_->ffn_down_ln, m->sm_count, stream)         \
+                                                   : launch_gemm_ln(t_->ffn_down_ln, m->sm_count, stream),             \
                "FFN down GEMM + LayerNorm");                                                                           \
     } else {                                                                                                           \
       MT_TIMED(MT_CLASS_FFN_DOWN, launch_gemm(t_->ffn_down, t_->down_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual,   \
@@ -1966,7 +1966,8 @@ int mt_kernel_linear_layernorm_tiles(const void* d_x, const void* d_w, const voi
   p.bias[0] = static_cast<const bf16*>(d_bias);
   p.gamma[0] = static_cast<const bf16*>(d_gamma);
   p.beta[0] = static_cast<const bf16*>(d_beta);
-  const cudaError_t e = tile_cols == 256 ? launch_gemm_ln_pair(p, as_stream(stream)) : launch_gemm_ln(p, as_stream(stream));
+  const int every = INT32_MAX;   // as many SMs as there are
+  const cudaError_t e = tile_cols == 256 ? launch_gemm_ln_pair(p, every, as_stream(stream)) : launch_gemm_ln(p, every, as_stream(stream));
   return e == cudaSuccess ? MT_OK : MT_ERR_CUDA;
 }
 

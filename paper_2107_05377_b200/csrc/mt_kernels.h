@@ -257,12 +257,12 @@ struct alignas(64) GemmLnParams {
 };
 // N must be 768 or 1024 (clusters of 6 or 8 CTAs), K a multiple of 64.
 bool gemm_ln_supported(int N);
-int gemm_ln_resident(int N);        // clusters resident on the current device at once (0: error)
-cudaError_t launch_gemm_ln(const GemmLnParams& p, cudaStream_t stream);
+int gemm_ln_resident(int N, int sm_count);   // clusters of a launch: resident at once, on at most sm_count SMs (0: error)
+cudaError_t launch_gemm_ln(const GemmLnParams& p, int sm_count, cudaStream_t stream);
 // The same on 256 x 256 accumulator tiles of CTA pairs, clusters of N / 256 pairs over 256 rows: identical bits, half the
 // operand bytes per tile - for launches with many row blocks.
-int gemm_ln_pair_resident(int N);
-cudaError_t launch_gemm_ln_pair(const GemmLnParams& p, cudaStream_t stream);
+int gemm_ln_pair_resident(int N, int sm_count);
+cudaError_t launch_gemm_ln_pair(const GemmLnParams& p, int sm_count, cudaStream_t stream);
 
 struct EmbedParams {
   const int32_t* token_ids;

@@ -1,5 +1,5 @@
 """What a forward launches, read from a captured graph: which kernel carries the residual projections of a plan that does not know
-how many of its rows are in use."""
+how many of its rows are in use, and how many CTAs a limit on the SMs leaves each persistent kernel."""
 import pytest
 import torch
 
@@ -43,4 +43,21 @@ def test_kernel_of_the_residual_projections_of_one_layer(cfg, B, known, kind):
     if kind != "separate":
         want[kind] = 4                       # attention output and FFN-down of the two layers on all tokens
     assert count == want, names
+    assert model.poll_status() == 0
+
+
+PERSISTENT = ("gemm_bf16_tcgen05", "gemm_ln_tcgen05", "gemm_ln_pair_tcgen05", "qkv_attention_tcgen05")
+
+
+@pytest.mark.parametrize("cfg,B,S,fused_ln", [(ONE, 28, 128, 2), (ONE, 48, 128, 2), (ONE, 48, 128, 1), (ONE, 48, 128, 3), (WIDE, 28, 128, 3),
+                                              (ONE, 64, 64, 0)])
+def test_sm_limit_holds_for_every_persistent_kernel(cfg, B, S, fused_ln):
+    limit = 40
+    model, run = model_and_run(cfg, B, S, fused_ln=fused_ln, sm_limit=limit)
+    seen = {}
+    for name, grid, _ in captured_kernels(run):
+        for kind in PERSISTENT:
+            if kind in name:
+                seen[kind] = max(seen.get(kind, 0), grid[0] * grid[1] * grid[2])
+    assert seen and max(seen.values()) <= limit, seen
     assert model.poll_status() == 0
