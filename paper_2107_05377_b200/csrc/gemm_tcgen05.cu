@@ -617,9 +617,9 @@ cudaError_t launch_one(const GemmParams& p, int sm_count, cudaStream_t stream) {
   if (err != cudaSuccess) return err;
   constexpr int tile_m = PAIR ? 2 * kGemmBlockM : (LOW ? LOW : kGemmBlockM);
   const int tiles = ((p.M + tile_m - 1) / tile_m) * (p.N / BN) * p.n_groups * (p.k_splits > 1 ? p.k_splits : 1);
-  const int workers_max = PAIR ? sm_count / 2 : sm_count;
+  const int fit = PAIR ? sm_count / 2 : sm_count;
+  const int workers_max = fit > 0 ? fit : 1;   // (a limit of one SM still takes a pair)
   const int workers = tiles < workers_max ? tiles : workers_max;
-  if (workers <= 0) return cudaSuccess;
   return launch_kernel(kernel, dim3(PAIR ? 2 * workers : workers), dim3(gemm_threads(BN, PAIR, EPI, FP8)), gemm_smem_bytes(BN, PAIR, EPI, FP8, LOW), stream,
                        p, PAIR ? 2u : 1u);
 }

@@ -61,3 +61,18 @@ def test_sm_limit_holds_for_every_persistent_kernel(cfg, B, S, fused_ln):
                 seen[kind] = max(seen.get(kind, 0), grid[0] * grid[1] * grid[2])
     assert seen and max(seen.values()) <= limit, seen
     assert model.poll_status() == 0
+
+
+def test_a_limit_of_one_sm_computes_the_same():
+    """96 x 128 rows are projected on CTA pairs, of which one SM holds none: one pair runs all the same."""
+    model, _ = model_and_run(ONE, 96, 128)
+    batch = synth.make_batch(ONE, 96, 128, 16, 128, seed=4)
+    out = {}
+    for limit in (1, 0):
+        model.workspace.zero_()              # (no earlier forward's activations)
+        model.set_option("sm_limit", limit)
+        out[limit] = torch.full((96, ONE.total_classes), float("nan"), device="cuda")
+        model.forward(*dev_batch(batch), out[limit])
+        torch.cuda.synchronize()
+        assert model.poll_status() == 0
+    assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
