@@ -136,7 +136,6 @@ struct PlanStep {
 struct Plan {
   std::vector<PlanStep> steps;
   bf16* embedding = nullptr;   // where the embedding output goes (StateBufs)
-  int32_t launches = 0;
   uint64_t last_use = 0;  // stamp of the last forward that ran this plan (least recently used goes first)
 };
 
@@ -566,7 +565,7 @@ int2* row_info(const mt_model* m) { return reinterpret_cast<int2*>(m->d_workspac
 // few tokens that q~ and z [B, heads, H] would outweigh K and V stay where they were.
 bool cls_pool_scratch(const mt_model* m) { return !m->fp8 && 3 * m->max_seq >= 2 * m->trunk.heads; }
 bool use_cls_pool(const mt_model* m, int64_t rows, int32_t seq) {
-  return m->cls_pool && m->cls_only && cls_pool_scratch(m) && rows > kSplitRowsMax && 3 * seq >= 2 * m->trunk.heads;
+  return m->cls_pool && m->d_workspace != nullptr && m->cls_only && cls_pool_scratch(m) && rows > kSplitRowsMax && 3 * seq >= 2 * m->trunk.heads;
 }
 
 // Tile width of a grouped GEMM launch (see gemm_block_n).  `rows` are the rows the launch is sized for;
@@ -640,12 +639,12 @@ int32_t down_split_count(const mt_model* m, int64_t rows) {
   if (m->ffn_down_split == 0 || m->fp8 || rows > kSplitRowsMax) return 1;
   return (m->trunk.ffn / kGemmBlockK) % kDownSplits == 0 ? kDownSplits : 1;
 }
-// Launches of steps 3-7 for `groups` layers (before mt_bind_memory; afterwards plans are built and counted).
+// Launches of steps 3-7 for `groups` layers.
 int32_t tail_launches(const mt_model* m, int32_t groups, int64_t rows) {
   const bool fused = fused_ln_kind(m, groups, rows) != 0;
-  // 8-bit operands: two quantisations, and the FFN-down projection keeps its LayerNorm as a launch of its own;
-  // so does a projection whose K is split
-  return (fused ? 3 : 5) + (m->fp8 ? 2 + (fused ? 1 : 0) : 0) + (fused && down_split_count(m, rows) > 1 ? 1 : 0);
+  const bool down_fused = fused && !m->fp8 && down_split_count(m, rows) == 1;
+  // 8-bit operands: f is quantised by a launch of its own, h1 too unless its LayerNorm, where that is a launch, does it
+  return (fused ? 1 : 2) + 1 + (down_fused ? 1 : 2) + (m->fp8 ? (fused ? 2 : 1) : 0);
 }
 
 void init_tail(const mt_model* m, LayerTail* t, int32_t rows, bool all_rows_valid, int32_t groups) {
@@ -982,12 +981,6 @@ cudaError_t build_cls_tail(const mt_model* m, const std::vector<int32_t>& tasks,
   return cudaSuccess;
 }
 
-int32_t chunk_launches(const mt_model* m, const std::vector<OpDesc>& ops, size_t first, size_t count, int64_t rows) {
-  size_t n_cls = 0;
-  for (size_t i = 0; i < count; ++i) n_cls += is_cls_op(m, ops[first + i]) ? 1 : 0;
-  return 1 + (m->fp8 ? 1 : 0) + (n_cls < count ? 1 + tail_launches(m, static_cast<int32_t>(count - n_cls), rows) : 0) +
-         (n_cls > 0 ? 1 : 0);
-}
 // Active tasks whose last branch layer is finished on first tokens right after wave w (1-based):
 // those whose last layer is in wave w with option early_heads, otherwise all of them after the last wave.
 std::vector<int32_t> cls_tasks_after_wave(const mt_model* m, const Schedule& s, size_t w) {
@@ -1001,20 +994,60 @@ std::vector<int32_t> cls_tasks_after_wave(const mt_model* m, const Schedule& s, 
   return out;
 }
 
-// Kernel launches of a built plan: the row starts, the embedding, and what mt_forward_tokens does for every step.
-int32_t plan_launches(const Plan& plan) {
-  auto tail = [](const LayerTail& t) {
-    return t.count == 0 ? 0 : (t.out_ln != 0 ? 1 : 2) + 1 + (t.down_ln != 0 ? 1 : 2) + (t.fp8 ? (t.out_ln != 0 ? 2 : 1) : 0);
-  };
-  int32_t n = 2;
-  for (const PlanStep& st : plan.steps) {
-    if (st.kind == 0) {
-      const Chunk& ck = st.chunk;
-      n += (ck.q_in.n_groups > 0 ? 1 : 0) + (ck.fused_qkv ? 1 : 0) + (ck.qkv.n_groups > 0 ? 1 : 0);
-      n += (ck.full.count > 0 && !ck.fused_qkv ? 1 : 0) + (ck.n_cls > 0 ? 1 : 0) + tail(ck.full);
-    } else {
-      n += st.kind == 2 ? tail(st.tail) : (st.kind == 4 ? 3 : (st.kind == 3 ? 1 : 2));
+// The layers of wave w (1-based) as the plan takes them.  With `pool` (use_cls_pool) the first-token attention is no part of
+// the wave.  That of all waves but the last goes beside the last two, from the start of the one before last, when all
+// its inputs are there: one fork and one join per forward, where a fork and a join per wave cost the caller's stream the
+// overlap of two launches each (23 x 101: 994 us against 1027; 32 x 128: 1009 against 1032).  With option "early_heads" each
+// stays in its own wave, since its tail follows at once.
+struct WaveOps {
+  std::vector<OpDesc> pooled;   // first-token attention without keys and values, ahead of the wave's layers
+  bool beside = false;          // ... on the side stream
+  std::vector<OpDesc> layers;
+};
+WaveOps wave_ops(const mt_model* m, const Schedule& s, size_t w, bool pool) {
+  WaveOps out;
+  const size_t last = s.waves.size();
+  out.beside = pool && !m->early_heads && w + 1 == last;
+  for (size_t v = 1; pool && v <= w; ++v)
+    if (m->early_heads || w == last ? v == w : out.beside)
+      for (const OpDesc& op : s.waves[v - 1])
+        if (is_cls_op(m, op)) out.pooled.push_back(op);
+  for (const OpDesc& op : s.waves[w - 1])
+    if (!pool || !is_cls_op(m, op)) out.layers.push_back(op);
+  return out;
+}
+
+// Kernel launches of a forward, from the schedule and the rules alone: what build_plan lays out and mt_forward_tokens enqueues.
+int32_t count_launches(const mt_model* m, const Schedule& s, int32_t batch, int32_t seq) {
+  const int64_t rows = static_cast<int64_t>(batch) * seq;
+  const bool pool = use_cls_pool(m, rows, seq);
+  auto launches_of = [](size_t n, size_t per_launch) { return static_cast<int32_t>((n + per_launch - 1) / per_launch); };
+  int32_t n = 2;   // row starts, embedding
+  for (size_t w = 0; w <= s.waves.size(); ++w) {
+    if (w >= 1) {
+      const WaveOps ops = wave_ops(m, s, w, pool);
+      n += 3 * launches_of(ops.pooled.size(), kMaxGroups);   // query, pooling, value projection
+      for (size_t first = 0; first < ops.layers.size(); first += m->n_slots) {
+        const size_t count = std::min<size_t>(m->n_slots, ops.layers.size() - first);
+        int32_t n_cls = 0;
+        for (size_t i = 0; i < count; ++i) n_cls += is_cls_op(m, ops.layers[first + i]) ? 1 : 0;
+        const int32_t n_full = static_cast<int32_t>(count) - n_cls;
+        const bool fused_qkv = n_full > 0 && use_qkv_attention(m, rows, seq);
+        // (inputs quantised), Q/K/V and attention of the layers on all tokens, of the last branch layers, the rest of the layer
+        n += (m->fp8 ? 1 : 0) + (fused_qkv ? 1 + (n_cls > 0 ? 1 : 0) : 1 + (n_full > 0 ? 1 : 0)) + (n_cls > 0 ? 1 : 0);
+        n += n_full > 0 ? tail_launches(m, n_full, rows) : 0;
+      }
+      const size_t n_tails = cls_tasks_after_wave(m, s, w).size();
+      for (size_t first = 0; first < n_tails; first += kMaxGroups)
+        n += tail_launches(m, static_cast<int32_t>(std::min<size_t>(kMaxGroups, n_tails - first)), batch);
     }
+    size_t n_compact = 0, n_token = 0;
+    for (int32_t t : s.heads[w]) {
+      n_compact += is_compact_task(m, t) ? 1 : 0;
+      n_token += is_token_task(m, t) ? 1 : 0;
+    }
+    n += launches_of(n_token, kMaxGroups) +
+         2 * (launches_of(n_compact, kMaxGroups) + launches_of(s.heads[w].size() - n_compact - n_token, kMaxGroups));
   }
   return n;
 }
@@ -1105,28 +1138,15 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
   };
   add_heads(s.heads[0]);
   for (size_t w = 1; w <= s.waves.size(); ++w) {
-    std::vector<OpDesc> ops = s.waves[w - 1];
-    if (pool) {
-      // The first-token attention is no part of the wave.  That of all waves but the last goes beside the last two, from the
-      // start of the one before last, when all its inputs are there: one fork and one join per forward, where a fork
-      // and a join per wave cost the caller's stream the overlap of two launches each (23 x 101: 994 us against 1027;
-      // 32 x 128: 1009 against 1032).  With option "early_heads" each stays in its own wave, since its tail follows at once.
-      std::vector<OpDesc> now;
-      const size_t last = s.waves.size();
-      const bool beside = !m->early_heads && w + 1 == last;
-      for (size_t v = 1; v <= w; ++v)
-        if (m->early_heads || w == last ? v == w : beside)
-          for (const OpDesc& op : s.waves[v - 1])
-            if (is_cls_op(m, op)) now.push_back(op);
-      for (size_t first = 0; first < now.size(); first += kMaxGroups) {
-        PlanStep st;
-        cudaError_t e = build_cls_pool(m, now, first, std::min<size_t>(kMaxGroups, now.size() - first), batch, seq, bufs, &st);
-        if (e != cudaSuccess) return e;
-        st.beside = beside;
-        plan->steps.push_back(std::move(st));
-      }
-      ops.erase(std::remove_if(ops.begin(), ops.end(), [&](const OpDesc& op) { return is_cls_op(m, op); }), ops.end());
+    const WaveOps wave = wave_ops(m, s, w, pool);
+    for (size_t first = 0; first < wave.pooled.size(); first += kMaxGroups) {
+      PlanStep st;
+      cudaError_t e = build_cls_pool(m, wave.pooled, first, std::min<size_t>(kMaxGroups, wave.pooled.size() - first), batch, seq, bufs, &st);
+      if (e != cudaSuccess) return e;
+      st.beside = wave.beside;
+      plan->steps.push_back(std::move(st));
     }
+    const std::vector<OpDesc>& ops = wave.layers;
     for (size_t first = 0; first < ops.size(); first += m->n_slots) {
       const size_t count = std::min<size_t>(m->n_slots, ops.size() - first);
       PlanStep st;
@@ -1148,7 +1168,6 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
     }
     add_heads(s.heads[w]);
   }
-  plan->launches = plan_launches(*plan);
   return heads_error;
 }
 
@@ -1525,34 +1544,7 @@ int mt_plan_launches(const mt_model* m, uint64_t task_mask, int32_t* n_launches)
   if (m == nullptr || n_launches == nullptr) return MT_ERR_INVALID_ARG;
   Schedule s;
   if (!build_schedule(m, task_mask, &s)) return fail(m, MT_ERR_INVALID_ARG, "task_mask selects no task");
-  if (m->d_workspace != nullptr) {
-    Plan plan;
-    cudaError_t e = build_plan(m, s, m->max_batch, m->max_seq, &plan);
-    if (e != cudaSuccess) return fail_cuda(m, e, "building the launch plan");
-    *n_launches = plan.launches;
-    return MT_OK;
-  }
-  int32_t n = 2;  // row starts, embedding
-  for (size_t w = 0; w <= s.waves.size(); ++w) {
-    if (w >= 1) {
-      const std::vector<OpDesc>& ops = s.waves[w - 1];
-      for (size_t first = 0; first < ops.size(); first += m->n_slots)
-        n += chunk_launches(m, ops, first, std::min<size_t>(m->n_slots, ops.size() - first),
-                            static_cast<int64_t>(m->max_batch) * m->max_seq);
-      const size_t n_cls_tasks = cls_tasks_after_wave(m, s, w).size();
-      for (size_t first = 0; first < n_cls_tasks; first += kMaxGroups)
-        n += tail_launches(m, static_cast<int32_t>(std::min<size_t>(kMaxGroups, n_cls_tasks - first)), m->max_batch);
-    }
-    size_t n_compact = 0, n_token = 0;
-    for (int32_t t : s.heads[w]) {
-      n_compact += is_compact_task(m, t) ? 1 : 0;
-      n_token += is_token_task(m, t) ? 1 : 0;
-    }
-    n += static_cast<int32_t>((n_token + kMaxGroups - 1) / kMaxGroups);
-    n += 2 * static_cast<int32_t>((n_compact + kMaxGroups - 1) / kMaxGroups +
-                                  (s.heads[w].size() - n_compact - n_token + kMaxGroups - 1) / kMaxGroups);
-  }
-  *n_launches = n;
+  *n_launches = count_launches(m, s, m->max_batch, m->max_seq);
   return MT_OK;
 }
 

@@ -1,5 +1,6 @@
 """What a forward launches, read from a captured graph: which kernel carries the residual projections of a plan that does not know
-how many of its rows are in use, and how many CTAs a limit on the SMs leaves each persistent kernel."""
+how many of its rows are in use, whether options choose the path that they name, the number of launches that the library
+states, and how many CTAs a limit on the SMs leaves each persistent kernel."""
 import pytest
 import torch
 
@@ -76,3 +77,32 @@ def test_a_limit_of_one_sm_computes_the_same():
         torch.cuda.synchronize()
         assert model.poll_status() == 0
     assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
+
+
+# branches of one, two and three layers at three depths, a task on the trunk, a token-level one; more than eight tails
+TREE = synth.TreeConfig(trunk_layers=3, vocab_size=2000, tasks=(
+    synth.TaskSpec(1, 1, 3), synth.TaskSpec(2, 1, 2), synth.TaskSpec(2, 3, 2), synth.TaskSpec(3, 2, 2), synth.TaskSpec(2, 0, 2),
+    synth.TaskSpec(1, 2, 3, token_level=True)) + (synth.TaskSpec(3, 1, 2),) * 6)
+
+
+@pytest.mark.parametrize("B,S", [(2, 50), (40, 17), (6, 100), (20, 128)])   # few rows, windows, pooled first tokens, both sizes of it
+@pytest.mark.parametrize("options", [{}, {"cls_pool": 0}, {"qkv_attention": 0}, {"early_heads": 1}, {"cls_only_last_layer": 0},
+                                     {"fused_ln": 0}, {"fused_ln": 3}, {"fp8_gemm": 1}, {"max_groups": 2}, {"ffn_down_split": 0}])
+def test_stated_launches_are_those_of_a_captured_forward(B, S, options):
+    cfg, options = TREE, dict(options)
+    _, blob, _ = cached_weights(cfg, 1)
+    model = mt.MTModel(cfg, B, S, fp8_gemm=bool(options.pop("fp8_gemm", 0)), max_groups=options.pop("max_groups", None))
+    model.load_weights(blob)
+    for key, value in options.items():
+        model.set_option(key, value)
+    ids = dev_batch(synth.make_batch(cfg, B, S, 1, S, seed=4))
+    logits = torch.empty(B, cfg.total_classes, device="cuda")
+    token_logits = torch.empty(B, S, cfg.total_token_classes, device="cuda")
+    names = [name for name, _, _ in captured_kernels(lambda: model.forward_tokens(*ids, logits, token_logits))]
+    assert model.plan_launches(model.full_mask()) == len(names), names
+    bf16 = model.weights_bytes() == mt.MTModel(cfg, B, S, bind=False).weights_bytes()
+    pooled = bf16 and B * S > 512 and 3 * S >= 2 * cfg.heads and options.get("cls_pool", 1) and options.get("cls_only_last_layer", 1)
+    windows = bf16 and B * S >= 256 and S <= 64 and options.get("qkv_attention", 1)
+    assert any("cls_pool_kernel" in n for n in names) == bool(pooled)
+    assert any("qkv_attention_tcgen05" in n for n in names) == bool(windows)
+    assert model.poll_status() == 0

@@ -119,6 +119,17 @@ def test_scheduler_masks_and_wavefront_of_the_8_task_tree(lib):
     m2.close()
 
 
+def test_launches_of_8_bit_layers(lib):
+    """With 8-bit operands a layer on all tokens quantises its input and f by launches of their own, and h1 in the LayerNorm
+    before the FFN where that is a launch (fused_ln 0: 9 launches) or by a third (1: the projection carries the LayerNorm)."""
+    m = binding.MTModel(small_cfg([(2, 0, 2)], trunk_layers=2), 4, 32, bind=False, fp8_gemm=True)
+    m.set_option("fused_ln", 0)
+    assert m.plan_launches(1) == 2 + 2 * 9 + 2
+    m.set_option("fused_ln", 1)
+    assert m.plan_launches(1) == 2 + 2 * 9 + 2
+    m.close()
+
+
 def test_token_level_tasks_in_the_plan(lib):
     """A token-level task needs every row of its last layer (no first-token shortcut) and gets its head,
     one launch, right after the wave that completes it; sequence-level tasks are planned as before."""
