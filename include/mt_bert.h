@@ -288,7 +288,7 @@ int mt_plan_cache_size(const mt_model* m);
 int mt_set_option(mt_model* m, const char* key, int64_t value);
 
 /* Per-launch timing.  With option "profile" = 1 (may be toggled at any time) every kernel launch of
- * mt_forward is bracketed by two CUDA events on the caller's stream (events are created on the host
+ * mt_forward (but the row starts, its first) is bracketed by two CUDA events on the caller's stream (events are created on the host
  * on first use).  mt_profile_read waits for the recorded events, adds the elapsed milliseconds and the
  * launch counts per kernel class since the last read into the two arrays (MT_NUM_CLASSES entries
  * each) and forgets them.  Classes follow the steps of the encoder layer. */

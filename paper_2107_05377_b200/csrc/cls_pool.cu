@@ -342,6 +342,12 @@ cudaError_t launch_query(const ClsPoolParams& p, cudaStream_t stream) {
   if (err != cudaSuccess) return err;
   return launch_kernel(kernel, dim3((p.batch + RT * 16 - 1) / (RT * 16), p.heads, p.n_groups), dim3(kCpThreads), smem, stream, p);
 }
+// sequences per CTA: a CTA reads 192 KB of weights (hidden 768) whatever their number, 64 rows of x fit
+template <int V>
+cudaError_t launch_query(const ClsPoolParams& p, cudaStream_t stream) {
+  if (p.batch <= 16) return launch_query<V, 1>(p, stream);
+  return p.batch <= 32 ? launch_query<V, 2>(p, stream) : launch_query<V, 4>(p, stream);
+}
 template <int V>
 cudaError_t launch_pool(const ClsPoolParams& p, cudaStream_t stream) {
   constexpr int smem = kCpStages * kCpWarps * kCpKeys * (V * 64 + 16) + kCpWarps * 16 * kCpPartPitch * 4 + 2 * 16 * (kCpKeys * 2 + 16) + 64;
@@ -349,20 +355,23 @@ cudaError_t launch_pool(const ClsPoolParams& p, cudaStream_t stream) {
   static PerDeviceOnce once;
   cudaError_t err = per_device_once(once, [&](int) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
   if (err != cudaSuccess) return err;
-  // sequences per CTA of the first kernel: a CTA reads 192 KB of weights (hidden 768) whatever their number, 64 rows of x fit
-  if (p.batch <= 16) err = launch_query<V, 1>(p, stream);
-  else if (p.batch <= 32) err = launch_query<V, 2>(p, stream);
-  else err = launch_query<V, 4>(p, stream);
-  if (err != cudaSuccess) return err;
   return launch_kernel(kernel, dim3(p.batch, p.n_groups), dim3(kCpThreads), smem, stream, p);
+}
+bool valid(const ClsPoolParams& p) {
+  return p.n_groups >= 1 && p.n_groups <= kMaxGroups && p.batch >= 1 && p.seq >= 1 && p.heads >= 1 && p.heads <= 16 &&
+         p.row_start != nullptr && p.lengths != nullptr;
 }
 
 }  // namespace
 
+cudaError_t launch_cls_query(const ClsPoolParams& p, cudaStream_t stream) {
+  if (!valid(p)) return cudaErrorInvalidValue;
+  if (p.heads * kHeadDim == 768) return launch_query<3>(p, stream);
+  if (p.heads * kHeadDim == 1024) return launch_query<4>(p, stream);
+  return cudaErrorInvalidValue;
+}
 cudaError_t launch_cls_pool(const ClsPoolParams& p, cudaStream_t stream) {
-  if (p.n_groups < 1 || p.n_groups > kMaxGroups || p.batch < 1 || p.seq < 1 || p.heads < 1 || p.heads > 16 || p.row_start == nullptr ||
-      p.lengths == nullptr)
-    return cudaErrorInvalidValue;
+  if (!valid(p)) return cudaErrorInvalidValue;
   if (p.heads * kHeadDim == 768) return launch_pool<3>(p, stream);
   if (p.heads * kHeadDim == 1024) return launch_pool<4>(p, stream);
   return cudaErrorInvalidValue;

@@ -1720,7 +1720,8 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
         MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
         MT_LAUNCH(cudaStreamWaitEvent(on, m->ev_fork, 0), "forking the side stream");
       }
-      MT_TIMED(MT_CLASS_ATTENTION, launch_cls_pool(st.cls_pool, on), "first-token attention kernels");
+      MT_TIMED(MT_CLASS_ATTENTION, launch_cls_query(st.cls_pool, on), "first-token query kernel");
+      MT_TIMED(MT_CLASS_ATTENTION, launch_cls_pool(st.cls_pool, on), "first-token pooling kernel");
       MT_TIMED(MT_CLASS_ATTENTION, launch_gemm(st.cls_v, kEpiBias, m->sm_count, on), "first-token value projection");
       if (beside) {
         MT_LAUNCH(cudaEventRecord(m->ev_join, on), "joining the side stream");
@@ -1744,7 +1745,8 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
         MT_TIMED(MT_CLASS_HEAD, launch_head(st.heads, stream), "head kernel");
       } else {
         st.heads.logits = d_logits;
-        MT_TIMED(MT_CLASS_HEAD, launch_pooler_head(st.heads, stream), "pooler/head kernel");
+        MT_TIMED(MT_CLASS_HEAD, launch_pooler(st.heads, stream), "pooler kernel");
+        MT_TIMED(MT_CLASS_HEAD, launch_head(st.heads, stream), "head kernel");
       }
       if (task_events != nullptr)
         for (int32_t t : st.head_tasks)

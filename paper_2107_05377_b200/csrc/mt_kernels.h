@@ -195,7 +195,7 @@ struct ClsAttnParams {
 cudaError_t launch_cls_attention(const ClsAttnParams& p, cudaStream_t stream);
 
 // The same without keys and values (cls_pool.cu): q~ = Wk^T (Wq x_0 + bq) per head, softmax over q~ . x_j / 8, z = the
-// weighted sum of the rows x_j per head; the context is then z Wv^T + bv, a GEMM with GemmParams::x_by_tile 2.  Two launches.
+// weighted sum of the rows x_j per head; the context is then z Wv^T + bv, a GEMM with GemmParams::x_by_tile 2.
 // Also gathers the fp32 residual, res[b, :] = in32[row_start[b], :].
 struct ClsPoolParams {
   const bf16* x[kMaxGroups];     // layer input [rows, H]
@@ -210,7 +210,8 @@ struct ClsPoolParams {
   const int32_t* row_start;      // [B + 1]
   int32_t n_groups, batch, seq, heads;
 };
-cudaError_t launch_cls_pool(const ClsPoolParams& p, cudaStream_t stream);
+cudaError_t launch_cls_query(const ClsPoolParams& p, cudaStream_t stream);   // q~
+cudaError_t launch_cls_pool(const ClsPoolParams& p, cudaStream_t stream);    // z and the residual
 
 // y = LN(x): x fp32; y is written as bf16 (the next GEMM's operand) and, if y32 is not null, also
 // as fp32 (the residual of the next sub-layer, so the residual stream is never rounded to bf16).
@@ -336,7 +337,8 @@ cudaError_t launch_row_starts(const int32_t* lengths, int32_t batch, int32_t seq
 cudaError_t launch_unpack_rows(const bf16* packed, const int32_t* lengths, const int32_t* row_start, bf16* padded,
                                int32_t batch, int32_t seq, int32_t hidden, int32_t compact, cudaStream_t stream);
 // Two launches: pooler (tanh features into `pooled`), then head (logits).
-cudaError_t launch_pooler_head(const HeadParams& p, cudaStream_t stream);
+cudaError_t launch_pooler(const HeadParams& p, cudaStream_t stream);
+cudaError_t launch_pooler_head(const HeadParams& p, cudaStream_t stream);   // both
 // The head alone, for a caller that has filled `pooled` itself (the pooler as a grouped GEMM).
 cudaError_t launch_head(const HeadParams& p, cudaStream_t stream);
 

@@ -603,16 +603,18 @@ cudaError_t launch_embed(const EmbedParams& p, cudaStream_t stream) {
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_pooler_head(const HeadParams& p, cudaStream_t stream) {
+cudaError_t launch_pooler(const HeadParams& p, cudaStream_t stream) {
   if (p.n_tasks < 1 || p.n_tasks > kMaxGroups || p.batch < 1 || p.hidden % 256 != 0 || p.hidden > 1024 ||
       p.pooled == nullptr)
     return cudaErrorInvalidValue;
   const size_t smem = static_cast<size_t>(kSeqPerCta) * p.hidden * sizeof(float);  // <= 32 KB
   const int chunks = (p.batch + kSeqPerCta - 1) / kSeqPerCta;
-  cudaError_t err = launch_kernel(pooler_kernel, dim3(p.hidden / kPoolFeaturesPerCta, p.n_tasks, chunks),
-                                  dim3(kHeadThreads), smem, stream, p);
-  if (err != cudaSuccess) return err;
-  return launch_kernel(head_kernel, dim3(chunks, p.n_tasks), dim3(kHeadThreads), 0, stream, p);
+  return launch_kernel(pooler_kernel, dim3(p.hidden / kPoolFeaturesPerCta, p.n_tasks, chunks), dim3(kHeadThreads), smem, stream, p);
+}
+
+cudaError_t launch_pooler_head(const HeadParams& p, cudaStream_t stream) {
+  const cudaError_t err = launch_pooler(p, stream);
+  return err != cudaSuccess ? err : launch_head(p, stream);
 }
 
 cudaError_t launch_head(const HeadParams& p, cudaStream_t stream) {

@@ -105,4 +105,7 @@ def test_stated_launches_are_those_of_a_captured_forward(B, S, options):
     windows = bf16 and B * S >= 256 and S <= 64 and options.get("qkv_attention", 1)
     assert any("cls_pool_kernel" in n for n in names) == bool(pooled)
     assert any("qkv_attention_tcgen05" in n for n in names) == bool(windows)
+    model.set_option("profile", 1)
+    model.forward_tokens(*ids, logits, token_logits)
+    assert sum(n for _, n in model.profile_read().values()) == len(names) - 1   # (the row starts are not timed)
     assert model.poll_status() == 0
