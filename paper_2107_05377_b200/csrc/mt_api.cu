@@ -56,6 +56,7 @@ struct TaskEntry {
   size_t pool_w, pool_b, cls_w, cls_b;
   size_t section_begin, section_bytes;
   int32_t col0;
+  int32_t pool_slot;   // scratch of the first-token attention without keys and values; -1: never needed
   bool loaded;
 };
 
@@ -286,7 +287,8 @@ struct mt_model {
   // workspace layout (byte offsets)
   size_t ws_status, ws_rows_valid, ws_row_start, ws_windows, ws_row_info, ws_tok, ws_seg, ws_len, ws_logits, ws_pooled, ws_partial, ws_trunk[2], ws_task0,
       ws_slot0, ws_cls0, ws_dump0;
-  size_t slot_q_off, cls_q_off, cls_pool_off;   // 8-bit scratch inside a slot / inside a task's first-token scratch
+  size_t slot_q_off, cls_q_off;   // 8-bit scratch inside a slot / inside a task's first-token scratch
+  size_t ws_pool0, pool_bytes;    // q~ and z of the tasks that have a pool_slot
   size_t cls_bytes, cls_h_bytes, cls_h32_bytes;  // per-task first-token scratch and its [B,H] bf16 / fp32 pieces
   size_t act_bytes;    // max_batch*max_seq*hidden bf16
   size_t act32_bytes;  // the same tensor in fp32
@@ -378,6 +380,11 @@ cudaError_t quantize_layer_weights(const mt_model* m, const std::vector<const La
   return cudaSuccess;
 }
 
+// Whether a forward within the model's limits can take the first-token attention without keys and values (use_cls_pool).
+bool cls_pool_scratch(const mt_model* m) {
+  return !m->fp8 && 3 * m->max_seq >= 2 * m->trunk.heads && static_cast<int64_t>(m->max_batch) * m->max_seq > kSplitRowsMax;
+}
+
 void layout_workspace(mt_model* m) {
   const size_t M = static_cast<size_t>(m->max_batch) * m->max_seq;
   const size_t H = m->trunk.hidden, F = m->trunk.ffn;
@@ -421,12 +428,16 @@ void layout_workspace(mt_model* m) {
     const size_t B = static_cast<size_t>(m->max_batch);
     m->cls_bytes += pad256(B * H) + pad256(B * F) + 2 * pad256(B * 4);
   }
-  // ... and q~ and z of the attention without keys and values, bf16 [B, heads, H] and [B, heads, 2, H]
-  m->cls_pool_off = m->cls_bytes;
-  if (!m->fp8 && 3 * m->max_seq >= 2 * m->trunk.heads)
-    m->cls_bytes += 3 * pad256(static_cast<size_t>(m->max_batch) * m->trunk.heads * H * 2);
   m->ws_cls0 = off;
   off += m->cls_bytes * m->tasks.size();
+  // q~ and z of the attention without keys and values, bf16 [B, heads, H] and [B, heads, 2, H], of the tasks whose last branch
+  // layer can have it, where a forward can be large enough
+  m->ws_pool0 = off;
+  m->pool_bytes = 3 * pad256(static_cast<size_t>(m->max_batch) * m->trunk.heads * H * 2);
+  int32_t pooled = 0;
+  for (TaskEntry& t : m->tasks)
+    t.pool_slot = cls_pool_scratch(m) && t.cfg.branch_layers > 0 && t.cfg.head_kind != MT_HEAD_TOKEN ? pooled++ : -1;
+  off += m->pool_bytes * pooled;
   m->n_dump = 0;
   m->ws_dump0 = off;
   if (m->debug_capture) {
@@ -563,7 +574,6 @@ int2* row_info(const mt_model* m) { return reinterpret_cast<int2*>(m->d_workspac
 // against 1005; 32 x 128: 1009 against 1046, 1555 against 1704 with 21 tasks; 256 x 128: 10.09 ms against 11.11).
 // The line depends on the rows of one layer alone, so a task gets the same bits whatever runs beside it.  Sequences of so
 // few tokens that q~ and z [B, heads, H] would outweigh K and V stay where they were.
-bool cls_pool_scratch(const mt_model* m) { return !m->fp8 && 3 * m->max_seq >= 2 * m->trunk.heads; }
 bool use_cls_pool(const mt_model* m, int64_t rows, int32_t seq) {
   return m->cls_pool && m->d_workspace != nullptr && m->cls_only && cls_pool_scratch(m) && rows > kSplitRowsMax && 3 * seq >= 2 * m->trunk.heads;
 }
@@ -942,7 +952,7 @@ cudaError_t build_cls_pool(const mt_model* m, const std::vector<OpDesc>& ops, si
     const LayerOffsets& lo = m->tasks[op.task].layers[op.layer - 1];
     bf16* in = layer_input(m, bufs, op);
     uint8_t* cs = m->d_workspace + m->ws_cls0 + m->cls_bytes * op.task;
-    bf16* qt = reinterpret_cast<bf16*>(cs + m->cls_pool_off);
+    bf16* qt = reinterpret_cast<bf16*>(m->d_workspace + m->ws_pool0 + m->pool_bytes * m->tasks[op.task].pool_slot);
     bf16* z = qt + pad256(static_cast<size_t>(m->max_batch) * m->trunk.heads * H * 2) / 2;
     p.x[i] = in;
     p.in32[i] = f32_of(m, in);

@@ -130,6 +130,25 @@ def test_launches_of_8_bit_layers(lib):
     m.close()
 
 
+@pytest.mark.parametrize("more,B,pooled", [((2, 1, 2), 9, True), ((2, 1, 2), 8, False), ((2, 0, 2), 9, False), ((2, 1, 2, True), 9, False)])
+def test_workspace_of_one_task_more(lib, more, B, pooled):
+    """A task adds its state, its first-token scratch, its logits and - only if its last branch layer can have its first-token
+    attention without keys and values, and a forward can have more than 512 rows - q~ and z: [B, heads, 3, hidden] bf16."""
+    S, H, F, heads = 64, 768, 3072, 12
+    pad = lambda n: (n + 255) // 256 * 256   # noqa: E731
+
+    def workspace(tasks):
+        m = binding.MTModel(small_cfg(tasks, trunk_layers=2), B, S, max_groups=1, bind=False)
+        n = m.workspace_bytes()
+        m.close()
+        return n
+    grown = workspace([(2, 1, 2), more]) - workspace([(2, 1, 2)])
+    state = pad(B * S * H * 2) + pad(B * S * H * 4)
+    first_token = 2 * pad(B * H * 2) + 3 * pad(B * H * 4) + pad(B * F * 2)
+    logits = 0 if len(more) > 3 else pad(B * 4 * 4) - pad(B * 2 * 4)
+    assert grown == state + first_token + logits + (3 * pad(B * heads * H * 2) if pooled else 0)
+
+
 def test_token_level_tasks_in_the_plan(lib):
     """A token-level task needs every row of its last layer (no first-token shortcut) and gets its head,
     one launch, right after the wave that completes it; sequence-level tasks are planned as before."""
