@@ -231,6 +231,7 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
     uint32_t acc_phase = 0;
     uint32_t stats_phase = 0;         // bit `parity`: phase of that statistics barrier
     int parity = 0;                   // statistics buffer of this tile
+    uint32_t open = 0;                // on their way: 1, 2: the tile's first, second residual box; 4: its statistics
 
     for (int tile = cluster; tile < total_tiles; tile += n_clusters) {
       const int m0 = (tile / p.n_groups) * 2 * kGemmBlockM + static_cast<int>(row_half) * kGemmBlockM;
@@ -245,6 +246,7 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
         mbar_expect_tx(my_res_bar, kLpStagingBytes);
         tma_load_2d(my_stage, &p.tmap_res[g], col0, row0, my_res_bar);
       }
+      open = 4 | 1;
       // this warp's 64 columns of bias, gamma and beta (128 bytes each) into L1 ahead of their use
       if (lane >= 1 && lane < 4) {
         const bf16* line = (lane == 1 ? p.bias[g] : (lane == 2 ? p.gamma[g] : p.beta[g])) + col0;
@@ -265,6 +267,7 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
         mbar_expect_tx(my_res_bar, kLpStagingBytes);
         tma_load_2d(my_stage, &p.tmap_res[g], col0 + 32, row0, my_res_bar);
       }
+      open = 4 | 2;
 
       if (!__all_sync(0xffffffffu, mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag))) break;
       tc_fence_after();
@@ -304,9 +307,10 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
         }
         tmem_st_32x16(taddr + c * 16, r);
       }
-      if (!res_ok) break;
-      __syncwarp();   // every lane has read the residual: the staging buffer now serves the stores
       tmem_st_wait();
+      if (!res_ok) break;
+      open = 4;
+      __syncwarp();   // every lane has read the residual: the staging buffer now serves the stores
 
       // this thread's segment of 64 values: mean and centred sum of squares, with the additions of the row-wise LayerNorm
       // kernel (eight sums of 8 in order, then a balanced tree)
@@ -336,7 +340,7 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
       }
 
       if (!__all_sync(0xffffffffu, mbar_wait_cluster(bar_stats + 8 * parity, (stats_phase >> parity) & 1u, abort_flag))) break;
-
+      open = 0;
       stats_phase ^= 1u << parity;
       // merge the segment statistics of this row, in column order
       float mean, rstd;
@@ -394,7 +398,6 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
       fence_async_shared();
       __syncwarp();
       if (lane == 0) {
-
         if (rows_in_range) tma_store_2d(&p.tmap_y[g], my_stage, col0, row0);
         tma_store_commit();
       }
@@ -405,7 +408,6 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
         if (lane == 0) tma_store_wait_read<0>();
         __syncwarp();
         tmem_ld_wait();
-
         if (h == 1) {   // the results are in registers: the MMA thread may reuse the accumulator
           tc_fence_before();
           __syncwarp();
@@ -421,11 +423,15 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
           if (rows_in_range) tma_store_2d(&p.tmap_y32[g], my_stage, col0 + h * 32, row0);
           tma_store_commit();
         }
-
       }
-
     }
-    if (lane == 0) tma_store_wait_read<0>();   // shared memory must outlive the stores that still read it
+    // shared memory must outlive the stores that still read it and (when the CTA is giving up) the copies that still write
+    // it: a residual box, the peers' statistics
+    if (lane == 0) {
+      tma_store_wait_read<0>();
+      if (open & 3) mbar_drain(my_res_bar, open & 2 ? 1u : 0u);
+      if (e == 0 && (open & 4)) mbar_drain(bar_stats + 8 * parity, (stats_phase >> parity) & 1u);
+    }
     __syncwarp();
   }
 

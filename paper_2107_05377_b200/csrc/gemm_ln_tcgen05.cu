@@ -196,6 +196,7 @@ __global__ void __launch_bounds__(kLnThreads, 1) gemm_ln_tcgen05(const __grid_co
     uint32_t res_phase = 0;           // both residual barriers complete once per tile
     uint32_t stats_phase[2] = {0, 0};
     int parity = 0;                   // statistics buffer of this tile
+    bool boxes_open = false, stats_open = false;   // this tile's residual / statistics are announced and not all in
 
     for (int tile = cluster; tile < total_tiles; tile += n_clusters) {
       const int m0 = (tile / p.n_groups) * kGemmBlockM;
@@ -212,6 +213,7 @@ __global__ void __launch_bounds__(kLnThreads, 1) gemm_ln_tcgen05(const __grid_co
         mbar_expect_tx(my_res_bar + 8, kLnStagingBytes);
         tma_load_2d(my_stage + kLnStagingBytes, &p.tmap_res[g], col0 + 32, row0, my_res_bar + 8);
       }
+      boxes_open = stats_open = true;
       // this warp's 64 columns of bias, gamma and beta (128 bytes each) into L1 ahead of their use
       if (lane < 3) {
         const bf16* line = (lane == 0 ? p.bias[g] : (lane == 1 ? p.gamma[g] : p.beta[g])) + col0;
@@ -242,6 +244,7 @@ __global__ void __launch_bounds__(kLnThreads, 1) gemm_ln_tcgen05(const __grid_co
       bool res_ok = mbar_wait(my_res_bar, res_phase, abort_flag);
       res_ok = mbar_wait(my_res_bar + 8, res_phase, abort_flag) && res_ok;
       if (!__all_sync(0xffffffffu, res_ok)) break;
+      boxes_open = false;
       res_phase ^= 1u;
       const bf16* bias = p.bias[g] + col0;
 #pragma unroll
@@ -284,6 +287,7 @@ __global__ void __launch_bounds__(kLnThreads, 1) gemm_ln_tcgen05(const __grid_co
         st_async_f2(map_to_cta(slot, static_cast<uint32_t>(peer)), mean_l, m2_l,
                     map_to_cta(bar_stats + 8 * parity, static_cast<uint32_t>(peer)));
       if (!__all_sync(0xffffffffu, mbar_wait_cluster(bar_stats + 8 * parity, stats_phase[parity], abort_flag))) break;
+      stats_open = false;
       stats_phase[parity] ^= 1u;
       // merge the 2 * cluster_size segment statistics of this row, in column order
       float mean, rstd;
@@ -359,7 +363,16 @@ __global__ void __launch_bounds__(kLnThreads, 1) gemm_ln_tcgen05(const __grid_co
         tma_store_commit();
       }
     }
-    if (lane == 0) tma_store_wait_read<0>();   // shared memory must outlive the stores that still read it
+    // shared memory must outlive the stores that still read it and (when the CTA is giving up) the copies that still write
+    // it: the residual boxes, the peers' statistics
+    if (lane == 0) {
+      tma_store_wait_read<0>();
+      if (boxes_open) {
+        mbar_drain(my_res_bar, res_phase);
+        mbar_drain(my_res_bar + 8, res_phase);
+      }
+      if (e == 0 && stats_open) mbar_drain(bar_stats + 8 * parity, stats_phase[parity]);
+    }
     __syncwarp();
   }
 
