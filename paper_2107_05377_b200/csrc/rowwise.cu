@@ -64,11 +64,9 @@ __device__ __forceinline__ void store_codes(const uint4 (&u)[V], uint2* q, float
   }
 }
 
-// PARTS: the row is put together from the partial sums of a split projection (LayerNormParams::n_parts > 0); a
-// separate instantiation, so that the plain kernel keeps its registers and occupancy.
 // QUANT: the bf16 row that leaves is quantised as well, codes and scale as by quantize_rows_kernel, which would be a launch
 // and a pass over the rows of its own (8-bit projections: 64 x 128 tokens 1657 -> 1641 us, 24 x 100 861 -> 844).
-template <int V, bool PARTS, bool QUANT>
+template <int V, bool QUANT>
 __global__ void __launch_bounds__(kRowThreads) layernorm_kernel(const LayerNormParams p) {
   constexpr int H = V * 256;
   const int lane = threadIdx.x & 31;
@@ -81,55 +79,13 @@ __global__ void __launch_bounds__(kRowThreads) layernorm_kernel(const LayerNormP
   grid_launch_dependents();
   if (row >= rows_in_use) return;
   float x[V][8];
-  if (PARTS) {
-    // the row from the partial sums of a GEMM whose K was split: the ranges in order, then the bias, then
-    // the residual - residual + ((part_0 + part_1 + ...) + bias)
-    const float* part = p.part[g] + static_cast<size_t>(row) * H;
-    const float* res = p.residual[g] + static_cast<size_t>(row) * H;
-    const size_t pitch = static_cast<size_t>(p.part_pitch) * H;
-    const int n_parts = p.n_parts;   // at most kMaxParts (checked by the launcher)
-    // every load of the row is issued before the first addition: one round trip to L2, not one per range
-    float4 pa[V][kMaxParts], pb[V][kMaxParts], ra[V], rb[V];
-    uint4 bias8[V];
+  const float* xin = p.x[g] + static_cast<size_t>(row) * H;
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const int col = (v * 32 + lane) * 8;
-#pragma unroll
-      for (int s = 0; s < kMaxParts; ++s) {
-        if (s < n_parts) {
-          pa[v][s] = *reinterpret_cast<const float4*>(part + s * pitch + col);
-          pb[v][s] = *reinterpret_cast<const float4*>(part + s * pitch + col + 4);
-        }
-      }
-      ra[v] = *reinterpret_cast<const float4*>(res + col);
-      rb[v] = *reinterpret_cast<const float4*>(res + col + 4);
-      bias8[v] = __ldg(reinterpret_cast<const uint4*>(p.bias[g] + col));
-    }
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      float acc[8] = {pa[v][0].x, pa[v][0].y, pa[v][0].z, pa[v][0].w, pb[v][0].x, pb[v][0].y, pb[v][0].z, pb[v][0].w};
-#pragma unroll
-      for (int s = 1; s < kMaxParts; ++s) {
-        if (s < n_parts) {
-          acc[0] += pa[v][s].x; acc[1] += pa[v][s].y; acc[2] += pa[v][s].z; acc[3] += pa[v][s].w;
-          acc[4] += pb[v][s].x; acc[5] += pb[v][s].y; acc[6] += pb[v][s].z; acc[7] += pb[v][s].w;
-        }
-      }
-      float bias[8];
-      unpack8(bias8[v], bias);
-      const float r[8] = {ra[v].x, ra[v].y, ra[v].z, ra[v].w, rb[v].x, rb[v].y, rb[v].z, rb[v].w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i) x[v][i] = r[i] + (acc[i] + bias[i]);
-    }
-  } else {
-    const float* xin = p.x[g] + static_cast<size_t>(row) * H;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const float4 a = *reinterpret_cast<const float4*>(xin + (v * 32 + lane) * 8);
-      const float4 b = *reinterpret_cast<const float4*>(xin + (v * 32 + lane) * 8 + 4);
-      x[v][0] = a.x; x[v][1] = a.y; x[v][2] = a.z; x[v][3] = a.w;
-      x[v][4] = b.x; x[v][5] = b.y; x[v][6] = b.z; x[v][7] = b.w;
-    }
+  for (int v = 0; v < V; ++v) {
+    const float4 a = *reinterpret_cast<const float4*>(xin + (v * 32 + lane) * 8);
+    const float4 b = *reinterpret_cast<const float4*>(xin + (v * 32 + lane) * 8 + 4);
+    x[v][0] = a.x; x[v][1] = a.y; x[v][2] = a.z; x[v][3] = a.w;
+    x[v][4] = b.x; x[v][5] = b.y; x[v][6] = b.z; x[v][7] = b.w;
   }
   float* y32 = p.y32[g] != nullptr ? p.y32[g] + static_cast<size_t>(row) * H : nullptr;
   uint4 y8[V];
@@ -147,7 +103,10 @@ __global__ void __launch_bounds__(kRowThreads) layernorm_kernel(const LayerNormP
 // The same for few rows: one CTA of V warps per row, warp v on columns v * 256 .. + 255.  A launch of a few hundred rows is
 // one row's chain of latencies, which this shortens: a third (a quarter) of the loads, sums and stores per lane, the
 // warps' segments exchanged through shared memory.  Same segments, same additions, same bits.  (128 rows: 0.95 us after the
-// dependency wait against 1.7 with a warp per row; put together from four ranges 1.5 against 3.9.)
+// dependency wait against 1.7 with a warp per row.)
+// PARTS: the row is put together from the partial sums of a split projection (LayerNormParams::n_parts > 0), which only launches of
+// few rows have: residual + ((part_0 + part_1 + ...) + bias), every load issued before the first addition (128 rows and four
+// ranges: 1.5 us against 3.9 with a warp per row).
 template <int V, bool PARTS, bool QUANT>
 __global__ void __launch_bounds__(V * 32) layernorm_row_kernel(const LayerNormParams p) {
   constexpr int H = V * 256;
@@ -571,26 +530,27 @@ cudaError_t launch_token_heads(const TokenHeadParams& p, cudaStream_t stream) {
 }
 
 namespace {
-template <int V, bool PARTS>
-cudaError_t launch_layernorm_as(const LayerNormParams& p, bool row_per_cta, cudaStream_t stream) {
-  const bool quant = p.q[0] != nullptr;
-  if (row_per_cta) {
-    auto kernel = quant ? layernorm_row_kernel<V, PARTS, true> : layernorm_row_kernel<V, PARTS, false>;
+template <int V>
+cudaError_t launch_layernorm_as(const LayerNormParams& p, cudaStream_t stream) {
+  const bool quant = p.q[0] != nullptr;   // (never of partial sums: 8-bit operands split no projection)
+  // Few rows in all: a CTA per row, for its shorter chain; beyond that a warp per row, which takes fewer instructions per
+  // row.  (6 x 128 tokens, launches of up to 4608 rows: 0.635 ms per forward with the line here, 0.647 with it at 1184, 0.682
+  // without.)
+  if (p.n_parts > 0 || static_cast<int64_t>(p.rows) * p.n_groups <= kRowPerCtaMax) {
+    auto kernel = p.n_parts > 0 ? layernorm_row_kernel<V, true, false>
+                                : (quant ? layernorm_row_kernel<V, false, true> : layernorm_row_kernel<V, false, false>);
     return launch_kernel(kernel, dim3(p.rows, p.n_groups), dim3(V * 32), 0, stream, p);
   }
-  auto kernel = quant ? layernorm_kernel<V, PARTS, true> : layernorm_kernel<V, PARTS, false>;
+  auto kernel = quant ? layernorm_kernel<V, true> : layernorm_kernel<V, false>;
   return launch_kernel(kernel, dim3((p.rows + kRowThreads / 32 - 1) / (kRowThreads / 32), p.n_groups), dim3(kRowThreads), 0, stream, p);
 }
 }  // namespace
 
 cudaError_t launch_layernorm(const LayerNormParams& p, cudaStream_t stream) {
   if (p.n_groups < 1 || p.n_groups > kMaxGroups || p.rows < 1 || p.n_parts < 0 || p.n_parts > kMaxParts) return cudaErrorInvalidValue;
-  // Few rows in all: a CTA per row, for its shorter chain; beyond that a warp per row, which takes fewer instructions per
-  // row.  (6 x 128 tokens, launches of up to 4608 rows: 0.635 ms per forward with the line here, 0.647 with it at 1184, 0.682
-  // without.)
-  const bool row_per_cta = static_cast<int64_t>(p.rows) * p.n_groups <= kRowPerCtaMax;
-  if (p.hidden == 768) return p.n_parts > 0 ? launch_layernorm_as<3, true>(p, row_per_cta, stream) : launch_layernorm_as<3, false>(p, row_per_cta, stream);
-  if (p.hidden == 1024) return p.n_parts > 0 ? launch_layernorm_as<4, true>(p, row_per_cta, stream) : launch_layernorm_as<4, false>(p, row_per_cta, stream);
+  if (p.n_parts > 0 && p.q[0] != nullptr) return cudaErrorInvalidValue;
+  if (p.hidden == 768) return launch_layernorm_as<3>(p, stream);
+  if (p.hidden == 1024) return launch_layernorm_as<4>(p, stream);
   return cudaErrorInvalidValue;
 }
 

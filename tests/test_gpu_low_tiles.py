@@ -56,3 +56,23 @@ def test_only_the_ffn_down_projection_is_summed_range_by_range(cfg, B, S):
         torch.cuda.synchronize()
         assert model.poll_status() == 0
     assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("rows,hidden,n_parts", [(1, 768, 1), (512, 1024, 4), (4736, 768, 2), (4737, 768, 3)])
+def test_rows_put_together_from_partial_sums_at_any_number_of_rows(rows, hidden, n_parts):
+    """residual + ((part_0 + part_1 + ...) + bias), in this order and in fp32, then the LayerNorm: the bits of the plain kernel on
+    the sum formed here, also beyond the rows up to which the plain kernel takes a CTA per row (4736)."""
+    gen = torch.Generator(device="cuda").manual_seed(rows)
+    rnd = lambda *shape: torch.randn(*shape, device="cuda", generator=gen)   # noqa: E731
+    pitch = (rows + 127) // 128 * 128
+    part, residual = rnd(n_parts * pitch, hidden), rnd(rows, hidden)
+    bias, gamma, beta = (rnd(hidden).bfloat16() for _ in range(3))
+    y, y32, want, want32 = (torch.full((rows, hidden), float("nan"), dtype=t, device="cuda")
+                            for t in (torch.bfloat16, torch.float32) * 2)
+    mt.mt_kernel_layernorm_partial(part, n_parts, pitch, residual, bias, gamma, beta, y, 1e-12, y_f32=y32)
+    total = part[:rows].clone()
+    for s in range(1, n_parts):
+        total += part[s * pitch:s * pitch + rows]
+    mt.mt_kernel_layernorm(residual + (total + bias.float()), gamma, beta, want, 1e-12, y_f32=want32)
+    torch.cuda.synchronize()
+    assert torch.equal(y, want) and torch.equal(y32, want32)
