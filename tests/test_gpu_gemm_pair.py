@@ -50,3 +50,19 @@ def test_bf16_results_of_wide_tiles(M, K, epilogue, block_n):
         assert torch.isnan(out[pair, bn][M:].float()).all(), "rows beyond M were written"
     assert torch.equal(out[True, block_n][:M], out[False, 128][:M])
     assert torch.equal(out[False, block_n][:M], out[False, 128][:M])
+
+
+@pytest.mark.parametrize("K", [64, 768])
+def test_pair_tiles_give_the_same_bits_every_time(K):
+    """Many tiles per cluster, again and again: the staging buffers are read, refilled by copies and read again within a tile, and
+    an order missing between two of them shows in some runs only (one did, in one forward of eight)."""
+    M, N = 20000, 768
+    x, w, b, res, gamma, beta = draw(M, N, K, seed=2)
+    y, y32 = torch.empty(M, N, dtype=torch.bfloat16, device="cuda"), torch.empty(M, N, device="cuda")
+    u, z, z32 = torch.empty_like(res), torch.empty_like(y), torch.empty_like(y32)
+    mt.mt_kernel_linear(x, w, b, res, u, 2)
+    mt.mt_kernel_layernorm(u, gamma, beta, z, 1e-12, y_f32=z32)
+    for _ in range(100):
+        y32.fill_(float("nan"))
+        mt.mt_kernel_linear_layernorm(x, w, b, res, gamma, beta, y, y32, 1e-12, tile_cols=256)
+        assert torch.equal(y32, z32) and torch.equal(y, z)
