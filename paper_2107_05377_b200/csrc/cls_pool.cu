@@ -34,26 +34,13 @@ constexpr int kCpKeys = 16;   // keys of one step
 constexpr int kCpStages = 3;  // steps of x in flight per warp
 constexpr int kCpPartPitch = kCpKeys + 8;   // floats of a head's row of partial scores (no bank is hit twice)
 
-__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 // Four B fragments (n-tiles j = 0 .. 3) from four rows of K, four consecutive columns each: lane (g, t) holds rows r0 .. r3 of
 // its t at columns g * 4 .. + 3, and tile j's column n is column n * 4 + j of the block.
 __device__ __forceinline__ void mma_rows4(float (&c)[4][4], const uint32_t (&a)[4], uint2 r0, uint2 r1, uint2 r2, uint2 r3) {
-  mma_16816(c[0], a[0], a[1], a[2], a[3], __byte_perm(r0.x, r1.x, 0x5410), __byte_perm(r2.x, r3.x, 0x5410));
-  mma_16816(c[1], a[0], a[1], a[2], a[3], __byte_perm(r0.x, r1.x, 0x7632), __byte_perm(r2.x, r3.x, 0x7632));
-  mma_16816(c[2], a[0], a[1], a[2], a[3], __byte_perm(r0.y, r1.y, 0x5410), __byte_perm(r2.y, r3.y, 0x5410));
-  mma_16816(c[3], a[0], a[1], a[2], a[3], __byte_perm(r0.y, r1.y, 0x7632), __byte_perm(r2.y, r3.y, 0x7632));
+  mma_bf16_16816(c[0], a, __byte_perm(r0.x, r1.x, 0x5410), __byte_perm(r2.x, r3.x, 0x5410));
+  mma_bf16_16816(c[1], a, __byte_perm(r0.x, r1.x, 0x7632), __byte_perm(r2.x, r3.x, 0x7632));
+  mma_bf16_16816(c[2], a, __byte_perm(r0.y, r1.y, 0x5410), __byte_perm(r2.y, r3.y, 0x5410));
+  mma_bf16_16816(c[3], a, __byte_perm(r0.y, r1.y, 0x7632), __byte_perm(r2.y, r3.y, 0x7632));
 }
 // Row g (half 0) or g + 8 (half 1) of the four tiles: this lane's columns t * 8 .. + 7 of the block of 32.
 __device__ __forceinline__ uint4 pack_row(const float (&c)[4][4], int half) {
@@ -120,8 +107,9 @@ __global__ void __launch_bounds__(kCpThreads) cls_query_kernel(const ClsPoolPara
       const uint8_t* at = smem + (r * 16 + g) * PITCH + c * 64 + t * 16;
       const uint4 lo = *reinterpret_cast<const uint4*>(at);
       const uint4 hi = *reinterpret_cast<const uint4*>(at + 8 * PITCH);
-      mma_16816(acc[r], lo.x, hi.x, lo.y, hi.y, wb[c].x, wb[c].y);
-      mma_16816(acc[r], lo.z, hi.z, lo.w, hi.w, wb[c].z, wb[c].w);
+      const uint32_t a0[4] = {lo.x, hi.x, lo.y, hi.y}, a1[4] = {lo.z, hi.z, lo.w, hi.w};
+      mma_bf16_16816(acc[r], a0, wb[c].x, wb[c].y);
+      mma_bf16_16816(acc[r], a1, wb[c].z, wb[c].w);
     }
   }
 #pragma unroll
@@ -239,7 +227,7 @@ __global__ void __launch_bounds__(kCpThreads, V == 3 ? 2 : 1) cls_pool_kernel(co
 
   for (int tile = 0; tile < n_tiles; ++tile) {
     if (tile + kCpStages - 1 < n_tiles) ask(tile + kCpStages - 1); else cp_async_commit();
-    cp_async_wait<kCpStages - 1>();
+    cp_async_wait_pending<kCpStages - 1>();
     __syncwarp();
     const uint8_t* xs = buf + tile % kCpStages * BUF;
     // this warp's part of the scores
@@ -249,8 +237,10 @@ __global__ void __launch_bounds__(kCpThreads, V == 3 ? 2 : 1) cls_pool_kernel(co
 #pragma unroll
       for (int ch = 0; ch < V; ++ch) {
         const uint4 kv = *reinterpret_cast<const uint4*>(xs + (nt * 8 + g) * PITCH + ch * 64 + t * 16);
-        mma_16816(c, qa[ch][0].x, qa[ch][1].x, qa[ch][0].y, qa[ch][1].y, kv.x, kv.y);
-        mma_16816(c, qa[ch][0].z, qa[ch][1].z, qa[ch][0].w, qa[ch][1].w, kv.z, kv.w);
+        const uint32_t a0[4] = {qa[ch][0].x, qa[ch][1].x, qa[ch][0].y, qa[ch][1].y};
+        const uint32_t a1[4] = {qa[ch][0].z, qa[ch][1].z, qa[ch][0].w, qa[ch][1].w};
+        mma_bf16_16816(c, a0, kv.x, kv.y);
+        mma_bf16_16816(c, a1, kv.z, kv.w);
       }
       float* out = parts + (warp * 16 + g) * kCpPartPitch + nt * 8 + 2 * t;
       *reinterpret_cast<float2*>(out) = make_float2(c[0], c[1]);

@@ -142,10 +142,7 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
         // before the CTA retires (the other CTAs are held by the exit barrier)
         for (int s = 0; s < prefetched; ++s) {
           mbar_arrive(bar_full + 8 * s);
-          const unsigned long long t0 = global_timer_ns();
-          while (!mbar_try_wait(bar_full + 8 * s, 0)) {
-            if (global_timer_ns() - t0 > kWaitLimitNs) break;
-          }
+          mbar_drain(bar_full + 8 * s, 0);
         }
       }
       for (int tile = cluster; tile < total_tiles && ok; tile += n_clusters) {
@@ -174,10 +171,7 @@ __global__ void __launch_bounds__(kLpThreads, 1) gemm_ln_pair_tcgen05(const __gr
         for (int i = 0; i < pending; ++i) {
           if (s == 0) { s = kLpStages; ph ^= 1u; }
           --s;
-          const unsigned long long t0 = global_timer_ns();
-          while (!mbar_try_wait(bar_full + 8 * s, ph)) {
-            if (global_timer_ns() - t0 > kWaitLimitNs) break;
-          }
+          mbar_drain(bar_full + 8 * s, ph);
         }
       }
     }

@@ -141,10 +141,7 @@ __global__ void __launch_bounds__(kLnThreads, 1) gemm_ln_tcgen05(const __grid_co
         for (int i = 0; i < pending; ++i) {
           if (s == 0) { s = kLnStages; ph ^= 1u; }
           --s;
-          const unsigned long long t0 = global_timer_ns();
-          while (!mbar_try_wait(bar_full + 8 * s, ph)) {
-            if (global_timer_ns() - t0 > kWaitLimitNs) break;
-          }
+          mbar_drain(bar_full + 8 * s, ph);
         }
       }
     }

@@ -226,10 +226,7 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
         // the early W tiles land before the CTA retires (in a pair, rank 1 is held by the exit barrier)
         for (int s = 0; s < prefetched; ++s) {
           mbar_arrive(bar_full + 8 * s);
-          const unsigned long long t0 = global_timer_ns();
-          while (!mbar_try_wait(bar_full + 8 * s, 0)) {
-            if (global_timer_ns() - t0 > kWaitLimitNs) break;
-          }
+          mbar_drain(bar_full + 8 * s, 0);
         }
       }
       for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
@@ -277,10 +274,7 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
         for (int i = 0; i < pending; ++i) {
           if (s == 0) { s = STAGES; ph ^= 1u; }
           --s;
-          const unsigned long long t0 = global_timer_ns();
-          while (!mbar_try_wait(bar_full + 8 * s, ph)) {
-            if (global_timer_ns() - t0 > kWaitLimitNs) break;
-          }
+          mbar_drain(bar_full + 8 * s, ph);
         }
       }
     }
@@ -549,9 +543,9 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
                 float x0 = __uint_as_float(v[q * 8 + 2 * j]) + bf16_lo(bw[j]);
                 float x1 = __uint_as_float(v[q * 8 + 2 * j + 1]) + bf16_hi(bw[j]);
                 if (EPI == kEpiBiasGelu) {
-                x0 = gelu_fitted(x0);
-                x1 = gelu_fitted(x1);
-              }
+                  x0 = gelu_fitted(x0);
+                  x1 = gelu_fitted(x1);
+                }
                 ow[j] = pack_bf16(x0, x1);
               }
               *reinterpret_cast<uint4*>(sbuf + staging_off(lane, half * 4 + q)) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
@@ -583,10 +577,7 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
     if (lane == 0) {
       tma_store_wait_read<0>();
       for (int i = n_done; i < n_req; ++i) {
-        const unsigned long long t0 = global_timer_ns();
-        while (!mbar_try_wait(my_res_bar + 8 * (i & 1), res_phase[i & 1])) {
-          if (global_timer_ns() - t0 > kWaitLimitNs) break;
-        }
+        mbar_drain(my_res_bar + 8 * (i & 1), res_phase[i & 1]);
       }
     }
     __syncwarp();

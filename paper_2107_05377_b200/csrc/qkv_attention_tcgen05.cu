@@ -71,12 +71,6 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
       : "memory");
 }
 
-__device__ __forceinline__ float qa_ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Byte offset of 16-byte chunk c (0..3) of row r in a warp's scratch (rows of 64 bytes; two rows per 128 bytes, chunks
 // exclusive-or'ed so that eight lanes touch eight bank groups both when a lane writes its row and when four read one).
 __device__ __forceinline__ int qa_scratch_off(int r, int c) { return r * 64 + ((c ^ ((r >> 1) & 3)) << 4); }
@@ -179,10 +173,7 @@ __global__ void __launch_bounds__(kQaThreads, 1) qkv_attention_tcgen05(const __g
       // no unit for this CTA after all: let the early W boxes land before it retires
       for (int s = 0; s < prefetched; ++s) {
         mbar_arrive(bar_full + 8 * s);
-        const unsigned long long t0 = global_timer_ns();
-        while (!mbar_try_wait(bar_full + 8 * s, 0)) {
-          if (global_timer_ns() - t0 > kWaitLimitNs) break;
-        }
+        mbar_drain(bar_full + 8 * s, 0);
       }
     }
     for (int unit = first_unit; unit < total && ok; unit += step) {
@@ -227,16 +218,10 @@ __global__ void __launch_bounds__(kQaThreads, 1) qkv_attention_tcgen05(const __g
       for (int i = 0; i < pending; ++i) {
         if (s == 0) { s = kQaStages; ph ^= 1u; }
         --s;
-        const unsigned long long t0 = global_timer_ns();
-        while (!mbar_try_wait(bar_full + 8 * s, ph)) {
-          if (global_timer_ns() - t0 > kWaitLimitNs) break;
-        }
+        mbar_drain(bar_full + 8 * s, ph);
       }
       for (int i = max(0, sets_issued - kQaColumnSets); i < sets_issued; ++i) {
-        const unsigned long long t0 = global_timer_ns();
-        while (!mbar_try_wait(bar_col + 8 * (i % kQaColumnSets), static_cast<uint32_t>((i / kQaColumnSets) & 1))) {
-          if (global_timer_ns() - t0 > kWaitLimitNs) break;
-        }
+        mbar_drain(bar_col + 8 * (i % kQaColumnSets), static_cast<uint32_t>((i / kQaColumnSets) & 1));
       }
     }
   } else if (warp == 1) {
@@ -414,8 +399,8 @@ __global__ void __launch_bounds__(kQaThreads, 1) qkv_attention_tcgen05(const __g
         uint32_t w[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
-          const float e0 = qa_ex2(fmaf(__uint_as_float(s[2 * j]), k2, -shift));
-          const float e1 = qa_ex2(fmaf(__uint_as_float(s[2 * j + 1]), k2, -shift));
+          const float e0 = ex2_approx(fmaf(__uint_as_float(s[2 * j]), k2, -shift));
+          const float e1 = ex2_approx(fmaf(__uint_as_float(s[2 * j + 1]), k2, -shift));
           row_sum += e0 + e1;
           w[j] = pack_bf16(e0, e1);
         }

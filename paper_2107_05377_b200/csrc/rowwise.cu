@@ -20,8 +20,9 @@ __device__ __forceinline__ uint32_t cvt_e4m3x2(float hi, float lo) {
 }
 // x / scale rounded to nearest, from the correctly rounded reciprocal of scale: a product, its exact remainder and one
 // correction (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990: the result is the
-// correctly rounded quotient, as long as nothing under- or overflows and scale's significand is not all ones).  A
-// zero keeps the sign of x, which the correction would lose.
+// correctly rounded quotient, as long as nothing under- or overflows and scale's significand is not all ones - which that of
+// a bf16 times fl(1 / 448) never is: the largest of the 128 is 0x7F6DB7).  A zero keeps the sign of x, which the correction
+// would lose.
 __device__ __forceinline__ float divide_by(float x, float scale, float rcp) {
   const float q = x * rcp;
   return copysignf(fmaf(fmaf(-q, scale, x), rcp, q), x);
@@ -44,7 +45,7 @@ __device__ __forceinline__ __nv_bfloat162 amax8(const uint4& u, __nv_bfloat162 a
 __device__ __forceinline__ float row_scale(float amax) { return amax == 0.f ? 1.0f : __fmul_rn(amax, 1.0f / 448.0f); }
 // (the quotients that decide a code are between 2^-10 and 448: with scale in this range no remainder underflows)
 __device__ __forceinline__ bool plain_division(float scale) {
-  return scale > 0x1p-60f && scale < 0x1p60f && (__float_as_uint(scale) & 0x7FFFFFu) != 0x7FFFFFu;
+  return scale > 0x1p-60f && scale < 0x1p60f;
 }
 __device__ __forceinline__ float warp_max(__nv_bfloat162 amax2) {
   float amax = fmaxf(__low2float(amax2), __high2float(amax2));

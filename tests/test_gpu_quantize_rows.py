@@ -1,7 +1,7 @@
 """The row-wise quantiser where its short division can go wrong: every row length it holds in registers and one that it does
 not, quotients over the whole range of the format (its subnormals and the ties between codes too), zeros of both signs, rows
-of zeros, scales outside the range of the short division and with an all-ones significand.  Codes and scales equal the
-oracle's bit for bit."""
+of zeros, scales outside the range of the short division and of every significand that a scale can have.  Codes and scales
+equal the oracle's bit for bit."""
 import numpy as np
 import pytest
 import torch
@@ -25,12 +25,6 @@ def test_codes_and_scales_equal_the_oracle(rows, cols):
     x[3::8, ::3] = -0.0
     x[4] = 0.0
     xt = torch.from_numpy(x).to(torch.bfloat16)
-    # an all-ones significand of amax / 448: the bf16 values of one binade that give it, if any, as the largest of a row
-    cand = torch.arange(0x3F80, 0x4000, dtype=torch.int32).to(torch.int16).view(torch.bfloat16)
-    scale = (cand.float() * np.float32(1.0 / 448.0)).view(torch.int32) & 0x7FFFFF
-    near = int(torch.argmax(scale))
-    xt[5] = (torch.rand(cols) * 0.9).to(torch.bfloat16)
-    xt[5, 0] = cand[near]
     q = torch.zeros(rows, cols, dtype=torch.uint8, device="cuda")
     s = torch.zeros(rows, device="cuda")
     mt.mt_kernel_quantize_rows(xt.cuda(), q, s)
@@ -38,6 +32,25 @@ def test_codes_and_scales_equal_the_oracle(rows, cols):
     want_q, want_s = f8.quantize_rows(xt.float().numpy().astype(np.float64))
     assert np.array_equal(s.cpu().numpy(), want_s)
     assert np.array_equal(q.cpu().numpy(), want_q)
+
+
+def test_every_significand_of_a_scale():
+    """The scales of the 128 bf16 values of a binade: none has the all-ones significand that the short division cannot take, and
+    every bf16 value from 2^-12 to the largest of its row gets the oracle's code (rows of 768: held in registers)."""
+    amax = torch.arange(0x3F80, 0x4000, dtype=torch.int32).to(torch.int16).view(torch.bfloat16)
+    scale = (amax.float() * np.float32(1.0 / 448.0)).view(torch.int32) & 0x7FFFFF
+    assert int(scale.max()) < 0x7FFFFF
+    values = torch.arange(0x3980, 0x4000, dtype=torch.int32).to(torch.int16).view(torch.bfloat16)   # 2^-12 .. 2
+    for piece in values.split(767):
+        rows = torch.zeros(128, 768, dtype=torch.bfloat16)
+        rows[:, 0] = amax
+        rows[:, 1:1 + len(piece)] = torch.where(piece[None] <= amax[:, None], piece[None], torch.zeros_like(piece[None]))
+        q = torch.zeros(128, 768, dtype=torch.uint8, device="cuda")
+        s = torch.zeros(128, device="cuda")
+        mt.mt_kernel_quantize_rows(rows.cuda(), q, s)
+        torch.cuda.synchronize()
+        want_q, want_s = f8.quantize_rows(rows.float().numpy().astype(np.float64))
+        assert np.array_equal(s.cpu().numpy(), want_s) and np.array_equal(q.cpu().numpy(), want_q)
 
 
 BASE = synth.TreeConfig(trunk_layers=2, tasks=(synth.TaskSpec(2, 2, 3), synth.TaskSpec(1, 1, 2), synth.TaskSpec(2, 0, 2)))
