@@ -492,8 +492,8 @@ def main():
             "e2e": {"value": aggregate_throughput(world, BATCH, args.steps, e2e_s), "unit": UNIT,
                     "h2d_bytes_per_step": 2 * BATCH * SEQ * 4 + BATCH * 4,
                     "d2h_bytes_per_step": BATCH * cfg.total_classes * 4},
-            "roofline": {"bound": "tensor", "kernel": "gemm_bf16_tcgen05 and gemm_ln_tcgen05 (QKV, attention-out, FFN-up, FFN-down launches; the two "
-                                   "residual GEMMs include the LayerNorm after them)",
+            "roofline": {"bound": "tensor", "kernel": "gemm_bf16_tcgen05, gemm_ln_tcgen05 and gemm_ln_pair_tcgen05 (QKV, attention-out, FFN-up, "
+                                   "FFN-down launches; the last two include the LayerNorm after the residual GEMM)",
                          "flops": "valid tokens only; the last layer of each branch counts its attention-output and FFN maps on one token "
                                   "per sequence",
                          "achieved": achieved, "peak": peaks["tflops"], "unit": "TFLOP/s",
