@@ -57,8 +57,13 @@ constexpr int kQaExchangeBytes = 2 * 2 * 2 * 128 * 4;      // [unit parity][max 
 constexpr int kQaScratchBytes = 32 * 64;                   // a warp's 32 rows x 32 columns of bf16 output
 constexpr uint32_t kQaColQ = 2 * kQaAccCols;               // tensor memory: Q (64 bf16 = 32 columns) and P (128 bf16 =
 constexpr uint32_t kQaColP = kQaColQ + 32;                 // 64 columns) behind the two accumulators
+// A value that is not finite stays in its own sequence: it leaves the V tile as zero - the sequences that share the window
+// have a probability of 0 for its row, and 0 times it would not be 0 - and is noted here by row and column; the output
+// of its sequence's rows in that column is NaN.  [unit parity][row] bits of 64 columns, [unit parity] last unit with any.
+// (The look at every value: 256 x 16 tokens 1461 -> 1469 us per forward, 100 x 40 1015 -> 1020.)
+constexpr int kQaNotFiniteBytes = 2 * 128 * 8 + 16;
 constexpr int kQaSmemBytes = kQaStages * (kQaABytes + kQaBBytes) + 2 * kQaTileBytes + kQaEpilogueWarps * kQaScratchBytes +
-                             kQaExchangeBytes + kQaColumnSets * kQaColumnBytes + 512 + 1024;
+                             kQaExchangeBytes + kQaColumnSets * kQaColumnBytes + kQaNotFiniteBytes + 512 + 1024;
 static_assert(kQaSmemBytes <= 227 * 1024, "shared memory of one CTA");
 
 // D[tmem] (+)= A[tmem] . B[smem]^T, 128 x N x 16: A has its rows on the lanes and two consecutive elements of K per column.
@@ -86,7 +91,9 @@ __global__ void __launch_bounds__(kQaThreads, 1) qkv_attention_tcgen05(const __g
   uint8_t* scratch_base = tiles + 2 * kQaTileBytes;
   float* exchange = reinterpret_cast<float*>(scratch_base + kQaEpilogueWarps * kQaScratchBytes);
   uint8_t* columns = scratch_base + kQaEpilogueWarps * kQaScratchBytes + kQaExchangeBytes;
-  uint8_t* book = columns + kQaColumnSets * kQaColumnBytes;
+  unsigned long long* not_finite = reinterpret_cast<unsigned long long*>(columns + kQaColumnSets * kQaColumnBytes);
+  volatile int* not_finite_unit = reinterpret_cast<volatile int*>(not_finite + 2 * 128);
+  uint8_t* book = columns + kQaColumnSets * kQaColumnBytes + kQaNotFiniteBytes;
   const uint32_t bar_full = smem_u32(book);
   const uint32_t bar_empty = bar_full + 8 * kQaStages;
   const uint32_t bar_acc_full = bar_empty + 8 * kQaStages;   // 2: the projection of a unit is complete
@@ -122,6 +129,7 @@ __global__ void __launch_bounds__(kQaThreads, 1) qkv_attention_tcgen05(const __g
     for (int q = 0; q < 4; ++q) mbar_init(bar_pair + 8 * q, 2);
     for (int c = 0; c < kQaColumnSets; ++c) mbar_init(bar_col + 8 * c, 1);
     *abort_flag = 0;
+    not_finite_unit[0] = not_finite_unit[1] = -1;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_shared();
   }
@@ -322,6 +330,7 @@ __global__ void __launch_bounds__(kQaThreads, 1) qkv_attention_tcgen05(const __g
       // (1) this half's 96 columns of Q | K | V: + bias, bf16, into the tiles; rows beyond the window are zeroed (their
       // accumulator rows are another window's or stale data, and 0 * V must stay finite)
       const uint32_t acc_addr = lane_base + static_cast<uint32_t>(acc * kQaAccCols);
+      uint32_t v_max = 0;   // largest magnitudes of this row's V, as bf16 bits
       // (32 of the 192 columns: packed to 16 words; Q's go to tensor memory, K's and V's into their tiles)
       auto convert = [&](uint32_t (&v)[32], int c) {
         const int col = half * 96 + c * 32;
@@ -338,6 +347,7 @@ __global__ void __launch_bounds__(kQaThreads, 1) qkv_attention_tcgen05(const __g
           for (int j = 0; j < 4; ++j) {
             w[j] = pack_bf16(__uint_as_float(v[q * 8 + 2 * j]) + bf16_lo(bw[j]), __uint_as_float(v[q * 8 + 2 * j + 1]) + bf16_hi(bw[j]));
             if (!row_valid) w[j] = 0u;
+            if (tile == 2) v_max = __vmaxu2(v_max, w[j] & 0x7FFF7FFFu);
           }
           if (tile > 0) *reinterpret_cast<uint4*>(tile_ptr + staging_off(row, (in_tile >> 3) + q)) = make_uint4(w[0], w[1], w[2], w[3]);
         }
@@ -354,6 +364,19 @@ __global__ void __launch_bounds__(kQaThreads, 1) qkv_attention_tcgen05(const __g
         tmem_ld_wait();
         convert(va, 2);
         if (half == 0) tmem_st_wait();
+      }
+      if (half == 1) {   // (this thread has all 64 columns of its row of V)
+        unsigned long long columns_hit = 0;
+        if (max(v_max & 0xFFFFu, v_max >> 16) >= 0x7F80u) {
+          for (int c = 0; c < 64; ++c) {
+            uint16_t* at = reinterpret_cast<uint16_t*>(tiles + kQaTileBytes + staging_off(row, c >> 3)) + (c & 7);
+            if ((*at & 0x7F80u) != 0x7F80u) continue;
+            *at = 0;
+            columns_hit |= 1ull << c;
+          }
+          not_finite_unit[parity] = unit;
+        }
+        not_finite[parity * 128 + row] = columns_hit;
       }
       fence_async_shared();
       tc_fence_before();
@@ -426,6 +449,13 @@ __global__ void __launch_bounds__(kQaThreads, 1) qkv_attention_tcgen05(const __g
       uint32_t o[32];
       tmem_ld_32x32(acc_addr + 128 + half * 32, o);
       tmem_ld_wait();
+      if (not_finite_unit[parity] == unit) {
+        uint32_t nan_columns = 0;
+        for (int j = key_lo; j < key_hi; ++j) nan_columns |= static_cast<uint32_t>(not_finite[parity * 128 + j] >> (half * 32));
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          if (nan_columns >> i & 1u) o[i] = 0x7FC00000u;
+      }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_acc_empty + 8 * acc);

@@ -87,3 +87,30 @@ def test_ctas_that_take_many_units(cfg, B, S, lo):
         torch.cuda.synchronize()
         at = cfg.logit_offsets[task]
         assert torch.equal(mine, logits[:, at:at + alone.cfg.total_classes])
+
+
+@pytest.mark.parametrize("B,S", [(16, 40), (300, 3)])
+def test_values_that_are_not_finite_stay_in_their_sequence(B, S):
+    """One sequence holds a token whose embedding is NaN: its own logits are NaN, and those of the sequences that share its
+    windows are what they are without it."""
+    cfg = synth.TreeConfig(trunk_layers=2, vocab_size=2000, tasks=(synth.TaskSpec(2, 2, 3), synth.TaskSpec(2, 0, 2)))
+    w = synth.make_weights(cfg, seed=5, random_affine=True)
+    w["emb"]["word"][1500] = 0x7FC0
+    model = mt.MTModel(cfg, B, S)
+    model.load_weights(synth.pack_weights(cfg, w))
+    batch = synth.make_batch(cfg, B, S, 2, S, seed=3)
+    batch.token_ids[batch.token_ids == 1500] = 1501
+    out = {}
+    for token in (1501, 1500, 1501):          # (and nothing of it is left for the next forward)
+        batch.token_ids[3, 1] = token
+        logits = torch.full((B, cfg.total_classes), float("inf"), device="cuda")
+        model.forward(*dev_batch(batch), logits)
+        torch.cuda.synchronize()
+        assert model.poll_status() == 0
+        if token in out:
+            assert torch.equal(out[token], logits)
+        out[token] = logits
+    others = [b for b in range(B) if b != 3]
+    assert torch.isfinite(out[1501]).all()
+    assert torch.equal(out[1500][others], out[1501][others])
+    assert torch.isnan(out[1500][3]).all()
