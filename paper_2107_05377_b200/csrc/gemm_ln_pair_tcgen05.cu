@@ -11,7 +11,7 @@
 // in the same order, so they - and the separate GEMM and LayerNorm launches - give identical bits, and the choice between
 // them may depend on the size of a launch.
 //
-// Epilogue: sixteen warps, a thread owns one row and one segment of 64 columns.  At 112 registers per thread the 64 values
+// Epilogue: sixteen warps, a thread owns one row and one segment of 64 columns.  At 96 registers per thread the 64 values
 // do not stay in registers - spilled, they cost 12 of 23 thousand clocks per tile, since L1 is nearly all shared
 // memory - but live in tensor memory, over the accumulator, and are read 16 at a time:
 //   pass 1: accumulator + bias + fp32 residual -> x, the sums (the residual arrives by TMA in two boxes through the warp's
