@@ -236,7 +236,7 @@ int mt_plan_cache_size(const mt_model* m);
  * slower on small ones; the results are bit-identical.  key "attention_tc" (0/1, default 1, any time): attention
  * for seq <= 128 runs on tcgen05 with its accumulators in tensor memory (1) or on mma.sync (0, also
  * used for every longer seq).  key "expected_tokens" (>= 0, default 0 = every row, any time): the caller's
- * estimate of the valid tokens per batch; with the packed layout the GEMM tile widths are chosen for
+ * estimate of the valid tokens per batch; with the packed layout the GEMM kernels and tile widths are chosen for
  * that many rows instead of batch*seq; it never changes a result.
  * key "fp8_gemm" (0/1, default 0; before mt_bind_memory, it enlarges both arenas): reduced precision in the
  * sense of Appendix E.  The Q/K/V, FFN-up and FFN-down projections run on E4M3 operands (tcgen05 kind::f8f6f4,
@@ -248,10 +248,12 @@ int mt_plan_cache_size(const mt_model* m);
  * about 3e-2 (measured on the 8-task tree; the tests state the bounds); merged == stand-alone still holds bit
  * for bit.
  * key "sm_limit" (>= 0, default 0 = all; any time): size the persistent GEMM grids for at most this many SMs
- * (for callers that share the GPU between several streams and want to leave room; measured no gain).
+ * (for callers that share the GPU between several streams and want to leave room; measured no gain); a launch of CTA
+ * pairs or clusters has at least one of them.
  * key "fused_ln" (0 never; 1 always, on 128-column tiles; 3 always, on 256 x 256 tiles of CTA pairs; 2 = chosen per
  * launch, the default: launches of at most "fused_ln_max_groups" (default 8) layers on all tokens whose row blocks fill
- * the clusters that are resident at once, and launches of at most "fused_ln_max_rows" (default 0) rows per layer; any
+ * the clusters that are resident at once - where the valid rows are not known (option "expected_tokens") also when
+ * fewer of them are in use -, and launches of at most "fused_ln_max_rows" (default 0) rows per layer; any
  * time): the attention-output and FFN-down projections carry the LayerNorm that follows them: the CTAs holding the
  * column blocks of the same 128 or 256 rows form a thread-block cluster and exchange per-row statistics through
  * distributed shared memory, so the pre-normalisation sum never goes to global memory and no LayerNorm launch
