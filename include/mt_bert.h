@@ -146,10 +146,14 @@ int mt_adopt_weights(mt_model* m, const mt_model* src);
  * The shared trunk runs once, to the deepest fork among the active tasks only; each active task's
  * branch starts from the trunk state at its fork depth; keys at positions >= length are excluded
  * from every softmax; the pooler reads position 0.  Asynchronous: only enqueues kernels on `stream`,
- * never synchronises, never allocates device memory.  The first call for a given
+ * never synchronises, never allocates device memory of its own.  The first call for a given
  * (batch, seq, task_mask) builds and caches a launch plan on the host (host memory and tensor-map
- * encoding only; the model's own second stream and its two events exist since mt_bind_memory) - make one
- * warm-up call before capturing mt_forward into a CUDA graph.  Option "profile" creates CUDA events here.
+ * encoding only; the model's own streams and its two events exist since mt_bind_memory) - make one
+ * warm-up call before capturing mt_forward into a CUDA graph.  A plan that has been launched 16 times is
+ * made a CUDA graph (0.7 ms, once; the driver keeps its nodes, some kilobytes each) and replayed from then on
+ * with the pointers of each call - not while `stream` is being captured, nor with task_events or options
+ * "profile" and "debug_capture"; if the graph cannot be built the kernels are launched as before, and option
+ * "replay" = 0 never builds one.  Option "profile" creates CUDA events here.
  * One mt_model serves one caller at a time: the cached plans carry per-call pointers.
  * Errors: INVALID_ARG, SHAPE, NOT_BOUND, NOT_LOADED, CUDA. */
 int mt_forward(mt_model* m, const int32_t* d_token_ids, const int32_t* d_segment_ids,
@@ -275,6 +279,7 @@ int mt_plan_cache_size(const mt_model* m);
  * the last branch layers runs without projecting keys and values: the query is taken through the key matrix and
  * the attended mean of the inputs through the value matrix (1), or as a Q/K/V projection and an attention over it (0).
  * Logits agree to rounding.
+ * key "replay" (0/1, default 1, any time): plans in frequent use run as CUDA graphs, see mt_forward;
  * key "overlap_cls" (0/1, default 1, any time): first-token attention beside layers on all tokens runs on a stream
  * that the library creates for itself (in mt_bind_memory), so that it overlaps their kernels.  With "cls_pool" it is
  * forked from the caller's stream before the wave before last and joined before the first-token tails (with

@@ -13,6 +13,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <tuple>
@@ -40,6 +41,9 @@ constexpr size_t split_pitch(size_t rows) { return (rows + 127) / 128 * 128; }
 constexpr int32_t kDownSplits = 4;
 // "Few rows": at most this many per layer (batch 4 x 128 tokens; the first-token tails of batches up to 512).
 constexpr int32_t kSplitRowsMax = 512;
+// A plan is made a graph when it has been launched this often: building one takes 0.7 ms of the host, a
+// replay saves 10 to 40 us.
+constexpr int32_t kReplayAfter = 16;
 
 inline size_t pad256(size_t n) { return (n + kAlign - 1) / kAlign * kAlign; }
 
@@ -93,7 +97,7 @@ struct LayerTail {
   // launches of few rows: the FFN-down projection as partial sums over `down_splits` ranges of K, put together
   // (ranges in order, bias, residual) by the LayerNorm kernel after it
   int32_t down_splits = 1;
-  GemmLnParams attn_out_ln, ffn_down_ln;
+  std::unique_ptr<GemmLnParams> attn_out_ln, ffn_down_ln;   // (then the plain projection's parameters stay empty)
   // 8-bit operands: the inputs of the FFN-up and FFN-down projections are quantised row by row first
   bool fp8 = false;
   QuantParams q_h1, q_f;
@@ -122,22 +126,59 @@ struct Chunk {
 };
 struct PlanStep {
   int kind;  // 0 = chunk, 1 = heads, 2 = cls tail, 3 = token-level heads, 4 = first-token attention without keys and values
-  ClsPoolParams cls_pool;           // (4)
-  GemmParams cls_v;
+  // (the parts a step does not have are not there: one is tens of kilobytes, and a first pass pays for every page)
+  std::unique_ptr<Chunk> chunk;     // (0)
+  std::unique_ptr<LayerTail> tail;  // (2)
+  std::unique_ptr<ClsPoolParams> cls_pool;   // (4)
+  std::unique_ptr<GemmParams> cls_v;
   bool beside = false;              // (4) on the side stream, joined before the first-token tails
   TokenHeadParams token_heads;
-  Chunk chunk;
   HeadParams heads;
-  bool pool_gemm = false;           // heads step: the pooler runs as a grouped GEMM (`pool`), then the head kernel
-  GemmParams pool;
+  std::unique_ptr<GemmParams> pool;   // heads step: the pooler as a grouped GEMM, then the head kernel (null: row-wise pooler)
   std::vector<int32_t> head_tasks;  // tasks of a heads step, in group order
-  LayerTail tail;
   std::vector<DumpCopy> dumps;
+};
+// What a call brings: device pointers that only the kernels of ReplayNode see (the others read the workspace).
+struct Call {
+  const int32_t *ids = nullptr, *segments = nullptr, *lengths = nullptr;
+  float *logits = nullptr, *token_logits = nullptr;
+  bool operator==(const Call& o) const {
+    return ids == o.ids && segments == o.segments && lengths == o.lengths && logits == o.logits && token_logits == o.token_logits;
+  }
+};
+// A kernel node of a replayed forward that takes pointers of the call.
+struct ReplayNode {
+  enum Kind { kRowStarts, kEmbed, kHead, kTokenHead } kind;
+  size_t step = 0;   // (heads) of the plan
+  RowStartsParams row_starts;
+  EmbedParams embed;
+  cudaGraphNode_t node = nullptr;
+  cudaKernelNodeParams launch = {};
+};
+// The launches of a plan as a CUDA graph (option "replay").  A forward of a small batch is a chain of some forty to eighty
+// dependent kernels of 3 to 8 us; launched one by one each starts about 0.35 us later than as the node of a graph, whose
+// parameters are on the device already.  us per forward, launched / replayed: 2 x 32 tokens 158 / 149, 1 x 128 387 / 362, 4 x 128
+// 500 / 474, 32 x 128 1023 / 992, 16 x 512 1959 / 1929.
+struct Replay {
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  bool pdl = true, refused = false;   // programmatic launch edges or not; could not be built (then never tried again)
+  Call call;                          // pointers that the executable graph holds at present
+  std::vector<ReplayNode> nodes;
+  Replay() = default;
+  Replay(const Replay&) = delete;
+  Replay& operator=(const Replay&) = delete;
+  ~Replay() {   // (an executable graph in flight is freed when it has completed)
+    if (exec != nullptr) cudaGraphExecDestroy(exec);
+    if (graph != nullptr) cudaGraphDestroy(graph);
+  }
 };
 struct Plan {
   std::vector<PlanStep> steps;
   bf16* embedding = nullptr;   // where the embedding output goes (StateBufs)
   uint64_t last_use = 0;  // stamp of the last forward that ran this plan (least recently used goes first)
+  int32_t launched = 0;   // forwards launched kernel by kernel that could have been replayed
+  std::unique_ptr<Replay> replay;
 };
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -273,6 +314,8 @@ struct mt_model {
   // wave's other kernels (fork after the projection, join before the next step); option "overlap_cls".
   bool overlap_cls;
   cudaStream_t side_stream;
+  bool replay;                  // option "replay": forwards of a plan in frequent use run as a CUDA graph
+  cudaStream_t replay_stream;   // where a forward is recorded as a graph
   cudaEvent_t ev_fork, ev_join;
   bool fp8;          // Q/K/V, FFN-up and FFN-down projections on E4M3 operands (set before mt_bind_memory)
   bool pool_gemm;    // the pooler of tasks with a compact final state runs as a grouped GEMM on the tensor cores
@@ -566,6 +609,9 @@ bool use_qkv_attention(const mt_model* m, int64_t rows, int32_t seq) {
 }
 int32_t* window_count(const mt_model* m) { return reinterpret_cast<int32_t*>(m->d_workspace + m->ws_windows); }
 int2* window_list(const mt_model* m) { return reinterpret_cast<int2*>(m->d_workspace + m->ws_windows + 256); }
+// The lengths of the forward under way, copied by its first kernel (or, from host buffers, put there): the later kernels need
+// no pointer of the caller's.
+int32_t* call_lengths(const mt_model* m) { return reinterpret_cast<int32_t*>(m->d_workspace + m->ws_len); }
 int2* row_info(const mt_model* m) { return reinterpret_cast<int2*>(m->d_workspace + m->ws_row_info); }
 
 // Whether the last branch layers get their first-token attention without projecting keys and values (cls_pool.cu): a few
@@ -706,16 +752,18 @@ void init_tail(const mt_model* m, LayerTail* t, int32_t rows, bool all_rows_vali
   t->count = 0;
   t->out_ln = fused_ln_kind(m, groups, rows);
   t->down_ln = !m->fp8 && t->down_splits == 1 ? t->out_ln : 0;
-  if (t->out_ln != 0 || t->down_ln != 0) {
-    auto init_ln = [&](GemmLnParams* g, int32_t K) {
+  {
+    auto init_ln = [&](std::unique_ptr<GemmLnParams>* at, int32_t K) {
+      *at = std::make_unique<GemmLnParams>();
+      GemmLnParams* g = at->get();
       memset(g, 0, sizeof(*g));
       g->M = rows; g->N = H; g->K = K;
       g->m_valid = rows_valid;
       g->eps = m->trunk.ln_eps;
       g->status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
     };
-    init_ln(&t->attn_out_ln, H);
-    init_ln(&t->ffn_down_ln, F);
+    if (t->out_ln != 0) init_ln(&t->attn_out_ln, H);
+    if (t->down_ln != 0) init_ln(&t->ffn_down_ln, F);
   }
 }
 
@@ -725,8 +773,8 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
                         float* u, bf16* h1, float* h1_32, bf16* f, bf16* out, float* out32, const QuantScratch* qs) {
   const int i = t->count;
   cudaError_t e;
-  if ((e = set_gemm_group(&t->attn_out, i, kEpiBiasResidual, ctx, w_ptr(m, lo->wo), w_ptr(m, lo->bo), residual, u)) !=
-      cudaSuccess)
+  if (t->out_ln == 0 && (e = set_gemm_group(&t->attn_out, i, kEpiBiasResidual, ctx, w_ptr(m, lo->wo), w_ptr(m, lo->bo), residual, u)) !=
+                            cudaSuccess)
     return e;
   t->ln1.x[i] = u; t->ln1.gamma[i] = w_ptr(m, lo->ln1_g); t->ln1.beta[i] = w_ptr(m, lo->ln1_b);
   t->ln1.y[i] = h1; t->ln1.y32[i] = h1_32;
@@ -766,8 +814,8 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
         return e;
       t->ln2.part[i] = part; t->ln2.residual[i] = h1_32; t->ln2.bias[i] = w_ptr(m, lo->b2);
       t->ln2.n_parts = t->down_splits; t->ln2.part_pitch = static_cast<int32_t>(pitch);
-    } else if ((e = set_gemm_group(&t->ffn_down, i, kEpiBiasResidual, f, w_ptr(m, lo->w2), w_ptr(m, lo->b2), h1_32, u)) !=
-               cudaSuccess) {
+    } else if (t->down_ln == 0 && (e = set_gemm_group(&t->ffn_down, i, kEpiBiasResidual, f, w_ptr(m, lo->w2), w_ptr(m, lo->b2),
+                                                      h1_32, u)) != cudaSuccess) {
       return e;
     }
   }
@@ -790,9 +838,9 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
     };
     // (a state is its bf16 copy followed by room for its fp32 copy: the fp32 result always has a home)
     float* out32_home = out32 != nullptr ? out32 : f32_of(m, out);
-    if ((e = set_ln(&t->attn_out_ln, ctx, lo->wo, lo->bo, lo->ln1_g, lo->ln1_b, residual, h1, h1_32)) != cudaSuccess) return e;
+    if (t->out_ln != 0 && (e = set_ln(t->attn_out_ln.get(), ctx, lo->wo, lo->bo, lo->ln1_g, lo->ln1_b, residual, h1, h1_32)) != cudaSuccess) return e;
     if (t->down_ln != 0 &&
-        (e = set_ln(&t->ffn_down_ln, f, lo->w2, lo->b2, lo->ln2_g, lo->ln2_b, h1_32, out, out32_home)) != cudaSuccess)
+        (e = set_ln(t->ffn_down_ln.get(), f, lo->w2, lo->b2, lo->ln2_g, lo->ln2_b, h1_32, out, out32_home)) != cudaSuccess)
       return e;
   }
   return cudaSuccess;
@@ -861,7 +909,8 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   ck->attn.batch = ck->attn_cls.batch = batch;
   ck->attn.seq = ck->attn_cls.seq = seq;
   ck->attn.heads = ck->attn_cls.heads = m->trunk.heads;
-  ck->attn.row_start = ck->attn_cls.row_start = row_start;  // lengths are patched per call
+  ck->attn.row_start = ck->attn_cls.row_start = row_start;
+  ck->attn.lengths = ck->attn_cls.lengths = call_lengths(m);
   ck->attn.packed = m->pack_tokens ? 1 : 0;
   ck->attn.tensor_memory = (m->attention_tc && seq <= kAttnTensorMemoryMaxSeq) ? 1 : 0;
   ck->attn.status = ck->qkv.status;
@@ -936,12 +985,15 @@ cudaError_t build_cls_pool(const mt_model* m, const std::vector<OpDesc>& ops, si
                            const StateBufs& bufs, PlanStep* st) {
   const int32_t H = m->trunk.hidden;
   st->kind = 4;
-  ClsPoolParams& p = st->cls_pool;
-  GemmParams& v = st->cls_v;
+  st->cls_pool = std::make_unique<ClsPoolParams>();
+  st->cls_v = std::make_unique<GemmParams>();
+  ClsPoolParams& p = *st->cls_pool;
+  GemmParams& v = *st->cls_v;
   memset(&p, 0, sizeof(p));
   memset(&v, 0, sizeof(v));
   p.batch = batch; p.seq = seq; p.heads = m->trunk.heads;
   p.row_start = reinterpret_cast<const int32_t*>(m->d_workspace + m->ws_row_start);
+  p.lengths = call_lengths(m);
   v.M = batch; v.N = H; v.K = 2 * H;
   v.block_n = 64;
   v.x_by_tile = 2;
@@ -970,7 +1022,8 @@ cudaError_t build_cls_pool(const mt_model* m, const std::vector<OpDesc>& ops, si
 // Steps 3-7 of the last branch layers of `tasks` on their first tokens ([B, H] rows), one group per task.
 cudaError_t build_cls_tail(const mt_model* m, const std::vector<int32_t>& tasks, size_t first, size_t count,
                            int32_t batch, PlanStep* st) {
-  init_tail(m, &st->tail, batch, true, static_cast<int32_t>(count));
+  st->tail = std::make_unique<LayerTail>();
+  init_tail(m, st->tail.get(), batch, true, static_cast<int32_t>(count));
   for (size_t i = 0; i < count; ++i) {
     const int32_t t = tasks[first + i];
     const TaskEntry& te = m->tasks[t];
@@ -984,7 +1037,7 @@ cudaError_t build_cls_tail(const mt_model* m, const std::vector<int32_t>& tasks,
     bf16* f = reinterpret_cast<bf16*>(cs + 2 * m->cls_h_bytes + 3 * m->cls_h32_bytes);
     bf16* out = task_buf(m, t);  // the task's state becomes [B, H]
     const QuantScratch qs = m->fp8 ? cls_quant(m, cs) : QuantScratch{};
-    cudaError_t e = add_to_tail(m, &st->tail, lo, ctx, res, u, h1, h1_32, f, out, nullptr, &qs);
+    cudaError_t e = add_to_tail(m, st->tail.get(), lo, ctx, res, u, h1, h1_32, f, out, nullptr, &qs);
     if (e != cudaSuccess) return e;
     if (m->debug_capture) st->dumps.push_back({out, dump_slot(m, t, te.cfg.branch_layers), true});
   }
@@ -1084,16 +1137,17 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
       st.heads.logits_stride = m->c_total;
       st.heads.pooled = reinterpret_cast<float*>(m->d_workspace + m->ws_pooled);
       st.heads.row_start = reinterpret_cast<const int32_t*>(m->d_workspace + m->ws_row_start);
-      st.pool_gemm = compact && m->pool_gemm;
-      if (st.pool_gemm) {
-        memset(&st.pool, 0, sizeof(st.pool));
-        st.pool.n_groups = static_cast<int32_t>(count);
-        st.pool.M = batch; st.pool.N = m->trunk.hidden; st.pool.K = m->trunk.hidden;
-        st.pool.pair = 0;
-        st.pool.block_n = gemm_block_n(st.pool.N, kEpiBiasTanhF32, batch, static_cast<int>(count), false, m->sm_count);
-        st.pool.m_valid = nullptr;
-        gemm_choose_low(&st.pool, static_cast<int>(count), m->sm_count);
-        st.pool.status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
+      if (compact && m->pool_gemm) {
+        st.pool = std::make_unique<GemmParams>();
+        GemmParams& pool_gemm = *st.pool;
+        memset(&pool_gemm, 0, sizeof(pool_gemm));
+        pool_gemm.n_groups = static_cast<int32_t>(count);
+        pool_gemm.M = batch; pool_gemm.N = m->trunk.hidden; pool_gemm.K = m->trunk.hidden;
+        pool_gemm.pair = 0;
+        pool_gemm.block_n = gemm_block_n(pool_gemm.N, kEpiBiasTanhF32, batch, static_cast<int>(count), false, m->sm_count);
+        pool_gemm.m_valid = nullptr;
+        gemm_choose_low(&pool_gemm, static_cast<int>(count), m->sm_count);
+        pool_gemm.status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
       }
       for (size_t i = 0; i < count; ++i) {
         const int32_t t = tasks[first + i];
@@ -1105,9 +1159,9 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
         ht.num_classes = te.cfg.num_classes; ht.col0 = te.col0;
         ht.compact = compact ? 1 : 0;
         st.head_tasks.push_back(t);
-        if (st.pool_gemm) {
+        if (st.pool != nullptr) {
           float* pooled = st.heads.pooled + i * static_cast<size_t>(batch) * m->trunk.hidden;
-          cudaError_t e = set_gemm_group(&st.pool, static_cast<int>(i), kEpiBiasTanhF32, ht.hidden, ht.pool_w,
+          cudaError_t e = set_gemm_group(st.pool.get(), static_cast<int>(i), kEpiBiasTanhF32, ht.hidden, ht.pool_w,
                                                           ht.pool_b, nullptr, pooled);
           if (e != cudaSuccess) heads_error = e;
         }
@@ -1128,6 +1182,7 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
       th.batch = batch; th.seq = seq; th.hidden = m->trunk.hidden;
       th.logits_stride = m->ct_total;
       th.row_start = reinterpret_cast<const int32_t*>(m->d_workspace + m->ws_row_start);
+      th.lengths = call_lengths(m);
       for (size_t i = 0; i < count; ++i) {
         const int32_t t = tasks[first + i];
         const TaskEntry& te = m->tasks[t];
@@ -1161,7 +1216,8 @@ cudaError_t build_plan(const mt_model* m, const Schedule& s, int32_t batch, int3
       const size_t count = std::min<size_t>(m->n_slots, ops.size() - first);
       PlanStep st;
       st.kind = 0;
-      cudaError_t e = build_chunk(m, ops, first, count, batch, seq, bufs, &st.chunk);
+      st.chunk = std::make_unique<Chunk>();
+      cudaError_t e = build_chunk(m, ops, first, count, batch, seq, bufs, st.chunk.get());
       if (e != cudaSuccess) return e;
       plan->steps.push_back(std::move(st));
     }
@@ -1227,7 +1283,8 @@ int mt_create(const mt_trunk_config* trunk, const mt_task_config* tasks, int32_t
   m->expected_tokens = 0;
   m->pool_gemm = true;
   m->overlap_cls = true;
-  m->side_stream = nullptr;
+  m->side_stream = m->replay_stream = nullptr;
+  m->replay = true;
   m->ev_fork = m->ev_join = nullptr;
   m->fused_ln = 2;
   m->fused_ln_max_groups = kMaxGroups;
@@ -1293,6 +1350,7 @@ void mt_destroy(mt_model* m) {
   if (m->ev_fork != nullptr) cudaEventDestroy(m->ev_fork);
   if (m->ev_join != nullptr) cudaEventDestroy(m->ev_join);
   if (m->side_stream != nullptr) cudaStreamDestroy(m->side_stream);
+  if (m->replay_stream != nullptr) cudaStreamDestroy(m->replay_stream);
   delete m;
 }
 
@@ -1359,6 +1417,12 @@ int mt_set_option(mt_model* m, const char* key, int64_t value) {
   }
   if (strcmp(key, "overlap_cls") == 0) {
     m->overlap_cls = value != 0;
+    m->plans.clear();
+    return MT_OK;
+  }
+  if (strcmp(key, "replay") == 0) {
+    m->replay = value != 0;
+    m->plans.clear();
     return MT_OK;
   }
   if (strcmp(key, "pool_gemm") == 0) {
@@ -1452,6 +1516,7 @@ int mt_bind_memory(mt_model* m, void* d_weights, size_t weights_bytes, void* d_w
   // that a forward never creates anything
   if (m->side_stream == nullptr) {
     if ((e = cudaStreamCreateWithFlags(&m->side_stream, cudaStreamNonBlocking)) != cudaSuccess ||
+        (e = cudaStreamCreateWithFlags(&m->replay_stream, cudaStreamNonBlocking)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&m->ev_fork, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming)) != cudaSuccess)
       return fail_cuda(m, e, "creating the side stream");
@@ -1558,6 +1623,240 @@ int mt_plan_launches(const mt_model* m, uint64_t task_mask, int32_t* n_launches)
   return MT_OK;
 }
 
+// Enqueues the kernels of a plan one by one; with `nodes` (the stream is being captured) notes those that take pointers of the call.
+static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch, int32_t seq, void* const* task_events,
+                       cudaStream_t stream, std::vector<ReplayNode>* nodes) {
+  uint32_t* status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
+  const size_t act_used = static_cast<size_t>(batch) * seq * m->trunk.hidden * sizeof(bf16);
+  cudaError_t e;
+#define MT_LAUNCH(call, what)                          \
+  do {                                                 \
+    e = (call);                                        \
+    if (e != cudaSuccess) return fail_cuda(m, e, what); \
+  } while (0)
+  // With option "profile" every kernel launch sits between two events of a pool that grows on the host.
+#define MT_TIMED(cls, call, what)                                                            \
+  do {                                                                                       \
+    if (m->profile) {                                                                        \
+      while (m->events.size() < m->events_used + 2) {                                        \
+        cudaEvent_t ev;                                                                      \
+        MT_LAUNCH(cudaEventCreate(&ev), "creating a timing event");                          \
+        m->events.push_back(ev);                                                             \
+      }                                                                                      \
+      MT_LAUNCH(cudaEventRecord(m->events[m->events_used], stream), "recording an event");   \
+    }                                                                                        \
+    MT_LAUNCH(call, what);                                                                   \
+    if (m->profile) {                                                                        \
+      MT_LAUNCH(cudaEventRecord(m->events[m->events_used + 1], stream), "recording an event"); \
+      m->events_used += 2;                                                                   \
+      m->event_class.push_back(cls);                                                         \
+    }                                                                                        \
+  } while (0)
+
+  // Steps 3-7 of the layers of a wave: three launches (each residual GEMM carries its LayerNorm) or five.
+#define MT_TAIL(tail)                                                                                                  \
+  do {                                                                                                                 \
+    LayerTail* t_ = (tail);                                                                                            \
+    if (t_->out_ln != 0) {                                                                                             \
+      MT_TIMED(MT_CLASS_ATTN_OUT, t_->out_ln == 2 ? launch_gemm_ln_pair(*t_->attn_out_ln, m->sm_count, stream)          \
+                                                  : launch_gemm_ln(*t_->attn_out_ln, m->sm_count, stream),              \
+               "attention output GEMM + LayerNorm");                                                                   \
+    } else {                                                                                                           \
+      MT_TIMED(MT_CLASS_ATTN_OUT, launch_gemm(t_->attn_out, kEpiBiasResidual, m->sm_count, stream), "attention output GEMM"); \
+      MT_TIMED(MT_CLASS_LN1, launch_layernorm(t_->ln1, stream), "LayerNorm 1");                                        \
+    }                                                                                                                  \
+    if (t_->fp8 && t_->out_ln != 0)                                                                                    \
+      MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_h1, stream), "quantising the FFN input");                    \
+    MT_TIMED(MT_CLASS_FFN_UP, launch_gemm(t_->ffn_up, kEpiBiasGelu, m->sm_count, stream), "FFN up GEMM");              \
+    if (t_->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_f, stream), "quantising the FFN intermediate");   \
+    if (t_->down_ln != 0) {                                                                                            \
+      MT_TIMED(MT_CLASS_FFN_DOWN, t_->down_ln == 2 ? launch_gemm_ln_pair(*t_->ffn_down_ln, m->sm_count, stream)         \
+                                                   : launch_gemm_ln(*t_->ffn_down_ln, m->sm_count, stream),             \
+               "FFN down GEMM + LayerNorm");                                                                           \
+    } else {                                                                                                           \
+      MT_TIMED(MT_CLASS_FFN_DOWN, launch_gemm(t_->ffn_down, t_->down_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual,   \
+                                              m->sm_count, stream), "FFN down GEMM");                                  \
+      MT_TIMED(MT_CLASS_LN2, launch_layernorm(t_->ln2, stream), "LayerNorm 2");                                        \
+    }                                                                                                                  \
+  } while (0)
+
+  int32_t* row_start = reinterpret_cast<int32_t*>(m->d_workspace + m->ws_row_start);
+  const bool fused_qkv = use_qkv_attention(m, static_cast<int64_t>(batch) * seq, seq);
+  // (a forward being recorded for replay: the kernels that take pointers of the call)
+  auto note = [&](ReplayNode::Kind kind, size_t step, const RowStartsParams& rs, const EmbedParams& em) -> cudaError_t {
+    if (nodes == nullptr) return cudaSuccess;
+    ReplayNode n;
+    n.kind = kind; n.step = step; n.row_starts = rs; n.embed = em;
+    cudaStreamCaptureStatus state;
+    const cudaGraphNode_t* last = nullptr;
+    size_t count = 0;
+    cudaError_t err = cudaStreamGetCaptureInfo_v3(stream, &state, nullptr, nullptr, &last, nullptr, &count);
+    if (err != cudaSuccess) return err;
+    if (state != cudaStreamCaptureStatusActive || count != 1) return cudaErrorUnknown;
+    n.node = last[0];
+    nodes->push_back(n);
+    return cudaSuccess;
+  };
+  RowStartsParams rs = {};
+  EmbedParams ep = {};
+  rs.lengths = call.lengths; rs.lengths_copy = call_lengths(m);
+  rs.batch = batch; rs.seq = seq; rs.packed = m->pack_tokens ? 1 : 0;
+  rs.row_start = row_start;
+  rs.rows_valid = reinterpret_cast<int32_t*>(m->d_workspace + m->ws_rows_valid);
+  rs.n_windows = fused_qkv ? window_count(m) : nullptr;
+  rs.windows = fused_qkv ? window_list(m) : nullptr;
+  MT_LAUNCH(launch_row_starts(rs, stream), "row-start kernel");
+  MT_LAUNCH(note(ReplayNode::kRowStarts, 0, rs, ep), "recording the forward");
+  ep.row_start = row_start;
+  ep.row_info = fused_qkv ? row_info(m) : nullptr;
+  ep.packed = m->pack_tokens ? 1 : 0;
+  ep.token_ids = call.ids; ep.segment_ids = call.segments; ep.lengths = call.lengths;
+  ep.word = w_ptr(m, m->emb_word); ep.pos = w_ptr(m, m->emb_pos); ep.type = w_ptr(m, m->emb_type);
+  ep.gamma = w_ptr(m, m->emb_ln_g); ep.beta = w_ptr(m, m->emb_ln_b);
+  ep.out = plan.embedding;
+  ep.out32 = f32_of(m, ep.out);
+  ep.batch = batch; ep.seq = seq; ep.hidden = m->trunk.hidden; ep.vocab = m->trunk.vocab_size;
+  ep.type_vocab = m->trunk.type_vocab; ep.eps = m->trunk.ln_eps; ep.status = status;
+  MT_TIMED(MT_CLASS_EMBED, launch_embed(ep, stream), "embedding kernel");
+  MT_LAUNCH(note(ReplayNode::kEmbed, 0, rs, ep), "recording the forward");
+  if (m->debug_capture)
+    MT_LAUNCH(cudaMemcpyAsync(m->d_workspace + m->ws_dump0, ep.out, act_used, cudaMemcpyDeviceToDevice, stream),
+              "debug capture");
+
+  bool pool_pending = false;   // ... of a step of kind 4: waited for before the first-token tails
+  bool side_pending = false;   // work on the side stream that the caller's stream has not waited for yet
+  for (size_t step = 0; step < plan.steps.size(); ++step) {
+    PlanStep& st = plan.steps[step];
+    if (side_pending || (pool_pending && st.kind == 2)) {
+      MT_LAUNCH(cudaStreamWaitEvent(stream, m->ev_join, 0), "joining the side stream");
+      side_pending = pool_pending = false;
+    }
+    if (st.kind == 0) {
+      Chunk& ck = *st.chunk;
+      if (m->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(ck.q_in, stream), "quantising the layer inputs");
+      const bool beside = m->overlap_cls && m->side_stream != nullptr && !m->profile && ck.n_cls > 0 && ck.full.count > 0;
+      if (ck.fused_qkv)
+        MT_TIMED(MT_CLASS_QKV, launch_qkv_attention(ck.qa, m->sm_count, stream), "QKV projection + attention kernel");
+      if (ck.qkv.n_groups > 0)
+        MT_TIMED(MT_CLASS_QKV, launch_gemm(ck.qkv, kEpiBias, m->sm_count, stream), "QKV GEMM");
+      if (beside) {
+        MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
+        MT_LAUNCH(cudaStreamWaitEvent(m->side_stream, m->ev_fork, 0), "forking the side stream");
+        MT_LAUNCH(launch_cls_attention(ck.attn_cls, m->side_stream), "first-token attention kernel");
+        MT_LAUNCH(cudaEventRecord(m->ev_join, m->side_stream), "joining the side stream");
+        side_pending = true;
+      }
+      if (ck.full.count > 0 && !ck.fused_qkv) MT_TIMED(MT_CLASS_ATTENTION, launch_attention(ck.attn, stream), "attention kernel");
+      if (ck.n_cls > 0 && !beside)
+        MT_TIMED(MT_CLASS_ATTENTION, launch_cls_attention(ck.attn_cls, stream), "first-token attention kernel");
+      if (ck.full.count > 0) MT_TAIL(&ck.full);
+      for (const DumpCopy& d : ck.dumps)
+        MT_LAUNCH(cudaMemcpyAsync(m->d_workspace + m->ws_dump0 + m->act_bytes * d.slot, d.src,
+                                  d.compact ? static_cast<size_t>(batch) * m->trunk.hidden * sizeof(bf16) : act_used,
+                                  cudaMemcpyDeviceToDevice, stream),
+                  "debug capture");
+    } else if (st.kind == 4) {
+      const bool beside = st.beside && m->overlap_cls && m->side_stream != nullptr && !m->profile;
+      cudaStream_t on = beside ? m->side_stream : stream;
+      if (beside) {
+        MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
+        MT_LAUNCH(cudaStreamWaitEvent(on, m->ev_fork, 0), "forking the side stream");
+      }
+      MT_TIMED(MT_CLASS_ATTENTION, launch_cls_query(*st.cls_pool, on), "first-token query kernel");
+      MT_TIMED(MT_CLASS_ATTENTION, launch_cls_pool(*st.cls_pool, on), "first-token pooling kernel");
+      MT_TIMED(MT_CLASS_ATTENTION, launch_gemm(*st.cls_v, kEpiBias, m->sm_count, on), "first-token value projection");
+      if (beside) {
+        MT_LAUNCH(cudaEventRecord(m->ev_join, on), "joining the side stream");
+        pool_pending = true;
+      }
+    } else if (st.kind == 2) {
+      MT_TAIL(st.tail.get());
+      for (const DumpCopy& d : st.dumps)
+        MT_LAUNCH(cudaMemcpyAsync(m->d_workspace + m->ws_dump0 + m->act_bytes * d.slot, d.src,
+                                  static_cast<size_t>(batch) * m->trunk.hidden * sizeof(bf16), cudaMemcpyDeviceToDevice,
+                                  stream),
+                  "debug capture");
+    } else {
+      if (st.kind == 3) {
+        st.token_heads.logits = call.token_logits;
+        MT_TIMED(MT_CLASS_HEAD, launch_token_heads(st.token_heads, stream), "token-level head kernel");
+        MT_LAUNCH(note(ReplayNode::kTokenHead, step, rs, ep), "recording the forward");
+      } else {
+        st.heads.logits = call.logits;
+        if (st.pool != nullptr) MT_TIMED(MT_CLASS_HEAD, launch_gemm(*st.pool, kEpiBiasTanhF32, m->sm_count, stream), "pooler GEMM");
+        else MT_TIMED(MT_CLASS_HEAD, launch_pooler(st.heads, stream), "pooler kernel");
+        MT_TIMED(MT_CLASS_HEAD, launch_head(st.heads, stream), "head kernel");
+        MT_LAUNCH(note(ReplayNode::kHead, step, rs, ep), "recording the forward");
+      }
+      if (task_events != nullptr)
+        for (int32_t t : st.head_tasks)
+          if (task_events[t] != nullptr)
+            MT_LAUNCH(cudaEventRecord(reinterpret_cast<cudaEvent_t>(task_events[t]), stream), "recording a task event");
+    }
+  }
+  if (side_pending || pool_pending) MT_LAUNCH(cudaStreamWaitEvent(stream, m->ev_join, 0), "joining the side stream");
+#undef MT_TAIL
+#undef MT_TIMED
+#undef MT_LAUNCH
+  return MT_OK;
+}
+
+// Records a forward of the plan as an executable graph.  Nothing of it fails the forward: without the graph it is launched.
+static void build_replay(mt_model* m, Plan& plan, const Call& call, int32_t batch, int32_t seq) {
+  plan.replay = std::make_unique<Replay>();
+  Replay& r = *plan.replay;
+  r.refused = true;
+  r.pdl = g_use_pdl;
+  // (captures of other threads go their own way, and nothing here is held against one)
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return;
+  cudaError_t e = cudaStreamBeginCapture(m->replay_stream, cudaStreamCaptureModeRelaxed);
+  if (e == cudaSuccess) {
+    const std::string before = m->last_error;
+    if (launch_plan(m, plan, call, batch, seq, nullptr, m->replay_stream, &r.nodes) != MT_OK) e = cudaErrorUnknown;
+    m->last_error = before;
+    const cudaError_t ended = cudaStreamEndCapture(m->replay_stream, &r.graph);
+    if (e == cudaSuccess) e = ended;
+  }
+  for (ReplayNode& n : r.nodes)
+    if (e == cudaSuccess) e = cudaGraphKernelNodeGetParams(n.node, &n.launch);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&r.exec, r.graph, 0);
+  if (e != cudaSuccess) cudaGetLastError();
+  r.call = call;
+  r.refused = e != cudaSuccess;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
+// Puts the pointers of this call into the executable graph (launches already enqueued keep theirs).
+static cudaError_t set_call(Plan& plan, const Call& call) {
+  Replay& r = *plan.replay;
+  if (r.call == call) return cudaSuccess;
+  r.call = Call();   // (until all nodes have the new pointers)
+  for (ReplayNode& n : r.nodes) {
+    void* args[1];
+    if (n.kind == ReplayNode::kRowStarts) {
+      n.row_starts.lengths = call.lengths;
+      args[0] = &n.row_starts;
+    } else if (n.kind == ReplayNode::kEmbed) {
+      n.embed.token_ids = call.ids; n.embed.segment_ids = call.segments; n.embed.lengths = call.lengths;
+      args[0] = &n.embed;
+    } else if (n.kind == ReplayNode::kHead) {
+      plan.steps[n.step].heads.logits = call.logits;
+      args[0] = &plan.steps[n.step].heads;
+    } else {
+      plan.steps[n.step].token_heads.logits = call.token_logits;
+      args[0] = &plan.steps[n.step].token_heads;
+    }
+    cudaKernelNodeParams launch = n.launch;
+    launch.kernelParams = args;
+    launch.extra = nullptr;
+    const cudaError_t e = cudaGraphExecKernelNodeSetParams(r.exec, n.node, &launch);
+    if (e != cudaSuccess) return e;
+  }
+  r.call = call;
+  return cudaSuccess;
+}
+
 int mt_forward(mt_model* m, const int32_t* d_token_ids, const int32_t* d_segment_ids, const int32_t* d_lengths,
                uint64_t task_mask, int32_t batch, int32_t seq, float* d_logits, void* stream_) {
   return mt_forward_events(m, d_token_ids, d_segment_ids, d_lengths, task_mask, batch, seq, d_logits, nullptr, stream_);
@@ -1613,161 +1912,30 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
   }
   Plan& plan = it->second;
   plan.last_use = ++m->use_clock;
-  uint32_t* status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
-  const size_t act_used = static_cast<size_t>(batch) * seq * m->trunk.hidden * sizeof(bf16);
-  cudaError_t e;
-#define MT_LAUNCH(call, what)                          \
-  do {                                                 \
-    e = (call);                                        \
-    if (e != cudaSuccess) return fail_cuda(m, e, what); \
-  } while (0)
-  // With option "profile" every kernel launch sits between two events of a pool that grows on the host.
-#define MT_TIMED(cls, call, what)                                                            \
-  do {                                                                                       \
-    if (m->profile) {                                                                        \
-      while (m->events.size() < m->events_used + 2) {                                        \
-        cudaEvent_t ev;                                                                      \
-        MT_LAUNCH(cudaEventCreate(&ev), "creating a timing event");                          \
-        m->events.push_back(ev);                                                             \
-      }                                                                                      \
-      MT_LAUNCH(cudaEventRecord(m->events[m->events_used], stream), "recording an event");   \
-    }                                                                                        \
-    MT_LAUNCH(call, what);                                                                   \
-    if (m->profile) {                                                                        \
-      MT_LAUNCH(cudaEventRecord(m->events[m->events_used + 1], stream), "recording an event"); \
-      m->events_used += 2;                                                                   \
-      m->event_class.push_back(cls);                                                         \
-    }                                                                                        \
-  } while (0)
-
-  // Steps 3-7 of the layers of a wave: three launches (each residual GEMM carries its LayerNorm) or five.
-#define MT_TAIL(tail)                                                                                                  \
-  do {                                                                                                                 \
-    LayerTail* t_ = (tail);                                                                                            \
-    if (t_->out_ln != 0) {                                                                                             \
-      MT_TIMED(MT_CLASS_ATTN_OUT, t_->out_ln == 2 ? launch_gemm_ln_pair(t_->attn_out_ln, m->sm_count, stream)          \
-                                                  : launch_gemm_ln(t_->attn_out_ln, m->sm_count, stream),              \
-               "attention output GEMM + LayerNorm");                                                                   \
-    } else {                                                                                                           \
-      MT_TIMED(MT_CLASS_ATTN_OUT, launch_gemm(t_->attn_out, kEpiBiasResidual, m->sm_count, stream), "attention output GEMM"); \
-      MT_TIMED(MT_CLASS_LN1, launch_layernorm(t_->ln1, stream), "LayerNorm 1");                                        \
-    }                                                                                                                  \
-    if (t_->fp8 && t_->out_ln != 0)                                                                                    \
-      MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_h1, stream), "quantising the FFN input");                    \
-    MT_TIMED(MT_CLASS_FFN_UP, launch_gemm(t_->ffn_up, kEpiBiasGelu, m->sm_count, stream), "FFN up GEMM");              \
-    if (t_->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_f, stream), "quantising the FFN intermediate");   \
-    if (t_->down_ln != 0) {                                                                                            \
-      MT_TIMED(MT_CLASS_FFN_DOWN, t_->down_ln == 2 ? launch_gemm_ln_pair(t_->ffn_down_ln, m->sm_count, stream)         \
-                                                   : launch_gemm_ln(t_->ffn_down_ln, m->sm_count, stream),             \
-               "FFN down GEMM + LayerNorm");                                                                           \
-    } else {                                                                                                           \
-      MT_TIMED(MT_CLASS_FFN_DOWN, launch_gemm(t_->ffn_down, t_->down_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual,   \
-                                              m->sm_count, stream), "FFN down GEMM");                                  \
-      MT_TIMED(MT_CLASS_LN2, launch_layernorm(t_->ln2, stream), "LayerNorm 2");                                        \
-    }                                                                                                                  \
-  } while (0)
-
-  int32_t* row_start = reinterpret_cast<int32_t*>(m->d_workspace + m->ws_row_start);
-  const bool fused_qkv = use_qkv_attention(m, static_cast<int64_t>(batch) * seq, seq);
-  MT_LAUNCH(launch_row_starts(d_lengths, batch, seq, m->pack_tokens ? 1 : 0, row_start,
-                              reinterpret_cast<int32_t*>(m->d_workspace + m->ws_rows_valid), fused_qkv ? window_count(m) : nullptr,
-                              fused_qkv ? window_list(m) : nullptr, stream),
-            "row-start kernel");
-  EmbedParams ep;
-  ep.row_start = row_start;
-  ep.row_info = fused_qkv ? row_info(m) : nullptr;
-  ep.packed = m->pack_tokens ? 1 : 0;
-  ep.token_ids = d_token_ids; ep.segment_ids = d_segment_ids; ep.lengths = d_lengths;
-  ep.word = w_ptr(m, m->emb_word); ep.pos = w_ptr(m, m->emb_pos); ep.type = w_ptr(m, m->emb_type);
-  ep.gamma = w_ptr(m, m->emb_ln_g); ep.beta = w_ptr(m, m->emb_ln_b);
-  ep.out = plan.embedding;
-  ep.out32 = f32_of(m, ep.out);
-  ep.batch = batch; ep.seq = seq; ep.hidden = m->trunk.hidden; ep.vocab = m->trunk.vocab_size;
-  ep.type_vocab = m->trunk.type_vocab; ep.eps = m->trunk.ln_eps; ep.status = status;
-  MT_TIMED(MT_CLASS_EMBED, launch_embed(ep, stream), "embedding kernel");
-  if (m->debug_capture)
-    MT_LAUNCH(cudaMemcpyAsync(m->d_workspace + m->ws_dump0, ep.out, act_used, cudaMemcpyDeviceToDevice, stream),
-              "debug capture");
-
-  bool pool_pending = false;   // ... of a step of kind 4: waited for before the first-token tails
-  bool side_pending = false;   // work on the side stream that the caller's stream has not waited for yet
-  for (PlanStep& st : plan.steps) {
-    if (side_pending || (pool_pending && st.kind == 2)) {
-      MT_LAUNCH(cudaStreamWaitEvent(stream, m->ev_join, 0), "joining the side stream");
-      side_pending = pool_pending = false;
+  const Call call = {d_token_ids, d_segment_ids, d_lengths, d_logits, d_token_logits};
+  // Replayed: plans in frequent use, on a stream that is not being captured, without anything recorded between the launches.
+  bool replay = m->replay && m->replay_stream != nullptr && task_events == nullptr && !m->profile && !m->debug_capture;
+  if (replay && (plan.replay == nullptr || !plan.replay->refused)) {
+    cudaStreamCaptureStatus state = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &state) != cudaSuccess) {
+      cudaGetLastError();
+      state = cudaStreamCaptureStatusInvalidated;
     }
-    if (st.kind == 0) {
-      Chunk& ck = st.chunk;
-      ck.attn.lengths = d_lengths;
-      ck.attn_cls.lengths = d_lengths;
-      if (m->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(ck.q_in, stream), "quantising the layer inputs");
-      const bool beside = m->overlap_cls && m->side_stream != nullptr && !m->profile && ck.n_cls > 0 && ck.full.count > 0;
-      if (ck.fused_qkv)
-        MT_TIMED(MT_CLASS_QKV, launch_qkv_attention(ck.qa, m->sm_count, stream), "QKV projection + attention kernel");
-      if (ck.qkv.n_groups > 0)
-        MT_TIMED(MT_CLASS_QKV, launch_gemm(ck.qkv, kEpiBias, m->sm_count, stream), "QKV GEMM");
-      if (beside) {
-        MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
-        MT_LAUNCH(cudaStreamWaitEvent(m->side_stream, m->ev_fork, 0), "forking the side stream");
-        MT_LAUNCH(launch_cls_attention(ck.attn_cls, m->side_stream), "first-token attention kernel");
-        MT_LAUNCH(cudaEventRecord(m->ev_join, m->side_stream), "joining the side stream");
-        side_pending = true;
-      }
-      if (ck.full.count > 0 && !ck.fused_qkv) MT_TIMED(MT_CLASS_ATTENTION, launch_attention(ck.attn, stream), "attention kernel");
-      if (ck.n_cls > 0 && !beside)
-        MT_TIMED(MT_CLASS_ATTENTION, launch_cls_attention(ck.attn_cls, stream), "first-token attention kernel");
-      if (ck.full.count > 0) MT_TAIL(&ck.full);
-      for (const DumpCopy& d : ck.dumps)
-        MT_LAUNCH(cudaMemcpyAsync(m->d_workspace + m->ws_dump0 + m->act_bytes * d.slot, d.src,
-                                  d.compact ? static_cast<size_t>(batch) * m->trunk.hidden * sizeof(bf16) : act_used,
-                                  cudaMemcpyDeviceToDevice, stream),
-                  "debug capture");
-    } else if (st.kind == 4) {
-      st.cls_pool.lengths = d_lengths;
-      const bool beside = st.beside && m->overlap_cls && m->side_stream != nullptr && !m->profile;
-      cudaStream_t on = beside ? m->side_stream : stream;
-      if (beside) {
-        MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
-        MT_LAUNCH(cudaStreamWaitEvent(on, m->ev_fork, 0), "forking the side stream");
-      }
-      MT_TIMED(MT_CLASS_ATTENTION, launch_cls_query(st.cls_pool, on), "first-token query kernel");
-      MT_TIMED(MT_CLASS_ATTENTION, launch_cls_pool(st.cls_pool, on), "first-token pooling kernel");
-      MT_TIMED(MT_CLASS_ATTENTION, launch_gemm(st.cls_v, kEpiBias, m->sm_count, on), "first-token value projection");
-      if (beside) {
-        MT_LAUNCH(cudaEventRecord(m->ev_join, on), "joining the side stream");
-        pool_pending = true;
-      }
-    } else if (st.kind == 2) {
-      MT_TAIL(&st.tail);
-      for (const DumpCopy& d : st.dumps)
-        MT_LAUNCH(cudaMemcpyAsync(m->d_workspace + m->ws_dump0 + m->act_bytes * d.slot, d.src,
-                                  static_cast<size_t>(batch) * m->trunk.hidden * sizeof(bf16), cudaMemcpyDeviceToDevice,
-                                  stream),
-                  "debug capture");
-    } else {
-      if (st.kind == 3) {
-        st.token_heads.logits = d_token_logits;
-        st.token_heads.lengths = d_lengths;
-        MT_TIMED(MT_CLASS_HEAD, launch_token_heads(st.token_heads, stream), "token-level head kernel");
-      } else if (st.pool_gemm) {
-        st.heads.logits = d_logits;
-        MT_TIMED(MT_CLASS_HEAD, launch_gemm(st.pool, kEpiBiasTanhF32, m->sm_count, stream), "pooler GEMM");
-        MT_TIMED(MT_CLASS_HEAD, launch_head(st.heads, stream), "head kernel");
-      } else {
-        st.heads.logits = d_logits;
-        MT_TIMED(MT_CLASS_HEAD, launch_pooler(st.heads, stream), "pooler kernel");
-        MT_TIMED(MT_CLASS_HEAD, launch_head(st.heads, stream), "head kernel");
-      }
-      if (task_events != nullptr)
-        for (int32_t t : st.head_tasks)
-          if (task_events[t] != nullptr)
-            MT_LAUNCH(cudaEventRecord(reinterpret_cast<cudaEvent_t>(task_events[t]), stream), "recording a task event");
-    }
+    replay = state == cudaStreamCaptureStatusNone;
+    if (replay && plan.replay == nullptr && ++plan.launched > kReplayAfter) build_replay(m, plan, call, batch, seq);
+    replay = replay && plan.replay != nullptr && !plan.replay->refused && plan.replay->pdl == g_use_pdl;
+  } else {
+    replay = false;
   }
-  if (side_pending || pool_pending) MT_LAUNCH(cudaStreamWaitEvent(stream, m->ev_join, 0), "joining the side stream");
-#undef MT_TAIL
-#undef MT_TIMED
-#undef MT_LAUNCH
+  if (replay && (set_call(plan, call) != cudaSuccess || cudaGraphLaunch(plan.replay->exec, stream) != cudaSuccess)) {
+    cudaGetLastError();
+    plan.replay->refused = true;
+    replay = false;
+  }
+  if (!replay) {
+    const int rc = launch_plan(m, plan, call, batch, seq, task_events, stream, nullptr);
+    if (rc != MT_OK) return rc;
+  }
   m->last_batch = batch;
   m->last_seq = seq;
   m->last_lengths = d_lengths;

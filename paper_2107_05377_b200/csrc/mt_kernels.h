@@ -330,8 +330,16 @@ cudaError_t launch_wait_probe(unsigned long long limit_ns, int arrive, uint32_t*
 // of the lengths clamped to [1, seq] (packed).  With windows != null (packed, seq <= kWindowRows) also the windows of
 // qkv_attention_tcgen05: *n_windows <= batch runs of consecutive sequences, each filled until the next sequence would
 // not fit in kWindowRows rows.
-cudaError_t launch_row_starts(const int32_t* lengths, int32_t batch, int32_t seq, int32_t packed, int32_t* row_start,
-                              int32_t* rows_valid, int32_t* n_windows, int2* windows, cudaStream_t stream);
+struct RowStartsParams {
+  const int32_t* lengths;
+  int32_t* lengths_copy;   // the lengths as they are, for the kernels that come later (may be `lengths` itself)
+  int32_t batch, seq, packed;
+  int32_t* row_start;
+  int32_t* rows_valid;
+  int32_t* n_windows;
+  int2* windows;
+};
+cudaError_t launch_row_starts(const RowStartsParams& p, cudaStream_t stream);
 // padded[b*seq + pos] = packed[row_start[b] + pos] for pos < length, 0 elsewhere (bf16 rows of `hidden`).
 // With compact != 0 the source is [B, H] (first tokens only) and only position 0 of a sequence is filled.
 cudaError_t launch_unpack_rows(const bf16* packed, const int32_t* lengths, const int32_t* row_start, bf16* padded,

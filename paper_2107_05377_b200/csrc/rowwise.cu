@@ -390,9 +390,10 @@ __global__ void __launch_bounds__(kRowThreads, V >= 16 ? 3 : 4) quantize_rows_ke
 
 // One warp: inclusive scan of the clamped lengths in chunks of 32, and the windows (next fit: a window is closed by the
 // first sequence that would not fit in kWindowRows rows; a ballot finds it, one step per window).
-__global__ void row_starts_kernel(const int32_t* lengths, int32_t batch, int32_t seq, int32_t packed,
-                                  int32_t* row_start, int32_t* rows_valid, int32_t* n_windows, int2* windows) {
+__global__ void row_starts_kernel(const RowStartsParams p) {
   const int lane = threadIdx.x;
+  const int batch = p.batch, seq = p.seq;
+  int2* windows = p.windows;
   grid_dependency_wait();
   grid_launch_dependents();
   int carry = 0;
@@ -401,11 +402,9 @@ __global__ void row_starts_kernel(const int32_t* lengths, int32_t batch, int32_t
     const int b = base + lane;
     int n = 0;
     if (b < batch) {
-      n = seq;
-      if (packed) {
-        n = lengths[b];
-        n = n < 1 ? 1 : (n > seq ? seq : n);
-      }
+      const int len = p.lengths[b];
+      p.lengths_copy[b] = len;
+      n = p.packed == 0 ? seq : (len < 1 ? 1 : (len > seq ? seq : len));
     }
     int incl = n;
 #pragma unroll
@@ -413,7 +412,7 @@ __global__ void row_starts_kernel(const int32_t* lengths, int32_t batch, int32_t
       const int up = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += up;
     }
-    if (b < batch) row_start[b] = carry + incl - n;
+    if (b < batch) p.row_start[b] = carry + incl - n;
     if (windows != nullptr) {
       // (lanes past the batch end where the last sequence does: they close nothing that it does not)
       for (;;) {
@@ -428,11 +427,11 @@ __global__ void row_starts_kernel(const int32_t* lengths, int32_t batch, int32_t
     carry += __shfl_sync(0xffffffffu, incl, 31);
   }
   if (lane == 0) {
-    row_start[batch] = carry;
-    *rows_valid = carry;
+    p.row_start[batch] = carry;
+    *p.rows_valid = carry;
     if (windows != nullptr) {
       windows[win_count] = make_int2(win_first, carry - win_first);   // (the last sequence is always in the open one)
-      *n_windows = win_count + 1;
+      *p.n_windows = win_count + 1;
     }
   }
 }
@@ -469,11 +468,11 @@ cudaError_t launch_quantize_rows(const QuantParams& p, cudaStream_t stream) {
   }
 }
 
-cudaError_t launch_row_starts(const int32_t* lengths, int32_t batch, int32_t seq, int32_t packed, int32_t* row_start,
-                              int32_t* rows_valid, int32_t* n_windows, int2* windows, cudaStream_t stream) {
-  if (batch < 1 || seq < 1 || (windows != nullptr && (n_windows == nullptr || packed == 0 || seq > kWindowRows)))
+cudaError_t launch_row_starts(const RowStartsParams& p, cudaStream_t stream) {
+  if (p.batch < 1 || p.seq < 1 || p.lengths == nullptr || p.lengths_copy == nullptr ||
+      (p.windows != nullptr && (p.n_windows == nullptr || p.packed == 0 || p.seq > kWindowRows)))
     return cudaErrorInvalidValue;
-  row_starts_kernel<<<1, 32, 0, stream>>>(lengths, batch, seq, packed, row_start, rows_valid, n_windows, windows);
+  row_starts_kernel<<<1, 32, 0, stream>>>(p);
   return cudaGetLastError();
 }
 

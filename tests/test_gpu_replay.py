@@ -1,0 +1,102 @@
+"""Forwards of a plan in frequent use run as a CUDA graph (option "replay"): the same bits as launched kernels, with the pointers of
+each call, whatever comes between the calls."""
+import pytest
+import torch
+
+from paper_2107_05377_b200 import binding as mt
+from paper_2107_05377_b200 import synth
+from gpu_util import cached_weights, dev_batch
+
+pytestmark = pytest.mark.gpu
+
+# sequence- and token-level tasks, a task that pools the trunk, first-token attention of both kinds by batch size
+TREE = synth.TreeConfig(trunk_layers=3, vocab_size=2000,
+                        tasks=(synth.TaskSpec(2, 2, 2), synth.TaskSpec(3, 0, 3), synth.TaskSpec(1, 1, 4, token_level=True),
+                               synth.TaskSpec(1, 2, 1)))
+
+
+def models(B, S):
+    _, blob, _ = cached_weights(TREE, 1)
+    out = []
+    for replay in (1, 0):
+        m = mt.MTModel(TREE, B, S)
+        m.load_weights(blob)
+        m.set_option("replay", replay)
+        out.append(m)
+    return out
+
+
+def call(model, ids, mask=None, stream=None):
+    B, S = ids[0].shape
+    out = torch.zeros(B, TREE.total_classes, device="cuda"), torch.zeros(B, S, TREE.total_token_classes, device="cuda")
+    torch.cuda.synchronize()     # (the zeros are there before another stream writes)
+    model.forward_tokens(*ids, *out, task_mask=mask, stream=stream)
+    return out
+
+
+def same(a, b):
+    torch.cuda.synchronize()
+    return all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+# few rows; more than 512 (pooled first-token attention on the second stream); windows
+@pytest.mark.parametrize("B,S", [(2, 40), (6, 128), (9, 60)])
+def test_replayed_and_launched_forwards_have_the_same_bits(B, S):
+    often, plain = models(B, S)
+    inputs = [dev_batch(synth.make_batch(TREE, B, S, 1, S, seed=k)) for k in range(3)]
+    want = [call(plain, ids) for ids in inputs]
+    other = torch.cuda.Stream()
+    for k in range(48):          # (the graph is built at the 17th call; new output arrays in every call)
+        assert same(call(often, inputs[k % 3], stream=other if k % 5 == 4 else None), want[k % 3]), k
+    # calls in a row, unsynchronised, on buffers that change under the same graph
+    outs = [call(often, inputs[k % 3]) for k in range(7)]
+    assert all(same(outs[k], want[k % 3]) for k in range(7))
+    assert often.poll_status() == 0
+
+
+def test_captures_options_and_other_plans_between_replays():
+    B, S = 3, 40
+    often, plain = models(B, S)
+    ids = dev_batch(synth.make_batch(TREE, B, S, 1, S, seed=5))
+    want = call(plain, ids)
+    for _ in range(20):
+        got = call(often, ids)
+    assert same(got, want)
+    # the caller's own capture records the kernels themselves
+    graph, outs = torch.cuda.CUDAGraph(), (torch.zeros_like(want[0]), torch.zeros_like(want[1]))
+    with torch.cuda.graph(graph):
+        often.forward_tokens(*ids, *outs)
+    graph.replay()
+    assert same(outs, want) and same(call(often, ids), want)
+    # a bad length in a replayed forward is flagged as in a launched one
+    bad = ids[2].clone()
+    bad[1] = S + 3
+    call(often, (ids[0], ids[1], bad))
+    assert often.poll_status() & 4
+    # plans dropped while replays may be under way: by the cache's limit, by an option
+    often.set_option("plan_cache", 1)
+    for mask in (1, 2, 1, 15):
+        expect = call(plain, ids, mask)
+        for _ in range(18):
+            got = call(often, ids, mask)
+        assert same(got, expect)
+    often.set_option("overlap_cls", 0)
+    assert same(call(often, ids), want)
+    often.close()
+
+
+def test_host_calls_are_replayed_too():
+    cfg = synth.config_tiny()
+    _, blob, _ = cached_weights(cfg, 0)
+    B, S = 2, 32
+    model = mt.MTModel(cfg, B, S)
+    model.load_weights(blob)
+    batches = [synth.make_batch(cfg, B, S, 1, S, seed=k) for k in range(2)]
+    want = []
+    for k in range(40):
+        b = batches[k % 2]
+        out = torch.zeros(B, cfg.total_classes).pin_memory()
+        model.forward_host(*[torch.from_numpy(a).pin_memory() for a in (b.token_ids, b.segment_ids, b.lengths)], out)
+        if k < 2:
+            want.append(out)
+        assert torch.equal(out, want[k % 2]), k
