@@ -257,7 +257,9 @@ int mt_plan_cache_size(const mt_model* m);
  * key "fused_ln" (0 never; 1 always, on 128-column tiles; 3 always, on 256 x 256 tiles of CTA pairs; 2 = chosen per
  * launch, the default: launches of at most "fused_ln_max_groups" (default 8) layers on all tokens whose row blocks fill
  * the clusters that are resident at once - where the valid rows are not known (option "expected_tokens") also when
- * fewer of them are in use -, and launches of at most "fused_ln_max_rows" (default 0) rows per layer; any
+ * fewer of them are in use -, launches of at most "fused_ln_max_rows" (default 0) rows per layer, and with bf16 operands the
+ * attention-output projections of launches of at most 512 rows per layer, on tiles of 16 to 64 rows, as long as the clusters of all
+ * of them run at once; any
  * time): the attention-output and FFN-down projections carry the LayerNorm that follows them: the CTAs holding the
  * column blocks of the same 128 or 256 rows form a thread-block cluster and exchange per-row statistics through
  * distributed shared memory, so the pre-normalisation sum never goes to global memory and no LayerNorm launch
@@ -385,6 +387,10 @@ int mt_kernel_linear_layernorm(const void* d_x, const void* d_w, const void* d_b
 int mt_kernel_linear_layernorm_tiles(const void* d_x, const void* d_w, const void* d_bias, const void* d_residual,
                                      const void* d_gamma, const void* d_beta, void* d_y, void* d_y_f32, int32_t M,
                                      int32_t N, int32_t K, float eps, int32_t tile_cols, uint32_t* d_status, void* stream);
+/* The same on tiles of tile_rows = 16, 32 or 64 rows and 128 columns (launches of few rows).  K % 128 == 0.  Identical bits. */
+int mt_kernel_linear_layernorm_low(const void* d_x, const void* d_w, const void* d_bias, const void* d_residual,
+                                   const void* d_gamma, const void* d_beta, void* d_y, void* d_y_f32, int32_t M,
+                                   int32_t N, int32_t K, float eps, int32_t tile_rows, uint32_t* d_status, void* stream);
 
 /* ctx[B*S, heads*64] = softmax(QK^T/8 masked to keys < length) V per (sequence, head), from the
  * packed projection qkv[B*S, 3*heads*64] = [Q | K | V].  Rows at positions >= length are written as 0.

@@ -64,6 +64,7 @@ SIGNATURES = {
     "mt_kernel_linear_fp8": (C.c_int, [_P, _P, _P, _P, _P, _P, _P, _I32, _I32, _I32, _I32, _P, _P]),
     "mt_kernel_linear_layernorm": (C.c_int, [_P, _P, _P, _P, _P, _P, _P, _P, _I32, _I32, _I32, C.c_float, _P, _P]),
     "mt_kernel_linear_layernorm_tiles": (C.c_int, [_P, _P, _P, _P, _P, _P, _P, _P, _I32, _I32, _I32, C.c_float, _I32, _P, _P]),
+    "mt_kernel_linear_layernorm_low": (C.c_int, [_P, _P, _P, _P, _P, _P, _P, _P, _I32, _I32, _I32, C.c_float, _I32, _P, _P]),
     "mt_kernel_attention": (C.c_int, [_P, _P, _P, _I32, _I32, _I32, _I32, _P, _P]),
     "mt_kernel_layernorm": (C.c_int, [_P, _P, _P, _P, _P, _I32, _I32, C.c_float, _P]),
     "mt_kernel_linear_partial": (C.c_int, [_P, _P, _P, _I32, _I32, _I32, _I32, _I32, _P, _P]),
@@ -150,6 +151,15 @@ def mt_kernel_linear_layernorm(x, w, bias, residual, gamma, beta, y, y_f32, eps:
     _check(lib().mt_kernel_linear_layernorm_tiles(_ptr(x), _ptr(w), _ptr(bias), _ptr(residual), _ptr(gamma), _ptr(beta),
                                                   _ptr(y), _ptr(y_f32), M, N, K, eps, tile_cols, _ptr(status),
                                                   _stream(stream)), "mt_kernel_linear_layernorm_tiles")
+
+
+def mt_kernel_linear_layernorm_low(x, w, bias, residual, gamma, beta, y, y_f32, eps: float, tile_rows: int, status=None,
+                                   stream=None) -> None:
+    M, K = x.shape
+    N = w.shape[0]
+    _check(lib().mt_kernel_linear_layernorm_low(_ptr(x), _ptr(w), _ptr(bias), _ptr(residual), _ptr(gamma), _ptr(beta),
+                                                _ptr(y), _ptr(y_f32), M, N, K, eps, tile_rows, _ptr(status),
+                                                _stream(stream)), "mt_kernel_linear_layernorm_low")
 
 
 def mt_kernel_attention(qkv, lengths, ctx, batch: int, seq: int, heads: int, stream=None,

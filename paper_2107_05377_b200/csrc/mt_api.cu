@@ -91,8 +91,9 @@ struct LayerTail {
   GemmParams attn_out, ffn_up, ffn_down;
   LayerNormParams ln1, ln2;
   int32_t count = 0;
-  // each residual GEMM together with the LayerNorm after it, as one cluster launch (fused_ln_kind: 0 no, 1 on 128-column
-  // tiles, 2 on 256 x 256 tiles of CTA pairs); the FFN-down projection not with 8-bit operands (that GEMM is the plain kernel)
+  // each residual GEMM together with the LayerNorm after it, as one cluster launch (ln_kinds: 0 no, 1 on 128-column tiles, 2 on
+  // 256 x 256 tiles of CTA pairs, 3 on low tiles); the FFN-down projection not with 8-bit operands (that GEMM is the plain
+  // kernel), nor split
   int32_t out_ln = 0, down_ln = 0;
   // launches of few rows: the FFN-down projection as partial sums over `down_splits` ranges of K, put together
   // (ranges in order, bias, residual) by the LayerNorm kernel after it
@@ -223,13 +224,13 @@ cudaError_t make_tmap(CUtensorMap* map, const void* base, int64_t rows, int64_t 
 
 // Tensor map of a row-major bf16 matrix [rows, cols] as {64, rows, cols / 64}: a box is some rows of several k-blocks, one
 // behind the other in shared memory, each with the 128-byte swizzle.
-cudaError_t make_tmap_kblocks(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows) {
+cudaError_t make_tmap_kblocks(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows, int box_kblocks) {
   EncodeTiledFn enc = nullptr;
   cudaError_t err = get_encoder(&enc);
   if (err != cudaSuccess) return err;
   const cuuint64_t dims[3] = {kGemmBlockK, static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(cols / kGemmBlockK)};
   const cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * sizeof(bf16), kGemmBlockK * sizeof(bf16)};
-  const cuuint32_t box[3] = {kGemmBlockK, static_cast<cuuint32_t>(box_rows), kGemmLowKBlocks};
+  const cuuint32_t box[3] = {kGemmBlockK, static_cast<cuuint32_t>(box_rows), static_cast<cuuint32_t>(box_kblocks)};
   const cuuint32_t elem[3] = {1, 1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, elem,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -266,8 +267,8 @@ cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, co
     if ((e = make_tmap_u8(&g->tmap_x[i], x, M, K, kGemmBlockM)) != cudaSuccess) return e;
     if ((e = make_tmap_u8(&g->tmap_w[i], w, N, K, g->block_n)) != cudaSuccess) return e;
   } else if (g->low != 0) {
-    if ((e = make_tmap_kblocks(&g->tmap_x[i], x, M, x_cols, g->low)) != cudaSuccess) return e;
-    if ((e = make_tmap_kblocks(&g->tmap_w[i], w, N, w_cols, 64)) != cudaSuccess) return e;
+    if ((e = make_tmap_kblocks(&g->tmap_x[i], x, M, x_cols, g->low, kGemmLowKBlocks)) != cudaSuccess) return e;
+    if ((e = make_tmap_kblocks(&g->tmap_w[i], w, N, w_cols, 64, kGemmLowKBlocks)) != cudaSuccess) return e;
   } else {
     if ((e = make_tmap(&g->tmap_x[i], x, M, x_cols, kGemmBlockM, kGemmBlockK, false)) != cudaSuccess) return e;
     if ((e = make_tmap(&g->tmap_w[i], w, N, w_cols, g->block_n / (g->pair != 0 ? 2 : 1), kGemmBlockK, false)) != cudaSuccess) return e;
@@ -277,6 +278,24 @@ cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, co
   g->group[i].bias = bias;
   g->group[i].out = y;
   return cudaSuccess;
+}
+
+// Tensor maps of group i of a residual GEMM with its LayerNorm, whose pointers are set.
+cudaError_t set_ln_maps(GemmLnParams* g, int i, const void* x, const void* w) {
+  cudaError_t err;
+  if (g->low != 0) {
+    if ((err = make_tmap_kblocks(&g->tmap_x[i], x, g->M, g->K, g->low, 2)) != cudaSuccess) return err;
+    return make_tmap_kblocks(&g->tmap_w[i], w, g->N, g->K, 128, 2);
+  }
+  if ((err = make_tmap(&g->tmap_x[i], x, g->M, g->K, kGemmBlockM, kGemmBlockK, false)) != cudaSuccess) return err;
+  if ((err = make_tmap(&g->tmap_w[i], w, g->N, g->K, 128, kGemmBlockK, false)) != cudaSuccess) return err;
+  if ((err = make_tmap(&g->tmap_res[i], g->residual[i], g->M, g->N, 32, 32, true)) != cudaSuccess) return err;
+  if ((err = make_tmap(&g->tmap_y[i], g->y[i], g->M, g->N, 32, 64, false)) != cudaSuccess) return err;
+  return make_tmap(&g->tmap_y32[i], g->y32[i], g->M, g->N, 32, 32, true);
+}
+// kind: 1 on 128-column tiles, 2 on tiles of CTA pairs, 3 on low tiles
+cudaError_t launch_ln_kind(int kind, const GemmLnParams& p, int sm_count, cudaStream_t stream) {
+  return kind == 3 ? launch_gemm_ln_low(p, stream) : (kind == 2 ? launch_gemm_ln_pair(p, sm_count, stream) : launch_gemm_ln(p, sm_count, stream));
 }
 
 }  // namespace
@@ -695,10 +714,35 @@ int32_t down_split_count(const mt_model* m, int64_t rows) {
   if (m->ffn_down_split == 0 || m->fp8 || rows > kSplitRowsMax) return 1;
   return (m->trunk.ffn / kGemmBlockK) % kDownSplits == 0 ? kDownSplits : 1;
 }
+// Rows of the low tiles on which the attention-output projections of `groups` layers of few rows carry their LayerNorm
+// (gemm_ln_low_tcgen05): the lowest whose clusters all run at once; 0: none.  us per forward of the eight-task tree, 64 / 32 / 16
+// rows wherever they fit in any number of rounds: 1 x 128 tokens 368 / 350 / 357, with this rule 344; 4 x 128 465 / 476 / 521,
+// 454; 2 x 32 on the six-layer tree 151 / 142 / 137, 137; two launches 364, 474, 148.  The FFN-down projection keeps its four
+// ranges of K as tiles of their own: on these tiles, four accumulators each, a CTA streams all of K = 3072 by itself (1 x 128 370,
+// 4 x 128 465, 2 x 32 156).
+int low_ln_rows(const mt_model* m, int32_t groups, int64_t rows) {
+  if (groups < 1 || m->fused_ln != 2 || m->fp8 || rows > kSplitRowsMax || m->d_workspace == nullptr || !gemm_ln_supported(m->trunk.hidden)) return 0;
+  const int64_t fit = gemm_ln_resident(m->trunk.hidden, m->sm_count);
+  for (int low : {16, 32, 64})
+    if ((rows + low - 1) / low * groups <= fit) return low;
+  return 0;
+}
+// How the residual GEMMs of `groups` layers carry their LayerNorm (launch_ln_kind; 0: they do not).
+struct LnKinds {
+  int out = 0, down = 0;
+  int low = 0;   // rows of the low tiles
+};
+LnKinds ln_kinds(const mt_model* m, int32_t groups, int64_t rows) {
+  LnKinds k;
+  k.low = low_ln_rows(m, groups, rows);
+  k.out = k.low != 0 ? 3 : fused_ln_kind(m, groups, rows);
+  if (!m->fp8 && down_split_count(m, rows) == 1) k.down = fused_ln_kind(m, groups, rows);
+  return k;
+}
 // Launches of steps 3-7 for `groups` layers.
 int32_t tail_launches(const mt_model* m, int32_t groups, int64_t rows) {
-  const bool fused = fused_ln_kind(m, groups, rows) != 0;
-  const bool down_fused = fused && !m->fp8 && down_split_count(m, rows) == 1;
+  const LnKinds kinds = ln_kinds(m, groups, rows);
+  const bool fused = kinds.out != 0, down_fused = kinds.down != 0;
   // 8-bit operands: f is quantised by a launch of its own, h1 too unless its LayerNorm, where that is a launch, does it
   return (fused ? 1 : 2) + 1 + (down_fused ? 1 : 2) + (m->fp8 ? (fused ? 2 : 1) : 0);
 }
@@ -750,20 +794,22 @@ void init_tail(const mt_model* m, LayerTail* t, int32_t rows, bool all_rows_vali
   t->ln1.hidden = t->ln2.hidden = H;
   t->ln1.eps = t->ln2.eps = m->trunk.ln_eps;
   t->count = 0;
-  t->out_ln = fused_ln_kind(m, groups, rows);
-  t->down_ln = !m->fp8 && t->down_splits == 1 ? t->out_ln : 0;
+  const LnKinds kinds = ln_kinds(m, groups, rows);
+  t->out_ln = kinds.out;
+  t->down_ln = kinds.down;
   {
-    auto init_ln = [&](std::unique_ptr<GemmLnParams>* at, int32_t K) {
+    auto init_ln = [&](std::unique_ptr<GemmLnParams>* at, int32_t K, int kind) {
       *at = std::make_unique<GemmLnParams>();
       GemmLnParams* g = at->get();
       memset(g, 0, sizeof(*g));
       g->M = rows; g->N = H; g->K = K;
+      g->low = kind == 3 ? kinds.low : 0;
       g->m_valid = rows_valid;
       g->eps = m->trunk.ln_eps;
       g->status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
     };
-    if (t->out_ln != 0) init_ln(&t->attn_out_ln, H);
-    if (t->down_ln != 0) init_ln(&t->ffn_down_ln, F);
+    if (t->out_ln != 0) init_ln(&t->attn_out_ln, H, t->out_ln);
+    if (t->down_ln != 0) init_ln(&t->ffn_down_ln, F, t->down_ln);
   }
 }
 
@@ -826,15 +872,10 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
   if (t->out_ln != 0 || t->down_ln != 0) {
     auto set_ln = [&](GemmLnParams* g, const void* x, size_t w, size_t b, size_t gamma, size_t beta, const float* res,
                       bf16* y, float* y32) -> cudaError_t {
-      cudaError_t err;
-      if ((err = make_tmap(&g->tmap_x[i], x, g->M, g->K, kGemmBlockM, kGemmBlockK, false)) != cudaSuccess) return err;
-      if ((err = make_tmap(&g->tmap_w[i], w_ptr(m, w), g->N, g->K, 128, kGemmBlockK, false)) != cudaSuccess) return err;
-      if ((err = make_tmap(&g->tmap_res[i], res, g->M, g->N, 32, 32, true)) != cudaSuccess) return err;
-      if ((err = make_tmap(&g->tmap_y[i], y, g->M, g->N, 32, 64, false)) != cudaSuccess) return err;
-      if ((err = make_tmap(&g->tmap_y32[i], y32, g->M, g->N, 32, 32, true)) != cudaSuccess) return err;
       g->bias[i] = w_ptr(m, b); g->gamma[i] = w_ptr(m, gamma); g->beta[i] = w_ptr(m, beta);
+      g->residual[i] = res; g->y[i] = y; g->y32[i] = y32;
       g->n_groups = i + 1;
-      return cudaSuccess;
+      return set_ln_maps(g, i, x, w_ptr(m, w));
     };
     // (a state is its bf16 copy followed by room for its fp32 copy: the fp32 result always has a home)
     float* out32_home = out32 != nullptr ? out32 : f32_of(m, out);
@@ -1658,8 +1699,7 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
   do {                                                                                                                 \
     LayerTail* t_ = (tail);                                                                                            \
     if (t_->out_ln != 0) {                                                                                             \
-      MT_TIMED(MT_CLASS_ATTN_OUT, t_->out_ln == 2 ? launch_gemm_ln_pair(*t_->attn_out_ln, m->sm_count, stream)          \
-                                                  : launch_gemm_ln(*t_->attn_out_ln, m->sm_count, stream),              \
+      MT_TIMED(MT_CLASS_ATTN_OUT, launch_ln_kind(t_->out_ln, *t_->attn_out_ln, m->sm_count, stream),                   \
                "attention output GEMM + LayerNorm");                                                                   \
     } else {                                                                                                           \
       MT_TIMED(MT_CLASS_ATTN_OUT, launch_gemm(t_->attn_out, kEpiBiasResidual, m->sm_count, stream), "attention output GEMM"); \
@@ -1670,8 +1710,7 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
     MT_TIMED(MT_CLASS_FFN_UP, launch_gemm(t_->ffn_up, kEpiBiasGelu, m->sm_count, stream), "FFN up GEMM");              \
     if (t_->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(t_->q_f, stream), "quantising the FFN intermediate");   \
     if (t_->down_ln != 0) {                                                                                            \
-      MT_TIMED(MT_CLASS_FFN_DOWN, t_->down_ln == 2 ? launch_gemm_ln_pair(*t_->ffn_down_ln, m->sm_count, stream)         \
-                                                   : launch_gemm_ln(*t_->ffn_down_ln, m->sm_count, stream),             \
+      MT_TIMED(MT_CLASS_FFN_DOWN, launch_ln_kind(t_->down_ln, *t_->ffn_down_ln, m->sm_count, stream),                  \
                "FFN down GEMM + LayerNorm");                                                                           \
     } else {                                                                                                           \
       MT_TIMED(MT_CLASS_FFN_DOWN, launch_gemm(t_->ffn_down, t_->down_splits > 1 ? kEpiPartialF32 : kEpiBiasResidual,   \
@@ -2118,10 +2157,9 @@ int mt_kernel_linear_layernorm(const void* d_x, const void* d_w, const void* d_b
                                           d_status, stream);
 }
 
-int mt_kernel_linear_layernorm_tiles(const void* d_x, const void* d_w, const void* d_bias, const void* d_residual,
-                                     const void* d_gamma, const void* d_beta, void* d_y, void* d_y_f32, int32_t M,
-                                     int32_t N, int32_t K, float eps, int32_t tile_cols, uint32_t* d_status, void* stream) {
-  if (tile_cols != 128 && tile_cols != 256) return MT_ERR_INVALID_ARG;
+static int linear_layernorm_kind(int kind, const void* d_x, const void* d_w, const void* d_bias, const void* d_residual, const void* d_gamma,
+                                 const void* d_beta, void* d_y, void* d_y_f32, int32_t M, int32_t N, int32_t K, float eps, int32_t low,
+                                 uint32_t* d_status, void* stream) {
   if (d_x == nullptr || d_w == nullptr || d_bias == nullptr || d_residual == nullptr || d_gamma == nullptr ||
       d_beta == nullptr || d_y == nullptr || d_y_f32 == nullptr || M < 1 || !gemm_ln_supported(N) || K < 64 || K % 64 != 0 ||
       !(eps >= 0.f))
@@ -2129,18 +2167,31 @@ int mt_kernel_linear_layernorm_tiles(const void* d_x, const void* d_w, const voi
   GemmLnParams p;
   memset(&p, 0, sizeof(p));
   p.n_groups = 1; p.M = M; p.N = N; p.K = K; p.eps = eps; p.status = d_status;
-  if (make_tmap(&p.tmap_x[0], d_x, M, K, kGemmBlockM, kGemmBlockK, false) != cudaSuccess ||
-      make_tmap(&p.tmap_w[0], d_w, N, K, 128, kGemmBlockK, false) != cudaSuccess ||
-      make_tmap(&p.tmap_res[0], d_residual, M, N, 32, 32, true) != cudaSuccess ||
-      make_tmap(&p.tmap_y[0], d_y, M, N, 32, 64, false) != cudaSuccess ||
-      make_tmap(&p.tmap_y32[0], d_y_f32, M, N, 32, 32, true) != cudaSuccess)
-    return MT_ERR_CUDA;
+  p.low = low;
   p.bias[0] = static_cast<const bf16*>(d_bias);
   p.gamma[0] = static_cast<const bf16*>(d_gamma);
   p.beta[0] = static_cast<const bf16*>(d_beta);
+  p.residual[0] = static_cast<const float*>(d_residual);
+  p.y[0] = static_cast<bf16*>(d_y);
+  p.y32[0] = static_cast<float*>(d_y_f32);
+  if (set_ln_maps(&p, 0, d_x, d_w) != cudaSuccess) return MT_ERR_CUDA;
   const int every = INT32_MAX;   // as many SMs as there are
-  const cudaError_t e = tile_cols == 256 ? launch_gemm_ln_pair(p, every, as_stream(stream)) : launch_gemm_ln(p, every, as_stream(stream));
-  return e == cudaSuccess ? MT_OK : MT_ERR_CUDA;
+  return launch_ln_kind(kind, p, every, as_stream(stream)) == cudaSuccess ? MT_OK : MT_ERR_CUDA;
+}
+
+int mt_kernel_linear_layernorm_tiles(const void* d_x, const void* d_w, const void* d_bias, const void* d_residual,
+                                     const void* d_gamma, const void* d_beta, void* d_y, void* d_y_f32, int32_t M,
+                                     int32_t N, int32_t K, float eps, int32_t tile_cols, uint32_t* d_status, void* stream) {
+  if (tile_cols != 128 && tile_cols != 256) return MT_ERR_INVALID_ARG;
+  return linear_layernorm_kind(tile_cols == 256 ? 2 : 1, d_x, d_w, d_bias, d_residual, d_gamma, d_beta, d_y, d_y_f32, M, N, K, eps, 0,
+                               d_status, stream);
+}
+
+int mt_kernel_linear_layernorm_low(const void* d_x, const void* d_w, const void* d_bias, const void* d_residual,
+                                   const void* d_gamma, const void* d_beta, void* d_y, void* d_y_f32, int32_t M,
+                                   int32_t N, int32_t K, float eps, int32_t tile_rows, uint32_t* d_status, void* stream) {
+  if ((tile_rows != 16 && tile_rows != 32 && tile_rows != 64) || K % 128 != 0) return MT_ERR_INVALID_ARG;
+  return linear_layernorm_kind(3, d_x, d_w, d_bias, d_residual, d_gamma, d_beta, d_y, d_y_f32, M, N, K, eps, tile_rows, d_status, stream);
 }
 
 int mt_kernel_attention(const void* d_qkv, const int32_t* d_lengths, void* d_ctx, int32_t batch, int32_t seq,

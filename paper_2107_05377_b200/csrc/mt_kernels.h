@@ -250,8 +250,13 @@ struct alignas(64) GemmLnParams {
   const bf16* bias[kMaxGroups];
   const bf16* gamma[kMaxGroups];
   const bf16* beta[kMaxGroups];
+  const float* residual[kMaxGroups];  // (low tiles) the residual and the results by pointer
+  bf16* y[kMaxGroups];
+  float* y32[kMaxGroups];
   int32_t n_groups;
   int32_t M, N, K;
+  int32_t low;             // 16, 32 or 64: tiles of that many rows (launch_gemm_ln_low).  The X and W maps are then dims
+                           // {64, rows, K / 64}, boxes {64, low | 128, 2}
   const int32_t* m_valid;  // device scalar: rows actually in use (<= M); null = all M rows
   float eps;
   uint32_t* status;        // sticky device status word (may be null)
@@ -264,6 +269,10 @@ cudaError_t launch_gemm_ln(const GemmLnParams& p, int sm_count, cudaStream_t str
 // operand bytes per tile - for launches with many row blocks.
 int gemm_ln_pair_resident(int N, int sm_count);
 cudaError_t launch_gemm_ln_pair(const GemmLnParams& p, int sm_count, cudaStream_t stream);
+
+// The same on tiles of 16, 32 or 64 rows and 128 columns, one cluster of N / 128 CTAs each: identical bits - for launches of so
+// few rows that all clusters run at once.  K a multiple of 128.
+cudaError_t launch_gemm_ln_low(const GemmLnParams& p, cudaStream_t stream);
 
 struct EmbedParams {
   const int32_t* token_ids;
