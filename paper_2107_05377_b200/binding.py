@@ -163,9 +163,9 @@ def mt_kernel_linear_layernorm_low(x, w, bias, residual, gamma, beta, y, y_f32, 
 
 
 def mt_kernel_attention(qkv, lengths, ctx, batch: int, seq: int, heads: int, stream=None,
-                        tensor_memory: bool = False, status=None) -> None:
+                        tensor_memory: int = 0, status=None) -> None:
     _check(lib().mt_kernel_attention(_ptr(qkv), _ptr(lengths), _ptr(ctx), batch, seq, heads,
-                                     1 if tensor_memory else 0, _ptr(status), _stream(stream)), "mt_kernel_attention")
+                                     int(tensor_memory), _ptr(status), _stream(stream)), "mt_kernel_attention")
 
 
 def mt_kernel_layernorm(x, gamma, beta, y, eps: float, y_f32=None, stream=None) -> None:

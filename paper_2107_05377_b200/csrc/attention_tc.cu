@@ -496,7 +496,327 @@ __global__ void __launch_bounds__(kTcThreads, 2) attention_tc_tiled_kernel(const
   if (warp == 0) tmem_dealloc(tmem_base, kTlTmemCols);
 }
 
+// ---- two threads per query row, any length ---------------------------------------------------------
+// (With 8-bit projections the kernels above stay: a rounding that falls otherwise here is a code that falls otherwise there.)
+// One CTA = one (layer of the wave, sequence, head, tile of 128 queries); the keys are walked in tiles of 128:
+//   S = Q . K_j^T (tensor memory);  P = exp((S - m) / 8), bf16, written over S;  l += rowsum P;  O += P . V_j (tensor memory)
+// m is the maximum of the row when it was last set: it moves only when a tile's maximum exceeds it by more than 8 powers of
+// two (P then stays below 2^8, whose bf16 rounding is as fine as below 1), and O and l are scaled down by that factor; so O
+// is accumulated by the tensor cores and usually not touched before the end, O / l.
+// Eight warps; a thread owns one query row and half of the keys of a tile (64), held in registers between the maximum, which the
+// two warps of a quarter exchange, and the exponentials.  Warp 0 also requests the tiles (K and V double buffered) and issues the
+// MMAs, P . V_j and S_{j+1} right behind it, when the P of all warps is in tensor memory, where it is read from.  (A ninth warp
+// for that leaves room for one CTA per SM - the registers of a quarter of the SM hold four warps of 112 - and was slower than one
+// thread per row: 38 us where that takes 31.)
+// What bounds it: the chain of a step; its exponentials take 1024 clocks of the special-function unit per tile of 128 x 128 and SM,
+// a fifth of the time.  16 sequences of 128 to 512 tokens, 12 heads: 31.4 us with one thread per row (S read twice, O in
+// registers, four barriers of the whole CTA per tile), 27.2 us here.
+// Keys at positions >= length take no part: their probabilities are 0 and the rows of V that share their sixteen with
+// valid ones are zeroed.
+constexpr int kSpWarps = 8;
+constexpr int kSpThreads = 32 * kSpWarps;
+constexpr uint32_t kSpTmemCols = 256;                 // S (P over it) 128, O 64
+constexpr uint32_t kSpColO = 128;
+constexpr float kSpSlack = 8.0f;                      // powers of two that a row's maximum may lag behind
+constexpr int kSpExchangeBytes = 2 * 2 * kTcRows * 4;   // [maximum | sum][half][row]
+constexpr int sp_smem_bytes(int kv_buffers) { return (1 + 2 * kv_buffers) * kTcTileBytes + kSpExchangeBytes + 128 + 1024; }
+
+__global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const __grid_constant__ AttnParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int kv_buffers = p.seq > kTcRows ? 2 : 1;
+  const uint32_t sQ = smem_u32(smem);                 // at the end the output tile
+  const uint32_t sK = sQ + kTcTileBytes;
+  const uint32_t sV = sK + kv_buffers * kTcTileBytes;
+  uint8_t* v_ptr = smem + (1 + kv_buffers) * kTcTileBytes;
+  float* exchange = reinterpret_cast<float*>(smem + (1 + 2 * kv_buffers) * kTcTileBytes);
+  uint8_t* book = smem + (1 + 2 * kv_buffers) * kTcTileBytes + kSpExchangeBytes;
+  const uint32_t bar_k = smem_u32(book);              // two: K_j has landed (with the first one Q)
+  const uint32_t bar_v = bar_k + 16;                  // two
+  const uint32_t bar_s = bar_v + 16;                  // S of a step is complete
+  const uint32_t bar_p = bar_s + 8;                   // P of a step is in tensor memory
+  const uint32_t bar_pv = bar_p + 8;                  // P . V of a step is complete
+  const uint32_t bar_pair = bar_pv + 8;               // four: the two warps of a quarter exchange their maxima
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(book + 88);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(book + 92);
+
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5;
+  const int lane = tid & 31;
+  const int head = blockIdx.x;
+  const int q_tiles = (p.seq + kTcRows - 1) / kTcRows;
+  const int b = blockIdx.y / q_tiles;
+  const int q0 = (blockIdx.y - b * q_tiles) * kTcRows;   // first query of this CTA within the sequence
+  const int g = blockIdx.z;
+  const int H = p.heads * kHeadDim;
+
+  // inputs of the forward and the output of its first kernel: readable before the dependency wait (see above)
+  int len = p.lengths[b];
+  len = len < 1 ? 1 : (len > p.seq ? p.seq : len);
+  const int row0 = p.row_start != nullptr ? p.row_start[b] : b * p.seq;
+  bf16* ctx = p.ctx[g];
+  const int rows_in_seq = min(kTcRows, p.seq - q0);           // rows of this tile that exist in the padded layout
+  const int rows_out = p.packed ? min(kTcRows, len - q0) : rows_in_seq;
+  if (q0 >= len) {
+    // a tile of padded query positions only: nothing in the packed layout, zeros in the padded one
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const int chunk = tid & 7;
+    for (int r = tid >> 3; r < rows_out; r += kSpThreads / 8)
+      *reinterpret_cast<uint4*>(ctx + static_cast<size_t>(row0 + q0 + r) * H + head * kHeadDim + chunk * 8) = make_uint4(0, 0, 0, 0);
+    return;
+  }
+
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar_k + 8 * i, 1);
+      mbar_init(bar_v + 8 * i, 1);
+    }
+    mbar_init(bar_s, 1);
+    mbar_init(bar_p, kSpWarps);
+    mbar_init(bar_pv, 1);
+    for (int q = 0; q < 4; ++q) mbar_init(bar_pair + 8 * q, 2);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_shared();
+    prefetch_tensormap(&p.tmap_qkv[g]);
+    prefetch_tensormap(&p.tmap_qkv64[g]);
+  }
+  if (warp == 0) tmem_alloc(smem_u32(tmem_slot), kSpTmemCols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  grid_dependency_wait();
+  grid_launch_dependents();
+
+  const int n_kt = (len + kTcRows - 1) / kTcRows;    // key tiles
+  const int rows_q = min(kTcRows, len - q0);         // valid query rows of this tile
+  bool ok = true;
+  int k_issued = 0, v_issued = 0;                    // (warp 0) tiles requested so far
+
+  // ------------------------------ copies and MMAs (warp 0; the elected lane issues) ------------------------------
+  const bool leader = warp == 0 && elect_one();
+  // (at most 64 rows left: a box of 64; the tile's other rows are never read, or only where their results are not)
+  auto request = [&](uint32_t dst, int col, int row, int rows, uint32_t bar) {
+    tma_load_2d(dst, rows <= 64 ? &p.tmap_qkv64[g] : &p.tmap_qkv[g], col, row0 + row, bar);
+  };
+  auto box_bytes = [](int rows) { return static_cast<uint32_t>(rows <= 64 ? kTcTileBytes / 2 : kTcTileBytes); };
+  auto request_k = [&](int j) {
+    const int rows = len - j * kTcRows;
+    if (leader) {
+      const uint32_t bar = bar_k + 8 * (j & 1);
+      mbar_expect_tx(bar, box_bytes(rows) + (j == 0 ? box_bytes(rows_q) : 0u));
+      if (j == 0) request(sQ, head * kHeadDim, q0, rows_q, bar);
+      request(sK + (j & 1) * kTcTileBytes, H + head * kHeadDim, j * kTcRows, rows, bar);
+    }
+    ++k_issued;
+  };
+  auto request_v = [&](int j) {
+    const int rows = len - j * kTcRows;
+    if (leader) {
+      mbar_expect_tx(bar_v + 8 * (j & 1), box_bytes(rows));
+      request(sV + (j & 1) * kTcTileBytes, 2 * H + head * kHeadDim, j * kTcRows, rows, bar_v + 8 * (j & 1));
+    }
+    ++v_issued;
+  };
+  // S = Q . K_j^T for the tile's keys, rounded up to sixteens
+  auto issue_s = [&](int j) {
+    if (!mbar_wait(bar_k + 8 * (j & 1), static_cast<uint32_t>((j >> 1) & 1), abort_flag)) return false;
+    tc_fence_after();
+    if (leader) {
+      const uint64_t dq = smem_desc_sw128(sQ);
+      const uint64_t dk = smem_desc_sw128(sK + (j & 1) * kTcTileBytes);
+      const uint32_t idesc = umma_idesc_bf16(kTcRows, (min(kTcRows, len - j * kTcRows) + 15) & ~15);
+#pragma unroll
+      for (int k = 0; k < kHeadDim / 16; ++k) umma_bf16(tmem_base, dq + 2 * k, dk + 2 * k, idesc, k > 0 ? 1u : 0u);
+      umma_commit(bar_s);
+    }
+    return true;
+  };
+  if (warp == 0) {
+    request_k(0);
+    request_v(0);
+    if (n_kt > 1) {
+      request_k(1);
+      request_v(1);
+    }
+    ok = issue_s(0);
+  }
+
+  // ------------------------------ softmax -----------------------------------
+  const int quarter = warp & 3;                      // TMEM lanes this warp may read
+  const int half = warp >> 2;                        // which 64 keys of a tile, which 32 columns of O
+  const int row = quarter * 32 + lane;
+  const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+  const uint32_t pair_bar = bar_pair + 8 * quarter;
+  const bool row_valid = row < rows_q;
+  const bool warp_valid = quarter * 32 < rows_q;     // (the others only keep the barriers' counts; their P is never used)
+  const float k2 = 0.125f * 1.4426950408889634f;     // exp(x / 8) = 2^(x k2)
+  float m = 0.0f, l = 0.0f;                          // reference maximum (times k2), sum of this half's probabilities
+  for (int j = 0; j < n_kt && ok; ++j) {
+    const uint32_t parity = static_cast<uint32_t>(j & 1);
+    const int keys = min(kTcRows, len - j * kTcRows);       // valid keys of this tile
+    const int mine = min(64, keys - half * 64);             // of this half (none: <= 0)
+    if (keys < kTcRows) {
+      // rows of V past the last key, up to the sixteen that the products take: 0 * V must stay finite
+      if (!__all_sync(0xffffffffu, mbar_wait(bar_v + 8 * (j & 1), static_cast<uint32_t>((j >> 1) & 1), abort_flag))) { ok = false; break; }
+      const int last = (keys + 15) & ~15;
+      for (int i = tid; i < (last - keys) * 8; i += 32 * kSpWarps)
+        *reinterpret_cast<uint4*>(v_ptr + (j & 1) * kTcTileBytes + (keys + (i >> 3)) * 128 + (i & 7) * 16) = make_uint4(0, 0, 0, 0);
+      fence_async_shared();
+    }
+    // (every completion of a barrier is waited for in turn: P . V of the step before is, too, when S of this one is)
+    if (!__all_sync(0xffffffffu, mbar_wait(bar_s, parity, abort_flag) && (j == 0 || mbar_wait(bar_pv, parity ^ 1u, abort_flag)))) {
+      ok = false;
+      break;
+    }
+    tc_fence_after();
+    if (warp == 0 && j > 0 && j + 1 < n_kt) request_v(j + 1);   // (into the buffer of the step before)
+    uint32_t s[64];
+    float tile_max = -INFINITY;
+    if (warp_valid && mine > 0) {
+      tmem_ld_32x32(lane_base + half * 64, *reinterpret_cast<uint32_t(*)[32]>(s));
+      tmem_ld_32x32(lane_base + half * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(s + 32));
+      tmem_ld_wait();
+      if (mine < 64) {
+#pragma unroll
+        for (int i = 0; i < 64; ++i)
+          if (i >= mine) s[i] = 0xff800000u;   // -inf: exponential 0
+      }
+      float t[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // (four chains)
+#pragma unroll
+      for (int i = 0; i < 64; ++i) t[i & 3] = fmaxf(t[i & 3], __uint_as_float(s[i]));
+      tile_max = fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3]));
+    }
+    // the other half's maximum; with it this warp also knows that the other one has read its S, which P is written over
+    exchange[half * kTcRows + row] = tile_max;
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(pair_bar);
+    if (!__all_sync(0xffffffffu, mbar_wait(pair_bar, parity, abort_flag))) { ok = false; break; }
+    tc_fence_after();
+    if (warp_valid) {
+      tile_max = fmaxf(tile_max, exchange[(half ^ 1) * kTcRows + row]) * k2;
+      if (j == 0) {
+        m = tile_max;
+      } else if (__any_sync(0xffffffffu, row_valid && tile_max > m + kSpSlack)) {
+        // scale O (complete up to the step before) down to the new maximum; both halves see the same rows and do the same
+        const float to = tile_max > m + kSpSlack ? tile_max : m;
+        const float alpha = to > m ? ex2_approx(m - to) : 1.0f;
+        uint32_t o[32];
+        tmem_ld_32x32(lane_base + kSpColO + half * 32, o);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+        tmem_st_32x32(lane_base + kSpColO + half * 32, o);
+        l *= alpha;
+        m = to;
+      }
+      if (mine > 0) {
+        float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint32_t w[16];
+          if (c == 0 || mine > 32) {                 // (uniform)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float e0 = ex2_approx(fmaf(__uint_as_float(s[c * 32 + 2 * i]), k2, -m));
+              const float e1 = ex2_approx(fmaf(__uint_as_float(s[c * 32 + 2 * i + 1]), k2, -m));
+              sum[i & 1] += e0;
+              sum[2 + (i & 1)] += e1;
+              w[i] = pack_bf16(e0, e1);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) w[i] = 0u;
+          }
+          tmem_st_32x16(lane_base + half * 32 + c * 16, w);
+        }
+        l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
+      }
+      tmem_st_wait();
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_p);
+    __syncwarp();
+    if (warp == 0) {
+      ok = mbar_wait(bar_p, parity, abort_flag) && mbar_wait(bar_v + 8 * (j & 1), static_cast<uint32_t>((j >> 1) & 1), abort_flag);
+      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      tc_fence_after();
+      if (leader) {
+        constexpr uint32_t idesc = umma_idesc_bf16_b_mn(kTcRows, kHeadDim);
+        const int steps = (keys + 15) / 16;
+        for (int k = 0; k < steps; ++k)   // sixteen keys = sixteen 128-byte rows of the V tile, eight columns of P
+          umma_bf16_ts(tmem_base + kSpColO, tmem_base + k * 8, smem_desc_sw128(sV + (j & 1) * kTcTileBytes + k * 16 * 128), idesc,
+                       (j | k) != 0 ? 1u : 0u);
+        umma_commit(bar_pv);
+      }
+      if (j + 2 < n_kt) request_k(j + 2);                   // (S of this step is complete: K_j is dead)
+      if (j + 1 < n_kt) ok = __all_sync(0xffffffffu, issue_s(j + 1)) != 0;   // (behind P . V_j, which reads the P that it overwrites)
+    }
+  }
+  // O / l: this half's 32 columns, to bf16, into the Q tile's place (all products have completed)
+  float* sums = exchange + 2 * kTcRows;
+  if (ok) {
+    sums[half * kTcRows + row] = l;
+    ok = __all_sync(0xffffffffu, mbar_wait(bar_pv, static_cast<uint32_t>((n_kt - 1) & 1), abort_flag)) != 0;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(pair_bar);
+    ok = __all_sync(0xffffffffu, mbar_wait(pair_bar, static_cast<uint32_t>(n_kt & 1), abort_flag)) != 0 && ok;
+  }
+  if (ok) {
+    tc_fence_after();
+    uint32_t o[32];
+    tmem_ld_32x32(lane_base + kSpColO + half * 32, o);
+    tmem_ld_wait();
+    const float inv = row_valid ? 1.0f / (sums[row] + sums[kTcRows + row]) : 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t w[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        w[i] = row_valid ? pack_bf16(__uint_as_float(o[q * 8 + 2 * i]) * inv, __uint_as_float(o[q * 8 + 2 * i + 1]) * inv) : 0u;
+      *reinterpret_cast<uint4*>(smem + staging_off(row, half * 4 + q)) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+  if (!ok && leader) {
+    // shared memory must not be handed to another CTA while copies may still land in it: every tile that was requested gets
+    // the usual limit to arrive
+    for (int j = max(0, k_issued - 2); j < k_issued; ++j) mbar_drain(bar_k + 8 * (j & 1), static_cast<uint32_t>((j >> 1) & 1));
+    for (int j = max(0, v_issued - 2); j < v_issued; ++j) mbar_drain(bar_v + 8 * (j & 1), static_cast<uint32_t>((j >> 1) & 1));
+  }
+  __syncwarp();
+  // out row by row as full 128-byte segments
+  tc_fence_before();
+  ok = __syncthreads_and(ok) != 0;
+  if (ok) {
+    const int chunk = tid & 7;
+    for (int r = tid >> 3; r < rows_out; r += kSpThreads / 8) {
+      const uint4 val = *reinterpret_cast<const uint4*>(smem + staging_off(r, chunk));
+      *reinterpret_cast<uint4*>(ctx + static_cast<size_t>(row0 + q0 + r) * H + head * kHeadDim + chunk * 8) = val;
+    }
+  } else if (tid == 0 && p.status != nullptr) {
+    atomicOr(p.status, kFlagWaitTimeout);
+  }
+  if (warp == 0) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem_base, kSpTmemCols);
+  }
+}
+
 }  // namespace
+
+// Beyond 128 tokens always (us per forward of the eight-task tree, one thread per row / two: 16 x 512 ragged 1937 / 1887, 60 x 512
+// for one task 5286 / 5180, 64 x 150 1917 / 1855, 8 x 256 837 / 823, 1 x 300 511 / 498).  Up to 128 a CTA has one step, whose latencies
+// count where few sequences leave the SMs idle (4 x 128 450 / 441, 2 x 100 404 / 389, 1 x 128 338 / 337), while with many, four CTAs
+// of the kernel with one thread per row per SM hide them better (32 x 128 992 / 1018, 256 x 128 9425 / 9675), and with at most 64
+// keys half of the threads have nothing to do (2 x 64 333 / 338).  The line depends on the shape of the batch alone, so a task gets
+// the same bits whatever runs beside it.
+bool attention_split_rows(int batch, int seq) { return seq > kTcRows || (seq > kTcRows / 2 && batch <= 4); }
 
 cudaError_t launch_attention_tc(const AttnParams& p, cudaStream_t stream) {
   if (p.n_groups < 1 || p.n_groups > kMaxGroups || p.batch < 1 || p.seq < 1 || p.seq > kAttnTensorMemoryMaxSeq)
@@ -505,14 +825,19 @@ cudaError_t launch_attention_tc(const AttnParams& p, cudaStream_t stream) {
   cudaError_t e = per_device_once(once, [&](int) {
     cudaError_t r = cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBytes);
     if (r != cudaSuccess) return r;
-    return cudaFuncSetAttribute(attention_tc_tiled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTlSmemBytes);
+    r = cudaFuncSetAttribute(attention_tc_tiled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTlSmemBytes);
+    if (r != cudaSuccess) return r;
+    return cudaFuncSetAttribute(attention_tc_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sp_smem_bytes(2));
   });
   if (e != cudaSuccess) return e;
+  const int q_tiles = (p.seq + kTcRows - 1) / kTcRows;
+  if (p.split_rows != 0)
+    return launch_kernel(attention_tc_split_kernel, dim3(p.heads, p.batch * q_tiles, p.n_groups), dim3(kSpThreads), sp_smem_bytes(q_tiles > 1 ? 2 : 1),
+                         stream, p);
   if (p.seq <= kTcRows) {
     dim3 grid(p.heads, p.batch, p.n_groups);
     return launch_kernel(attention_tc_kernel, grid, dim3(kTcThreads), kTcSmemBytes, stream, p);
   }
-  const int q_tiles = (p.seq + kTcRows - 1) / kTcRows;
   dim3 grid(p.heads, p.batch * q_tiles, p.n_groups);
   return launch_kernel(attention_tc_tiled_kernel, grid, dim3(kTcThreads), kTlSmemBytes, stream, p);
 }

@@ -153,13 +153,15 @@ struct alignas(64) AttnParams {
   const int32_t* row_start;     // [B + 1] or null
   int32_t packed;               // 1: no padded rows exist, nothing is written beyond a sequence's length
   int32_t n_groups, batch, seq, heads;
-  int32_t tensor_memory;        // 1: the tcgen05 kernel (seq <= 128, tmap_qkv filled); 0: the mma.sync kernel
+  int32_t tensor_memory;        // 1: the tcgen05 kernels (seq <= 512, tmap_qkv and tmap_qkv64 filled); 0: the mma.sync kernel
+  int32_t split_rows;           // 1: of them the one with two threads per query row (attention_split_rows)
   uint32_t* status;             // sticky device status word (may be null)
 };
 // Longest sequence the tensor-memory attention kernels handle (up to 128 tokens: one CTA holds all keys of a
 // sequence; longer: tiles of 128 queries walk the keys in tiles of 128).
 constexpr int kAttnTensorMemoryMaxSeq = 512;
 constexpr int kAttnTileRows = 128;   // rows of the Q/K/V boxes of the tensor maps
+bool attention_split_rows(int batch, int seq);   // whether that one is the better (bf16 projections)
 cudaError_t launch_attention(const AttnParams& p, cudaStream_t stream);
 cudaError_t launch_attention_tc(const AttnParams& p, cudaStream_t stream);
 

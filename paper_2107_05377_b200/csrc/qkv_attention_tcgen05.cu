@@ -66,16 +66,6 @@ constexpr int kQaSmemBytes = kQaStages * (kQaABytes + kQaBBytes) + 2 * kQaTileBy
                              kQaExchangeBytes + kQaColumnSets * kQaColumnBytes + kQaNotFiniteBytes + 512 + 1024;
 static_assert(kQaSmemBytes <= 227 * 1024, "shared memory of one CTA");
 
-// D[tmem] (+)= A[tmem] . B[smem]^T, 128 x N x 16: A has its rows on the lanes and two consecutive elements of K per column.
-__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(desc_b), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
 // Byte offset of 16-byte chunk c (0..3) of row r in a warp's scratch (rows of 64 bytes; two rows per 128 bytes, chunks
 // exclusive-or'ed so that eight lanes touch eight bank groups both when a lane writes its row and when four read one).
 __device__ __forceinline__ int qa_scratch_off(int r, int c) { return r * 64 + ((c ^ ((r >> 1) & 3)) << 4); }
