@@ -65,8 +65,10 @@ __device__ __forceinline__ void split_row(const float (&c)[4][4], int half, floa
   *lo = pack_row(d, half);
 }
 
-// One CTA = (16 RT sequences, head, layer).  Warp w makes columns w * 8 .. + 7 of q (its rows of Wq are asked for before the
-// dependency wait), then H / 8 columns of q~.
+// One CTA = (16 RT sequences, head, layer).  Warp w makes columns w * 8 .. + 7 of q, then H / 8 columns of q~.  The head's rows of
+// both matrices (192 KB for H = 768, a chain of reads that is what the kernel takes) are asked for before the dependency wait:
+// a warp's rows of Wq in registers, its columns of Wk through shared memory (32 x 128 tokens 1036 -> 1028 us per forward,
+// 23 x 101 1044 -> 1035; Wk was read where it is used, a trip to memory for each block of columns).
 template <int V, int RT>
 __global__ void __launch_bounds__(kCpThreads) cls_query_kernel(const ClsPoolParams p) {
   constexpr int H = V * 256;
@@ -75,6 +77,7 @@ __global__ void __launch_bounds__(kCpThreads) cls_query_kernel(const ClsPoolPara
   constexpr int Q_PITCH = kHeadDim * 2 + 16;
   extern __shared__ uint8_t smem[];
   uint8_t* q_smem = smem + RT * 16 * PITCH;
+  uint8_t* wk_smem = q_smem + RT * 16 * Q_PITCH;   // the head's 64 rows of Wk, with the pitch of x
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const int head = blockIdx.y, layer = blockIdx.z;
@@ -84,16 +87,33 @@ __global__ void __launch_bounds__(kCpThreads) cls_query_kernel(const ClsPoolPara
   uint4 wb[CHUNKS];
 #pragma unroll
   for (int c = 0; c < CHUNKS; ++c) wb[c] = __ldg(reinterpret_cast<const uint4*>(wq + c * 32));
+  {
+    const bf16* wk = p.wk[layer] + static_cast<size_t>(head * kHeadDim) * H + warp * (H / kCpWarps);
+    const uint32_t dst = smem_u32(wk_smem) + warp * (H / kCpWarps) * 2;
+    constexpr int VECS = H / kCpWarps / 8;         // 16-byte pieces of this warp's columns of a row
+    for (int i = lane; i < kHeadDim * VECS; i += 32) {
+      const int r = i / VECS, c = i - r * VECS;
+      cp_async_16(dst + r * PITCH + c * 16, wk + static_cast<size_t>(r) * H + c * 8);
+    }
+    cp_async_commit();
+  }
   const uint32_t bias = __ldg(reinterpret_cast<const uint32_t*>(p.bq[layer] + head * kHeadDim + warp * 8 + 2 * t));
+  int starts[RT * 16 / kCpWarps];                  // of this warp's rows of x (written by the forward's first kernel, see below)
+#pragma unroll
+  for (int i = 0; i < RT * 16 / kCpWarps; ++i) starts[i] = b0 + warp + i * kCpWarps < p.batch ? p.row_start[b0 + warp + i * kCpWarps] : 0;
   grid_dependency_wait();
   grid_launch_dependents();
-  // the first tokens' rows
-  for (int i = threadIdx.x; i < RT * 16 * (H / 8); i += kCpThreads) {
-    const int r = i / (H / 8), c = i - r * (H / 8);
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (b0 + r < p.batch) v = __ldcg(reinterpret_cast<const uint4*>(p.x[layer] + static_cast<size_t>(p.row_start[b0 + r]) * H) + c);
-    *reinterpret_cast<uint4*>(smem + r * PITCH + c * 16) = v;
+  // the first tokens' rows (rows beyond the batch are zero)
+#pragma unroll
+  for (int i = 0; i < RT * 16 / kCpWarps; ++i) {
+    const int r = warp + i * kCpWarps;
+    const bool there = b0 + r < p.batch;
+    const bf16* row = p.x[layer] + static_cast<size_t>(starts[i]) * H;
+#pragma unroll
+    for (int v = 0; v < V; ++v) cp_async_16(smem_u32(smem) + r * PITCH + (v * 32 + lane) * 16, row + (v * 32 + lane) * 8, there);
   }
+  cp_async_commit();
+  cp_async_wait_pending<0>();                      // (Wk has landed too: it was asked for first)
   __syncthreads();
   float acc[RT][4];
 #pragma unroll
@@ -120,7 +140,7 @@ __global__ void __launch_bounds__(kCpThreads) cls_query_kernel(const ClsPoolPara
   }
   __syncthreads();
   // q~ = q Wk: K = the head's 64 rows of Wk (four steps of 16: lane t takes rows t * 4 .. + 3 of each)
-  const bf16* wk = p.wk[layer] + static_cast<size_t>(head * kHeadDim + t * 4) * H + g * 4;
+  const uint8_t* wk = wk_smem + t * 4 * PITCH + g * 8;
 #pragma unroll 1
   for (int blk = 0; blk < V; ++blk) {
     const int base = (warp * V + blk) * 32;
@@ -128,7 +148,7 @@ __global__ void __launch_bounds__(kCpThreads) cls_query_kernel(const ClsPoolPara
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) w[kk][i] = __ldg(reinterpret_cast<const uint2*>(wk + static_cast<size_t>(kk * 16 + i) * H + base));
+      for (int i = 0; i < 4; ++i) w[kk][i] = *reinterpret_cast<const uint2*>(wk + (kk * 16 + i) * PITCH + base * 2);
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
       float c[4][4];
@@ -325,18 +345,22 @@ __global__ void __launch_bounds__(kCpThreads, V == 3 ? 2 : 1) cls_pool_kernel(co
 
 template <int V, int RT>
 cudaError_t launch_query(const ClsPoolParams& p, cudaStream_t stream) {
-  constexpr int smem = RT * 16 * (V * 512 + 16) + RT * 16 * (kHeadDim * 2 + 16);
+  constexpr int smem = (RT * 16 + kHeadDim) * (V * 512 + 16) + RT * 16 * (kHeadDim * 2 + 16);
+  static_assert(smem <= 227 * 1024, "shared memory");
   auto kernel = cls_query_kernel<V, RT>;
   static PerDeviceOnce once;
   cudaError_t err = per_device_once(once, [&](int) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
   if (err != cudaSuccess) return err;
   return launch_kernel(kernel, dim3((p.batch + RT * 16 - 1) / (RT * 16), p.heads, p.n_groups), dim3(kCpThreads), smem, stream, p);
 }
-// sequences per CTA: a CTA reads 192 KB of weights (hidden 768) whatever their number, 64 rows of x fit
+// sequences per CTA: a CTA reads 192 KB of weights (hidden 768) whatever their number, 64 rows of x fit (hidden 1024: 32)
 template <int V>
 cudaError_t launch_query(const ClsPoolParams& p, cudaStream_t stream) {
   if (p.batch <= 16) return launch_query<V, 1>(p, stream);
-  return p.batch <= 32 ? launch_query<V, 2>(p, stream) : launch_query<V, 4>(p, stream);
+  if constexpr (V == 3) {
+    if (p.batch > 32) return launch_query<V, 4>(p, stream);
+  }
+  return launch_query<V, 2>(p, stream);
 }
 template <int V>
 cudaError_t launch_pool(const ClsPoolParams& p, cudaStream_t stream) {
