@@ -12,7 +12,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmt_bert.so")
-SOURCES = ["mt_api.cu", "gemm_tcgen05.cu", "attention.cu", "cls_pool.cu", "attention_tc.cu", "qkv_attention_tcgen05.cu", "gemm_ln_tcgen05.cu", "gemm_ln_pair_tcgen05.cu", "gemm_ln_low_tcgen05.cu", "rowwise.cu", "noalloc.cu", "wait_probe.cu"]
+SOURCES = ["mt_api.cu", "gemm_tcgen05.cu", "attention.cu", "cls_pool.cu", "attention_tc.cu", "qkv_attention_tcgen05.cu", "gemm_ln_tcgen05.cu", "gemm_ln_pair_tcgen05.cu", "gemm_ln_low_tcgen05.cu", "gemm_low_tcgen05.cu", "rowwise.cu", "noalloc.cu", "wait_probe.cu"]
 
 
 def sources():
@@ -23,7 +23,7 @@ def needs_build() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = sources() + [os.path.join(CSRC, "mt_kernels.h"), os.path.join(CSRC, "tc_ptx.cuh"), os.path.join(CSRC, "rowwise.cuh"), os.path.join(CSRC, "cluster_ptx.cuh"), os.path.join(HERE, "..", "include", "mt_bert.h")]
+    deps = sources() + [os.path.join(CSRC, "mt_kernels.h"), os.path.join(CSRC, "tc_ptx.cuh"), os.path.join(CSRC, "rowwise.cuh"), os.path.join(CSRC, "cluster_ptx.cuh"), os.path.join(CSRC, "gemm_low.cuh"), os.path.join(HERE, "..", "include", "mt_bert.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 

@@ -20,31 +20,17 @@
 // One cluster, one block of rows: nothing is persistent.  Every wait is bounded, as in gemm_bf16_tcgen05.
 
 #include "cluster_ptx.cuh"
+#include "gemm_low.cuh"
 #include "rowwise.cuh"
 
 namespace mt {
 namespace {
 
-constexpr int kLlCols = 128;                      // columns of a CTA
-constexpr int kLlEpilogueWarps = 8;
-constexpr int kLlThreads = 32 * (2 + kLlEpilogueWarps);
-constexpr int kLlStageK = 2;                      // k-blocks of a stage
-constexpr int kLlWBytes = kLlStageK * kLlCols * 128;
 constexpr int kLlMaxSegments = 16;
-constexpr int kLlPitch = kLlCols + 4;             // floats between rows of the turned accumulator
-__host__ __device__ constexpr int ll_x_bytes(int rows) { return kLlStageK * rows * 128; }
-__host__ __device__ constexpr int ll_stages(int rows) { return rows == 16 ? 6 : (rows == 32 ? 5 : 4); }
 __host__ __device__ constexpr int ll_stats_bytes(int rows) { return kLlMaxSegments * rows * 8; }
 __host__ __device__ constexpr int ll_smem_bytes(int rows) { return ll_stages(rows) * (kLlWBytes + ll_x_bytes(rows)) + ll_stats_bytes(rows) + 256 + 1024; }
 static_assert(ll_smem_bytes(16) <= 227 * 1024 && ll_smem_bytes(32) <= 227 * 1024 && ll_smem_bytes(64) <= 227 * 1024, "shared memory");
-static_assert(64 * kLlPitch * 4 <= 4 * kLlWBytes, "the turned accumulator goes over the ring");
 
-__device__ __forceinline__ void tmem_ld_32x8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr)
-               : "memory");
-}
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 

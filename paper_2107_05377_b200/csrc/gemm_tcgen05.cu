@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
   static_assert(!FP8 || !PAIR, "the 8-bit operands run as single CTAs");
   constexpr int KB_ELEMS = FP8 ? 2 * kGemmBlockK : kGemmBlockK;   // elements of K in a 128-byte row
   static_assert(LOW == 0 || LOW == 64 || LOW == 32, "tile heights implemented: 128, 64, 32");
-  static_assert(LOW == 0 || (BN == 64 && !PAIR && !FP8), "low tiles: 64 columns, single CTAs, bf16");
+  static_assert(LOW == 0 || (BN == 64 && !PAIR && !FP8 && EPI == kEpiBias), "low tiles: 64 columns, single CTAs, bf16 results");
   constexpr int STAGES = gemm_stages(BN, PAIR, EPI, FP8, LOW);
   constexpr int A_BYTES = gemm_a_bytes(LOW);
   constexpr int KPS = LOW ? kGemmLowKBlocks : 1;         // k-blocks of a stage
@@ -646,18 +646,6 @@ cudaError_t launch_any(const GemmParams& p, int epilogue, int sm_count, cudaStre
   }
 }
 
-template <int LOW>
-cudaError_t launch_low(const GemmParams& p, int epilogue, int sm_count, cudaStream_t stream) {
-  switch (epilogue) {
-    case kEpiBias: return launch_one<64, kEpiBias, false, false, LOW>(p, sm_count, stream);
-    case kEpiBiasGelu: return launch_one<64, kEpiBiasGelu, false, false, LOW>(p, sm_count, stream);
-    case kEpiBiasResidual: return launch_one<64, kEpiBiasResidual, false, false, LOW>(p, sm_count, stream);
-    case kEpiBiasTanhF32: return launch_one<64, kEpiBiasTanhF32, false, false, LOW>(p, sm_count, stream);
-    case kEpiPartialF32: return launch_one<64, kEpiPartialF32, false, false, LOW>(p, sm_count, stream);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
 }  // namespace
 
 int gemm_block_n(int N, int epilogue, int64_t rows, int groups, bool pair, int sm_count) {
@@ -693,13 +681,28 @@ int gemm_block_n(int N, int epilogue, int64_t rows, int groups, bool pair, int s
   }
   return best;
 }
-// Low tiles (64 rows x 64 columns, 32 rows where a layer has no more; single CTAs) where a launch has so few rows that all
-// of them run at once: then the chain of k-blocks one CTA walks is what the launch costs, not the bytes it stages.  (32-row
-// tiles of more rows read the weights that much more often: 1 x 128 tokens 397 us per forward against 386.)  Never changes
-// a bit.
+// Tiles of few rows, where a launch has so few that all of them run at once: then the chain of loads one CTA walks is what the
+// launch costs, not the bytes it stages.  Never changes a bit.
+// Turned tiles (gemm_low_tcgen05) of 32 rows, 16 where a layer has no more, 64 where 32 do not all fit.  (us per forward with 64 x 64
+// tiles that were not turned / turned from 16, 32, 64 rows on: 2 x 32 tokens 137 / 128, 126, 136; 1 x 128 346 / 335, 326, 330;
+// 3 x 57 host to host 248 / 214, 209, 227; 4 x 128 458 / 443, 441, 445.)
+// Not turned, 64 or 32 rows x 64 columns: where the X of a column tile is its own (x_by_tile: a head's 64 columns).
 void gemm_choose_low(GemmParams* p, int groups, int sm_count) {
   const int splits = p->k_splits > 1 ? p->k_splits : 1;
-  if (p->fp8 || p->N % 64 != 0 || p->K % (kGemmBlockK * kGemmLowKBlocks * splits * (p->x_by_tile > 1 ? p->x_by_tile : 1)) != 0) return;
+  if (p->x_by_tile == 0) {
+    if (p->fp8 || p->N % 128 != 0 || p->K % (2 * kGemmBlockK * splits) != 0) return;
+    for (int rows : {16, 32, 64}) {
+      if (rows == 16 && p->M > 16) continue;
+      const int64_t tiles = static_cast<int64_t>((p->M + rows - 1) / rows) * (p->N / 128) * (groups < 1 ? 1 : groups) * splits;
+      if (tiles > sm_count) continue;
+      p->turned = rows;
+      p->pair = 0;
+      p->block_n = 128;
+      return;
+    }
+    return;
+  }
+  if (p->fp8 || p->N % 64 != 0 || p->K % (kGemmBlockK * kGemmLowKBlocks * splits * p->x_by_tile) != 0) return;
   const int low = p->M <= 32 ? 32 : 64;
   const int64_t tiles = static_cast<int64_t>((p->M + low - 1) / low) * (p->N / 64) * (groups < 1 ? 1 : groups) * splits;
   if (tiles > sm_count) return;
@@ -731,11 +734,13 @@ cudaError_t launch_gemm(const GemmParams& p, int epilogue, int sm_count, cudaStr
   if (p.x_by_tile != 0 && (p.x_by_tile < 0 || p.x_by_tile > 2 || p.block_n != 64 || p.pair || p.fp8 || p.k_splits > 1 ||
                            p.K % (p.x_by_tile * kGemmBlockK * (p.low != 0 ? kGemmLowKBlocks : 1)) != 0))
     return cudaErrorInvalidValue;
+  if (p.turned != 0) return launch_gemm_low(p, epilogue, stream);
   if (p.low != 0) {
     if (p.pair || p.block_n != 64 || p.K % (kGemmBlockK * kGemmLowKBlocks * (p.k_splits > 1 ? p.k_splits : 1)) != 0)
       return cudaErrorInvalidValue;
-    return p.low == 64 ? launch_low<64>(p, epilogue, sm_count, stream)
-                       : (p.low == 32 ? launch_low<32>(p, epilogue, sm_count, stream) : cudaErrorInvalidValue);
+    if (epilogue != kEpiBias) return cudaErrorInvalidValue;   // (the value projection of the first-token attention)
+    if (p.low == 64) return launch_one<64, kEpiBias, false, false, 64>(p, sm_count, stream);
+    return p.low == 32 ? launch_one<64, kEpiBias, false, false, 32>(p, sm_count, stream) : cudaErrorInvalidValue;
   }
   return p.pair ? launch_any<true>(p, epilogue, sm_count, stream) : launch_any<false>(p, epilogue, sm_count, stream);
 }

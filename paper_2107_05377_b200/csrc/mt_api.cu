@@ -265,6 +265,10 @@ cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, co
   if (g->fp8 != 0) {
     if ((e = make_tmap_u8(&g->tmap_x[i], x, M, K, kGemmBlockM)) != cudaSuccess) return e;
     if ((e = make_tmap_u8(&g->tmap_w[i], w, N, K, g->block_n)) != cudaSuccess) return e;
+  } else if (g->turned != 0) {
+    if ((e = make_tmap_kblocks(&g->tmap_x[i], x, M, K, g->turned, 2)) != cudaSuccess) return e;
+    if ((e = make_tmap_kblocks(&g->tmap_w[i], w, N, K, 128, 2)) != cudaSuccess) return e;
+    g->group[i].residual = residual;
   } else if (g->low != 0) {
     if ((e = make_tmap_kblocks(&g->tmap_x[i], x, M, x_cols, g->low, kGemmLowKBlocks)) != cudaSuccess) return e;
     if ((e = make_tmap_kblocks(&g->tmap_w[i], w, N, w_cols, 64, kGemmLowKBlocks)) != cudaSuccess) return e;

@@ -103,7 +103,8 @@ enum GemmEpilogue { kEpiBias = 0, kEpiBiasGelu = 1, kEpiBiasResidual = 2, kEpiBi
 // The output and the residual are reached through the tensor maps of GemmParams.
 struct GemmGroup {
   const bf16* bias;
-  void* out;             // (low tiles with bf16 results) the output by pointer
+  void* out;             // (low and turned tiles) the output by pointer
+  const float* residual; // (turned tiles) the same of the residual
   const float* scale_x;  // (8-bit operands) one scale per row of X, [M]
   const float* scale_w;  // (8-bit operands) one scale per row of W, [N]
 };
@@ -121,6 +122,8 @@ struct alignas(64) GemmParams {
   int32_t block_n;         // tile width along N: 128, 192 or 256 (gemm_block_n); N % block_n == 0
   int32_t low;             // 64 or 32: tiles of that many rows (block_n 64, single CTAs, bf16); 0: 128.  The X and W maps are
                            // then dims {64, rows, K / 64}, box {64, low | 64, kGemmLowKBlocks}
+  int32_t turned;          // 64, 32 or 16: tiles of that many rows and 128 columns (launch_gemm_low; single CTAs, bf16); 0: not.  The X
+                           // and W maps are then dims {64, rows, K / 64}, boxes {64, turned | 128, 2}
   int32_t x_by_tile;       // s = 1 or 2: column tile n (block_n 64) multiplies columns n K .. n K + K - 1 of X, which has N / 64 * K
                            // of them: s pieces of K / s columns, summands of X, each against all K / s columns of W
   int32_t k_splits;        // ranges K is split into (kEpiPartialF32 only; otherwise 1): (K / 64) % k_splits == 0
@@ -140,6 +143,7 @@ void gemm_choose_low(GemmParams* p, int groups, int sm_count);   // after N, M, 
 // Width in elements of the 128-byte output box (64 bf16 or 32 fp32 columns; 32 rows).
 int gemm_out_box_cols(int epilogue);
 cudaError_t launch_gemm(const GemmParams& p, int epilogue, int sm_count, cudaStream_t stream);
+cudaError_t launch_gemm_low(const GemmParams& p, int epilogue, cudaStream_t stream);   // (launch_gemm with `turned` set)
 
 // Token layout.  The rows of sequence b start at row_start[b] (device array of batch + 1 ints written
 // by launch_row_starts: b * seq for the padded layout, the running sum of the lengths for the packed
