@@ -115,6 +115,7 @@ struct DumpCopy {
 // and values of all tokens) and the first-token attention (`attn_cls`, `n_cls` groups); the rest of
 // those layers, a few rows each, is run for all tasks together after the last wave (a `cls tail` step).
 struct Chunk {
+  QuantParams q_in;   // 8-bit operands: the layers' inputs, quantised row by row before the Q/K/V projection
   bool fused_qkv = false;
   QkvAttnParams qa;
   GemmParams qkv;
@@ -358,7 +359,6 @@ struct mt_model {
   size_t act_bytes;    // max_batch*max_seq*hidden bf16
   size_t act32_bytes;  // the same tensor in fp32
   size_t state_bytes;  // one hidden state = its bf16 copy (GEMM operand) followed by its fp32 copy (residual)
-  size_t stored_bytes; // a state that outlives its layer: with 8-bit operands its E4M3 copy and a scale per row follow
   size_t slot_bytes;
   int32_t n_slots, n_dump;
   size_t ws_total;
@@ -457,7 +457,6 @@ void layout_workspace(mt_model* m) {
   m->act_bytes = pad256(M * H * sizeof(bf16));
   m->act32_bytes = pad256(M * H * sizeof(float));
   m->state_bytes = m->act_bytes + m->act32_bytes;
-  m->stored_bytes = m->state_bytes + (m->fp8 ? pad256(M * H) + pad256(M * 4) : 0);
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t at = off; off += pad256(bytes); return at; };
   m->ws_status = take(256);
@@ -473,16 +472,16 @@ void layout_workspace(mt_model* m) {
   m->ws_pooled = take(static_cast<size_t>(kMaxGroups) * m->max_batch * H * sizeof(float));
   // partial sums of the FFN-down projection in launches of few rows: fp32 [group][range of K][row pitch][H]
   m->ws_partial = take(static_cast<size_t>(kMaxGroups) * kDownSplits * split_pitch(std::min<size_t>(M, kSplitRowsMax)) * H * sizeof(float));
-  m->ws_trunk[0] = take(m->stored_bytes);
-  m->ws_trunk[1] = take(m->stored_bytes);
+  m->ws_trunk[0] = take(m->state_bytes);
+  m->ws_trunk[1] = take(m->state_bytes);
   m->ws_task0 = off;
-  off += m->stored_bytes * m->tasks.size();
+  off += m->state_bytes * m->tasks.size();
   m->n_slots = std::min<int32_t>(m->max_groups, static_cast<int32_t>(m->tasks.size()) + 1);
   // slot = qkv [M,3H] bf16 + ctx [M,H] bf16 + u [M,H] fp32 + h1 [M,H] bf16 and fp32 + f [M,F] bf16
   m->slot_bytes = pad256(M * 3 * H * 2) + m->act_bytes + m->act32_bytes + m->state_bytes + pad256(M * F * 2);
   m->slot_q_off = m->slot_bytes;
-  // 8-bit operands: E4M3 copies of h1 ([M,H]) and of f ([M,F]), each with a scale per row
-  if (m->fp8) m->slot_bytes += pad256(M * H) + pad256(M * F) + 2 * pad256(M * 4);
+  // 8-bit operands: E4M3 copies of the layer input and of h1 ([M,H]) and of f ([M,F]), each with a scale per row
+  if (m->fp8) m->slot_bytes += 2 * pad256(M * H) + pad256(M * F) + 3 * pad256(M * 4);
   m->ws_slot0 = off;
   off += m->slot_bytes * m->n_slots;
   // per task, for its last branch layer on first tokens: ctx bf16, residual fp32, u fp32, h1 bf16 + fp32 (all
@@ -567,29 +566,39 @@ const bf16* w_ptr(const mt_model* m, size_t off) { return reinterpret_cast<const
 
 // Where the state of a stream lives: trunk depth d in ping-pong buffer d & 1, a task in its own buffer.
 bf16* trunk_buf(const mt_model* m, int32_t depth) { return ws_ptr(m, m->ws_trunk[depth & 1]); }
-bf16* task_buf(const mt_model* m, int32_t task) { return ws_ptr(m, m->ws_task0 + m->stored_bytes * task); }
+bf16* task_buf(const mt_model* m, int32_t task) { return ws_ptr(m, m->ws_task0 + m->state_bytes * task); }
 // fp32 copy of a state: stored right after its bf16 copy
 float* f32_of(const mt_model* m, bf16* state) {
   return reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(state) + m->act_bytes);
 }
 
-// (8-bit operands) E4M3 copy of a stored state and its scales: behind the fp32 copy.  Whoever writes the state writes them.
-uint8_t* codes_of(const mt_model* m, bf16* state) { return reinterpret_cast<uint8_t*>(state) + m->state_bytes; }
-float* scales_of(const mt_model* m, bf16* state) {
-  return reinterpret_cast<float*>(codes_of(m, state) + pad256(static_cast<size_t>(m->max_batch) * m->max_seq * m->trunk.hidden));
-}
-
-// 8-bit scratch at `p` of a slot (rows = max_batch * max_seq) or of a task's first tokens (rows = max_batch).
+// 8-bit scratch of a slot (rows = max_batch * max_seq; xq/sx: the layer input) or of a task's first-token
+// scratch (rows = max_batch; no xq).
 struct QuantScratch {
+  uint8_t* xq; float* sx;
   uint8_t* h1q; float* sh1;
   uint8_t* fq; float* sf;
 };
-QuantScratch quant_scratch(const mt_model* m, uint8_t* p, size_t rows) {
-  const size_t H = m->trunk.hidden, F = m->trunk.ffn;
+QuantScratch slot_quant(const mt_model* m, uint8_t* slot) {
+  const size_t M = static_cast<size_t>(m->max_batch) * m->max_seq, H = m->trunk.hidden, F = m->trunk.ffn;
+  uint8_t* p = slot + m->slot_q_off;
   QuantScratch q;
-  q.h1q = p; p += pad256(rows * H);
-  q.sh1 = reinterpret_cast<float*>(p); p += pad256(rows * 4);
-  q.fq = p; p += pad256(rows * F);
+  q.xq = p; p += pad256(M * H);
+  q.sx = reinterpret_cast<float*>(p); p += pad256(M * 4);
+  q.h1q = p; p += pad256(M * H);
+  q.sh1 = reinterpret_cast<float*>(p); p += pad256(M * 4);
+  q.fq = p; p += pad256(M * F);
+  q.sf = reinterpret_cast<float*>(p);
+  return q;
+}
+QuantScratch cls_quant(const mt_model* m, uint8_t* cs) {
+  const size_t B = static_cast<size_t>(m->max_batch), H = m->trunk.hidden, F = m->trunk.ffn;
+  uint8_t* p = cs + m->cls_q_off;
+  QuantScratch q;
+  q.xq = nullptr; q.sx = nullptr;
+  q.h1q = p; p += pad256(B * H);
+  q.sh1 = reinterpret_cast<float*>(p); p += pad256(B * 4);
+  q.fq = p; p += pad256(B * F);
   q.sf = reinterpret_cast<float*>(p);
   return q;
 }
@@ -919,10 +928,15 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   ck->qkv.pair = use_pair(m, M, n_qkv);
   choose_block_n(m, &ck->qkv, kEpiBias, false, n_qkv);
   if (!m->fp8) gemm_choose_low(&ck->qkv, n_qkv, m->sm_count);
+  memset(&ck->q_in, 0, sizeof(ck->q_in));
   if (m->fp8) {
     ck->qkv.fp8 = 1;
     ck->qkv.pair = 0;
     ck->qkv.block_n = 256;
+    ck->q_in.n_groups = static_cast<int32_t>(count);
+    ck->q_in.rows = M;
+    ck->q_in.cols = H;
+    ck->q_in.rows_valid = reinterpret_cast<const int32_t*>(m->d_workspace + m->ws_rows_valid);
   }
   ck->qkv.m_valid = reinterpret_cast<const int32_t*>(m->d_workspace + m->ws_rows_valid);
   ck->qkv.status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
@@ -963,9 +977,10 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
     cudaError_t e;
     // 1. qkv = in . [Wq;Wk;Wv]^T + [bq;bk;bv] on every token (the three matrices and biases are
     //    contiguous in the arena); keys and values are needed for all tokens even in a `cls` layer
-    const QuantScratch qs = m->fp8 ? quant_scratch(m, slot + m->slot_q_off, static_cast<size_t>(m->max_batch) * m->max_seq) : QuantScratch{};
+    const QuantScratch qs = m->fp8 ? slot_quant(m, slot) : QuantScratch{};
     const bool cls = is_cls_op(m, op);
-    const void* x_op = m->fp8 ? static_cast<const void*>(codes_of(m, in)) : in;   // the projection's operands
+    if (m->fp8) { ck->q_in.x[i] = in; ck->q_in.q[i] = qs.xq; ck->q_in.scale[i] = qs.sx; }
+    const void* x_op = m->fp8 ? static_cast<const void*>(qs.xq) : in;   // the projection's operands
     const void* w_op = m->fp8 ? static_cast<const void*>(m->d_weights + lo->q_qkv) : w_ptr(m, lo->wq);
     const float* w_scale = m->fp8 ? reinterpret_cast<const float*>(m->d_weights + lo->s_qkv) : nullptr;
     if (ck->fused_qkv && !cls) {
@@ -979,7 +994,7 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
     } else {
       const int a = n_qkv_set++;
       if ((e = set_gemm_group(&ck->qkv, a, kEpiBias, x_op, w_op, w_ptr(m, lo->bq), nullptr, qkv)) != cudaSuccess) return e;
-      ck->qkv.group[a].scale_x = m->fp8 ? scales_of(m, in) : nullptr;
+      ck->qkv.group[a].scale_x = qs.sx;
       ck->qkv.group[a].scale_w = w_scale;
     }
     if (!cls) {
@@ -995,10 +1010,6 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
       if ((e = add_to_tail(m, &ck->full, lo, ctx, f32_of(m, in), u, h1, f32_of(m, h1), f, out, f32_of(m, out), &qs)) !=
           cudaSuccess)
         return e;
-      if (m->fp8) {   // (the next layer's projection reads the state's codes)
-        ck->full.ln2.q[a] = codes_of(m, out);
-        ck->full.ln2.scale[a] = scales_of(m, out);
-      }
       if (m->debug_capture) ck->dumps.push_back({out, dump_slot(m, op.task, op.layer), false});
     } else {
       // 2'. first-token attention into the task's compact [B, H] scratch, which also gathers the first
@@ -1071,7 +1082,7 @@ cudaError_t build_cls_tail(const mt_model* m, const std::vector<int32_t>& tasks,
     float* h1_32 = reinterpret_cast<float*>(cs + 2 * m->cls_h_bytes + 2 * m->cls_h32_bytes);
     bf16* f = reinterpret_cast<bf16*>(cs + 2 * m->cls_h_bytes + 3 * m->cls_h32_bytes);
     bf16* out = task_buf(m, t);  // the task's state becomes [B, H]
-    const QuantScratch qs = m->fp8 ? quant_scratch(m, cs + m->cls_q_off, static_cast<size_t>(m->max_batch)) : QuantScratch{};
+    const QuantScratch qs = m->fp8 ? cls_quant(m, cs) : QuantScratch{};
     cudaError_t e = add_to_tail(m, st->tail.get(), lo, ctx, res, u, h1, h1_32, f, out, nullptr, &qs);
     if (e != cudaSuccess) return e;
     if (m->debug_capture) st->dumps.push_back({out, dump_slot(m, t, te.cfg.branch_layers), true});
@@ -1131,8 +1142,8 @@ int32_t count_launches(const mt_model* m, const Schedule& s, int32_t batch, int3
         for (size_t i = 0; i < count; ++i) n_cls += is_cls_op(m, ops.layers[first + i]) ? 1 : 0;
         const int32_t n_full = static_cast<int32_t>(count) - n_cls;
         const bool fused_qkv = n_full > 0 && use_qkv_attention(m, rows, seq);
-        // Q/K/V and attention of the layers on all tokens, of the last branch layers, the rest of the layer
-        n += (fused_qkv ? 1 + (n_cls > 0 ? 1 : 0) : 1 + (n_full > 0 ? 1 : 0)) + (n_cls > 0 ? 1 : 0);
+        // (inputs quantised), Q/K/V and attention of the layers on all tokens, of the last branch layers, the rest of the layer
+        n += (m->fp8 ? 1 : 0) + (fused_qkv ? 1 + (n_cls > 0 ? 1 : 0) : 1 + (n_full > 0 ? 1 : 0)) + (n_cls > 0 ? 1 : 0);
         n += n_full > 0 ? tail_launches(m, n_full, rows) : 0;
       }
       const size_t n_tails = cls_tasks_after_wave(m, s, w).size();
@@ -1748,8 +1759,6 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
   ep.gamma = w_ptr(m, m->emb_ln_g); ep.beta = w_ptr(m, m->emb_ln_b);
   ep.out = plan.embedding;
   ep.out32 = f32_of(m, ep.out);
-  ep.q = m->fp8 ? codes_of(m, ep.out) : nullptr;
-  ep.scale = m->fp8 ? scales_of(m, ep.out) : nullptr;
   ep.batch = batch; ep.seq = seq; ep.hidden = m->trunk.hidden; ep.vocab = m->trunk.vocab_size;
   ep.type_vocab = m->trunk.type_vocab; ep.eps = m->trunk.ln_eps; ep.status = status;
   MT_TIMED(MT_CLASS_EMBED, launch_embed(ep, stream), "embedding kernel");
@@ -1768,6 +1777,7 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
     }
     if (st.kind == 0) {
       Chunk& ck = *st.chunk;
+      if (m->fp8) MT_TIMED(MT_CLASS_QUANT, launch_quantize_rows(ck.q_in, stream), "quantising the layer inputs");
       const bool beside = m->overlap_cls && m->side_stream != nullptr && !m->profile && ck.n_cls > 0 && ck.full.count > 0;
       if (ck.fused_qkv)
         MT_TIMED(MT_CLASS_QKV, launch_qkv_attention(ck.qa, m->sm_count, stream), "QKV projection + attention kernel");
@@ -2260,7 +2270,7 @@ int mt_kernel_embed(const int32_t* d_token_ids, const int32_t* d_segment_ids, co
       batch < 1 || seq < 1 || vocab < 1 || type_vocab < 1)
     return MT_ERR_INVALID_ARG;
   if (hidden != 768 && hidden != 1024) return MT_ERR_UNSUPPORTED;
-  EmbedParams p = {};
+  EmbedParams p;
   p.token_ids = d_token_ids; p.segment_ids = d_segment_ids; p.lengths = d_lengths;
   p.word = static_cast<const bf16*>(d_word); p.pos = static_cast<const bf16*>(d_pos);
   p.type = static_cast<const bf16*>(d_type); p.gamma = static_cast<const bf16*>(d_gamma);

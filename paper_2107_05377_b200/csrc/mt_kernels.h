@@ -291,8 +291,6 @@ struct EmbedParams {
   int2* row_info;            // null, or (packed layout) {first row, row after the last} of the row's sequence, per row
   int32_t packed;            // 1: positions >= length are skipped
   int32_t batch, seq, hidden, vocab, type_vocab;
-  uint8_t* q;                // null, or E4M3 codes of the bf16 rows, ...
-  float* scale;              // ... and their scales (see QuantParams)
   float eps;
   uint32_t* status;
 };

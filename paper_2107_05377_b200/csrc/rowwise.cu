@@ -198,77 +198,50 @@ __global__ void __launch_bounds__(V * 32) layernorm_row_kernel(const LayerNormPa
   }
 }
 
-// The kernel before this one only lays out the rows (and came after everything else in the stream): tokens, lengths and tables are
-// read before the dependency wait, and up to kOwnStartBatch sequences a warp adds up the lengths before its own instead
-// of waiting for row_start, so that a trip to tokens and tables is off the chain.  QUANT: the bf16 rows are quantised as well, as
-// in layernorm_kernel.
-constexpr int kOwnStartBatch = 256;
-template <int V, bool QUANT>
+template <int V>
 __global__ void __launch_bounds__(kRowThreads) embed_kernel(const EmbedParams p) {
   constexpr int H = V * 256;
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5);
-  const bool exists = row < p.batch * p.seq;
-  const int b = exists ? row / p.seq : 0;
-  const int pos = exists ? row - b * p.seq : 0;
-  const bool own_start = p.row_start == nullptr || p.packed == 0 || p.batch <= kOwnStartBatch;
-  if (p.row_start == nullptr) grid_dependency_wait();   // (not in a forward: after any kernel)
-  bool stored = exists;
-  int out_row = row, len = p.seq;
-  float x[V][8];
-  if (exists) {
-    int tok = p.token_ids[row];
-    int seg = p.segment_ids[row];
-    uint32_t flags = 0;
-    if (tok < 0 || tok >= p.vocab) { flags |= kFlagBadToken; tok = tok < 0 ? 0 : p.vocab - 1; }
-    if (seg < 0 || seg >= p.type_vocab) { flags |= kFlagBadSegment; seg = seg < 0 ? 0 : p.type_vocab - 1; }
-    auto clamped = [&](int n) { return n < 1 ? 1 : (n > p.seq ? p.seq : n); };
-    if (pos == 0 || p.row_start != nullptr) {
-      const int n = p.lengths[b];
-      if (pos == 0 && (n < 1 || n > p.seq)) flags |= kFlagBadLength;
-      if (p.row_start != nullptr) len = clamped(n);
-    }
-    if (flags != 0 && lane == 0 && p.status != nullptr) atomicOr(p.status, flags);
-    stored = p.row_start == nullptr || p.packed == 0 || pos < len;   // packed layout: padded positions do not exist
-    if (stored) {
-      if (p.row_start != nullptr && p.packed != 0 && own_start) {
-        int start = 0;
-        for (int i = lane; i < b; i += 32) start += clamped(p.lengths[i]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) start += __shfl_xor_sync(0xffffffffu, start, o);
-        out_row = start + pos;
-      }
-      const bf16* w = p.word + static_cast<size_t>(tok) * H;
-      const bf16* q = p.pos + static_cast<size_t>(pos) * H;
-      const bf16* t = p.type + static_cast<size_t>(seg) * H;
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        const int col = (v * 32 + lane) * 8;
-        float a[8], c[8], d[8];
-        unpack8(__ldg(reinterpret_cast<const uint4*>(w + col)), a);
-        unpack8(__ldg(reinterpret_cast<const uint4*>(q + col)), c);
-        unpack8(__ldg(reinterpret_cast<const uint4*>(t + col)), d);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[v][i] = a[i] + c[i] + d[i];
-      }
-    }
-  }
   grid_dependency_wait();
   grid_launch_dependents();
-  if (!stored) return;
-  if (!own_start) out_row = p.row_start[b] + pos;
-  if (p.row_info != nullptr && lane == 0) p.row_info[out_row] = make_int2(out_row - pos, out_row - pos + len);
-  float* out32 = p.out32 != nullptr ? p.out32 + static_cast<size_t>(out_row) * H : nullptr;
-  uint4 y8[V];
-  normalise_store<V>(x, p.gamma, p.beta, p.out + static_cast<size_t>(out_row) * H, out32, lane, p.eps, y8);
-  if (QUANT) {
-    __nv_bfloat162 amax2 = __float2bfloat162_rn(0.f);
-#pragma unroll
-    for (int v = 0; v < V; ++v) amax2 = amax8(y8[v], amax2);
-    const float scale = row_scale(warp_max(amax2));
-    if (lane == 0) p.scale[out_row] = scale;
-    store_codes(y8, reinterpret_cast<uint2*>(p.q + static_cast<size_t>(out_row) * H) + lane, scale);
+  if (row >= p.batch * p.seq) return;
+  const int b = row / p.seq;
+  const int pos = row - b * p.seq;
+  int tok = p.token_ids[row];
+  int seg = p.segment_ids[row];
+  uint32_t flags = 0;
+  if (tok < 0 || tok >= p.vocab) { flags |= kFlagBadToken; tok = tok < 0 ? 0 : p.vocab - 1; }
+  if (seg < 0 || seg >= p.type_vocab) { flags |= kFlagBadSegment; seg = seg < 0 ? 0 : p.type_vocab - 1; }
+  if (pos == 0) {
+    const int len = p.lengths[b];
+    if (len < 1 || len > p.seq) flags |= kFlagBadLength;
   }
+  if (flags != 0 && lane == 0 && p.status != nullptr) atomicOr(p.status, flags);
+  int out_row = row;
+  if (p.row_start != nullptr) {
+    int len = p.lengths[b];
+    len = len < 1 ? 1 : (len > p.seq ? p.seq : len);
+    if (p.packed && pos >= len) return;  // packed layout: padded positions do not exist
+    out_row = p.row_start[b] + pos;
+    if (p.row_info != nullptr && lane == 0) p.row_info[out_row] = make_int2(out_row - pos, out_row - pos + len);
+  }
+  const bf16* w = p.word + static_cast<size_t>(tok) * H;
+  const bf16* q = p.pos + static_cast<size_t>(pos) * H;
+  const bf16* t = p.type + static_cast<size_t>(seg) * H;
+  float x[V][8];
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const int col = (v * 32 + lane) * 8;
+    float a[8], c[8], d[8];
+    unpack8(__ldg(reinterpret_cast<const uint4*>(w + col)), a);
+    unpack8(__ldg(reinterpret_cast<const uint4*>(q + col)), c);
+    unpack8(__ldg(reinterpret_cast<const uint4*>(t + col)), d);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[v][i] = a[i] + c[i] + d[i];
+  }
+  float* out32 = p.out32 != nullptr ? p.out32 + static_cast<size_t>(out_row) * H : nullptr;
+  normalise_store<V>(x, p.gamma, p.beta, p.out + static_cast<size_t>(out_row) * H, out32, lane, p.eps);
 }
 
 // Pooler + head, two launches.
@@ -585,9 +558,8 @@ cudaError_t launch_embed(const EmbedParams& p, cudaStream_t stream) {
   const int rows = p.batch * p.seq;
   if (rows < 1) return cudaErrorInvalidValue;
   dim3 grid((rows + kRowThreads / 32 - 1) / (kRowThreads / 32));
-  const bool quant = p.q != nullptr;
-  if (p.hidden == 768) return launch_kernel(quant ? embed_kernel<3, true> : embed_kernel<3, false>, grid, dim3(kRowThreads), 0, stream, p);
-  if (p.hidden == 1024) return launch_kernel(quant ? embed_kernel<4, true> : embed_kernel<4, false>, grid, dim3(kRowThreads), 0, stream, p);
+  if (p.hidden == 768) return launch_kernel(embed_kernel<3>, grid, dim3(kRowThreads), 0, stream, p);
+  if (p.hidden == 1024) return launch_kernel(embed_kernel<4>, grid, dim3(kRowThreads), 0, stream, p);
   return cudaErrorInvalidValue;
 }
 
