@@ -810,13 +810,12 @@ __global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const
 
 }  // namespace
 
-// Beyond 128 tokens always (us per forward of the eight-task tree, one thread per row / two: 16 x 512 ragged 1937 / 1887, 60 x 512
-// for one task 5286 / 5180, 64 x 150 1917 / 1855, 8 x 256 837 / 823, 1 x 300 511 / 498).  Up to 128 a CTA has one step, whose latencies
-// count where few sequences leave the SMs idle (4 x 128 450 / 441, 2 x 100 404 / 389, 1 x 128 338 / 337), while with many, four CTAs
-// of the kernel with one thread per row per SM hide them better (32 x 128 992 / 1018, 256 x 128 9425 / 9675), and with at most 64
-// keys half of the threads have nothing to do (2 x 64 333 / 338).  The line depends on the shape of the batch alone, so a task gets
-// the same bits whatever runs beside it.
-bool attention_split_rows(int batch, int seq) { return seq > kTcRows || (seq > kTcRows / 2 && batch <= 4); }
+// Beyond 128 tokens (us per forward of the eight-task tree, one thread per row / two: 16 x 512 ragged 1937 / 1887, 60 x 512 for one
+// task 5286 / 5180, 64 x 150 1917 / 1855, 8 x 256 837 / 823, 1 x 300 511 / 498).  Up to 128 a CTA has one step, whose latencies
+// four CTAs per SM of the kernel with one thread per row hide better (32 x 128 992 / 1018, 256 x 128 9425 / 9675); a few sequences of
+// 65 to 128 tokens would gain (4 x 128 450 / 441, 2 x 100 404 / 389), shorter ones not (2 x 64 333 / 338), but a line between them
+// would change the logits of a short sequence by 1e-3 when its batch is padded beyond 64.
+bool attention_split_rows(int seq) { return seq > kTcRows; }
 
 cudaError_t launch_attention_tc(const AttnParams& p, cudaStream_t stream) {
   if (p.n_groups < 1 || p.n_groups > kMaxGroups || p.batch < 1 || p.seq < 1 || p.seq > kAttnTensorMemoryMaxSeq)

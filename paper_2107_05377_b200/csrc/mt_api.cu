@@ -958,7 +958,7 @@ cudaError_t build_chunk(const mt_model* m, const std::vector<OpDesc>& ops, size_
   ck->attn.lengths = ck->attn_cls.lengths = call_lengths(m);
   ck->attn.packed = m->pack_tokens ? 1 : 0;
   ck->attn.tensor_memory = (m->attention_tc && seq <= kAttnTensorMemoryMaxSeq) ? 1 : 0;
-  ck->attn.split_rows = !m->fp8 && attention_split_rows(batch, seq) ? 1 : 0;
+  ck->attn.split_rows = !m->fp8 && attention_split_rows(seq) ? 1 : 0;
   ck->attn.status = ck->qkv.status;
 
   int n_qkv_set = 0;
@@ -2213,7 +2213,7 @@ int mt_kernel_attention(const void* d_qkv, const int32_t* d_lengths, void* d_ctx
   p.status = d_status;
   if (tensor_memory != 0) {
     p.tensor_memory = 1;
-    p.split_rows = tensor_memory != 2 && attention_split_rows(batch, seq) ? 1 : 0;   // (2: never)
+    p.split_rows = tensor_memory != 2 && attention_split_rows(seq) ? 1 : 0;   // (2: never)
     if (make_tmap(&p.tmap_qkv[0], d_qkv, static_cast<int64_t>(batch) * seq, 3 * static_cast<int64_t>(heads) * kHeadDim,
                   kAttnTileRows, kHeadDim, false) != cudaSuccess ||
         make_tmap(&p.tmap_qkv64[0], d_qkv, static_cast<int64_t>(batch) * seq, 3 * static_cast<int64_t>(heads) * kHeadDim,
