@@ -395,7 +395,7 @@ int mt_kernel_linear_layernorm_low(const void* d_x, const void* d_w, const void*
 /* ctx[B*S, heads*64] = softmax(QK^T/8 masked to keys < length) V per (sequence, head), from the
  * packed projection qkv[B*S, 3*heads*64] = [Q | K | V].  Rows at positions >= length are written as 0.
  * tensor_memory != 0 (seq <= 512 only, else MT_ERR_INVALID_ARG) selects the tcgen05 kernels (beyond 128 tokens the
- * one of bf16 projections, 2: the one of 8-bit projections), whose
+ * one with two threads per query row of bf16 projections, 2: the one with one thread of 8-bit projections; the same bits), whose
  * score and output accumulators live in tensor memory; 0 the mma.sync kernel, which takes any seq
  * (see option "attention_tc").  d_status (device, may be NULL) receives MT_FLAG_WAIT_TIMEOUT. */
 int mt_kernel_attention(const void* d_qkv, const int32_t* d_lengths, void* d_ctx,

@@ -496,49 +496,49 @@ __global__ void __launch_bounds__(kTcThreads, 2) attention_tc_tiled_kernel(const
   if (warp == 0) tmem_dealloc(tmem_base, kTlTmemCols);
 }
 
-// ---- two threads per query row, any length ---------------------------------------------------------
-// (With 8-bit projections the kernels above stay: a rounding that falls otherwise here is a code that falls otherwise there.)
-// One CTA = one (layer of the wave, sequence, head, tile of 128 queries); the keys are walked in tiles of 128:
-//   S = Q . K_j^T (tensor memory);  P = exp((S - m) / 8), bf16, written over S;  l += rowsum P;  O += P . V_j (tensor memory)
-// m is the maximum of the row when it was last set: it moves only when a tile's maximum exceeds it by more than 8 powers of
-// two (P then stays below 2^8, whose bf16 rounding is as fine as below 1), and O and l are scaled down by that factor; so O
-// is accumulated by the tensor cores and usually not touched before the end, O / l.
-// Eight warps; a thread owns one query row and half of the keys of a tile (64), held in registers between the maximum, which the
-// two warps of a quarter exchange, and the exponentials.  Warp 0 also requests the tiles (K and V double buffered) and issues the
-// MMAs, P . V_j and S_{j+1} right behind it, when the P of all warps is in tensor memory, where it is read from.  (A ninth warp
-// for that leaves room for one CTA per SM - the registers of a quarter of the SM hold four warps of 112 - and was slower than one
-// thread per row: 38 us where that takes 31.)
+// ---- more than 128 tokens, two threads per query row ---------------------------------------------------
+// The tiles, the running maximum and the sums of attention_tc_tiled_kernel, in its order: the same bits, and with one tile of keys
+// those of attention_tc_kernel, so that a short sequence has the same result however far its batch is padded.
+// Eight warps; a thread owns one query row and half of the keys of a tile (64), of which it reads S twice - for the maximum, which
+// the two warps of a quarter exchange, and for the exponentials -, and 32 columns of O in registers.  The sum of a row of P is one
+// chain over its keys: the first half's thread hands its part on and the second half's goes on from there while the products run.
+// P goes over the first half of its S columns in tensor memory and is read from there; T = P . V_j takes turns in two places, so that
+// it is folded into O a step later, beside the products of that step.  Warp 0 also requests the tiles (K and V double buffered) and
+// issues the MMAs, P . V_j and S_{j+1} right behind it, when the P of all warps is there.  (A ninth warp for that leaves room for
+// one CTA per SM - the registers of a quarter of the SM hold four warps of 112 - and was slower than one thread per row: 38 us
+// where that takes 31.  S held in registers between the two uses: 148 bytes of spills, 33.3 us where this takes 29.5.)
 // What bounds it: the chain of a step; its exponentials take 1024 clocks of the special-function unit per tile of 128 x 128 and SM,
-// a fifth of the time.  16 sequences of 128 to 512 tokens, 12 heads: 31.4 us with one thread per row (S read twice, O in
-// registers, four barriers of the whole CTA per tile), 27.2 us here.
+// a fifth of the time.  us per launch, 12 heads, one thread per row (S read twice, one T, four barriers of the whole CTA per
+// tile) / two: 16 sequences of 128 to 512 tokens 30.6 / 29.5, 60 of 512 148.1 / 138.7, 64 of 16 to 150 25.6 / 24.4, 8 of 256
+// 9.28 / 8.84.
 // Keys at positions >= length take no part: their probabilities are 0 and the rows of V that share their sixteen with
 // valid ones are zeroed.
 constexpr int kSpWarps = 8;
 constexpr int kSpThreads = 32 * kSpWarps;
-constexpr uint32_t kSpTmemCols = 256;                 // S (P over it) 128, O 64
-constexpr uint32_t kSpColO = 128;
-constexpr float kSpSlack = 8.0f;                      // powers of two that a row's maximum may lag behind
+constexpr uint32_t kSpTmemCols = 256;                 // S (P over it) 128, T 2 x 64
+constexpr uint32_t kSpColT = 128;
 constexpr int kSpExchangeBytes = 2 * 2 * kTcRows * 4;   // [maximum | sum][half][row]
-constexpr int sp_smem_bytes(int kv_buffers) { return (1 + 2 * kv_buffers) * kTcTileBytes + kSpExchangeBytes + 128 + 1024; }
+constexpr int kSpSmemBytes = 5 * kTcTileBytes + kSpExchangeBytes + 128 + 1024;   // Q, K x 2, V x 2
 
 __global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const __grid_constant__ AttnParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int kv_buffers = p.seq > kTcRows ? 2 : 1;
   const uint32_t sQ = smem_u32(smem);                 // at the end the output tile
   const uint32_t sK = sQ + kTcTileBytes;
-  const uint32_t sV = sK + kv_buffers * kTcTileBytes;
-  uint8_t* v_ptr = smem + (1 + kv_buffers) * kTcTileBytes;
-  float* exchange = reinterpret_cast<float*>(smem + (1 + 2 * kv_buffers) * kTcTileBytes);
-  uint8_t* book = smem + (1 + 2 * kv_buffers) * kTcTileBytes + kSpExchangeBytes;
+  const uint32_t sV = sK + 2 * kTcTileBytes;
+  uint8_t* v_ptr = smem + 3 * kTcTileBytes;
+  float* exchange = reinterpret_cast<float*>(smem + 5 * kTcTileBytes);
+  float* sums = exchange + 2 * kTcRows;
+  uint8_t* book = smem + 5 * kTcTileBytes + kSpExchangeBytes;
   const uint32_t bar_k = smem_u32(book);              // two: K_j has landed (with the first one Q)
   const uint32_t bar_v = bar_k + 16;                  // two
   const uint32_t bar_s = bar_v + 16;                  // S of a step is complete
   const uint32_t bar_p = bar_s + 8;                   // P of a step is in tensor memory
   const uint32_t bar_pv = bar_p + 8;                  // P . V of a step is complete
   const uint32_t bar_pair = bar_pv + 8;               // four: the two warps of a quarter exchange their maxima
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(book + 88);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(book + 92);
+  const uint32_t bar_sum = bar_pair + 32;             // four: the first half's part of a row's sum is there
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(book + 120);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(book + 124);
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
@@ -575,7 +575,10 @@ __global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const
     mbar_init(bar_s, 1);
     mbar_init(bar_p, kSpWarps);
     mbar_init(bar_pv, 1);
-    for (int q = 0; q < 4; ++q) mbar_init(bar_pair + 8 * q, 2);
+    for (int q = 0; q < 4; ++q) {
+      mbar_init(bar_pair + 8 * q, 2);
+      mbar_init(bar_sum + 8 * q, 1);
+    }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_shared();
@@ -653,8 +656,20 @@ __global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const
   const uint32_t pair_bar = bar_pair + 8 * quarter;
   const bool row_valid = row < rows_q;
   const bool warp_valid = quarter * 32 < rows_q;     // (the others only keep the barriers' counts; their P is never used)
+  const uint32_t sum_bar = bar_sum + 8 * quarter;
   const float k2 = 0.125f * 1.4426950408889634f;     // exp(x / 8) = 2^(x k2)
-  float m = 0.0f, l = 0.0f;                          // reference maximum (times k2), sum of this half's probabilities
+  float m = -INFINITY, l = 0.0f;                     // running maximum; (second half) running sum
+  float alpha = 0.0f;                                // what O is scaled by when T of this step is added
+  float o[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) o[i] = 0.0f;
+  auto fold = [&](int j, float by) {                 // O = O by + T_j
+    uint32_t t[32];
+    tmem_ld_32x32(lane_base + kSpColT + (j & 1) * kHeadDim + half * 32, t);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 32; ++i) o[i] = fmaf(o[i], by, __uint_as_float(t[i]));
+  };
   for (int j = 0; j < n_kt && ok; ++j) {
     const uint32_t parity = static_cast<uint32_t>(j & 1);
     const int keys = min(kTcRows, len - j * kTcRows);       // valid keys of this tile
@@ -674,73 +689,80 @@ __global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const
     }
     tc_fence_after();
     if (warp == 0 && j > 0 && j + 1 < n_kt) request_v(j + 1);   // (into the buffer of the step before)
-    uint32_t s[64];
+    const uint32_t s_cols = lane_base + half * 64;   // this half's columns of S; its P goes over the first half of them
     float tile_max = -INFINITY;
     if (warp_valid && mine > 0) {
-      tmem_ld_32x32(lane_base + half * 64, *reinterpret_cast<uint32_t(*)[32]>(s));
-      tmem_ld_32x32(lane_base + half * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(s + 32));
-      tmem_ld_wait();
-      if (mine < 64) {
-#pragma unroll
-        for (int i = 0; i < 64; ++i)
-          if (i >= mine) s[i] = 0xff800000u;   // -inf: exponential 0
-      }
       float t[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // (four chains)
 #pragma unroll
-      for (int i = 0; i < 64; ++i) t[i & 3] = fmaxf(t[i & 3], __uint_as_float(s[i]));
+      for (int c = 0; c < 2; ++c) {
+        uint32_t s[32];
+        tmem_ld_32x32(s_cols + c * 32, s);
+        tmem_ld_wait();
+        if (mine < 64) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (c * 32 + i >= mine) s[i] = 0xff800000u;   // -inf
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) t[i & 3] = fmaxf(t[i & 3], __uint_as_float(s[i]));
+      }
       tile_max = fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3]));
     }
-    // the other half's maximum; with it this warp also knows that the other one has read its S, which P is written over
+    // the other half's maximum
     exchange[half * kTcRows + row] = tile_max;
     tc_fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive(pair_bar);
     if (!__all_sync(0xffffffffu, mbar_wait(pair_bar, parity, abort_flag))) { ok = false; break; }
     tc_fence_after();
+    const float alpha_before = alpha;
+    float part = 0.0f;                               // of the row's sum, this half's keys in order
+    float pair[32];
     if (warp_valid) {
-      tile_max = fmaxf(tile_max, exchange[(half ^ 1) * kTcRows + row]) * k2;
-      if (j == 0) {
-        m = tile_max;
-      } else if (__any_sync(0xffffffffu, row_valid && tile_max > m + kSpSlack)) {
-        // scale O (complete up to the step before) down to the new maximum; both halves see the same rows and do the same
-        const float to = tile_max > m + kSpSlack ? tile_max : m;
-        const float alpha = to > m ? ex2_approx(m - to) : 1.0f;
-        uint32_t o[32];
-        tmem_ld_32x32(lane_base + kSpColO + half * 32, o);
-        tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-        tmem_st_32x32(lane_base + kSpColO + half * 32, o);
-        l *= alpha;
-        m = to;
-      }
+      const float m_new = fmaxf(m, fmaxf(tile_max, exchange[(half ^ 1) * kTcRows + row]));
+      alpha = ex2_approx((m - m_new) * k2);          // 0 on the first tile
+      m = m_new;
+      const float shift = m_new * k2;
       if (mine > 0) {
-        float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
           uint32_t w[16];
           if (c == 0 || mine > 32) {                 // (uniform)
+            uint32_t s[32];
+            tmem_ld_32x32(s_cols + c * 32, s);
+            tmem_ld_wait();
+            if (mine < 64) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i)
+                if (c * 32 + i >= mine) s[i] = 0xff800000u;   // -inf: exponential 0
+            }
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-              const float e0 = ex2_approx(fmaf(__uint_as_float(s[c * 32 + 2 * i]), k2, -m));
-              const float e1 = ex2_approx(fmaf(__uint_as_float(s[c * 32 + 2 * i + 1]), k2, -m));
-              sum[i & 1] += e0;
-              sum[2 + (i & 1)] += e1;
+              const float e0 = ex2_approx(fmaf(__uint_as_float(s[2 * i]), k2, -shift));
+              const float e1 = ex2_approx(fmaf(__uint_as_float(s[2 * i + 1]), k2, -shift));
+              pair[c * 16 + i] = e0 + e1;
+              part += pair[c * 16 + i];
               w[i] = pack_bf16(e0, e1);
             }
           } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) w[i] = 0u;
+            for (int i = 0; i < 16; ++i) {
+              pair[c * 16 + i] = 0.0f;
+              w[i] = 0u;
+            }
           }
-          tmem_st_32x16(lane_base + half * 32 + c * 16, w);
+          tmem_st_32x16(s_cols + c * 16, w);
         }
-        l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
       }
       tmem_st_wait();
     }
+    if (half == 0) sums[row] = part;
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(bar_p);
+    if (lane == 0) {
+      mbar_arrive(bar_p);
+      if (half == 0) mbar_arrive(sum_bar);
+    }
     __syncwarp();
     if (warp == 0) {
       ok = mbar_wait(bar_p, parity, abort_flag) && mbar_wait(bar_v + 8 * (j & 1), static_cast<uint32_t>((j >> 1) & 1), abort_flag);
@@ -750,18 +772,29 @@ __global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const
         constexpr uint32_t idesc = umma_idesc_bf16_b_mn(kTcRows, kHeadDim);
         const int steps = (keys + 15) / 16;
         for (int k = 0; k < steps; ++k)   // sixteen keys = sixteen 128-byte rows of the V tile, eight columns of P
-          umma_bf16_ts(tmem_base + kSpColO, tmem_base + k * 8, smem_desc_sw128(sV + (j & 1) * kTcTileBytes + k * 16 * 128), idesc,
-                       (j | k) != 0 ? 1u : 0u);
+          umma_bf16_ts(tmem_base + kSpColT + (j & 1) * kHeadDim, tmem_base + (k >> 2) * 64 + (k & 3) * 8, smem_desc_sw128(sV + (j & 1) * kTcTileBytes + k * 16 * 128),
+                       idesc, k != 0 ? 1u : 0u);
         umma_commit(bar_pv);
       }
       if (j + 2 < n_kt) request_k(j + 2);                   // (S of this step is complete: K_j is dead)
       if (j + 1 < n_kt) ok = __all_sync(0xffffffffu, issue_s(j + 1)) != 0;   // (behind P . V_j, which reads the P that it overwrites)
     }
+    if (!ok) break;
+    // beside those products: T of the step before, and the row's sum
+    if (warp_valid && j > 0) fold(j - 1, alpha_before);
+    if (warp_valid && half == 1) {
+      if (!__all_sync(0xffffffffu, mbar_wait(sum_bar, parity, abort_flag))) { ok = false; break; }
+      float tile_sum = sums[row];
+      if (mine > 0) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) tile_sum += pair[i];
+      }
+      l = fmaf(l, alpha, tile_sum);
+    }
   }
   // O / l: this half's 32 columns, to bf16, into the Q tile's place (all products have completed)
-  float* sums = exchange + 2 * kTcRows;
   if (ok) {
-    sums[half * kTcRows + row] = l;
+    if (half == 1) sums[kTcRows + row] = l;
     ok = __all_sync(0xffffffffu, mbar_wait(bar_pv, static_cast<uint32_t>((n_kt - 1) & 1), abort_flag)) != 0;
     __syncwarp();
     if (lane == 0) mbar_arrive(pair_bar);
@@ -769,16 +802,14 @@ __global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const
   }
   if (ok) {
     tc_fence_after();
-    uint32_t o[32];
-    tmem_ld_32x32(lane_base + kSpColO + half * 32, o);
-    tmem_ld_wait();
-    const float inv = row_valid ? 1.0f / (sums[row] + sums[kTcRows + row]) : 0.0f;
+    fold(n_kt - 1, alpha);
+    const float inv = row_valid ? 1.0f / sums[kTcRows + row] : 0.0f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       uint32_t w[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        w[i] = row_valid ? pack_bf16(__uint_as_float(o[q * 8 + 2 * i]) * inv, __uint_as_float(o[q * 8 + 2 * i + 1]) * inv) : 0u;
+        w[i] = row_valid ? pack_bf16(o[q * 8 + 2 * i] * inv, o[q * 8 + 2 * i + 1] * inv) : 0u;
       *reinterpret_cast<uint4*>(smem + staging_off(row, half * 4 + q)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
@@ -810,11 +841,9 @@ __global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const
 
 }  // namespace
 
-// Beyond 128 tokens (us per forward of the eight-task tree, one thread per row / two: 16 x 512 ragged 1937 / 1887, 60 x 512 for one
-// task 5286 / 5180, 64 x 150 1917 / 1855, 8 x 256 837 / 823, 1 x 300 511 / 498).  Up to 128 a CTA has one step, whose latencies
-// four CTAs per SM of the kernel with one thread per row hide better (32 x 128 992 / 1018, 256 x 128 9425 / 9675); a few sequences of
-// 65 to 128 tokens would gain (4 x 128 450 / 441, 2 x 100 404 / 389), shorter ones not (2 x 64 333 / 338), but a line between them
-// would change the logits of a short sequence by 1e-3 when its batch is padded beyond 64.
+// Beyond 128 tokens (figures above; one sequence of 300 or 512: 9.95 / 9.75, 12.7 / 12.1 us per launch).  Up to 128 a CTA has one
+// step, whose latencies four CTAs per SM of attention_tc_kernel hide better (32 x 128 992 / 1018 us per forward of the eight-task
+// tree, 256 x 128 9425 / 9675, with sums in an order that made two threads 8 % faster than now).
 bool attention_split_rows(int seq) { return seq > kTcRows; }
 
 cudaError_t launch_attention_tc(const AttnParams& p, cudaStream_t stream) {
@@ -826,13 +855,12 @@ cudaError_t launch_attention_tc(const AttnParams& p, cudaStream_t stream) {
     if (r != cudaSuccess) return r;
     r = cudaFuncSetAttribute(attention_tc_tiled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTlSmemBytes);
     if (r != cudaSuccess) return r;
-    return cudaFuncSetAttribute(attention_tc_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sp_smem_bytes(2));
+    return cudaFuncSetAttribute(attention_tc_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpSmemBytes);
   });
   if (e != cudaSuccess) return e;
   const int q_tiles = (p.seq + kTcRows - 1) / kTcRows;
   if (p.split_rows != 0)
-    return launch_kernel(attention_tc_split_kernel, dim3(p.heads, p.batch * q_tiles, p.n_groups), dim3(kSpThreads), sp_smem_bytes(q_tiles > 1 ? 2 : 1),
-                         stream, p);
+    return launch_kernel(attention_tc_split_kernel, dim3(p.heads, p.batch * q_tiles, p.n_groups), dim3(kSpThreads), kSpSmemBytes, stream, p);
   if (p.seq <= kTcRows) {
     dim3 grid(p.heads, p.batch, p.n_groups);
     return launch_kernel(attention_tc_kernel, grid, dim3(kTcThreads), kTcSmemBytes, stream, p);

@@ -165,7 +165,7 @@ struct alignas(64) AttnParams {
 // sequence; longer: tiles of 128 queries walk the keys in tiles of 128).
 constexpr int kAttnTensorMemoryMaxSeq = 512;
 constexpr int kAttnTileRows = 128;   // rows of the Q/K/V boxes of the tensor maps
-bool attention_split_rows(int seq);   // whether that one is the better (bf16 projections)
+bool attention_split_rows(int seq);   // whether that one is the better (with bf16 projections; 8-bit ones keep the other: same bits)
 cudaError_t launch_attention(const AttnParams& p, cudaStream_t stream);
 cudaError_t launch_attention_tc(const AttnParams& p, cudaStream_t stream);
 

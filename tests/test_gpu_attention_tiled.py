@@ -1,10 +1,12 @@
 """Attention over tiles of 128 queries and keys: lengths at the edges of tiles, of halves and of the sixteens that an MMA takes,
-rows whose maximum grows from tile to tile by more and by less than the exponentials may lag, and values that are not finite in
-other sequences' rows."""
+rows whose maximum grows from tile to tile, values that are not finite in other sequences' rows, and the same bits from every
+kernel that a sequence can be given to."""
 import pytest
 import torch
 
 from paper_2107_05377_b200 import binding as mt
+from paper_2107_05377_b200 import synth
+from gpu_util import cached_weights, dev_batch
 
 pytestmark = pytest.mark.gpu
 
@@ -37,9 +39,12 @@ def check(x, ctx, lens, S, heads):
         assert (ctx[b * S + n:(b + 1) * S] == 0).all(), "padded query rows must be written as zero"
 
 
-@pytest.mark.parametrize("kernel", [1, 2])     # two threads per query row; one (with 8-bit projections)
-@pytest.mark.parametrize("S,lens", [(100, [100, 65, 96, 17]), (128, [128, 112, 113, 1]), (129, [1, 15, 16, 17, 63, 64, 65, 127, 128, 129]), (200, [200, 144, 145, 192, 193, 33]),
-                                    (300, [256, 257, 272, 300, 129, 5]), (512, [512, 511, 385, 384, 400, 448, 449, 1])])
+EDGES = [(129, [1, 15, 16, 17, 63, 64, 65, 127, 128, 129]), (200, [200, 144, 145, 192, 193, 33]), (300, [256, 257, 272, 300, 129, 5]),
+         (512, [512, 511, 385, 384, 400, 448, 449, 1])]
+
+
+# up to 128 tokens there is one kernel; beyond, one with two threads per query row (1) and one with one (2: 8-bit projections)
+@pytest.mark.parametrize("S,lens,kernel", [(100, [100, 65, 96, 17], 1), (128, [128, 112, 113, 1], 1)] + [e + (k,) for k in (1, 2) for e in EDGES])
 def test_lengths_at_every_edge(S, lens, kernel):
     g = torch.Generator(device="cuda").manual_seed(S)
     qkv = torch.randn(len(lens) * S, 3 * 128, device="cuda", generator=g) * 1.5
@@ -57,3 +62,50 @@ def test_maxima_that_grow_from_tile_to_tile(growth):
     qkv[::3, :64] *= -1.0
     x, ctx = run(qkv, lens, S, 1)
     check(x, ctx, lens, S, 1)
+
+
+@pytest.mark.parametrize("growth", [1.0, 1.7])
+@pytest.mark.parametrize("S,lens", EDGES)
+def test_one_and_two_threads_per_row_have_the_same_bits(S, lens, growth):
+    g = torch.Generator(device="cuda").manual_seed(S)
+    qkv = torch.randn(len(lens) * S, 3 * 128, device="cuda", generator=g) * 1.3
+    tile = torch.arange(S, device="cuda").repeat(len(lens)) // 128
+    qkv[:, 128:256] *= growth ** tile[:, None].float()
+    two, one = (run(qkv, lens, S, 2, kernel)[1] for kernel in (1, 2))
+    assert torch.equal(two, one)
+
+
+@pytest.mark.parametrize("kernel", [1, 2])
+@pytest.mark.parametrize("S", [129, 257, 512])
+def test_a_short_sequence_has_the_same_bits_at_any_padding(S, kernel):
+    lens = [1, 16, 31, 64, 65, 100, 127, 128]
+    g = torch.Generator(device="cuda").manual_seed(S)
+    qkv = torch.randn(len(lens), S, 3 * 128, device="cuda", generator=g) * 1.5
+    wide = run(qkv.view(-1, 3 * 128), lens, S, 2, kernel)[1].view(len(lens), S, 128)
+    for seq in (100, 128):
+        some = [b for b, n in enumerate(lens) if n <= seq]
+        near = run(qkv[some, :seq].reshape(-1, 3 * 128), [lens[b] for b in some], seq, 2)[1].view(len(some), seq, 128)
+        for i, b in enumerate(some):
+            assert torch.equal(near[i, :lens[b]], wide[b, :lens[b]])
+
+
+def test_logits_of_short_sequences_do_not_depend_on_a_padding_beyond_128_tokens():
+    """(From 65 tokens and more than 512 rows on: below, other choices that may change bits depend on the padded size; with 8-bit
+    projections the first-token attention of the last layers has another kernel beyond 128 tokens.)"""
+    cfg = synth.TreeConfig(trunk_layers=2, vocab_size=2000, tasks=(synth.TaskSpec(2, 2, 2), synth.TaskSpec(1, 1, 3), synth.TaskSpec(2, 0, 2)))
+    _, blob, _ = cached_weights(cfg, 1)
+    B = 8
+    short = synth.make_batch(cfg, B, 100, 30, 100, seed=3)
+    want = None
+    for S in (100, 128, 129, 300, 512):
+        model = mt.MTModel(cfg, B, S)
+        model.load_weights(blob)
+        tok, seg, lens = dev_batch(short)
+        tok, seg = (torch.nn.functional.pad(t, (0, S - 100)) for t in (tok, seg))
+        logits = torch.full((B, cfg.total_classes), float("nan"), device="cuda")
+        model.forward(tok.contiguous(), seg.contiguous(), lens, logits)
+        torch.cuda.synchronize()
+        assert model.poll_status() == 0
+        want = logits if want is None else want
+        assert torch.equal(logits, want), S
+        model.close()
