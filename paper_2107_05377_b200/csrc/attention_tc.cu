@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(kSpThreads, 2) attention_tc_split_kernel(const
       request_k(1);
       request_v(1);
     }
-    ok = issue_s(0);
+    ok = __all_sync(0xffffffffu, issue_s(0)) != 0;
   }
 
   // ------------------------------ softmax -----------------------------------
