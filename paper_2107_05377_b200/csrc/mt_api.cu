@@ -12,6 +12,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -2162,6 +2163,12 @@ int mt_kernel_linear_layernorm(const void* d_x, const void* d_w, const void* d_b
                                           d_status, stream);
 }
 
+static bool misaligned16(std::initializer_list<const void*> pointers) {
+  uintptr_t bits = 0;
+  for (const void* p : pointers) bits |= reinterpret_cast<uintptr_t>(p);
+  return bits % 16 != 0;
+}
+
 static int linear_layernorm_kind(int kind, const void* d_x, const void* d_w, const void* d_bias, const void* d_residual, const void* d_gamma,
                                  const void* d_beta, void* d_y, void* d_y_f32, int32_t M, int32_t N, int32_t K, float eps, int32_t low,
                                  uint32_t* d_status, void* stream) {
@@ -2196,6 +2203,8 @@ int mt_kernel_linear_layernorm_low(const void* d_x, const void* d_w, const void*
                                    const void* d_gamma, const void* d_beta, void* d_y, void* d_y_f32, int32_t M,
                                    int32_t N, int32_t K, float eps, int32_t tile_rows, uint32_t* d_status, void* stream) {
   if ((tile_rows != 16 && tile_rows != 32 && tile_rows != 64) || K % 128 != 0) return MT_ERR_INVALID_ARG;
+  // these tiles reach them by pointer, sixteen bytes at a time, and not through tensor maps, whose encoding looks at the address
+  if (misaligned16({d_residual, d_gamma, d_beta, d_y, d_y_f32})) return MT_ERR_INVALID_ARG;
   return linear_layernorm_kind(3, d_x, d_w, d_bias, d_residual, d_gamma, d_beta, d_y, d_y_f32, M, N, K, eps, tile_rows, d_status, stream);
 }
 

@@ -231,3 +231,11 @@ def test_blob_sizes_match_the_generator(lib):
     with pytest.raises(binding.MTError):
         m.set_option("nonsense", 1)
     m.close()
+
+
+@pytest.mark.parametrize("which", ["residual", "gamma", "beta", "y", "y_f32"])
+def test_low_tiles_refuse_what_they_cannot_read_in_sixteen_bytes(lib, which):
+    """Looked at on the host, before anything else: no kernel runs on these addresses."""
+    names = ["x", "w", "bias", "residual", "gamma", "beta", "y", "y_f32"]
+    at = [(i + 1 << 20) + (8 if n == which else 0) for i, n in enumerate(names)]
+    assert lib.mt_kernel_linear_layernorm_low(*at, 16, 768, 768, 1e-12, 16, None, None) == -1
