@@ -373,6 +373,14 @@ int mt_debug_wait_probe(uint64_t limit_ns, int32_t arrive, uint32_t* d_status, u
 int mt_kernel_linear_partial(const void* d_x, const void* d_w, void* d_part, int32_t M, int32_t N, int32_t K,
                              int32_t k_splits, int32_t split_pitch, uint32_t* d_status, void* stream);
 
+/* The linear maps above on tiles of tile_rows = 16, 32 or 64 rows and 128 columns, as launches of few rows take them: epilogues 0, 1
+ * and 2 of mt_kernel_linear, 3: tanh(+bias), Y fp32 (the pooler), 4: partial sums as mt_kernel_linear_partial has them (d_bias
+ * unused; k_splits is 1 and split_pitch unused otherwise).  K % (128 * k_splits) == 0.  d_rows (device, may be NULL): rows in use,
+ * at most M; the others are not written.  Identical bits. */
+int mt_kernel_linear_low(const void* d_x, const void* d_w, const void* d_bias, const void* d_residual, void* d_y, int32_t M,
+                         int32_t N, int32_t K, int32_t epilogue, int32_t tile_rows, int32_t k_splits, int32_t split_pitch,
+                         const int32_t* d_rows, uint32_t* d_status, void* stream);
+
 /* Y = LN(X[M,K] . W[N,K]^T + bias[N] + residual[M,N]) * gamma[N] + beta[N] in one launch: the residual
  * sub-layer followed by LayerNorm, as the encoder layer has it twice (after attention, after the FFN).
  * X, W, bias, gamma, beta bf16; residual fp32; Y is written twice, d_y bf16 [M,N] and d_y_f32 fp32 [M,N].

@@ -65,6 +65,7 @@ SIGNATURES = {
     "mt_kernel_linear_layernorm": (C.c_int, [_P, _P, _P, _P, _P, _P, _P, _P, _I32, _I32, _I32, C.c_float, _P, _P]),
     "mt_kernel_linear_layernorm_tiles": (C.c_int, [_P, _P, _P, _P, _P, _P, _P, _P, _I32, _I32, _I32, C.c_float, _I32, _P, _P]),
     "mt_kernel_linear_layernorm_low": (C.c_int, [_P, _P, _P, _P, _P, _P, _P, _P, _I32, _I32, _I32, C.c_float, _I32, _P, _P]),
+    "mt_kernel_linear_low": (C.c_int, [_P, _P, _P, _P, _P, _I32, _I32, _I32, _I32, _I32, _I32, _I32, _P, _P, _P]),
     "mt_kernel_attention": (C.c_int, [_P, _P, _P, _I32, _I32, _I32, _I32, _P, _P]),
     "mt_kernel_layernorm": (C.c_int, [_P, _P, _P, _P, _P, _I32, _I32, C.c_float, _P]),
     "mt_kernel_linear_partial": (C.c_int, [_P, _P, _P, _I32, _I32, _I32, _I32, _I32, _P, _P]),
@@ -160,6 +161,14 @@ def mt_kernel_linear_layernorm_low(x, w, bias, residual, gamma, beta, y, y_f32, 
     _check(lib().mt_kernel_linear_layernorm_low(_ptr(x), _ptr(w), _ptr(bias), _ptr(residual), _ptr(gamma), _ptr(beta),
                                                 _ptr(y), _ptr(y_f32), M, N, K, eps, tile_rows, _ptr(status),
                                                 _stream(stream)), "mt_kernel_linear_layernorm_low")
+
+
+def mt_kernel_linear_low(x, w, bias, residual, y, epilogue: int, tile_rows: int, k_splits: int = 1, split_pitch: int = 0, rows=None,
+                         status=None, stream=None) -> None:
+    M, K = x.shape
+    N = w.shape[0]
+    _check(lib().mt_kernel_linear_low(_ptr(x), _ptr(w), _ptr(bias), _ptr(residual), _ptr(y), M, N, K, epilogue, tile_rows, k_splits,
+                                      split_pitch, _ptr(rows), _ptr(status), _stream(stream)), "mt_kernel_linear_low")
 
 
 def mt_kernel_attention(qkv, lengths, ctx, batch: int, seq: int, heads: int, stream=None,

@@ -2077,6 +2077,12 @@ int mt_debug_copy_hidden(mt_model* m, int32_t task, int32_t layer, void* d_out, 
 
 // ---- single steps ------------------------------------------------------------------------------
 
+static bool misaligned16(std::initializer_list<const void*> pointers) {
+  uintptr_t bits = 0;
+  for (const void* p : pointers) bits |= reinterpret_cast<uintptr_t>(p);
+  return bits % 16 != 0;
+}
+
 void mt_kernel_linear_force_block_n(int32_t block_n) { g_force_block_n = block_n; }
 
 int mt_kernel_linear(const void* d_x, const void* d_w, const void* d_bias, const void* d_residual, void* d_y, int32_t M,
@@ -2121,6 +2127,29 @@ int mt_kernel_linear_partial(const void* d_x, const void* d_w, void* d_part, int
   return launch_gemm(p, kEpiPartialF32, sms, as_stream(stream)) == cudaSuccess ? MT_OK : MT_ERR_CUDA;
 }
 
+int mt_kernel_linear_low(const void* d_x, const void* d_w, const void* d_bias, const void* d_residual, void* d_y, int32_t M,
+                         int32_t N, int32_t K, int32_t epilogue, int32_t tile_rows, int32_t k_splits, int32_t split_pitch,
+                         const int32_t* d_rows, uint32_t* d_status, void* stream) {
+  const bool partial = epilogue == kEpiPartialF32;
+  if (d_x == nullptr || d_w == nullptr || d_y == nullptr || (d_bias == nullptr && !partial) || M < 1 || N < 128 || N % 128 != 0 ||
+      epilogue < kEpiBias || epilogue > kEpiPartialF32 || (epilogue == kEpiBiasResidual && d_residual == nullptr) ||
+      (tile_rows != 16 && tile_rows != 32 && tile_rows != 64) || k_splits < 1 || k_splits > 64 || (k_splits > 1 && !partial) ||
+      K < 128 || K % (128 * k_splits) != 0 || (partial && (split_pitch < M || split_pitch % 128 != 0)) ||
+      misaligned16({d_bias, d_residual, d_y}))
+    return MT_ERR_INVALID_ARG;
+  GemmParams p;
+  memset(&p, 0, sizeof(p));
+  p.n_groups = 1; p.M = M; p.N = N; p.K = K; p.status = d_status;
+  p.block_n = 128;
+  p.turned = tile_rows;
+  p.k_splits = k_splits; p.split_pitch = split_pitch;
+  p.m_valid = d_rows;
+  if (set_gemm_group(&p, 0, epilogue, d_x, d_w, static_cast<const bf16*>(d_bias), static_cast<const float*>(d_residual), d_y) !=
+      cudaSuccess)
+    return MT_ERR_CUDA;
+  return launch_gemm(p, epilogue, 0, as_stream(stream)) == cudaSuccess ? MT_OK : MT_ERR_CUDA;   // (a CTA per tile, whatever the SMs)
+}
+
 int mt_kernel_quantize_rows(const void* d_x, void* d_q, float* d_scale, int32_t rows, int32_t cols, void* stream) {
   if (d_x == nullptr || d_q == nullptr || d_scale == nullptr || rows < 1 || cols < 256 || cols % 256 != 0)
     return MT_ERR_INVALID_ARG;
@@ -2161,12 +2190,6 @@ int mt_kernel_linear_layernorm(const void* d_x, const void* d_w, const void* d_b
                                int32_t K, float eps, uint32_t* d_status, void* stream) {
   return mt_kernel_linear_layernorm_tiles(d_x, d_w, d_bias, d_residual, d_gamma, d_beta, d_y, d_y_f32, M, N, K, eps, 128,
                                           d_status, stream);
-}
-
-static bool misaligned16(std::initializer_list<const void*> pointers) {
-  uintptr_t bits = 0;
-  for (const void* p : pointers) bits |= reinterpret_cast<uintptr_t>(p);
-  return bits % 16 != 0;
 }
 
 static int linear_layernorm_kind(int kind, const void* d_x, const void* d_w, const void* d_bias, const void* d_residual, const void* d_gamma,
