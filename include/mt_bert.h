@@ -225,6 +225,10 @@ int mt_plan_launches(const mt_model* m, uint64_t task_mask, int32_t* n_launches)
  * Returns the count, or MT_ERR_INVALID_ARG for a null model. */
 int mt_plan_cache_size(const mt_model* m);
 
+/* Forwards that have run as a CUDA graph since mt_create (see mt_forward; host side, no device access), or MT_ERR_INVALID_ARG for
+ * a null model. */
+int64_t mt_replayed_forwards(const mt_model* m);
+
 /* Options.  key "max_groups" (1..8): upper bound on layers fused into one grouped launch;
  * key "debug_capture" (0/1): keep a copy of every layer output for mt_debug_copy_hidden (changes
  * mt_workspace_bytes); both must be set before mt_bind_memory.  key "profile" (0/1): see

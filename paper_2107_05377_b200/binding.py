@@ -53,6 +53,7 @@ SIGNATURES = {
     "mt_poll_status": (C.c_int, [_P, _P, C.POINTER(C.c_uint32)]),
     "mt_plan_summary": (C.c_int, [_P, _U64, C.POINTER(_I32), C.POINTER(_I32), C.POINTER(_I32), C.POINTER(_I32)]),
     "mt_plan_launches": (C.c_int, [_P, _U64, C.POINTER(_I32)]),
+    "mt_replayed_forwards": (C.c_int64, [_P]),
     "mt_plan_cache_size": (C.c_int, [_P]),
     "mt_set_option": (C.c_int, [_P, C.c_char_p, C.c_int64]),
     "mt_debug_copy_hidden": (C.c_int, [_P, _I32, _I32, _P, _P]),
@@ -303,6 +304,9 @@ class MTModel:
 
     def plan_cache_size(self) -> int:
         return lib().mt_plan_cache_size(self.handle)
+
+    def replayed_forwards(self) -> int:
+        return lib().mt_replayed_forwards(self.handle)
 
     # -- device -------------------------------------------------------------
     def bind(self, device: str = "cuda:0") -> None:

@@ -340,6 +340,7 @@ struct mt_model {
   cudaStream_t side_stream;
   bool replay;                  // option "replay": forwards of a plan in frequent use run as a CUDA graph
   cudaStream_t replay_stream;   // where a forward is recorded as a graph
+  int64_t replayed;             // forwards that ran as one
   cudaEvent_t ev_fork, ev_join;
   bool fp8;          // Q/K/V, FFN-up and FFN-down projections on E4M3 operands (set before mt_bind_memory)
   bool pool_gemm;    // the pooler of tasks with a compact final state runs as a grouped GEMM on the tensor cores
@@ -1332,6 +1333,7 @@ int mt_create(const mt_trunk_config* trunk, const mt_task_config* tasks, int32_t
   m->overlap_cls = true;
   m->side_stream = m->replay_stream = nullptr;
   m->replay = true;
+  m->replayed = 0;
   m->ev_fork = m->ev_join = nullptr;
   m->fused_ln = 2;
   m->fused_ln_max_groups = kMaxGroups;
@@ -1662,6 +1664,8 @@ int mt_plan_summary(const mt_model* m, uint64_t task_mask, int32_t* n_layers, in
 
 int mt_plan_cache_size(const mt_model* m) { return m == nullptr ? MT_ERR_INVALID_ARG : static_cast<int>(m->plans.size()); }
 
+int64_t mt_replayed_forwards(const mt_model* m) { return m == nullptr ? MT_ERR_INVALID_ARG : m->replayed; }
+
 int mt_plan_launches(const mt_model* m, uint64_t task_mask, int32_t* n_launches) {
   if (m == nullptr || n_launches == nullptr) return MT_ERR_INVALID_ARG;
   Schedule s;
@@ -1977,7 +1981,9 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
     plan.replay->refused = true;
     replay = false;
   }
-  if (!replay) {
+  if (replay) {
+    ++m->replayed;
+  } else {
     const int rc = launch_plan(m, plan, call, batch, seq, task_events, stream, nullptr);
     if (rc != MT_OK) return rc;
   }

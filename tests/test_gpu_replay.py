@@ -1,5 +1,7 @@
 """Forwards of a plan in frequent use run as a CUDA graph (option "replay"): the same bits as launched kernels, with the pointers of
-each call, whatever comes between the calls."""
+each call, whatever comes between the calls - and they do run as one, from the call on that the plan has been launched often enough."""
+import ctypes as C
+
 import pytest
 import torch
 
@@ -8,6 +10,8 @@ from paper_2107_05377_b200 import synth
 from gpu_util import cached_weights, dev_batch
 
 pytestmark = pytest.mark.gpu
+
+LAUNCHED = 16     # times that a plan is launched kernel by kernel first
 
 # sequence- and token-level tasks, a task that pools the trunk, first-token attention of both kinds by batch size
 TREE = synth.TreeConfig(trunk_layers=3, vocab_size=2000,
@@ -46,11 +50,13 @@ def test_replayed_and_launched_forwards_have_the_same_bits(B, S):
     inputs = [dev_batch(synth.make_batch(TREE, B, S, 1, S, seed=k)) for k in range(3)]
     want = [call(plain, ids) for ids in inputs]
     other = torch.cuda.Stream()
-    for k in range(48):          # (the graph is built at the 17th call; new output arrays in every call)
+    for k in range(LAUNCHED + 32):   # (new output arrays in every call)
         assert same(call(often, inputs[k % 3], stream=other if k % 5 == 4 else None), want[k % 3]), k
+        assert often.replayed_forwards() == max(0, k + 1 - LAUNCHED)
     # calls in a row, unsynchronised, on buffers that change under the same graph
     outs = [call(often, inputs[k % 3]) for k in range(7)]
     assert all(same(outs[k], want[k % 3]) for k in range(7))
+    assert often.replayed_forwards() == 32 + 7 and plain.replayed_forwards() == 0
     assert often.poll_status() == 0
 
 
@@ -59,15 +65,29 @@ def test_captures_options_and_other_plans_between_replays():
     often, plain = models(B, S)
     ids = dev_batch(synth.make_batch(TREE, B, S, 1, S, seed=5))
     want = call(plain, ids)
-    for _ in range(20):
+    for _ in range(LAUNCHED + 4):
         got = call(often, ids)
-    assert same(got, want)
+    assert same(got, want) and often.replayed_forwards() == 4
     # the caller's own capture records the kernels themselves
     graph, outs = torch.cuda.CUDAGraph(), (torch.zeros_like(want[0]), torch.zeros_like(want[1]))
     with torch.cuda.graph(graph):
         often.forward_tokens(*ids, *outs)
+    assert often.replayed_forwards() == 4
     graph.replay()
-    assert same(outs, want) and same(call(often, ids), want)
+    assert same(outs, want) and same(call(often, ids), want) and often.replayed_forwards() == 5
+    # events of tasks and per-launch timing lie between the launches
+    out = (torch.zeros_like(want[0]), torch.zeros_like(want[1]))
+    events = [torch.cuda.Event() for _ in TREE.tasks]
+    for e in events:
+        e.record()
+    torch.cuda.synchronize()
+    rc = mt.lib().mt_forward_tokens(often.handle, *(t.data_ptr() for t in ids), often.full_mask(), B, S, *(t.data_ptr() for t in out),
+                                    (C.c_void_p * len(events))(*(e.cuda_event for e in events)), None)
+    assert rc == 0 and same(out, want) and often.replayed_forwards() == 5
+    often.set_option("profile", 1)
+    assert same(call(often, ids), want) and often.replayed_forwards() == 5
+    often.set_option("profile", 0)
+    assert same(call(often, ids), want) and often.replayed_forwards() == 6
     # a bad length in a replayed forward is flagged as in a launched one
     bad = ids[2].clone()
     bad[1] = S + 3
@@ -77,9 +97,10 @@ def test_captures_options_and_other_plans_between_replays():
     often.set_option("plan_cache", 1)
     for mask in (1, 2, 1, 15):
         expect = call(plain, ids, mask)
-        for _ in range(18):
+        before = often.replayed_forwards()
+        for _ in range(LAUNCHED + 2):
             got = call(often, ids, mask)
-        assert same(got, expect)
+        assert same(got, expect) and often.replayed_forwards() == before + 2
     often.set_option("overlap_cls", 0)
     assert same(call(often, ids), want)
     often.close()
@@ -93,10 +114,11 @@ def test_host_calls_are_replayed_too():
     model.load_weights(blob)
     batches = [synth.make_batch(cfg, B, S, 1, S, seed=k) for k in range(2)]
     want = []
-    for k in range(40):
+    for k in range(LAUNCHED + 24):
         b = batches[k % 2]
         out = torch.zeros(B, cfg.total_classes).pin_memory()
         model.forward_host(*[torch.from_numpy(a).pin_memory() for a in (b.token_ids, b.segment_ids, b.lengths)], out)
         if k < 2:
             want.append(out)
         assert torch.equal(out, want[k % 2]), k
+    assert model.replayed_forwards() == 24
