@@ -157,6 +157,16 @@ struct ReplayNode {
   cudaGraphNode_t node = nullptr;
   cudaKernelNodeParams launch = {};
 };
+// Building, updating and dropping a graph are calls that a stream capture may forbid, and end, from any thread of the process (the
+// mode of cudaStreamBeginCapture); they touch no stream that is being captured, so this thread asks for leave while it makes them.
+struct CaptureLeave {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CaptureLeave() { ok = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess; }
+  ~CaptureLeave() {
+    if (ok) cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  bool ok;
+};
 // The launches of a plan as a CUDA graph (option "replay").  A forward of a small batch is a chain of some forty to eighty
 // dependent kernels of 3 to 8 us; launched one by one each starts about 0.35 us later than as the node of a graph, whose
 // parameters are on the device already.  us per forward, launched / replayed: 2 x 32 tokens 158 / 149, 1 x 128 387 / 362, 4 x 128
@@ -171,6 +181,8 @@ struct Replay {
   Replay(const Replay&) = delete;
   Replay& operator=(const Replay&) = delete;
   ~Replay() {   // (an executable graph in flight is freed when it has completed)
+    if (exec == nullptr && graph == nullptr) return;
+    const CaptureLeave leave;
     if (exec != nullptr) cudaGraphExecDestroy(exec);
     if (graph != nullptr) cudaGraphDestroy(graph);
   }
@@ -1856,9 +1868,8 @@ static void build_replay(mt_model* m, Plan& plan, const Call& call, int32_t batc
   Replay& r = *plan.replay;
   r.refused = true;
   r.pdl = g_use_pdl;
-  // (captures of other threads go their own way, and nothing here is held against one)
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return;
+  const CaptureLeave leave;
+  if (!leave.ok) return;
   cudaError_t e = cudaStreamBeginCapture(m->replay_stream, cudaStreamCaptureModeRelaxed);
   if (e == cudaSuccess) {
     const std::string before = m->last_error;
@@ -1873,7 +1884,6 @@ static void build_replay(mt_model* m, Plan& plan, const Call& call, int32_t batc
   if (e != cudaSuccess) cudaGetLastError();
   r.call = call;
   r.refused = e != cudaSuccess;
-  cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 // Puts the pointers of this call into the executable graph (launches already enqueued keep theirs).

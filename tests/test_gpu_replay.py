@@ -106,6 +106,38 @@ def test_captures_options_and_other_plans_between_replays():
     often.close()
 
 
+def test_a_callers_capture_outlives_what_becomes_of_graphs_meanwhile():
+    """While a stream is being captured (in the mode that forbids what might disturb it, from every thread), forwards on another
+    stream are made a graph, replayed with new pointers and dropped, and the captured forward itself drops one."""
+    B, S = 3, 40
+    often, plain = models(B, S)
+    inputs = [dev_batch(synth.make_batch(TREE, B, S, 1, S, seed=k)) for k in range(2)]
+    short = dev_batch(synth.make_batch(TREE, B, 25, 1, 25, seed=7))
+    want, want_short = [call(plain, ids) for ids in inputs], call(plain, short)
+    often.set_option("plan_cache", 1)
+    for _ in range(LAUNCHED):
+        call(often, inputs[0])
+    outs = [(torch.zeros_like(want[0][0]), torch.zeros_like(want[0][1])) for _ in range(4)]
+    out_short = [tuple(torch.zeros_like(t) for t in want_short) for _ in range(2)]
+    other, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        plain.forward_tokens(*inputs[0], *outs[3])
+        for k in range(3):
+            often.forward_tokens(*inputs[k % 2], *outs[k], stream=other)
+        assert often.replayed_forwards() == 3
+        often.forward_tokens(*short, *out_short[0], stream=other)
+        for _ in range(LAUNCHED + 1):
+            often.forward_tokens(*inputs[0], *outs[2], stream=other)
+        assert often.replayed_forwards() == 4
+        often.forward_tokens(*short, *out_short[1])     # captured: drops the graph under way
+    torch.cuda.synchronize()
+    assert all(same(outs[k], want[k % 2]) for k in range(3)) and same(out_short[0], want_short)
+    graph.replay()
+    assert same(outs[3], want[0]) and same(out_short[1], want_short)
+    assert often.poll_status() == 0
+
+
 def test_host_calls_are_replayed_too():
     cfg = synth.config_tiny()
     _, blob, _ = cached_weights(cfg, 0)
