@@ -149,8 +149,8 @@ int mt_adopt_weights(mt_model* m, const mt_model* src);
  * never synchronises, never allocates device memory of its own.  The first call for a given
  * (batch, seq, task_mask) builds and caches a launch plan on the host (host memory and tensor-map
  * encoding only; the model's own streams and its two events exist since mt_bind_memory) - make one
- * warm-up call before capturing mt_forward into a CUDA graph.  A plan that has been launched 16 times is
- * made a CUDA graph (0.7 ms, once; the driver keeps its nodes, some kilobytes each) and replayed from then on
+ * warm-up call before capturing mt_forward into a CUDA graph.  A plan that has been launched 32 times is
+ * made a CUDA graph (0.2 to 1 ms of the host, once; the driver keeps its nodes, some kilobytes each) and replayed from then on
  * with the pointers of each call - not while `stream` is being captured, nor with task_events or options
  * "profile" and "debug_capture"; if the graph cannot be built the kernels are launched as before, and option
  * "replay" = 0 never builds one.  Option "profile" creates CUDA events here.

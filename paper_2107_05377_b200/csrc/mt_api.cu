@@ -42,9 +42,11 @@ constexpr size_t split_pitch(size_t rows) { return (rows + 127) / 128 * 128; }
 constexpr int32_t kDownSplits = 4;
 // "Few rows": at most this many per layer (batch 4 x 128 tokens; the first-token tails of batches up to 512).
 constexpr int32_t kSplitRowsMax = 512;
-// A plan is made a graph when it has been launched this often: building one takes 0.7 ms of the host, a
-// replay saves 10 to 40 us.
-constexpr int32_t kReplayAfter = 16;
+// A plan is made a graph when it has been launched this often.  Building one takes the host 0.23 ms (34 launches: 2 x 32 tokens), 0.4
+// to 0.55 (46 to 77) or 1 ms (117), twice that the first time in a process; a replay saves 11 us of a forward of 34 launches, 24 of 67
+// (1 x 128), 33 (32 x 128), 44 of 117.  That is 16 to 36 forwards: a plan that has been launched as often will have cost at
+// most about twice what the better of both ways would have, however soon it falls out of use.
+constexpr int32_t kReplayAfter = 32;
 
 inline size_t pad256(size_t n) { return (n + kAlign - 1) / kAlign * kAlign; }
 

@@ -11,7 +11,7 @@ from gpu_util import cached_weights, dev_batch
 
 pytestmark = pytest.mark.gpu
 
-LAUNCHED = 16     # times that a plan is launched kernel by kernel first
+LAUNCHED = 32     # times that a plan is launched kernel by kernel first
 
 # sequence- and token-level tasks, a task that pools the trunk, first-token attention of both kinds by batch size
 TREE = synth.TreeConfig(trunk_layers=3, vocab_size=2000,
