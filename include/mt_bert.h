@@ -10,8 +10,10 @@
  * the checkpoints into it, mt_forward() evaluates it.
  *
  * Conventions
- *  - All device memory and all streams belong to the caller.  The library allocates only host
- *    metadata.  Pointers named d_* are DEVICE pointers, everything else is a HOST pointer.
+ *  - The device memory that a forward works in belongs to the caller.  The library allocates host metadata; what it
+ *    has the driver create - two streams and two events in mt_bind_memory, events with option "profile", and CUDA
+ *    graphs unless option "replay" is 0 - takes the driver device memory of its own (see mt_forward).
+ *    Pointers named d_* are DEVICE pointers, everything else is a HOST pointer.
  *  - cudaStream_t is passed as a plain `void*` (the value of the stream handle; NULL = default stream).
  *  - Weights and the operands of every matrix product are bf16; accumulation, LayerNorm statistics
  *    and the residual stream (every LayerNorm input and the residual it is added to) are fp32; logits
@@ -149,11 +151,13 @@ int mt_adopt_weights(mt_model* m, const mt_model* src);
  * never synchronises, never allocates device memory of its own.  The first call for a given
  * (batch, seq, task_mask) builds and caches a launch plan on the host (host memory and tensor-map
  * encoding only; the model's own streams and its two events exist since mt_bind_memory) - make one
- * warm-up call before capturing mt_forward into a CUDA graph.  A plan that has been launched 32 times is
- * made a CUDA graph (0.2 to 1 ms of the host, once; the driver keeps its nodes, some kilobytes each) and replayed from then on
- * with the pointers of each call - not while `stream` is being captured, nor with task_events or options
- * "profile" and "debug_capture"; if the graph cannot be built the kernels are launched as before, and option
- * "replay" = 0 never builds one.  Option "profile" creates CUDA events here.
+ * warm-up call before capturing mt_forward into a CUDA graph.  Option "profile" creates CUDA events here.
+ * A plan that has been launched 32 times is made a CUDA graph by the next call (0.2 to 1 ms of the host, once) and
+ * replayed from then on with the pointers of each call - not while `stream` is being captured, nor with task_events
+ * or options "profile" and "debug_capture".  The driver keeps a graph in device memory (some 0.7 MB for 67 launches),
+ * of at most 32 graphs per model, and holds it for later ones when they are dropped.  A caller that has handed out all
+ * device memory, or wants no such call, sets option "replay" to 0: no graph is ever built.  If one cannot be built
+ * the kernels are launched as before.
  * One mt_model serves one caller at a time: the cached plans carry per-call pointers.
  * Errors: INVALID_ARG, SHAPE, NOT_BOUND, NOT_LOADED, CUDA. */
 int mt_forward(mt_model* m, const int32_t* d_token_ids, const int32_t* d_segment_ids,

@@ -47,6 +47,9 @@ constexpr int32_t kSplitRowsMax = 512;
 // (1 x 128), 33 (32 x 128), 44 of 117.  That is 16 to 36 forwards: a plan that has been launched as often will have cost at
 // most about twice what the better of both ways would have, however soon it falls out of use.
 constexpr int32_t kReplayAfter = 32;
+// Graphs of a model at a time, whatever option "plan_cache" says: the driver keeps each of them in device memory, some 0.7 MB of it
+// for 67 launches (62 graphs: 45 MB, kept for the next ones when they are dropped).
+constexpr int32_t kMaxReplays = 32;
 
 inline size_t pad256(size_t n) { return (n + kAlign - 1) / kAlign * kAlign; }
 
@@ -1888,6 +1891,21 @@ static void build_replay(mt_model* m, Plan& plan, const Call& call, int32_t batc
   r.refused = e != cudaSuccess;
 }
 
+// The graph not used for longest goes when there are kMaxReplays; its plan stays.
+static void make_room_for_replay(mt_model* m) {
+  int32_t count = 0;
+  Plan* oldest = nullptr;
+  for (auto& entry : m->plans) {
+    Plan& p = entry.second;
+    if (p.replay == nullptr || p.replay->refused) continue;
+    ++count;
+    if (oldest == nullptr || p.last_use < oldest->last_use) oldest = &p;
+  }
+  if (count < kMaxReplays) return;
+  oldest->replay.reset();
+  oldest->launched = 0;
+}
+
 // Puts the pointers of this call into the executable graph (launches already enqueued keep theirs).
 static cudaError_t set_call(Plan& plan, const Call& call) {
   Replay& r = *plan.replay;
@@ -1983,7 +2001,10 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
       state = cudaStreamCaptureStatusInvalidated;
     }
     replay = state == cudaStreamCaptureStatusNone;
-    if (replay && plan.replay == nullptr && ++plan.launched > kReplayAfter) build_replay(m, plan, call, batch, seq);
+    if (replay && plan.replay == nullptr && ++plan.launched > kReplayAfter) {
+      make_room_for_replay(m);
+      build_replay(m, plan, call, batch, seq);
+    }
     replay = replay && plan.replay != nullptr && !plan.replay->refused && plan.replay->pdl == g_use_pdl;
   } else {
     replay = false;

@@ -138,6 +138,28 @@ def test_a_callers_capture_outlives_what_becomes_of_graphs_meanwhile():
     assert often.poll_status() == 0
 
 
+def test_a_model_has_at_most_32_graphs():
+    cfg = synth.config_tiny()
+    _, blob, _ = cached_weights(cfg, 0)
+    model = mt.MTModel(cfg, 1, 33)
+    model.load_weights(blob)
+    model.set_option("plan_cache", 64)
+    ids = [dev_batch(synth.make_batch(cfg, 1, S, S, S, seed=S)) for S in range(1, 34)]
+    out = torch.zeros(1, cfg.total_classes, device="cuda")
+    for k, one in enumerate(ids):
+        for _ in range(LAUNCHED + 1):
+            model.forward(*one, out)
+        assert model.replayed_forwards() == k + 1
+    assert model.plan_cache_size() == 33
+    # the first one's graph went when the last one's was built, the others are there
+    for k in (1, 32, 0, 2):
+        before = model.replayed_forwards()
+        model.forward(*ids[k], out)
+        assert model.replayed_forwards() == before + (k != 0)
+    torch.cuda.synchronize()
+    assert model.poll_status() == 0
+
+
 def test_host_calls_are_replayed_too():
     cfg = synth.config_tiny()
     _, blob, _ = cached_weights(cfg, 0)
