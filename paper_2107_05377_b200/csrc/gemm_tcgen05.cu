@@ -53,9 +53,10 @@ constexpr int kStagingBytes = 4096;  // 32 rows x 128 bytes, one epilogue chunk 
 #endif
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kBookBytes = 512 + 1024;   // barriers/bookkeeping + slack for manual 1024-byte alignment
-// LOW = 64 or 32: tiles of that many rows and 64 columns (launches of few rows; 0: the full 128).  The MMA still covers 128
-// rows, of which the others are whatever follows in shared memory; their rows of the accumulator are never read.
-// Their stages hold kGemmLowKBlocks k-blocks, fetched by one copy each (three-dimensional tensor maps).
+// LOW = 64 or 32: tiles of that many rows and 64 columns (the value projection of the first-token attention in batches of few
+// sequences; 0: the full 128).  The MMA still covers 128 rows, of which the others are whatever follows in shared memory; their rows
+// of the accumulator are never read.  Their stages hold kGemmLowKBlocks k-blocks, fetched by one copy each (three-dimensional tensor
+// maps), and their results go straight from registers to memory, without staging.
 __host__ __device__ constexpr int gemm_a_bytes(int low = 0) {
   return (low ? low * kGemmLowKBlocks : kGemmBlockM) * kGemmBlockK * 2;
 }
@@ -66,9 +67,8 @@ __host__ __device__ constexpr int gemm_b_bytes(int bn, bool pair, int low = 0) {
 __host__ __device__ constexpr int gemm_staging_bufs(int bn, bool pair, int epi, bool fp8) {
   return epi == kEpiBiasResidual ? 2 : (((bn == 256 && !pair) || gemm_epilogue_warps(bn, pair, epi, fp8) > 8) ? 1 : MT_GEMM_NBUF);
 }
-// Epilogue warps with rows to work on: all eight, or (LOW) those whose quarter of tensor memory the tile's rows reach.
 __host__ __device__ constexpr int gemm_staging_warps(int bn, bool pair, int epi, bool fp8, int low) {
-  return low ? 2 * (low / 32) : gemm_epilogue_warps(bn, pair, epi, fp8);
+  return low ? 0 : gemm_epilogue_warps(bn, pair, epi, fp8);
 }
 __host__ __device__ constexpr int gemm_stages(int bn, bool pair, int epi, bool fp8, int low = 0) {
   const int room = kSmemLimit - kBookBytes - gemm_staging_warps(bn, pair, epi, fp8, low) * gemm_staging_bufs(bn, pair, epi, fp8) * kStagingBytes;
@@ -90,13 +90,11 @@ __host__ __device__ constexpr int gemm_smem_bytes(int bn, bool pair, int epi, bo
 // FP8: the operands are E4M3 bytes with one fp32 scale per row of X and per row of W (GemmParams::scale_x,
 // scale_w); a shared-memory row of 128 bytes then holds 128 elements of K, an instruction covers 32 of them,
 // and the epilogue multiplies the accumulator by scale_x[row] * scale_w[column] before the bias.
-// LOW: tiles of 64 or 32 rows and 64 columns.  A launch of one or two row blocks is a chain of latencies: with 16 (12) KB a
-// k-block all twelve of K = 768 fit in the ring, so the whole operands are asked for at once; a stage is four k-blocks, so
-// that a copy, a wait and a commit are paid for three times and not twelve (each costs the issuing warp 100 to 200 clocks);
-// more CTAs share the launch; and X, which comes in at about 30 bytes per clock and CTA once the previous kernel has
-// ended (32 KB after 1.15 us, 96 KB after 2.3), is a half or a quarter of the full tile's.  128 rows of the eight-task tree:
-// accumulator complete 2.8 us after the dependency wait against 3.3 with 128-row tiles of the same width, results bf16
-// 0.6 us later (straight from registers) against 1.1 to 1.7.
+// LOW: tiles of 64 or 32 rows and 64 columns.  A launch of one or two row blocks is a chain of latencies: a stage is four k-blocks,
+// so that a copy, a wait and a commit are paid for a quarter as often (each costs the issuing warp 100 to 200 clocks); more CTAs
+// share the launch; and X, which comes in at about 30 bytes per clock and CTA once the previous kernel has ended (32 KB after
+// 1.15 us, 96 KB after 2.3), is a half or a quarter of the full tile's.  (128 rows, 64 columns, K = 768: accumulator complete 2.8 us
+// after the dependency wait against 3.3 with 128-row tiles of the same width, results 0.6 us later against 1.1 to 1.7.)
 template <int BN, int EPI, bool PAIR, bool FP8 = false, int LOW = 0>
 __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16_tcgen05(const __grid_constant__ GemmParams p) {
   static_assert(!FP8 || !PAIR, "the 8-bit operands run as single CTAs");
@@ -331,10 +329,9 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
     constexpr int CHUNK_COLS = (LOW || EPI == kEpiBiasResidual || EPI == kEpiBiasTanhF32 || EPI == kEpiPartialF32) ? 32 : 64;
     constexpr int CHUNKS = BN / CHUNK_COLS;
     const bool has_rows = LOW == 0 || quarter < LOW / 32;                // (LOW) the others only keep the barriers' counts
-    const int slot = LOW ? col_group * (LOW / 32) + quarter : e;         // (not used without rows)
-    const uint32_t my_stage = sStage + static_cast<uint32_t>(slot * NBUF * kStagingBytes);
+    const uint32_t my_stage = sStage + static_cast<uint32_t>(e * NBUF * kStagingBytes);
     const uint32_t my_res_bar = bar_res + 16 * e;       // two barriers, one per staging buffer
-    uint8_t* my_stage_ptr = smem + STAGES * (A_BYTES + B_BYTES) + slot * NBUF * kStagingBytes;
+    uint8_t* my_stage_ptr = smem + STAGES * (A_BYTES + B_BYTES) + e * NBUF * kStagingBytes;
     int acc = 0;
     uint32_t acc_phase = 0;
     int buf = 0;                  // staging buffer of the next chunk
@@ -358,7 +355,7 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
     // its present chunk has read it, so up to two requests are kept in flight: both chunks of a 128-wide tile
     // are asked for before the tile's main loop ends (at the kernel's start for a CTA's first tile) instead of
     // the second one only when the first is being worked on.
-    int req_tile = has_rows ? worker : total_tiles, req_chunk = col_group;   // the next chunk to ask for
+    int req_tile = worker, req_chunk = col_group;   // the next chunk to ask for
     int n_req = 0, n_done = 0;                      // chunks asked for / chunks whose store has been issued
     auto refill = [&]() {
       while (n_req < n_done + 2 && req_tile < total_tiles) {
@@ -382,7 +379,7 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
       const int out_row0 = m0 + quarter * 32 + (EPI == kEpiPartialF32 ? (rem_s % k_splits) * p.split_pitch : 0);
       // (LOW) the tile's bias - this warp has one chunk of 32 columns - is on its way while the MMAs run
       uint4 low_bias[LOW ? 4 : 1];
-      if (LOW && EPI != kEpiPartialF32 && has_rows) {
+      if (LOW && has_rows) {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
           low_bias[LOW ? q : 0] = __ldg(reinterpret_cast<const uint4*>(p.group[g].bias + n0 + col_group * 32) + q);
@@ -432,7 +429,7 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
           const uint4* bias4 = reinterpret_cast<const uint4*>(bias + col);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const uint4 b = LOW ? low_bias[LOW ? q : 0] : __ldg(bias4 + q);
+            const uint4 b = __ldg(bias4 + q);
             const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
             float4* s0 = reinterpret_cast<float4*>(sbuf + staging_off(lane, 2 * q));
             float4* s1 = reinterpret_cast<float4*>(sbuf + staging_off(lane, 2 * q + 1));
@@ -472,7 +469,7 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
           const uint4* bias4 = reinterpret_cast<const uint4*>(bias + col);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const uint4 b = LOW ? low_bias[LOW ? q : 0] : __ldg(bias4 + q);
+            const uint4 b = __ldg(bias4 + q);
             const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
             float4 r0, r1;
             r0.x = tanhf(__uint_as_float(v[q * 8 + 0]) + bf16_lo(bw[0]));
@@ -499,15 +496,8 @@ __global__ void __launch_bounds__(gemm_threads(BN, PAIR, EPI, FP8), 1) gemm_bf16
             const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
             uint32_t ow[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              float x0 = __uint_as_float(v[q * 8 + 2 * j]) + bf16_lo(bw[j]);
-              float x1 = __uint_as_float(v[q * 8 + 2 * j + 1]) + bf16_hi(bw[j]);
-              if (EPI == kEpiBiasGelu) {
-                x0 = gelu_fitted(x0);
-                x1 = gelu_fitted(x1);
-              }
-              ow[j] = pack_bf16(x0, x1);
-            }
+            for (int j = 0; j < 4; ++j)
+              ow[j] = pack_bf16(__uint_as_float(v[q * 8 + 2 * j]) + bf16_lo(bw[j]), __uint_as_float(v[q * 8 + 2 * j + 1]) + bf16_hi(bw[j]));
             if (row < m_rows) *reinterpret_cast<uint4*>(out + q * 8) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
           }
           continue;
@@ -652,7 +642,8 @@ int gemm_block_n(int N, int epilogue, int64_t rows, int groups, bool pair, int s
   if (epilogue == kEpiBiasTanhF32) return 128;
   if (epilogue == kEpiPartialF32) {
     // (`groups` counts the ranges of K too) 64-wide tiles while they all run at once, else 128-wide (measured at
-    // N = 768, K = 3072 in four ranges: 128 rows 5.4 against 6.0 us, 512 rows 8.8 against 6.7 us)
+    // N = 768, K = 3072 in four ranges: 128 rows 5.4 against 6.0 us, 512 rows 8.8 against 6.7 us).  A forward has turned tiles
+    // wherever the 64-wide ones would all run at once (gemm_choose_low): these are the single step's (mt_kernel_linear_partial).
     const int64_t tiles64 = ((rows + kGemmBlockM - 1) / kGemmBlockM) * (N / 64) * groups;
     return (N % 128 != 0 || tiles64 <= sm_count) ? 64 : 128;
   }
@@ -688,8 +679,8 @@ int gemm_block_n(int N, int epilogue, int64_t rows, int groups, bool pair, int s
 // 3 x 57 host to host 248 / 214, 209, 227; 4 x 128 458 / 443, 441, 445.)
 // Not turned, 64 or 32 rows x 64 columns: where the X of a column tile is its own (x_by_tile: a head's 64 columns).
 void gemm_choose_low(GemmParams* p, int groups, int sm_count) {
-  const int splits = p->k_splits > 1 ? p->k_splits : 1;
   if (p->x_by_tile == 0) {
+    const int splits = p->k_splits > 1 ? p->k_splits : 1;
     if (p->fp8 || p->N % 128 != 0 || p->K % (2 * kGemmBlockK * splits) != 0) return;
     for (int rows : {16, 32, 64}) {
       if (rows == 16 && p->M > 16) continue;
@@ -702,9 +693,9 @@ void gemm_choose_low(GemmParams* p, int groups, int sm_count) {
     }
     return;
   }
-  if (p->fp8 || p->N % 64 != 0 || p->K % (kGemmBlockK * kGemmLowKBlocks * splits * p->x_by_tile) != 0) return;
+  if (p->fp8 || p->N % 64 != 0 || p->K % (kGemmBlockK * kGemmLowKBlocks * p->x_by_tile) != 0) return;
   const int low = p->M <= 32 ? 32 : 64;
-  const int64_t tiles = static_cast<int64_t>((p->M + low - 1) / low) * (p->N / 64) * (groups < 1 ? 1 : groups) * splits;
+  const int64_t tiles = static_cast<int64_t>((p->M + low - 1) / low) * (p->N / 64) * (groups < 1 ? 1 : groups);
   if (tiles > sm_count) return;
   p->low = low;
   p->pair = 0;
@@ -736,9 +727,7 @@ cudaError_t launch_gemm(const GemmParams& p, int epilogue, int sm_count, cudaStr
     return cudaErrorInvalidValue;
   if (p.turned != 0) return launch_gemm_low(p, epilogue, stream);
   if (p.low != 0) {
-    if (p.pair || p.block_n != 64 || p.K % (kGemmBlockK * kGemmLowKBlocks * (p.k_splits > 1 ? p.k_splits : 1)) != 0)
-      return cudaErrorInvalidValue;
-    if (epilogue != kEpiBias) return cudaErrorInvalidValue;   // (the value projection of the first-token attention)
+    if (p.x_by_tile == 0 || epilogue != kEpiBias) return cudaErrorInvalidValue;   // (the value projection of the first-token attention)
     if (p.low == 64) return launch_one<64, kEpiBias, false, false, 64>(p, sm_count, stream);
     return p.low == 32 ? launch_one<64, kEpiBias, false, false, 32>(p, sm_count, stream) : cudaErrorInvalidValue;
   }

@@ -120,8 +120,8 @@ struct alignas(64) GemmParams {
   const int32_t* m_valid;  // device scalar: rows actually in use (<= M); null = all M rows
   int32_t pair;            // 1: run as pairs of CTAs on 256-row tiles (the W maps then fetch half a tile's rows)
   int32_t block_n;         // tile width along N: 128, 192 or 256 (gemm_block_n); N % block_n == 0
-  int32_t low;             // 64 or 32: tiles of that many rows (block_n 64, single CTAs, bf16); 0: 128.  The X and W maps are
-                           // then dims {64, rows, K / 64}, box {64, low | 64, kGemmLowKBlocks}
+  int32_t low;             // 64 or 32: tiles of that many rows (with x_by_tile and bf16 results; block_n 64, single CTAs); 0: 128.  The
+                           // X and W maps are then dims {64, rows, K / 64}, box {64, low | 64, kGemmLowKBlocks}
   int32_t turned;          // 64, 32 or 16: tiles of that many rows and 128 columns (launch_gemm_low; single CTAs, bf16); 0: not.  The X
                            // and W maps are then dims {64, rows, K / 64}, boxes {64, turned | 128, 2}
   int32_t x_by_tile;       // s = 1 or 2: column tile n (block_n 64) multiplies columns n K .. n K + K - 1 of X, which has N / 64 * K
