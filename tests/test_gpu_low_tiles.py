@@ -1,7 +1,7 @@
 """Forwards of few rows: GEMM tiles of 16, 32 and 64 rows taken transposed, the attention output with its LayerNorm on such tiles, the
-FFN-down projection as partial sums, a LayerNorm CTA per row.  Parity with the oracle at every hidden state where the sizes can go wrong: a single row, tiles just full and just begun, the last
-size before full tiles and the first after, and a hidden size of 1024 (more k-blocks than the ring of stages holds);
-and the same bits from run to run."""
+FFN-down projection as partial sums, a LayerNorm CTA per row.  Parity with the oracle at every hidden state where the sizes can go
+wrong: a single row, tiles just full and just begun, the last size before full tiles and the first after, and a hidden size of 1024
+(more k-blocks than the ring of stages holds); and the same bits from run to run."""
 import numpy as np
 import pytest
 import torch
