@@ -295,10 +295,11 @@ cudaError_t set_gemm_group(GemmParams* g, int i, int epilogue, const void* x, co
     if ((e = make_tmap(&g->tmap_x[i], x, M, x_cols, kGemmBlockM, kGemmBlockK, false)) != cudaSuccess) return e;
     if ((e = make_tmap(&g->tmap_w[i], w, N, w_cols, g->block_n / (g->pair != 0 ? 2 : 1), kGemmBlockK, false)) != cudaSuccess) return e;
   }
-  if ((e = make_tmap(&g->tmap_out[i], y, M, N, 32, gemm_out_box_cols(epilogue), f32_out)) != cudaSuccess) return e;
-  if (res && (e = make_tmap(&g->tmap_res[i], residual, M, N, 32, 32, true)) != cudaSuccess) return e;
   g->group[i].bias = bias;
   g->group[i].out = y;
+  if (g->turned != 0 || g->low != 0) return cudaSuccess;   // (the result and the residual by pointer)
+  if ((e = make_tmap(&g->tmap_out[i], y, M, N, 32, gemm_out_box_cols(epilogue), f32_out)) != cudaSuccess) return e;
+  if (res && (e = make_tmap(&g->tmap_res[i], residual, M, N, 32, 32, true)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 
@@ -878,8 +879,8 @@ cudaError_t add_to_tail(const mt_model* m, LayerTail* t, const LayerOffsets* lo,
                     static_cast<size_t>(i) * t->down_splits * pitch * m->trunk.hidden;
       if ((e = set_gemm_group(&t->ffn_down, i, kEpiPartialF32, f, w_ptr(m, lo->w2), nullptr, nullptr, part)) != cudaSuccess)
         return e;
-      if ((e = make_tmap(&t->ffn_down.tmap_out[i], part, static_cast<int>(t->down_splits * pitch), t->ffn_down.N, 32, 32,
-                         true)) != cudaSuccess)
+      if (t->ffn_down.turned == 0 && (e = make_tmap(&t->ffn_down.tmap_out[i], part, static_cast<int>(t->down_splits * pitch),
+                                                    t->ffn_down.N, 32, 32, true)) != cudaSuccess)
         return e;
       t->ln2.part[i] = part; t->ln2.residual[i] = h1_32; t->ln2.bias[i] = w_ptr(m, lo->b2);
       t->ln2.n_parts = t->down_splits; t->ln2.part_pitch = static_cast<int32_t>(pitch);
