@@ -219,7 +219,7 @@ int mt_plan_summary(const mt_model* m, uint64_t task_mask, int32_t* n_layers, in
                     int32_t* trunk_depth, int32_t* groups_per_wave);
 /* Kernel launches one mt_forward at batch = max_batch, seq = max_seq enqueues for this mask.  Before mt_bind_memory the
  * device is not known: the count is then that of the plan with options "qkv_attention" and "cls_pool" 0 and with
- * "fused_ln" 2 taken as fusing launches of one or two layers. */
+ * "fused_ln" 2 taken as fusing launches of one or two layers of more than 1024 rows together, and no others. */
 int mt_plan_launches(const mt_model* m, uint64_t task_mask, int32_t* n_launches);
 
 /* Launch plans currently cached (host side; no device access).  mt_forward keeps one plan per distinct
