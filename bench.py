@@ -43,8 +43,8 @@ L2_FLUSH_BYTES = 256 << 20    # larger than the 126 MB L2
 # launches of the forwards of `bench.py --steps 2`); the figure and the digest of the kernel sources it was
 # taken on are two lines of the launch-list summary under profiles/, and it is reported only while the
 # sources still have that digest.
-GEMM_SOURCES = ("gemm_tcgen05.cu", "gemm_ln_tcgen05.cu", "gemm_ln_pair_tcgen05.cu", "gemm_ln_low_tcgen05.cu", "gemm_low_tcgen05.cu", "gemm_low.cuh", "cluster_ptx.cuh", "tc_ptx.cuh",
-                "rowwise.cuh")
+GEMM_SOURCES = ("gemm_tcgen05.cu", "gemm_ln_tcgen05.cu", "gemm_ln_pair_tcgen05.cu", "gemm_ln_low_tcgen05.cu", "gemm_low_tcgen05.cu",
+                "gemm_low.cuh", "cluster_ptx.cuh", "tc_ptx.cuh", "rowwise.cuh")
 TRAFFIC_SUMMARY = os.path.join("profiles", "bench_glue8_b32_s128_launch_list.md")
 NOMINAL_BF16_TFLOPS = 2250.0   # dense bf16 of the part, for context beside the measured peak
 STEADY_SECONDS = 2.0
@@ -492,8 +492,9 @@ def main():
             "e2e": {"value": aggregate_throughput(world, BATCH, args.steps, e2e_s), "unit": UNIT,
                     "h2d_bytes_per_step": 2 * BATCH * SEQ * 4 + BATCH * 4,
                     "d2h_bytes_per_step": BATCH * cfg.total_classes * 4},
-            "roofline": {"bound": "tensor", "kernel": "gemm_bf16_tcgen05, gemm_ln_tcgen05 and gemm_ln_pair_tcgen05 (QKV, attention-out, FFN-up, "
-                                   "FFN-down launches; the last two include the LayerNorm after the residual GEMM)",
+            "roofline": {"bound": "tensor", "kernel": "gemm_bf16_tcgen05, gemm_low_tcgen05, gemm_ln_tcgen05, gemm_ln_pair_tcgen05 and gemm_ln_low_tcgen05 "
+                                   "(QKV, attention-out, FFN-up, FFN-down launches; the last three include the LayerNorm after the "
+                                   "residual GEMM)",
                          "flops": "valid tokens only; the last layer of each branch counts its attention-output and FFN maps on one token "
                                   "per sequence",
                          "achieved": achieved, "peak": peaks["tflops"], "unit": "TFLOP/s",

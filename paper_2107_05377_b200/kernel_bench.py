@@ -2,6 +2,7 @@
 
     python -m paper_2107_05377_b200.kernel_bench linear --m 4096 --n 2304 --k 768 --epilogue 0
     python -m paper_2107_05377_b200.kernel_bench linear_ln --m 4096 --n 768 --k 3072   # residual GEMM + LayerNorm, one launch
+    python -m paper_2107_05377_b200.kernel_bench linear --m 128 --tile-rows 32      # the tiles of launches of few rows (linear_ln too)
     python -m paper_2107_05377_b200.kernel_bench attention --batch 32 --seq 128 --heads 12
     python -m paper_2107_05377_b200.kernel_bench layernorm --rows 4096 --hidden 768
     python -m paper_2107_05377_b200.kernel_bench embed --batch 256 --seq 128
@@ -70,16 +71,20 @@ def _time(fn, iters, warmup, flush):
     return total / iters
 
 
-def bench_linear(m, n, k, epilogue, iters, warmup, flush):
+def bench_linear(m, n, k, epilogue, iters, warmup, flush, tile_rows=0):
     x = torch.randn(m, k, device="cuda").to(torch.bfloat16)
     w = (0.02 * torch.randn(n, k, device="cuda")).to(torch.bfloat16)
     b = (0.02 * torch.randn(n, device="cuda")).to(torch.bfloat16)
     r = torch.randn(m, n, device="cuda") if epilogue == 2 else None
     y = torch.empty(m, n, device="cuda", dtype=torch.float32 if epilogue == 2 else torch.bfloat16)
-    ms = _time(lambda: mt.mt_kernel_linear(x, w, b, r, y, epilogue, cta_pair=CTA_PAIR), iters, warmup, flush)
+    if tile_rows:
+        run = lambda: mt.mt_kernel_linear_low(x, w, b, r, y, epilogue, tile_rows)   # noqa: E731
+    else:
+        run = lambda: mt.mt_kernel_linear(x, w, b, r, y, epilogue, cta_pair=CTA_PAIR)   # noqa: E731
+    ms = _time(run, iters, warmup, flush)
     flops = 2.0 * m * n * k
     bytes_ = 2.0 * (m * k + n * k) + (8.0 if epilogue == 2 else 2.0) * m * n
-    return {"kernel": "linear", "M": m, "N": n, "K": k, "epilogue": epilogue, "us": 1e3 * ms,
+    return {"kernel": "linear", "tile_rows": tile_rows, "M": m, "N": n, "K": k, "epilogue": epilogue, "us": 1e3 * ms,
             "tflops": flops / ms / 1e9, "min_gbytes_per_s": bytes_ / ms / 1e6}
 
 
@@ -100,7 +105,7 @@ def bench_linear_fp8(m, n, k, epilogue, iters, warmup, flush):
             "tflops": 2.0 * m * n * k / ms / 1e9, "quantize_rows_us": 1e3 * ms_q}
 
 
-def bench_linear_ln(m, n, k, iters, warmup, flush, tile_cols=128):
+def bench_linear_ln(m, n, k, iters, warmup, flush, tile_cols=128, tile_rows=0):
     x = torch.randn(m, k, device="cuda").to(torch.bfloat16)
     w = (0.02 * torch.randn(n, k, device="cuda")).to(torch.bfloat16)
     b = (0.02 * torch.randn(n, device="cuda")).to(torch.bfloat16)
@@ -109,10 +114,14 @@ def bench_linear_ln(m, n, k, iters, warmup, flush, tile_cols=128):
     r = torch.randn(m, n, device="cuda")
     y = torch.empty(m, n, device="cuda", dtype=torch.bfloat16)
     y32 = torch.empty(m, n, device="cuda")
-    ms = _time(lambda: mt.mt_kernel_linear_layernorm(x, w, b, r, g, be, y, y32, 1e-12, tile_cols=tile_cols), iters, warmup, flush)
+    if tile_rows:
+        run = lambda: mt.mt_kernel_linear_layernorm_low(x, w, b, r, g, be, y, y32, 1e-12, tile_rows)   # noqa: E731
+    else:
+        run = lambda: mt.mt_kernel_linear_layernorm(x, w, b, r, g, be, y, y32, 1e-12, tile_cols=tile_cols)   # noqa: E731
+    ms = _time(run, iters, warmup, flush)
     flops = 2.0 * m * n * k
     bytes_ = 2.0 * (m * k + n * k) + (4.0 + 2.0 + 4.0) * m * n
-    return {"kernel": "linear_ln", "tile_cols": tile_cols, "M": m, "N": n, "K": k, "us": 1e3 * ms, "tflops": flops / ms / 1e9,
+    return {"kernel": "linear_ln", "tile_rows": tile_rows, "tile_cols": tile_cols, "M": m, "N": n, "K": k, "us": 1e3 * ms, "tflops": flops / ms / 1e9,
             "min_gbytes_per_s": bytes_ / ms / 1e6}
 
 
@@ -176,6 +185,7 @@ def main():
     ap.add_argument("--flush", action="store_true")
     ap.add_argument("--graph", action="store_true", help="replay the launches from a CUDA graph")
     ap.add_argument("--tile-cols", type=int, default=128, help="linear_ln: accumulator tile width, 128 or 256")
+    ap.add_argument("--tile-rows", type=int, default=0, help="linear, linear_ln: tiles of 16, 32 or 64 rows and 128 columns (0: full ones)")
     ap.add_argument("--block-n", type=int, default=0, help="linear: force the tile width (0 = automatic)")
     ap.add_argument("--pair", action="store_true", help="linear: pairs of CTAs on 256-row tiles (cta_group::2)")
     ap.add_argument("--mma-sync", action="store_true", help="attention: the mma.sync kernel also where seq <= 128")
@@ -187,11 +197,11 @@ def main():
     mt.lib().mt_kernel_linear_force_block_n(a.block_n)
     torch.manual_seed(0)
     if a.kernel == "linear":
-        print(json.dumps(bench_linear(a.m, a.n, a.k, a.epilogue, a.iters, a.warmup, a.flush)))
+        print(json.dumps(bench_linear(a.m, a.n, a.k, a.epilogue, a.iters, a.warmup, a.flush, a.tile_rows)))
     elif a.kernel == "linear_fp8":
         print(json.dumps(bench_linear_fp8(a.m, a.n, a.k, a.epilogue, a.iters, a.warmup, a.flush)))
     elif a.kernel == "linear_ln":
-        print(json.dumps(bench_linear_ln(a.m, a.n, a.k, a.iters, a.warmup, a.flush, a.tile_cols)))
+        print(json.dumps(bench_linear_ln(a.m, a.n, a.k, a.iters, a.warmup, a.flush, a.tile_cols, a.tile_rows)))
     elif a.kernel == "attention":
         print(json.dumps(bench_attention(a.batch, a.seq, a.heads, a.len_lo, a.iters, a.warmup, a.flush)))
     elif a.kernel == "layernorm":
