@@ -246,8 +246,7 @@ int64_t mt_replayed_forwards(const mt_model* m);
  * time): run GEMM launches as pairs of CTAs on 256-row tiles (tcgen05 cta_group::2, each CTA stages half
  * of a weight tile) instead of single CTAs on 128-row tiles; faster on large launches (+11 % at 8192^3),
  * slower on small ones; the results are bit-identical.  key "attention_tc" (0/1, default 1, any time): attention
- * for seq <= 128 runs on tcgen05 with its accumulators in tensor memory (1) or on mma.sync (0, also
- * used for every longer seq).  key "expected_tokens" (>= 0, default 0 = every row, any time): the caller's
+ * on all tokens runs on tcgen05 with its accumulators in tensor memory (1) or on mma.sync (0).  key "expected_tokens" (>= 0, default 0 = every row, any time): the caller's
  * estimate of the valid tokens per batch; with the packed layout the GEMM kernels and tile widths are chosen for
  * that many rows instead of batch*seq; it never changes a result.
  * key "fp8_gemm" (0/1, default 0; before mt_bind_memory, it enlarges both arenas): reduced precision in the

@@ -343,7 +343,7 @@ struct mt_model {
   int64_t expected_tokens;  // caller's estimate of the valid tokens per batch (0 = every row); tunes tile shapes only
   bool qkv_attention; // Q/K/V projection and attention of layers on all tokens in one launch where it applies (use_qkv_attention)
   bool cls_pool;      // first-token attention without projecting keys and values (use_cls_pool)
-  bool attention_tc;  // attention on tcgen05 with tensor-memory accumulators when seq <= 128 (else mma.sync)
+  bool attention_tc;  // attention on all tokens on tcgen05 with tensor-memory accumulators (else mma.sync)
   int32_t gemm_pair;  // GEMMs as pairs of CTAs on 256-row tiles (cta_group::2): 0 never, 1 always, 2 by launch size
   bool early_heads;  // every task's head (and first-token tail) runs right after the wave that finishes its branch
   int32_t fused_ln;  // each residual GEMM and the LayerNorm after it as one cluster launch: 0 never, 1 always on
