@@ -11,7 +11,7 @@
  *
  * Conventions
  *  - The device memory that a forward works in belongs to the caller.  The library allocates host metadata; what it
- *    has the driver create - two streams and two events in mt_bind_memory, events with option "profile", and CUDA
+ *    has the driver create - a stream and two events in mt_bind_memory, events with option "profile", and CUDA
  *    graphs unless option "replay" is 0 - takes the driver device memory of its own (see mt_forward).
  *    Pointers named d_* are DEVICE pointers, everything else is a HOST pointer.
  *  - cudaStream_t is passed as a plain `void*` (the value of the stream handle; NULL = default stream).
@@ -150,7 +150,7 @@ int mt_adopt_weights(mt_model* m, const mt_model* src);
  * from every softmax; the pooler reads position 0.  Asynchronous: only enqueues kernels on `stream`,
  * never synchronises, never allocates device memory of its own.  The first call for a given
  * (batch, seq, task_mask) builds and caches a launch plan on the host (host memory and tensor-map
- * encoding only; the model's own streams and its two events exist since mt_bind_memory) - make one
+ * encoding only; the model's own stream and its two events exist since mt_bind_memory) - make one
  * warm-up call before capturing mt_forward into a CUDA graph.  Option "profile" creates CUDA events here.
  * A plan that has been launched 32 times is made a CUDA graph by the next call (0.2 to 1 ms of the host, once) and
  * replayed from then on with the pointers of each call - not while `stream` is being captured, nor with task_events

@@ -27,6 +27,47 @@ using namespace mt;
 
 namespace mt {
 bool g_use_pdl = true;
+thread_local GraphRecorder* t_recorder = nullptr;
+
+cudaError_t GraphRecorder::add(const void* kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const void* param,
+                               unsigned cluster_x, bool programmatic) {
+  void* args[1] = {const_cast<void*>(param)};
+  cudaKernelNodeParams p = {};
+  p.func = const_cast<void*>(kernel);
+  p.gridDim = grid;
+  p.blockDim = block;
+  p.sharedMemBytes = static_cast<unsigned>(smem);
+  p.kernelParams = args;
+  cudaGraphNode_t node = nullptr;
+  cudaError_t e = cudaGraphAddKernelNode(&node, graph, nullptr, 0, &p);
+  if (e != cudaSuccess) return e;
+  if (cluster_x > 1) {
+    cudaLaunchAttributeValue v = {};
+    v.clusterDim.x = cluster_x;
+    v.clusterDim.y = v.clusterDim.z = 1;
+    if ((e = cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributeClusterDimension, &v)) != cudaSuccess) return e;
+  }
+  Front& f = front[side != nullptr && stream == side ? 1 : 0];
+  for (cudaGraphNode_t before : f.after) {
+    cudaGraphEdgeData edge = {};
+    if (programmatic && f.alone) {
+      edge.from_port = cudaGraphKernelNodePortProgrammatic;   // (when all its CTAs have let their dependents start)
+      edge.type = cudaGraphDependencyTypeProgrammatic;
+    }
+    if ((e = cudaGraphAddDependencies_v2(graph, &before, &node, &edge, 1)) != cudaSuccess) return e;
+  }
+  f.after.assign(1, node);
+  f.alone = true;
+  last_node = node;
+  last_launch = p;
+  last_launch.kernelParams = nullptr;
+  return cudaSuccess;
+}
+void GraphRecorder::Front::wait_for(const Front& other) {
+  for (cudaGraphNode_t n : other.after)
+    if (std::find(after.begin(), after.end(), n) == after.end()) after.push_back(n);
+  alone = false;
+}
 }
 static int g_force_block_n = 0;   // tile width forced on mt_kernel_linear (tuning aid), 0 = chosen by gemm_block_n
 
@@ -357,7 +398,6 @@ struct mt_model {
   bool overlap_cls;
   cudaStream_t side_stream;
   bool replay;                  // option "replay": forwards of a plan in frequent use run as a CUDA graph
-  cudaStream_t replay_stream;   // where a forward is recorded as a graph
   int64_t replayed;             // forwards that ran as one
   cudaEvent_t ev_fork, ev_join;
   bool fp8;          // Q/K/V, FFN-up and FFN-down projections on E4M3 operands (set before mt_bind_memory)
@@ -1349,7 +1389,7 @@ int mt_create(const mt_trunk_config* trunk, const mt_task_config* tasks, int32_t
   m->expected_tokens = 0;
   m->pool_gemm = true;
   m->overlap_cls = true;
-  m->side_stream = m->replay_stream = nullptr;
+  m->side_stream = nullptr;
   m->replay = true;
   m->replayed = 0;
   m->ev_fork = m->ev_join = nullptr;
@@ -1417,7 +1457,6 @@ void mt_destroy(mt_model* m) {
   if (m->ev_fork != nullptr) cudaEventDestroy(m->ev_fork);
   if (m->ev_join != nullptr) cudaEventDestroy(m->ev_join);
   if (m->side_stream != nullptr) cudaStreamDestroy(m->side_stream);
-  if (m->replay_stream != nullptr) cudaStreamDestroy(m->replay_stream);
   delete m;
 }
 
@@ -1583,7 +1622,6 @@ int mt_bind_memory(mt_model* m, void* d_weights, size_t weights_bytes, void* d_w
   // that a forward never creates anything
   if (m->side_stream == nullptr) {
     if ((e = cudaStreamCreateWithFlags(&m->side_stream, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaStreamCreateWithFlags(&m->replay_stream, cudaStreamNonBlocking)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&m->ev_fork, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming)) != cudaSuccess)
       return fail_cuda(m, e, "creating the side stream");
@@ -1692,9 +1730,11 @@ int mt_plan_launches(const mt_model* m, uint64_t task_mask, int32_t* n_launches)
   return MT_OK;
 }
 
-// Enqueues the kernels of a plan one by one; with `nodes` (the stream is being captured) notes those that take pointers of the call.
+// Enqueues the kernels of a plan one by one, or (`nodes`: this thread records) adds them to a graph and notes those that take pointers of
+// the call.
 static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch, int32_t seq, void* const* task_events,
                        cudaStream_t stream, std::vector<ReplayNode>* nodes) {
+  GraphRecorder* const recorder = t_recorder;   // (with `nodes`)
   uint32_t* status = reinterpret_cast<uint32_t*>(m->d_workspace + m->ws_status);
   const size_t act_used = static_cast<size_t>(batch) * seq * m->trunk.hidden * sizeof(bf16);
   cudaError_t e;
@@ -1750,19 +1790,13 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
   int32_t* row_start = reinterpret_cast<int32_t*>(m->d_workspace + m->ws_row_start);
   const bool fused_qkv = use_qkv_attention(m, static_cast<int64_t>(batch) * seq, seq);
   // (a forward being recorded for replay: the kernels that take pointers of the call)
-  auto note = [&](ReplayNode::Kind kind, size_t step, const RowStartsParams& rs, const EmbedParams& em) -> cudaError_t {
-    if (nodes == nullptr) return cudaSuccess;
+  auto note = [&](ReplayNode::Kind kind, size_t step, const RowStartsParams& rs, const EmbedParams& em) {
+    if (nodes == nullptr) return;
     ReplayNode n;
     n.kind = kind; n.step = step; n.row_starts = rs; n.embed = em;
-    cudaStreamCaptureStatus state;
-    const cudaGraphNode_t* last = nullptr;
-    size_t count = 0;
-    cudaError_t err = cudaStreamGetCaptureInfo_v3(stream, &state, nullptr, nullptr, &last, nullptr, &count);
-    if (err != cudaSuccess) return err;
-    if (state != cudaStreamCaptureStatusActive || count != 1) return cudaErrorUnknown;
-    n.node = last[0];
+    n.node = recorder->last_node;
+    n.launch = recorder->last_launch;
     nodes->push_back(n);
-    return cudaSuccess;
   };
   RowStartsParams rs = {};
   EmbedParams ep = {};
@@ -1773,7 +1807,7 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
   rs.n_windows = fused_qkv ? window_count(m) : nullptr;
   rs.windows = fused_qkv ? window_list(m) : nullptr;
   MT_LAUNCH(launch_row_starts(rs, stream), "row-start kernel");
-  MT_LAUNCH(note(ReplayNode::kRowStarts, 0, rs, ep), "recording the forward");
+  note(ReplayNode::kRowStarts, 0, rs, ep);
   ep.row_start = row_start;
   ep.row_info = fused_qkv ? row_info(m) : nullptr;
   ep.packed = m->pack_tokens ? 1 : 0;
@@ -1785,17 +1819,32 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
   ep.batch = batch; ep.seq = seq; ep.hidden = m->trunk.hidden; ep.vocab = m->trunk.vocab_size;
   ep.type_vocab = m->trunk.type_vocab; ep.eps = m->trunk.ln_eps; ep.status = status;
   MT_TIMED(MT_CLASS_EMBED, launch_embed(ep, stream), "embedding kernel");
-  MT_LAUNCH(note(ReplayNode::kEmbed, 0, rs, ep), "recording the forward");
+  note(ReplayNode::kEmbed, 0, rs, ep);
   if (m->debug_capture)
     MT_LAUNCH(cudaMemcpyAsync(m->d_workspace + m->ws_dump0, ep.out, act_used, cudaMemcpyDeviceToDevice, stream),
               "debug capture");
 
+  // the side stream waits for what is enqueued on the caller's so far; its work so far is what the caller's stream then waits for
+  auto fork_side = [&]() -> cudaError_t {
+    if (recorder != nullptr) {
+      recorder->fork();
+      return cudaSuccess;
+    }
+    const cudaError_t err = cudaEventRecord(m->ev_fork, stream);
+    return err != cudaSuccess ? err : cudaStreamWaitEvent(m->side_stream, m->ev_fork, 0);
+  };
+  auto side_done = [&]() { return recorder != nullptr ? cudaSuccess : cudaEventRecord(m->ev_join, m->side_stream); };
+  auto join_side = [&]() -> cudaError_t {
+    if (recorder == nullptr) return cudaStreamWaitEvent(stream, m->ev_join, 0);
+    recorder->join();
+    return cudaSuccess;
+  };
   bool pool_pending = false;   // ... of a step of kind 4: waited for before the first-token tails
   bool side_pending = false;   // work on the side stream that the caller's stream has not waited for yet
   for (size_t step = 0; step < plan.steps.size(); ++step) {
     PlanStep& st = plan.steps[step];
     if (side_pending || (pool_pending && st.kind == 2)) {
-      MT_LAUNCH(cudaStreamWaitEvent(stream, m->ev_join, 0), "joining the side stream");
+      MT_LAUNCH(join_side(), "joining the side stream");
       side_pending = pool_pending = false;
     }
     if (st.kind == 0) {
@@ -1807,10 +1856,9 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
       if (ck.qkv.n_groups > 0)
         MT_TIMED(MT_CLASS_QKV, launch_gemm(ck.qkv, kEpiBias, m->sm_count, stream), "QKV GEMM");
       if (beside) {
-        MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
-        MT_LAUNCH(cudaStreamWaitEvent(m->side_stream, m->ev_fork, 0), "forking the side stream");
+        MT_LAUNCH(fork_side(), "forking the side stream");
         MT_LAUNCH(launch_cls_attention(ck.attn_cls, m->side_stream), "first-token attention kernel");
-        MT_LAUNCH(cudaEventRecord(m->ev_join, m->side_stream), "joining the side stream");
+        MT_LAUNCH(side_done(), "joining the side stream");
         side_pending = true;
       }
       if (ck.full.count > 0 && !ck.fused_qkv) MT_TIMED(MT_CLASS_ATTENTION, launch_attention(ck.attn, stream), "attention kernel");
@@ -1825,15 +1873,12 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
     } else if (st.kind == 4) {
       const bool beside = st.beside && m->overlap_cls && m->side_stream != nullptr && !m->profile;
       cudaStream_t on = beside ? m->side_stream : stream;
-      if (beside) {
-        MT_LAUNCH(cudaEventRecord(m->ev_fork, stream), "forking the side stream");
-        MT_LAUNCH(cudaStreamWaitEvent(on, m->ev_fork, 0), "forking the side stream");
-      }
+      if (beside) MT_LAUNCH(fork_side(), "forking the side stream");
       MT_TIMED(MT_CLASS_ATTENTION, launch_cls_query(*st.cls_pool, on), "first-token query kernel");
       MT_TIMED(MT_CLASS_ATTENTION, launch_cls_pool(*st.cls_pool, on), "first-token pooling kernel");
       MT_TIMED(MT_CLASS_ATTENTION, launch_gemm(*st.cls_v, kEpiBias, m->sm_count, on), "first-token value projection");
       if (beside) {
-        MT_LAUNCH(cudaEventRecord(m->ev_join, on), "joining the side stream");
+        MT_LAUNCH(side_done(), "joining the side stream");
         pool_pending = true;
       }
     } else if (st.kind == 2) {
@@ -1847,13 +1892,13 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
       if (st.kind == 3) {
         st.token_heads.logits = call.token_logits;
         MT_TIMED(MT_CLASS_HEAD, launch_token_heads(st.token_heads, stream), "token-level head kernel");
-        MT_LAUNCH(note(ReplayNode::kTokenHead, step, rs, ep), "recording the forward");
+        note(ReplayNode::kTokenHead, step, rs, ep);
       } else {
         st.heads.logits = call.logits;
         if (st.pool != nullptr) MT_TIMED(MT_CLASS_HEAD, launch_gemm(*st.pool, kEpiBiasTanhF32, m->sm_count, stream), "pooler GEMM");
         else MT_TIMED(MT_CLASS_HEAD, launch_pooler(st.heads, stream), "pooler kernel");
         MT_TIMED(MT_CLASS_HEAD, launch_head(st.heads, stream), "head kernel");
-        MT_LAUNCH(note(ReplayNode::kHead, step, rs, ep), "recording the forward");
+        note(ReplayNode::kHead, step, rs, ep);
       }
       if (task_events != nullptr)
         for (int32_t t : st.head_tasks)
@@ -1861,7 +1906,7 @@ static int launch_plan(mt_model* m, Plan& plan, const Call& call, int32_t batch,
             MT_LAUNCH(cudaEventRecord(reinterpret_cast<cudaEvent_t>(task_events[t]), stream), "recording a task event");
     }
   }
-  if (side_pending || pool_pending) MT_LAUNCH(cudaStreamWaitEvent(stream, m->ev_join, 0), "joining the side stream");
+  if (side_pending || pool_pending) MT_LAUNCH(join_side(), "joining the side stream");
 #undef MT_TAIL
 #undef MT_TIMED
 #undef MT_LAUNCH
@@ -1876,16 +1921,19 @@ static void build_replay(mt_model* m, Plan& plan, const Call& call, int32_t batc
   r.pdl = g_use_pdl;
   const CaptureLeave leave;
   if (!leave.ok) return;
-  cudaError_t e = cudaStreamBeginCapture(m->replay_stream, cudaStreamCaptureModeRelaxed);
+  cudaError_t e = cudaGraphCreate(&r.graph, 0);
   if (e == cudaSuccess) {
+    struct Recording {
+      GraphRecorder recorder;
+      Recording() { t_recorder = &recorder; }
+      ~Recording() { t_recorder = nullptr; }
+    } recording;
+    recording.recorder.graph = r.graph;
+    recording.recorder.side = m->side_stream;
     const std::string before = m->last_error;
-    if (launch_plan(m, plan, call, batch, seq, nullptr, m->replay_stream, &r.nodes) != MT_OK) e = cudaErrorUnknown;
+    if (launch_plan(m, plan, call, batch, seq, nullptr, nullptr, &r.nodes) != MT_OK) e = cudaErrorUnknown;
     m->last_error = before;
-    const cudaError_t ended = cudaStreamEndCapture(m->replay_stream, &r.graph);
-    if (e == cudaSuccess) e = ended;
   }
-  for (ReplayNode& n : r.nodes)
-    if (e == cudaSuccess) e = cudaGraphKernelNodeGetParams(n.node, &n.launch);
   if (e == cudaSuccess) e = cudaGraphInstantiate(&r.exec, r.graph, 0);
   if (e != cudaSuccess) cudaGetLastError();
   r.call = call;
@@ -1994,7 +2042,7 @@ int mt_forward_tokens(mt_model* m, const int32_t* d_token_ids, const int32_t* d_
   plan.last_use = ++m->use_clock;
   const Call call = {d_token_ids, d_segment_ids, d_lengths, d_logits, d_token_logits};
   // Replayed: plans in frequent use, on a stream that is not being captured, without anything recorded between the launches.
-  bool replay = m->replay && m->replay_stream != nullptr && task_events == nullptr && !m->profile && !m->debug_capture;
+  bool replay = m->replay && task_events == nullptr && !m->profile && !m->debug_capture;
   if (replay && (plan.replay == nullptr || !plan.replay->refused)) {
     cudaStreamCaptureStatus state = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &state) != cudaSuccess) {

@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include <mutex>
+#include <vector>
 
 namespace mt {
 
@@ -59,10 +60,34 @@ cudaError_t per_device_once(PerDeviceOnce& state, F&& setup, int* device_out = n
   return cudaSuccess;
 }
 
-// cluster_x > 1 launches the grid as thread-block clusters of that many CTAs along x.
+// Collects the launches of a forward as kernel nodes of a CUDA graph, in the order of their streams: the caller's and one
+// beside it, which fork() and join() tie together as events would.  Built node by node and not by capturing a stream: while any
+// stream of a process is being captured, a cudaDeviceSynchronize of another thread fails.
+struct GraphRecorder {
+  cudaGraph_t graph = nullptr;
+  cudaStream_t side = nullptr;
+  // what the next kernel of a stream waits for; alone: it is the kernel before it in the stream and nothing else
+  struct Front {
+    std::vector<cudaGraphNode_t> after;
+    bool alone = false;
+    void wait_for(const Front& other);
+  } front[2];
+  cudaGraphNode_t last_node = nullptr;
+  cudaKernelNodeParams last_launch = {};   // (but kernelParams)
+  cudaError_t add(const void* kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const void* param, unsigned cluster_x,
+                  bool programmatic);
+  void fork() { front[1].wait_for(front[0]); }   // the stream beside waits for what the caller's has so far
+  void join() { front[0].wait_for(front[1]); }
+};
+// Set while this thread records a forward (GraphRecorder instead of the stream).
+extern thread_local GraphRecorder* t_recorder;
+
+// cluster_x > 1 launches the grid as thread-block clusters of that many CTAs along x; programmatic: see g_use_pdl.
 template <typename Param>
 cudaError_t launch_kernel(void (*kernel)(Param), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                          const Param& param, unsigned cluster_x = 1) {
+                          const Param& param, unsigned cluster_x = 1, bool programmatic = true) {
+  if (t_recorder != nullptr)
+    return t_recorder->add(reinterpret_cast<const void*>(kernel), grid, block, smem, stream, &param, cluster_x, programmatic && g_use_pdl);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -70,7 +95,7 @@ cudaError_t launch_kernel(void (*kernel)(Param), dim3 grid, dim3 block, size_t s
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   unsigned n = 0;
-  if (g_use_pdl) {
+  if (programmatic && g_use_pdl) {
     attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[n].val.programmaticStreamSerializationAllowed = 1;
     ++n;

@@ -472,8 +472,7 @@ cudaError_t launch_row_starts(const RowStartsParams& p, cudaStream_t stream) {
   if (p.batch < 1 || p.seq < 1 || p.lengths == nullptr || p.lengths_copy == nullptr ||
       (p.windows != nullptr && (p.n_windows == nullptr || p.packed == 0 || p.seq > kWindowRows)))
     return cudaErrorInvalidValue;
-  row_starts_kernel<<<1, 32, 0, stream>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(row_starts_kernel, dim3(1), dim3(32), 0, stream, p, 1, false);   // (whatever came before has completed)
 }
 
 cudaError_t launch_unpack_rows(const bf16* packed, const int32_t* lengths, const int32_t* row_start, bf16* padded,

@@ -1,6 +1,7 @@
 """Forwards of a plan in frequent use run as a CUDA graph (option "replay"): the same bits as launched kernels, with the pointers of
 each call, whatever comes between the calls - and they do run as one, from the call on that the plan has been launched often enough."""
 import ctypes as C
+import threading
 
 import pytest
 import torch
@@ -136,6 +137,37 @@ def test_a_callers_capture_outlives_what_becomes_of_graphs_meanwhile():
     graph.replay()
     assert same(outs[3], want[0]) and same(out_short[1], want_short)
     assert often.poll_status() == 0
+
+
+def test_graphs_are_built_beside_a_thread_that_waits_for_the_device():
+    """A wait for the whole device fails while any stream is being captured, so a graph is not built by capturing one."""
+    cfg = synth.config_tiny()
+    _, blob, _ = cached_weights(cfg, 0)
+    model = mt.MTModel(cfg, 1, 24)
+    model.load_weights(blob)
+    ids = [dev_batch(synth.make_batch(cfg, 1, S, S, S, seed=S)) for S in range(1, 25)]
+    out = torch.zeros(1, cfg.total_classes, device="cuda")
+    errors, waits, done = [], [0], threading.Event()
+
+    def wait():
+        try:
+            while not done.is_set():
+                torch.cuda.synchronize()
+                waits[0] += 1
+        except Exception as e:   # noqa: BLE001
+            errors.append(e)
+    thread = threading.Thread(target=wait)
+    thread.start()
+    for rep in range(4):
+        for one in ids:
+            for _ in range(LAUNCHED + 1):
+                model.forward(*one, out)
+        assert model.replayed_forwards() == (rep + 1) * len(ids)
+        model.set_option("replay", 1)        # (drops the plans: the graphs are built anew)
+    done.set()
+    thread.join()
+    assert not errors and waits[0] > 0
+    assert model.poll_status() == 0
 
 
 def test_a_model_has_at_most_32_graphs():
