@@ -152,12 +152,12 @@ int mt_adopt_weights(mt_model* m, const mt_model* src);
  * (batch, seq, task_mask) builds and caches a launch plan on the host (host memory and tensor-map
  * encoding only; the model's own stream and its two events exist since mt_bind_memory) - make one
  * warm-up call before capturing mt_forward into a CUDA graph.  Option "profile" creates CUDA events here.
- * A plan that has been launched 32 times is made a CUDA graph by the next call (0.2 to 1 ms of the host, once) and
- * replayed from then on with the pointers of each call - not while `stream` is being captured, nor with task_events
- * or options "profile" and "debug_capture".  The driver keeps a graph in device memory (some 0.7 MB for 67 launches),
- * of at most 32 graphs per model, and holds it for later ones when they are dropped.  A caller that has handed out all
- * device memory, or wants no such call, sets option "replay" to 0: no graph is ever built.  If one cannot be built
- * the kernels are launched as before.
+ * A plan that has been launched 32 times is made a CUDA graph by the next call (0.2 to 1 ms of the host, once; up to
+ * 4 ms the first time in a process) and replayed from then on with the pointers of each call - not while `stream` is
+ * being captured, nor with task_events or options "profile" and "debug_capture".  The driver keeps a graph in device
+ * memory (some 0.6 MB for 67 launches), of at most 32 graphs per model, and holds it for later ones when they are
+ * dropped.  A caller that has handed out all device memory, or wants no such call, sets option "replay" to 0: no graph
+ * is ever built.  If one cannot be built the kernels are launched as before.
  * One mt_model serves one caller at a time: the cached plans carry per-call pointers.
  * Errors: INVALID_ARG, SHAPE, NOT_BOUND, NOT_LOADED, CUDA. */
 int mt_forward(mt_model* m, const int32_t* d_token_ids, const int32_t* d_segment_ids,

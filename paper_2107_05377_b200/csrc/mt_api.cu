@@ -83,13 +83,13 @@ constexpr size_t split_pitch(size_t rows) { return (rows + 127) / 128 * 128; }
 constexpr int32_t kDownSplits = 4;
 // "Few rows": at most this many per layer (batch 4 x 128 tokens; the first-token tails of batches up to 512).
 constexpr int32_t kSplitRowsMax = 512;
-// A plan is made a graph when it has been launched this often.  Building one and its first replay take 0.3 ms more than launching (34
-// launches: 2 x 32 tokens), 0.4 to 0.55 (46 to 77) or 1.05 (117), twice that the first time in a process; a replay saves 11 us of a
-// forward of 34 launches, 24 of 67 (1 x 128), 33 (32 x 128), 44 of 117.  That is 16 to 36 forwards: a plan that has been launched
-// as often will have cost at most about twice what the better of both ways would have, however soon it falls out of use.
+// A plan is made a graph when it has been launched this often.  Building one and its first replay take 0.25 ms more than launching
+// (34 launches: 2 x 32 tokens), 0.35 to 0.6 (46 to 77) or 1.03 (117), the first time in a process 1 to 4 ms; a replay saves 10 us of
+// a forward of 34 launches, 24 of 67 (1 x 128), 35 (32 x 128), 50 of 117.  That is 14 to 27 forwards: a plan that has been launched
+// as often will have cost hardly more than twice what the better of both ways would have, however soon it falls out of use.
 constexpr int32_t kReplayAfter = 32;
-// Graphs of a model at a time, whatever option "plan_cache" says: the driver keeps each of them in device memory, some 0.7 MB of it
-// for 67 launches (62 graphs: 45 MB, kept for the next ones when they are dropped).
+// Graphs of a model at a time, whatever option "plan_cache" says: the driver keeps each of them in device memory, some 0.6 MB of it
+// for 67 launches, and what dropped ones had for later ones (18 MB after 62 shapes).
 constexpr int32_t kMaxReplays = 32;
 
 inline size_t pad256(size_t n) { return (n + kAlign - 1) / kAlign * kAlign; }
